@@ -122,7 +122,7 @@ extern "C" int32_t dg_mesh_create(int64_t nv, const double *xy, int64_t nt, cons
   *out = nullptr;
   HostMesh hm;
   std::string msg;
-  const int32_t rc = build_host_mesh(nv, xy, nt, tri, canon, bc, TPB, hm, msg);
+  const int32_t rc = build_host_mesh(nv, xy, nt, tri, canon, bc, tile_cells(DG_PREC_FP64), hm, msg);
   if (rc != DG_OK) return fail(rc, "%s", msg.c_str());
   auto m = new (std::nothrow) dg_mesh();
   if (!m) return fail(DG_ENOMEM, "host allocation failed");
@@ -135,7 +135,7 @@ extern "C" int32_t dg_mesh_create(int64_t nv, const double *xy, int64_t nt, cons
   m->vxy_host = std::move(hm.vxy);
   const std::vector<int32_t> &conn = hm.conn, &e_cell = hm.e_cell, &etile = hm.etile, &cedge = hm.cedge;
   const std::vector<int8_t> &e_loc = hm.e_loc;
-  const int64_t ntiles = num_blocks(nt);
+  const int64_t ntiles = num_tiles(nt, DG_PREC_FP64);   // the edge ranges serve the FP64 form
   if ((int64_t)etile.size() != ntiles + 1) { delete m; return fail(DG_EINVAL, "tile count mismatch"); }
   m->ne = (int64_t)e_cell.size();
   double *part = nullptr, *mins = nullptr;
@@ -170,7 +170,7 @@ extern "C" int32_t dg_mesh_create(int64_t nv, const double *xy, int64_t nt, cons
   MTRY(cudaMemcpy(m->e_loc, e_loc.data(), m->ne, cudaMemcpyHostToDevice));
   MTRY(cudaMemcpy(m->etile, etile.data(), sizeof(int32_t) * (ntiles + 1), cudaMemcpyHostToDevice));
   MTRY(cudaMemcpy(m->cedge, cedge.data(), sizeof(int32_t) * 3 * nt, cudaMemcpyHostToDevice));
-  MTRY(dalloc(&part, 4 * num_blocks(nt)));
+  MTRY(dalloc(&part, 4 * ((nt + TPB - 1) / TPB)));
   MTRY(dalloc(&mins, 4));
   MTRY(cudaMemcpy(m->vxy, m->vxy_host.data(), sizeof(double) * 6 * nt, cudaMemcpyHostToDevice));
   MTRY(cudaMemcpy(m->conn, conn.data(), sizeof(int32_t) * 3 * nt, cudaMemcpyHostToDevice));
@@ -399,7 +399,7 @@ extern "C" int32_t dg_init(const dg_mesh *mesh, const dg_config *cfg, const doub
   const int64_t nt = mesh->nt;
   const int nq = cfg->k + 1;
   const size_t rs = real_size(s);
-  const int64_t nblk = num_blocks(nt);
+  const int64_t nblk = num_tiles(nt, cfg->precision);
   int32_t rc = DG_OK;
   cudaError_t e = cudaSuccess;
 #define STRY(x)                                                                                          \
@@ -418,7 +418,7 @@ extern "C" int32_t dg_init(const dg_mesh *mesh, const dg_config *cfg, const doub
   STRY(alloc_state(s, &s->uh));
   STRY(alloc_state(s, &s->us));
   const int64_t xc = uses_exchange(cfg->precision) ? nt : 1;   // exchange buffers: FP64 form only
-  STRY(cudaMalloc(&s->tr, rs * xc * 3 * nq * trace_stride(cfg->precision)));
+  STRY(cudaMalloc(&s->tr, rs * xc * 3 * nq * TR_STRIDE));
   STRY(cudaMalloc(&s->vd, rs * xc * VD_CELL));
   STRY(cudaMalloc(&s->hs, rs * xc * 12));
   STRY(cudaMalloc(&s->ej, rs * (uses_exchange(cfg->precision) ? std::max<int64_t>(mesh->ne, 1) : 1) * EJ_STRIDE));

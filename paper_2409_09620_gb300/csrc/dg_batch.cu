@@ -363,7 +363,7 @@ struct BatchCore {
       d.k = c.k;
       d.oe = c.phys.oe;
       d.bp = c.phys.bp;
-      d.ntiles = num_blocks(c.mesh.nt);
+      d.ntiles = num_tiles(c.mesh.nt, prec);
       host_sv.push_back(d);
     }
     if (host_sv.size() > sv_cap) {
@@ -377,7 +377,7 @@ struct BatchCore {
       return set_error(DG_ECUDA, "solve table upload");
     if (auto_chunk) {
       int64_t tiles = 0;
-      for (const SolveDev &d : host_sv) tiles += d.ntiles;
+      for (const SolveDev &d : host_sv) tiles += d.ntiles * tile_cells(prec) / TPB;   // of TPB cells
       const int64_t resident = (int64_t)num_sms * std::max(1, max_blocks_per_sm(form));
       int tpw = 1;
       while (tpw < 8 && tiles / (2 * tpw) >= 2 * resident) tpw *= 2;
@@ -395,7 +395,7 @@ struct BatchCore {
     if (max_blocks_per_sm(launch_form) < 1)
       return set_error(DG_EINVAL, "the device does not support cooperative launches");
     std::vector<WorkItem> work;
-    const int64_t tpw = cells_per_block / TPB;
+    const int64_t tpw = cells_per_block / tile_cells(prec);
     for (size_t i = 0; i < host_sv.size(); ++i)
       for (int64_t t = 0; t < host_sv[i].ntiles; t += tpw)
         work.push_back(WorkItem{(int)i, 0, t, std::min<int64_t>(tpw, host_sv[i].ntiles - t)});
@@ -665,7 +665,7 @@ extern "C" int32_t dg_batch_autotune(dg_batch *b, int32_t steps, int32_t *best_c
     StateBuf un, uh, us;
     solver_states(s, &un, &uh, &us);
     Snap &q = snaps[i];
-    const size_t ntr = uses_exchange(core.prec) ? rs * nt * 3 * nq * trace_stride(core.prec) : 0;
+    const size_t ntr = uses_exchange(core.prec) ? rs * nt * 3 * nq * TR_STRIDE : 0;
     q = Snap{nullptr, nullptr, nullptr, sizeof(double) * 4 * nt, rs * 4 * (nb - 1) * nt, ntr, {}};
     if (cudaMalloc(&q.avg, q.navg) != cudaSuccess || cudaMalloc(&q.hi, q.nhi) != cudaSuccess ||
         (q.ntr && cudaMalloc(&q.tr, q.ntr) != cudaSuccess)) {

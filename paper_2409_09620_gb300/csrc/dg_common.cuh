@@ -14,9 +14,10 @@
 //             vd[nt][3][16]    value (4), physical gradient (8), 1/rho and sound speed
 //                              of u_h at each vertex (2 padding values)
 //             hs[nt][12]       physical Hessian (xx, xy, yy) of u_h per component (P2)
-//             ej[ne][16]       per edge: beta and the square roots of the OE jump sums
-// Every kernel is one thread per cell; reductions are per-block partials
-// reduced in a fixed order, so results are bitwise reproducible.
+//             ej[ne][16]       per edge: the OE jump terms of each component
+// The mixed form's kernels are one thread per cell, the FP64 form's four lanes
+// per cell; reductions are per-block partials reduced in a fixed order, so
+// results are bitwise reproducible.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -25,7 +26,13 @@
 
 namespace dg {
 
-constexpr int TPB = 128;                 // cells per block
+constexpr int TPB = 128;                 // threads per block of the stage kernels
+// cells per tile (one block's work, one reduction partial): one thread per
+// cell in the mixed form, four lanes per cell in the FP64 form
+template <typename Real> struct TileCells { static constexpr int value = sizeof(Real) == 4 ? TPB : TPB / 4; };
+__host__ __device__ constexpr int tile_cells(int precision) {
+  return precision == 0 ? TileCells<double>::value : TileCells<float>::value;
+}
 constexpr int FIN_THREADS = 1024;        // threads (virtual lanes) of the finalize reductions
 
 template <int K> struct Deg;
@@ -43,7 +50,7 @@ struct MeshDev {
   int64_t ne;
   const int32_t *e_cell;   // [ne] owning cell
   const int8_t *e_loc;     // [ne] its local edge
-  const int32_t *etile;    // [ntiles + 1] first edge owned by each tile of TPB cells
+  const int32_t *etile;    // [ntiles + 1] first edge owned by each tile of the FP64 form
   const int32_t *cedge;    // [3][nt] edge index of (cell, local edge)
   // FP32 copies of the geometry the mixed-precision kernels read (the same
   // rounded values, without a conversion per read), and 1/|K| in FP64
@@ -53,35 +60,14 @@ struct MeshDev {
   const double *psi_node;  // [2][5][nt] P2 basis psi_1..psi_5 at the two internal nodes
 };
 
-// geometry in the working precision of a kernel
-template <typename Real> struct Geo;
-template <> struct Geo<double> {
-  static __device__ __forceinline__ const double *jinv(const MeshDev &m) { return m.jinv; }
-  static __device__ __forceinline__ const double *nrm(const MeshDev &m) { return m.nrm; }
-  static __device__ __forceinline__ const double *len(const MeshDev &m) { return m.len; }
-  static __device__ __forceinline__ const double *hgeo(const MeshDev &m) { return m.hgeo; }
-};
-template <> struct Geo<float> {
-  static __device__ __forceinline__ const float *jinv(const MeshDev &m) { return m.jinv_f; }
-  static __device__ __forceinline__ const float *nrm(const MeshDev &m) { return m.nrm_f; }
-  static __device__ __forceinline__ const float *len(const MeshDev &m) { return m.len_f; }
-  static __device__ __forceinline__ const float *hgeo(const MeshDev &m) { return m.hgeo_f; }
-};
-
-// values per edge Gauss point in the trace buffer tr[nt][3][Q][TS]: u and
-// F(u).n in the FP64 form (TS = 8); u only in the FP32 form (TS = 4), whose
-// stage kernel recomputes F(u).n in FP32 on both sides of the edge.  The two
-// cells of an edge have exactly opposite normals, so the recomputed fluxes
-// are the negated values the other cell uses, bit for bit.
-template <typename Real> struct TraceStride { static constexpr int value = sizeof(Real) == 4 ? 4 : 8; };
-__host__ __device__ constexpr int trace_stride(int precision) { return precision == 0 ? 8 : 4; }
 // the exchange buffers (traces, vertex records, Hessians, edge records) are
 // used by the FP64 form only; the mixed form's passes read the states directly
 __host__ __device__ constexpr bool uses_exchange(int precision) { return precision == 0; }
-// per-edge OE record ej[ne][EJ_STRIDE]: beta, then sqrt(2 J) of the trapezoidal
-// jump sums J for q = rho, (m_n|m_t max | m1), (m2), E and j = 0..k (13 used)
+// values per edge Gauss point in the trace buffer tr[nt][3][Q][8]: u and F(u).n
+constexpr int TR_STRIDE = 8;
+// per-edge OE record ej[ne][4][4]: A^{k,j} beta sqrt(J) of the trapezoidal jump
+// sums J, per component and derivative order j = 0..k (one padding value)
 constexpr int EJ_STRIDE = 16;
-__host__ __device__ constexpr int ej_row(int q, int j, int K) { return 1 + q * (K + 1) + j; }
 // per-cell vertex record vd[nt][3][VD_STRIDE]: value (4), gradient (8), 1/rho, sound speed
 constexpr int VD_STRIDE = 16;
 constexpr int VD_CELL = 3 * VD_STRIDE;
@@ -291,7 +277,8 @@ __device__ __forceinline__ bool nonzero_bits(float x) { return (__float_as_int(x
 
 // F(u) . n and the spectral radius |v.n| + c (+inf for rho <= 0) with one reciprocal
 template <typename T>
-__device__ __forceinline__ T flux_speed_ri(const T u[4], T ri, T nx, T ny, T gm1, T gamma, T f[4]) {
+__device__ __forceinline__ T flux_speed(const T u[4], T nx, T ny, T gm1, T gamma, T f[4]) {
+  const T ri = T(1) / u[0];
   const T p = gm1 * fma(T(-0.5) * fdot2(u[1], u[1], u[2], u[2]), ri, u[3]);
   const T mn = fdot2(u[1], nx, u[2], ny);
   const T vn = mn * ri;
@@ -302,39 +289,6 @@ __device__ __forceinline__ T flux_speed_ri(const T u[4], T ri, T nx, T ny, T gm1
   if (!gt0(u[0])) return T(INFINITY);
   const T pc = gt0(p) ? p : T(0);
   return fabs(vn) + sqrt(gamma * pc * ri);
-}
-template <typename T>
-__device__ __forceinline__ T flux_speed(const T u[4], T nx, T ny, T gm1, T gamma, T f[4]) {
-  return flux_speed_ri(u, T(1) / u[0], nx, ny, gm1, gamma, f);
-}
-
-// 1 / x[p] for n values from one division (Montgomery's batch inversion:
-// prefix products, one reciprocal, back-substitution with two multiplies
-// per value; each result within about 2n roundings of 1 / x[p]).  If a prefix product is not a normal number (a
-// zero, a non-finite or an extreme value) every value is divided instead.
-template <int n>
-__device__ __forceinline__ void batch_reciprocal(const double x[n], double r[n]) {
-  double c[n];
-  c[0] = x[0];
-  unsigned bad = 0;
-#pragma unroll
-  for (int p = 0; p < n; ++p) {
-    if (p > 0) c[p] = c[p - 1] * x[p];
-    const unsigned ex = unsigned(__double_as_longlong(c[p]) >> 52) & 0x7ffu;
-    bad |= (ex == 0u) | (ex == 0x7ffu);
-  }
-  if (bad) {
-#pragma unroll
-    for (int p = 0; p < n; ++p) r[p] = 1.0 / x[p];
-    return;
-  }
-  double inv = 1.0 / c[n - 1];
-#pragma unroll
-  for (int p = n - 1; p > 0; --p) {
-    r[p] = inv * c[p - 1];
-    inv = inv * x[p];
-  }
-  r[0] = inv;
 }
 
 // spectral radius |v.n| + c; +inf for rho <= 0, pressure clamped at 0
@@ -716,30 +670,6 @@ __device__ __forceinline__ void step_begin_thread(Scalars *sc) {
   } else {
     sc->dt = 0.0;
     sc->active = 0;
-  }
-}
-
-// Deviation from the average of the extra limiter point(s) of the classical
-// decomposition, from the deviations at the edge Gauss points (the first 3Q
-// rows of d): P1 has no internal term (its edge weights sum to one), so the
-// edge point 0 is repeated; P2 takes the weighted internal state u_* of
-// Sec. 4.1 with edge weights 1/9: u_* - ubar = -(1/9) sum w_nu dev / (1 - 3/9).
-template <int K, typename T, int ROWS>
-__device__ __forceinline__ void zxs_extra_points(T d[ROWS][4]) {
-  constexpr int NQ = K + 1, NE = 3 * NQ;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    T v;
-    if (K == 1) {
-      v = d[0][c];
-    } else {
-      T acc = T(0);
-#pragma unroll
-      for (int p = 0; p < NE; ++p) acc += T(gauss_w(NQ, p % NQ)) * d[p][c];
-      v = T(-1.0 / 6.0) * acc;
-    }
-    d[NE][c] = v;
-    d[NE + 1][c] = v;
   }
 }
 

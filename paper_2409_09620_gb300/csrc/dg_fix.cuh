@@ -1,0 +1,150 @@
+// dg_fix.cuh -- block fixed-point arithmetic for the FP64 form's contractions
+// with constant tables (basis values at points, quadrature sums), plain C++
+// where compiled without CUDA (host self-test).
+//
+// GB300 runs an FP64 warp instruction in 64 cycles per scheduler when all
+// operands are registers and in 76 when one is an immediate or a constant
+// (a compile-time basis value always is; DADD and DMUL always take 76), while
+// a 32 x 32 + 64 bit integer multiply-add takes about 2.  A sum
+// sum_j c_j x_j with constants c_j therefore runs on the integer units, about
+// 9 cycles per term, beside the FP64 pipe:
+//
+//   * the values x_j of a block (a cell's modes of one component, its fluxes
+//     at the volume points, ...) share the exponent E of the largest:
+//     x_j = (h 2^29 + l) 2^(E - 1080), |h 2^29 + l| < 2^58, truncated at 2^-58
+//     of the block's largest magnitude (FP64 rounds at 2^-53 of each term);
+//   * a constant |c| <= 4 is (h 2^29 + l) 2^-56 with |l| <= 2^28;
+//   * the products h h and h l + l h accumulate exactly in two 64-bit
+//     integers (l l, below 2^-57 of the block, is dropped), so the order of
+//     the terms does not matter;
+//   * the result converts to FP64 with one rounding.
+//
+// The error of a sum is a few 2^-57 of the block's largest magnitude, below
+// that of the FMA chain it replaces (tests/test_fix_host.py).  Zeros stay
+// zero, subnormals count as zero and blocks below 2^-959 keep an absolute
+// 2^-1016; a block that holds an infinity or a NaN has E = 0x7ff, and the
+// callers turn its results into NaN.
+#pragma once
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define FX_HD __host__ __device__ __forceinline__
+#define FX_CONST __host__ __device__ constexpr
+#else
+#define FX_HD inline
+#define FX_CONST constexpr
+#endif
+
+namespace dg {
+
+constexpr int FX_LIMB = 29;          // bits of the low limb
+constexpr int FX_ONE = 56;           // a constant c is stored as round(c 2^56)
+constexpr int FX_EMIN = 64, FX_ENAN = 0x7ff;   // smallest block exponent used; exponent of a non-finite block
+
+FX_HD int fx_hiword(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2hiint(x);
+#else
+  int64_t b;
+  std::memcpy(&b, &x, 8);
+  return (int)(b >> 32);
+#endif
+}
+FX_HD unsigned fx_loword(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(x);
+#else
+  int64_t b;
+  std::memcpy(&b, &x, 8);
+  return (unsigned)b;
+#endif
+}
+FX_HD double fx_make(int hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(hi, (int)lo);
+#else
+  const int64_t b = (int64_t)(((uint64_t)(unsigned)hi << 32) | lo);
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+// 127 + floor(log2 |r|), 0 for r = 0: the exponent field of r rounded toward
+// zero to FP32 (the conversion runs beside the integer pipe)
+FX_HD int fx_log2_127(int64_t r) {
+#ifdef __CUDA_ARCH__
+  return (__float_as_int(__ll2float_rz(r)) >> 23) & 0xff;
+#else
+  return r == 0 ? 0 : 190 - __builtin_clzll((uint64_t)(r < 0 ? -r : r));
+#endif
+}
+
+// constant: c = (h 2^29 + l) 2^-56, |l| <= 2^28
+struct FxC {
+  int h, l;
+};
+FX_CONST FxC fxc(double c) {
+  const double s = c * double(1LL << FX_ONE);
+  const int64_t v = (int64_t)(s < 0.0 ? s - 0.5 : s + 0.5);
+  const int64_t h = (v + (1LL << (FX_LIMB - 1))) >> FX_LIMB;
+  return FxC{(int)h, (int)(v - h * (1LL << FX_LIMB))};
+}
+
+// exponent of a block from the bitwise-positive high words of its values
+FX_HD int fx_abs_hi(double x) { return fx_hiword(x) & 0x7fffffff; }
+FX_HD int fx_exp(int max_abs_hi) {
+  const int e = max_abs_hi >> 20;
+  return e < FX_EMIN ? FX_EMIN : e;
+}
+
+// a value of a block with exponent E (|x| < 2^(E - 1022))
+struct Fx {
+  int h, l;
+};
+FX_HD Fx fx_from(double x, int E) {
+  const int hi = fx_hiword(x);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const uint64_t m = (((uint64_t)mh << 32) | fx_loword(x)) << 5;
+  // E >= 64, so a zero or subnormal x (exponent field 0) shifts out
+  int s = E - ((hi >> 20) & 0x7ff);
+  s = s > 63 ? 63 : s;
+  const uint64_t v = m >> s;
+  const int g = (hi >> 31) | 1;        // sign
+  return Fx{(int)(v >> FX_LIMB) * g, ((int)v & ((1 << FX_LIMB) - 1)) * g};
+}
+
+// sum of products, exact but for the dropped l l
+struct FxAcc {
+  int64_t a, b;
+};
+FX_HD void fx_mac(FxAcc &s, FxC c, Fx x) {
+  if (c.h != 0) {
+    s.a += (int64_t)c.h * x.h;
+    s.b += (int64_t)c.h * x.l;
+  }
+  if (c.l != 0) s.b += (int64_t)c.l * x.h;
+}
+FX_HD int64_t fx_sum(const FxAcc &s) {
+  return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + (s.b >> (FX_ONE - FX_LIMB));
+}
+// r 2^(E - 1080) rounded to nearest; |r| < 2^63
+FX_HD double fx_to(int64_t r, int E) {
+  const int e8 = fx_log2_127(r);
+  const int64_t g = r >> 63;
+  const uint64_t m = (uint64_t)(r ^ g) << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62 (|r| - 1 for r < 0)
+  const uint64_t q = (m + 512u) >> 10;
+  int f = E + e8 - 185;                // exponent field, less the one that q carries
+  f = f < 0 ? 0 : (f > 2046 ? 2046 : f);
+  f = e8 == 0 ? 0 : f;
+  const int hi = ((int)(q >> 32) + (f << 20)) | ((int)(g >> 32) & (int)0x80000000);
+  return fx_make(hi, (unsigned)q);
+}
+// r1 2^(E1 - 1080) + r2 2^(E2 - 1080) as r 2^(E - 1080)
+FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
+  E = (E1 > E2 ? E1 : E2) + 1;
+  const int s1 = E - E1, s2 = E - E2;
+  return (r1 >> (s1 > 63 ? 63 : s1)) + (r2 >> (s2 > 63 ? 63 : s2));
+}
+
+}  // namespace dg

@@ -55,7 +55,8 @@ void launch_fin_alpha(const StageCtx &c, int stage);
 void launch_step_begin(const StageCtx &c);
 void launch_set_active(const StageCtx &c, int active);
 void launch_set_inv_normalisers(const StageCtx &c);
-int64_t num_blocks(int64_t nt);
+// tiles of a mesh: the blocks of a stage kernel in the given precision, one reduction partial each
+int64_t num_tiles(int64_t nt, int prec);
 
 // access to a solver's launch context and buffers (dg_api.cu)
 const StageCtx &solver_ctx(const dg_solver *s);

@@ -155,7 +155,9 @@ __global__ void k_set_active(Scalars *sc, int active) {
 // ==========================================================================
 // Launch wrappers
 // ==========================================================================
-static inline unsigned nblocks(int64_t nt) { return (unsigned)((nt + TPB - 1) / TPB); }
+static inline unsigned nblocks(int64_t nt) { return (unsigned)((nt + TPB - 1) / TPB); }   // one thread per cell
+template <typename Real>
+static inline unsigned ntiles(int64_t nt) { return (unsigned)((nt + TileCells<Real>::value - 1) / TileCells<Real>::value); }
 
 void launch_geometry(cudaStream_t s, int64_t nt, const double *vxy, const GeomPtrs &g, double *part_min,
                      double *out_min4) {
@@ -169,20 +171,20 @@ template <int K, typename Real>
 static void rk_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> v, StateDev<Real> un,
                     StateDev<Real> uh, const void *tr, void *vd, void *hs, double *part_sum, const Scalars *sc,
                     double a, double b, double c_in) {
-  k_rk<K, Real><<<nblocks(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
+  k_rk<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
                                               sc, a, b, c_in);
 }
 template <int K, typename Real>
 static void stats_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, double *part_dev,
                        const void *vd, const void *hs, void *ej, const Scalars *sc, double c_out) {
-  k_stats<K, Real><<<nblocks(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
+  k_stats<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
                                                  sc, c_out);
 }
 template <int K, typename Real>
 static void oebp_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, StateDev<Real> out,
                       const void *ej, void *tr, double *pa, long long *pc, const Scalars *sc, int do_oe,
                       int do_bp, double c_out, int end_of_step) {
-  k_oe_bp<K, Real><<<nblocks(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe,
+  k_oe_bp<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe,
                                                  do_bp, c_out, end_of_step);
 }
 
@@ -208,7 +210,7 @@ void launch_rk_only(const StageCtx &c, const StateBuf &v, const StateBuf &un, co
 }
 
 void launch_fin_mean(const StageCtx &c) {
-  const int64_t nt = nblocks(c.mesh.nt);
+  const int64_t nt = num_tiles(c.mesh.nt, c.prec);
   k_fin_mean<<<(unsigned)num_groups(nt), TPB, 0, c.stream>>>(c.part_sum, c.fin, nt, c.sc);
 }
 
@@ -226,7 +228,7 @@ void launch_stats_only(const StageCtx &c, const StateBuf &uh, double c_out) {
 }
 
 void launch_fin_dev(const StageCtx &c) {
-  const int64_t nt = nblocks(c.mesh.nt);
+  const int64_t nt = num_tiles(c.mesh.nt, c.prec);
   k_fin_dev<<<(unsigned)num_groups(nt), TPB, 0, c.stream>>>(c.part_dev, c.fin, nt, c.sc, c.phys.oe == 2);
 }
 
@@ -245,7 +247,7 @@ void launch_oe_bp_only(const StageCtx &c, const StateBuf &uh, const StateBuf &ou
 
 // alpha and counters; after stage 2 also t += dt (stage < 0: outside a step)
 void launch_fin_alpha(const StageCtx &c, int stage) {
-  const int64_t nt = nblocks(c.mesh.nt);
+  const int64_t nt = num_tiles(c.mesh.nt, c.prec);
   k_fin_alpha<<<(unsigned)num_groups(nt), TPB, 0, c.stream>>>(c.part_alpha, c.part_cnt, c.fin, nt, c.sc, stage);
 }
 
@@ -261,7 +263,7 @@ void launch_set_inv_normalisers(const StageCtx &c) {
   k_set_inv_normalisers<<<1, 32, 0, c.stream>>>(c.sc, c.phys.oe == 2);
 }
 
-int64_t num_blocks(int64_t nt) { return nblocks(nt); }
+int64_t num_tiles(int64_t nt, int prec) { return (nt + tile_cells(prec) - 1) / tile_cells(prec); }
 
 size_t stage_kernels_local_bytes(int k, int prec) {
   size_t n = 0;

@@ -1,0 +1,714 @@
+// dg_stage_fp64.cuh -- stage kernels of the FP64 form (Ding, Cui & Wu, arXiv
+// 2409.09620, Sec. 4.5).
+//
+// What bounds them: GB300's FP64 pipe takes 64 cycles per warp instruction and
+// scheduler (76 with an immediate or constant operand), whatever the number
+// of active lanes, and a dependent instruction waits as long.  So
+//
+//   * four lanes share a cell, one per conserved component: a tile of 32 cells
+//     is a block of 128 threads.  A quarter of the serial chain per thread,
+//     four times the warps of one thread per cell on a small mesh, and few
+//     enough registers for several blocks per SM;
+//   * sums with compile-time coefficients (values at points, quadrature sums,
+//     vertex derivatives) run in block fixed point on the integer units
+//     beside the FP64 pipe (dg_fix.cuh);
+//   * work that needs all four components (fluxes, wave speeds) is dealt out
+//     one (cell, point) per lane through shared memory.  The warp that starts
+//     depends on the tile: warp w sits on scheduler w mod 4, and 6 or 9 points
+//     are no multiple of 4.
+//
+// Threads beyond the last cell repeat the last cell and store nothing.
+//
+// Measured against one thread per cell with every sum on the FP64 pipe: double
+// Mach reflection, 1,036,800 P2 cells, ms per launch: k_rk 2.37 -> 1.50,
+// k_stats 0.96 -> 1.05, k_oe_bp 1.39 -> 0.90, step 14.16 -> 10.38; isentropic
+// vortex, 2,048 P1 cells, step 250 -> 135 us.
+#pragma once
+
+namespace dg {
+
+constexpr int FT = TileCells<double>::value;   // cells per tile
+static_assert(4 * FT == TPB, "four lanes per cell");
+
+// a cell's four components of one point, in shared memory
+struct __align__(16) Vec4d {
+  double c[4];
+};
+
+// one component's average and modes
+template <int NB>
+__device__ __forceinline__ void load_comp(const StateDev<double> &s, int64_t nt, int64_t K, int c, double x[NB]) {
+  x[0] = s.avg[c * nt + K];
+#pragma unroll
+  for (int l = 1; l < NB; ++l) x[l] = s.hi[(c * (NB - 1) + (l - 1)) * nt + K];
+}
+// block fixed point of a component's coefficients; returns the block's exponent
+template <int NB>
+__device__ __forceinline__ int fx_block(const double x[NB], Fx f[NB]) {
+  int mx = 0;
+#pragma unroll
+  for (int l = 0; l < NB; ++l) mx = max(mx, fx_abs_hi(x[l]));
+  const int E = fx_exp(mx);
+#pragma unroll
+  for (int l = 0; l < NB; ++l) f[l] = fx_from(x[l], E);
+  return E;
+}
+// value of the component's polynomial at a fixed reference point: sum_l psi_l(x) f_l
+template <int NB>
+__device__ __forceinline__ int64_t fx_point(const Fx f[NB], double xi, double eta) {
+  FxAcc s{0, 0};
+#pragma unroll
+  for (int l = 0; l < NB; ++l) fx_mac(s, fxc(psi(l, xi, eta)), f[l]);
+  return fx_sum(s);
+}
+// fx_to, NaN for a block that holds a non-finite value
+__device__ __forceinline__ double fx_out(int64_t r, int E) {
+  const double x = fx_to(r, E);
+  return E >= FX_ENAN ? NAN : x;
+}
+// component c of four values held by every lane
+__device__ __forceinline__ double pick4(const double v[4], int c) {
+  const double a = c & 1 ? v[1] : v[0], b = c & 1 ? v[3] : v[2];
+  return c & 2 ? b : a;
+}
+
+// ==========================================================================
+// K1: u_h = a u_n + b (v + dt L(v))
+// ==========================================================================
+// one tile; block partial -> part_sum[4 * tile]
+template <int K>
+__device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> v, StateDev<double> un,
+                                             StateDev<double> uh, const double *__restrict__ tr,
+                                             double *__restrict__ vdo, double *__restrict__ hso, double *part_sum,
+                                             const Scalars *sc, double a, double b, double c_in, int64_t tile) {
+  constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ, NV = Deg<K>::NV;
+  __shared__ Vec4d s_u[NV][FT], s_g[NV][FT];
+  const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
+  const int lane = threadIdx.x & 31, warp0 = ((threadIdx.x >> 5) + (int)tile) & 3;
+  const int64_t nt = m.nt, K0 = tile * FT;
+  const bool live = K0 + lc < nt;
+  const int64_t Kc = live ? K0 + lc : nt - 1;
+  const double gm1 = phys_gm1<double>(ph), dt = sc->dt, alpha = sc->alpha;
+
+  // ---- values at the volume points -----------------------------------------
+  {
+    double x[NB];
+    Fx f[NB];
+    load_comp<NB>(v, nt, Kc, c, x);
+    const int E = fx_block<NB>(x, f);
+#pragma unroll
+    for (int mu = 0; mu < NV; ++mu)
+      s_u[mu][lc].c[c] = fx_out(fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu)), E);
+  }
+  __syncthreads();
+  // ---- volume fluxes, one (cell, point) per lane -----------------------------
+  // F . grad Psi = (F . grad xi) dPsi/dxi + (F . grad eta) dPsi/deta; |K| rides on the gradients
+  {
+    const int64_t Kl = K0 + lane < nt ? K0 + lane : nt - 1;
+    const double ar = m.area[Kl];
+    const double jx = ar * m.jinv[Kl], jy = ar * m.jinv[nt + Kl], ex = ar * m.jinv[2 * nt + Kl],
+                 ey = ar * m.jinv[3 * nt + Kl];
+#pragma unroll 1
+    for (int p = warp0; p < NV; p += 4) {
+      Vec4d u = s_u[p][lane], g1, g2;
+      flux_dir2(u.c, jx, jy, ex, ey, gm1, g1.c, g2.c);
+      s_u[p][lane] = g1;
+      s_g[p][lane] = g2;
+    }
+  }
+  // ---- edge fluxes of this component -------------------------------------------
+  double tv[3 * NQ];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int32_t cn = m.conn[i * nt + Kc];
+    const double li = m.len[i * nt + Kc];
+#pragma unroll
+    for (int nu = 0; nu < NQ; ++nu) {
+      const double *po = tr + ((Kc * 3 + i) * NQ + nu) * 8;
+      const double um = po[c], fm = po[4 + c];
+      double up, fp;
+      if (cn >= 0) {
+        const double *pn = tr + (((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)) * 8;
+        up = pn[c];
+        fp = -pn[4 + c];   // F(u+).n of this cell's normal
+      } else {
+        const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
+        double px = 0.0, py = 0.0, ow[4], av[4], gh[4], gf[4];
+        const double t_in = fma(c_in, sc->dt, sc->t);
+        if (cn == -7) {
+          const double s = gauss_s(NQ, nu);
+          const double xa = m.vxy[(2 * ((i + 1) % 3)) * nt + Kc], ya = m.vxy[(2 * ((i + 1) % 3) + 1) * nt + Kc];
+          const double xb = m.vxy[(2 * ((i + 2) % 3)) * nt + Kc], yb = m.vxy[(2 * ((i + 2) % 3) + 1) * nt + Kc];
+          px = fma(xb - xa, s, xa);
+          py = fma(yb - ya, s, ya);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          ow[q] = po[q];
+          av[q] = v.avg[q * nt + Kc];
+        }
+        ghost_state(-cn, ow, av, nx, ny, px, py, t_in, ph, gh);
+        flux_dir(gh, nx, ny, gm1, gf);
+        up = pick4(gh, c);
+        fp = pick4(gf, c);
+      }
+      // l_i w_nu / 2: the 1/2 of the LF flux rides on the weight (a power of
+      // two).  The two cells of an edge form exactly opposite products.
+      const double lw = li * (0.5 * gauss_w(NQ, nu));
+      tv[i * NQ + nu] = lw * fma(-alpha, up - um, fm + fp);
+    }
+  }
+  __syncthreads();
+  // ---- quadrature sums, mass inverse, SSP-RK combination ---------------------------
+  // volume |K| sum_mu w_mu F . grad Psi_l, edges - sum_i l_i sum_nu w_nu Fhat Psi_l
+  double h[NB];
+  {
+    int64_t rv[NB];
+    int Ev;
+    {
+      double g1[NV], g2[NV];
+      int mx = 0;
+#pragma unroll
+      for (int mu = 0; mu < NV; ++mu) {
+        g1[mu] = s_u[mu][lc].c[c];
+        g2[mu] = s_g[mu][lc].c[c];
+        mx = max(mx, max(fx_abs_hi(g1[mu]), fx_abs_hi(g2[mu])));
+      }
+      Ev = fx_exp(mx);
+      FxAcc s[NB];
+#pragma unroll
+      for (int l = 1; l < NB; ++l) s[l] = FxAcc{0, 0};
+#pragma unroll
+      for (int mu = 0; mu < NV; ++mu) {
+        const double xi = vol_xi(NV, mu), eta = vol_eta(NV, mu), w = vol_w(NV, mu);
+        const Fx f1 = fx_from(g1[mu], Ev), f2 = fx_from(g2[mu], Ev);
+#pragma unroll
+        for (int l = 1; l < NB; ++l) {
+          fx_mac(s[l], fxc(w * psi_x(l, xi, eta)), f1);
+          fx_mac(s[l], fxc(w * psi_y(l, xi, eta)), f2);
+        }
+      }
+#pragma unroll
+      for (int l = 1; l < NB; ++l) rv[l] = fx_sum(s[l]);
+    }
+    int mx = 0;
+#pragma unroll
+    for (int p = 0; p < 3 * NQ; ++p) mx = max(mx, fx_abs_hi(tv[p]));
+    const int Ee = fx_exp(mx);
+    FxAcc s[NB];
+#pragma unroll
+    for (int l = 0; l < NB; ++l) s[l] = FxAcc{0, 0};
+#pragma unroll
+    for (int p = 0; p < 3 * NQ; ++p) {
+      const double sg = gauss_s(NQ, p % NQ);
+      const Fx f = fx_from(tv[p], Ee);
+#pragma unroll
+      for (int l = 0; l < NB; ++l) fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg))), f);
+    }
+    const double dta = dt * m.iarea[Kc];
+    const bool first = a == 0.0 && b == 1.0;   // the first stage skips the zero term and the load of u_n
+    const bool bad = max(Ev, Ee) >= FX_ENAN;
+    double x[NB], xn[NB];
+    load_comp<NB>(v, nt, Kc, c, x);
+    if (!first) load_comp<NB>(un, nt, Kc, c, xn);
+#pragma unroll
+    for (int l = 0; l < NB; ++l) {
+      int E = Ee;
+      int64_t r = fx_sum(s[l]);
+      if (l > 0) r = fx_add(rv[l], Ev, r, Ee, E);
+      const double d = bad ? NAN : fx_to(r, E);
+      const double L = fma(dta * inv_mass_c(l), d, x[l]);
+      h[l] = first ? L : fdot2(a, xn[l], b, L);
+    }
+  }
+  if (live) {
+    uh.avg[c * nt + Kc] = h[0];
+#pragma unroll
+    for (int l = 1; l < NB; ++l) uh.hi[(c * (NB - 1) + (l - 1)) * nt + Kc] = h[l];
+  }
+  double mass = live ? m.area[Kc] * h[0] : 0.0;
+
+  // ---- vertex derivatives of u_h for the OE jumps ------------------------------
+  {
+    const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
+    Fx f[NB];
+    const int E = fx_block<NB>(h, f);
+    double *vo = vdo + Kc * VD_CELL;
+    double gx = 0.0, ge = 0.0;
+#pragma unroll
+    for (int vv = 0; vv < 3; ++vv) {
+      const double val = fx_out(fx_point<NB>(f, vert_xi(vv), vert_eta(vv)), E);
+      if (K == 2 || vv == 0) {   // P1 has one gradient
+        FxAcc sx{0, 0}, se{0, 0};   // derivative coefficients reach 48: as c / 64
+#pragma unroll
+        for (int l = 1; l < NB; ++l) {
+          fx_mac(sx, fxc(psi_x(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
+          fx_mac(se, fxc(psi_y(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
+        }
+        gx = fx_out(fx_sum(sx), E + 6);
+        ge = fx_out(fx_sum(se), E + 6);
+      }
+      s_u[vv][lc].c[c] = val;   // this warp's slots; read after the barrier below
+      if (live) {
+        double *rec = vo + vv * VD_STRIDE;
+        rec[c] = val;
+        *reinterpret_cast<double2 *>(rec + 4 + 2 * c) = make_double2(fdot2(gx, jx, ge, ex), fdot2(gx, jy, ge, ey));
+      }
+    }
+    if (K == 2) {
+      // physical second derivatives (xx, xy, yy) from the reference ones:
+      // lane r forms the factors of row r of J^-T H J^-1, shared by the components
+      const double p0 = c == 2 ? jy : jx, p1 = c == 2 ? ey : ex, q0 = c == 0 ? jx : jy, q1 = c == 0 ? ex : ey;
+      const double wa = p0 * q0, wb = fdot2(p0, q1, q0, p1), wc = p1 * q1;
+      FxAcc s0{0, 0}, s1{0, 0}, s2{0, 0};
+#pragma unroll
+      for (int l = 3; l < NB; ++l) {
+        fx_mac(s0, fxc(psi_2(l, 0) / 64.0), f[l]);
+        fx_mac(s1, fxc(psi_2(l, 1) / 64.0), f[l]);
+        fx_mac(s2, fxc(psi_2(l, 2) / 64.0), f[l]);
+      }
+      const double hxx = fx_out(fx_sum(s0), E + 6), hxe = fx_out(fx_sum(s1), E + 6), hee = fx_out(fx_sum(s2), E + 6);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const double ga = __shfl_sync(0xffffffffu, wa, (lane & ~3) + r), gb = __shfl_sync(0xffffffffu, wb, (lane & ~3) + r),
+                     gc = __shfl_sync(0xffffffffu, wc, (lane & ~3) + r);
+        const double d2 = fma(hxx, ga, fdot2(hxe, gb, hee, gc));
+        if (live) hso[Kc * 12 + 3 * c + r] = d2;
+      }
+    }
+  }
+  __syncthreads();
+  // 1/rho and sound speed at the vertices, for the wave speeds beta of the OE (+inf for rho <= 0)
+  if (warp0 < 3 && K0 + lane < nt) {
+    const double gamma = phys_gamma<double>(ph);
+    const Vec4d u = s_u[warp0][lane];
+    double ri = 0.0, cs = INFINITY;
+    if (gt0(u.c[0])) {
+      ri = 1.0 / u.c[0];
+      double p = gm1 * fma(-0.5 * fdot2(u.c[1], u.c[1], u.c[2], u.c[2]), ri, u.c[3]);
+      p = gt0(p) ? p : 0.0;
+      cs = sqrt(gamma * p * ri);
+    }
+    *reinterpret_cast<double2 *>(vdo + (K0 + lane) * VD_CELL + warp0 * VD_STRIDE + 12) = make_double2(ri, cs);
+  }
+  // block sums of |K| u^(0): the cells of a warp, then the warps in order
+  __shared__ double s_m[TPB / 32][4];
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
+  if (lane < 4) s_m[threadIdx.x >> 5][lane] = mass;
+  __syncthreads();
+  if (threadIdx.x < 4)
+    part_sum[4 * tile + threadIdx.x] =
+        ((s_m[0][threadIdx.x] + s_m[1][threadIdx.x]) + s_m[2][threadIdx.x]) + s_m[3][threadIdx.x];
+  __syncthreads();
+}
+
+// ==========================================================================
+// K2: sup deviations from the domain mean at the volume points
+// ==========================================================================
+template <int K>
+__device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<double> uh, double *part_dev,
+                                                const Scalars *sc, int64_t tile) {
+  constexpr int NB = Deg<K>::NB, NV = Deg<K>::NV;
+  const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
+  const int64_t nt = m.nt, K0 = tile * FT;
+  const int64_t Kc = K0 + lc < nt ? K0 + lc : nt - 1;   // a repeated cell changes no maximum
+  double x[NB];
+  load_comp<NB>(uh, nt, Kc, c, x);
+  x[0] -= sc->mean[c];
+  int mx = 0;
+#pragma unroll
+  for (int l = 0; l < NB; ++l) mx = max(mx, fx_abs_hi(x[l]));
+  // the two momentum components share a block, so that their squares compare
+  const bool mom = c == 1 || c == 2;
+  const int mp = __shfl_xor_sync(0xffffffffu, mx, 3);
+  const int E = fx_exp(mom ? max(mx, mp) : mx);
+  Fx f[NB];
+#pragma unroll
+  for (int l = 0; l < NB; ++l) f[l] = fx_from(x[l], E);
+  // maxima in fixed point; the point of the largest |m|^2 is found from the
+  // top 64 bits of the squares (2^-62 of the largest), its norm taken in FP64
+  uint64_t top = 0, best = 0;
+  int64_t b1 = 0, b2 = 0;
+#pragma unroll
+  for (int mu = 0; mu < NV; ++mu) {
+    const int64_t r = fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu));
+    const uint64_t ab = (uint64_t)(r < 0 ? -r : r);
+    top = ab > top ? ab : top;
+    const uint64_t sq = __umul64hi(ab, ab);
+    const uint64_t s = sq + (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)sq, 3);
+    const int64_t q = __shfl_xor_sync(0xffffffffu, (long long)r, 3);
+    if (mu == 0 || s > best) { best = s; b1 = r; b2 = q; }
+  }
+  const double d = fx_out((int64_t)top, E);
+  const double m1 = fx_out(b1, E), m2 = fx_out(b2, E);
+  // rho, |m|, E, |m1|, |m2|; the lanes of the other components hold 0
+  double dr[5] = {c == 0 ? d : 0.0, c == 1 ? sqrt(fdot2(m1, m1, m2, m2)) : 0.0, c == 3 ? d : 0.0, c == 1 ? d : 0.0,
+                  c == 2 ? d : 0.0};
+  block_reduce<5>(dr, part_dev + 5 * tile, OpMaxNN());
+}
+
+// --------------------------------------------------------------------------
+// OE jump data of one edge, computed once for both cells that share it: per
+// component and derivative order j, A^{k,j} beta sqrt(J) of the trapezoidal
+// sums J = 1/2 sum_{|alpha| = j} C_j^alpha1 [d^alpha q]^2 over the two
+// endpoints (eqs. OEScalar:Coef2 with the trapezoidal rule, RIOESys:Coef1/
+// Coef2), seen from the owning cell; beta is the largest spectral radius of
+// both sides at both endpoints.  Jump sums are even in the sign of the jump
+// and of the normal, so both cells share them.  With RIOE both momentum rows
+// hold the larger of the normal and tangential sums.
+// Edges [etile[tile], etile[tile + 1]), four lanes per edge, one per component;
+// for beta the lanes take the four (endpoint, side) pairs.
+// --------------------------------------------------------------------------
+template <int K>
+__device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph, const double *__restrict__ avg,
+                                               const double *__restrict__ vdi, const double *__restrict__ hsi,
+                                               double *__restrict__ ej, const Scalars *sc, double c_out,
+                                               int64_t tile) {
+  const int64_t nt = m.nt;
+  const int64_t e0 = m.etile[tile], e1 = m.etile[tile + 1];
+  const double gamma = phys_gamma<double>(ph);
+  const int cw = ph.oe == 2;
+  const int c = threadIdx.x & 3;
+  const int slot = ((threadIdx.x >> 2) + 8 * (int)(tile & 3)) & 31;   // an uneven last round moves over the schedulers
+  const bool mom = !cw && (c == 1 || c == 2);
+  for (int64_t eb = e0; eb < e1; eb += FT) {
+    if (eb + (slot & ~7) >= e1) continue;   // no edge left for this warp
+    const bool live = eb + slot < e1;
+    const int64_t e = live ? eb + slot : e1 - 1;
+    const int64_t Kc = m.e_cell[e];
+    const int i = m.e_loc[e];
+    const int32_t cn = m.conn[i * nt + Kc];
+    const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
+    const double *vme = vdi + Kc * VD_CELL;
+    double jv[2], jg[2][2], jh[3] = {0.0, 0.0, 0.0}, r;
+    if (cn >= 0) {
+      const int64_t nb = cn >> 2;
+      const int jn = cn & 3;
+      const double *vnb = vdi + nb * VD_CELL;
+#pragma unroll
+      for (int ev = 0; ev < 2; ++ev) {   // v_c then v_d, and the neighbour's copy of it
+        int ov = i + 1 + ev, xv = jn + 2 - ev;
+        ov = ov >= 3 ? ov - 3 : ov;
+        xv = xv >= 3 ? xv - 3 : xv;
+        const double *ro = vme + ov * VD_STRIDE, *rx = vnb + xv * VD_STRIDE;
+        const double2 go = *reinterpret_cast<const double2 *>(ro + 4 + 2 * c),
+                      gx = *reinterpret_cast<const double2 *>(rx + 4 + 2 * c);
+        jv[ev] = ro[c] - rx[c];
+        jg[ev][0] = go.x - gx.x;
+        jg[ev][1] = go.y - gx.y;
+      }
+      if (K == 2) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) jh[q] = hsi[Kc * 12 + 3 * c + q] - hsi[nb * 12 + 3 * c + q];
+      }
+      int vv = c & 1 ? (c & 2 ? jn + 1 : i + 2) : (c & 2 ? jn + 2 : i + 1);
+      vv = vv >= 3 ? vv - 3 : vv;
+      const double *rr = (c & 2 ? vnb : vme) + vv * VD_STRIDE;
+      r = fma(fabs(fdot2(rr[1], nx, rr[2], ny)), rr[12], rr[13]);
+    } else {
+      // boundary edge: the exterior polynomial from all components of this side
+      const double t_out = fma(c_out, sc->dt, sc->t);
+      double ab[4], hme[12];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) ab[q] = avg[q * nt + Kc];   // the exterior state of a transmissive edge
+#pragma unroll
+      for (int q = 0; q < 12; ++q) hme[q] = K == 2 ? hsi[Kc * 12 + q] : 0.0;
+      r = 0.0;
+#pragma unroll 1
+      for (int ev = 0; ev < 2; ++ev) {
+        int ov = i + 1 + ev;
+        ov = ov >= 3 ? ov - 3 : ov;
+        const double *ro = vme + ov * VD_STRIDE;
+        double val[4], grd[8], xv[4], xg[8], xh[12];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) val[q] = ro[q];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) grd[q] = ro[4 + q];
+        double px = 0.0, py = 0.0;
+        if (cn == -7) { px = m.vxy[(2 * ov) * nt + Kc]; py = m.vxy[(2 * ov + 1) * nt + Kc]; }
+        ghost_vertex(-cn, val, grd, hme, ab, nx, ny, px, py, t_out, ph, xv, xg, xh);
+        const double r_own = fma(fabs(fdot2(val[1], nx, val[2], ny)), ro[12], ro[13]);
+        // a mirror state has the same spectral radius
+        r = max_nn(r, max_nn(r_own, cn == -1 ? r_own : wave_speed(xv, nx, ny, gamma)));
+        double gv[4], gw[4], dv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          dv[q] = val[q] - xv[q];
+          gv[q] = grd[2 * q] - xg[2 * q];
+          gw[q] = grd[2 * q + 1] - xg[2 * q + 1];
+        }
+        const double d0 = pick4(dv, c), d1 = pick4(gv, c), d2 = pick4(gw, c);
+        if (ev == 0) {
+          jv[0] = d0; jg[0][0] = d1; jg[0][1] = d2;
+          // the Hessian of the exterior state is constant: taken at v_c only
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const double dh[4] = {hme[q] - xh[q], hme[3 + q] - xh[3 + q], hme[6 + q] - xh[6 + q], hme[9 + q] - xh[9 + q]};
+            jh[q] = K == 2 ? pick4(dh, c) : 0.0;
+          }
+        } else {
+          jv[1] = d0; jg[1][0] = d1; jg[1][1] = d2;
+        }
+      }
+    }
+    r = max_nn(r, __shfl_xor_sync(0xffffffffu, r, 1));
+    const double beta = max_nn(r, __shfl_xor_sync(0xffffffffu, r, 2));
+    // RIOE: rotate the momentum jumps to (m_n, m_t) with the owner's normal
+    const double sy = c == 2 ? -ny : ny;
+    auto rot = [&](double q) {
+      const double p = __shfl_xor_sync(0xffffffffu, q, 3);
+      const double t = fdot2(q, nx, p, sy);
+      return mom ? t : q;
+    };
+    double J[K + 1];
+#pragma unroll
+    for (int ev = 0; ev < 2; ++ev) {
+      const double q = rot(jv[ev]), g0 = rot(jg[ev][0]), g1 = rot(jg[ev][1]);
+      // 2 J: the 1/2 of the trapezoidal rule moves into A (sqrt(1/2))
+      J[0] = ev == 0 ? q * q : fma(q, q, J[0]);
+      J[1] = ev == 0 ? fdot2(g0, g0, g1, g1) : fma(g0, g0, fma(g1, g1, J[1]));
+    }
+    if (K == 2) {   // the Hessian jump counts at both endpoints
+      const double h0 = rot(jh[0]), h1 = rot(jh[1]), h2 = rot(jh[2]);
+      const double f = fma(h0, h0, fma(h1 + h1, h1, h2 * h2));
+      J[K] = f + f;
+    }
+    const bool finite = is_finite_bits(beta);
+    double er[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j <= K; ++j) {
+      const double Jp = __shfl_xor_sync(0xffffffffu, J[j], 3);
+      if (mom) J[j] = max_nn(J[j], Jp);   // delta_m = max(delta_mn, delta_mt)
+      const double s = sqrt(J[j]);
+      // A^{k,j} = (2j + 1) / ((2k - 1) j!); a zero jump adds nothing, also where beta is
+      // +inf (a vertex with rho <= 0) and 0 * inf would be NaN
+      constexpr double r2 = 0.70710678118654752440;
+      const double A = (2.0 * j + 1.0) / ((2.0 * K - 1.0) * (j == 2 ? 2.0 : 1.0)) * r2;
+      er[j] = finite || nonzero_bits(s) ? (A * beta) * s : 0.0;
+    }
+    if (live) vstore<4>(ej + e * EJ_STRIDE + 4 * c, er);
+  }
+}
+
+// ==========================================================================
+// K3: RIOE + BP limiter + traces / alpha of the limited state
+// ==========================================================================
+// |x| truncated to FP32 from its high word: in [t, t (1 + 2^-20)] up to
+// 2^-126; +inf above the FP32 range or if not finite
+__device__ __forceinline__ float abs_f32_down(double x) {
+  const int t = (fx_hiword(x) & 0x7fffffff) - 0x38000000;
+  return __int_as_float(min(max(t, 0), 0x0ff00000) << 3);
+}
+
+template <int K>
+__device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> uh,
+                                                StateDev<double> out, const double *__restrict__ ej,
+                                                double *__restrict__ tr, double *part_alpha, long long *part_cnt,
+                                                const Scalars *sc, int do_oe, int do_bp, double c_out,
+                                                int end_of_step, int64_t tile) {
+  constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ;
+  constexpr int NE = 3 * NQ;          // edge Gauss points
+  __shared__ Vec4d s_u[NE + 2][FT], s_a[FT];
+  const unsigned FULL = 0xffffffffu;
+  const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
+  const int lane = threadIdx.x & 31, warp0 = ((threadIdx.x >> 5) + (int)tile) & 3, q0 = lane & ~3;
+  const int64_t nt = m.nt, K0 = tile * FT;
+  const bool live = K0 + lc < nt;
+  const int64_t Kc = live ? K0 + lc : nt - 1;
+  const double dt = sc->dt;
+  long long cnt[2] = {0, 0};
+  double x[NB];
+  load_comp<NB>(uh, nt, Kc, c, x);
+  s_a[lc].c[c] = x[0];
+
+  // ---------------------------- RIOE ---------------------------------------
+  if (do_oe) {
+    // sigma^j = sum_i (beta_i / h_i) delta_i^j with delta = A^{k,j} h^j sqrt(J) / D: the
+    // edge records hold A beta sqrt(J), the edge sum is scaled by 1 / D once (a constant
+    // component, 1 / D = 0, gets sigma = 0)
+    double sig[K + 1];
+#pragma unroll
+    for (int j = 0; j <= K; ++j) sig[j] = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double *er = ej + (int64_t)m.cedge[i * nt + Kc] * EJ_STRIDE + 4 * c;
+      const double2 e01 = *reinterpret_cast<const double2 *>(er);
+      sig[0] = fma(m.hgeo[(3 + i) * nt + Kc], e01.x, sig[0]);
+      sig[1] += e01.y;
+      if (K == 2) sig[K] = fma(m.hgeo[i * nt + Kc], er[2], sig[K]);
+    }
+    const double iD = sc->invD[c];
+    // exact solution of the damping ODE: mode of degree d times exp(-dt sum_{j<=d} sigma^j)
+    const double s = nonzero_bits(iD) ? iD * dt : 0.0;
+    double sacc = sig[0];
+#pragma unroll
+    for (int d = 1; d <= K; ++d) {
+      sacc += sig[d];
+      const double fac = exp_neg(nonzero_bits(iD) ? s * sacc : 0.0);
+#pragma unroll
+      for (int l = 1; l < NB; ++l)
+        if (degree_of(l) == d) x[l] *= fac;
+    }
+  }
+
+  // ---------------------------- BP limiter ----------------------------------
+  // A bound over the whole cell settles the usual (smooth) cell without its
+  // limiter points: with |Psi_l| <= 4 on K, every point's density is at least
+  // rho_bar - 4 sum |rho_l|, its energy at least E_bar - 4 sum |E_l| and the L1
+  // norm of its momentum at most |m1_bar| + |m2_bar| + 4 sum (|m1_l| + |m2_l|).
+  // If these keep rho and the internal energy above the thresholds with a
+  // margin (1e-5 relative) far above the rounding of this FP32 bound and of
+  // the point evaluations, every point passes the paper's tests and theta = 1,
+  // as the points themselves would give.
+  bool todo = false;
+  if (do_bp) {
+    float S = 0.0f;
+#pragma unroll
+    for (int l = 1; l < NB; ++l) S += abs_f32_down(x[l]);
+    const float D = fmaf(4.00002f, S, 1e-37f), A = abs_f32_down(x[0]);
+    const float B = fmaf(1.000002f, A, D);              // upper bound of |component|
+    const float lo = x[0] > 0.0 ? A - D : -1.0f;        // lower bound of rho, E
+    const float r_lo = __shfl_sync(FULL, lo, q0), r_hi = __shfl_sync(FULL, B, q0);
+    const float M_hi = __shfl_sync(FULL, B, q0 + 1) + __shfl_sync(FULL, B, q0 + 2);
+    const float E_lo = __shfl_sync(FULL, lo, q0 + 3), E_hi = __shfl_sync(FULL, B, q0 + 3);
+    const float M2 = M_hi * M_hi;
+    const bool settled = r_lo >= fmaf(1e-5f, r_hi, 2e-13f) &&
+                         r_lo * E_lo - 0.5f * M2 >= fmaf(1e-5f, fmaf(E_hi, r_lo, M2), 2e-13f * r_lo);
+    todo = !settled;
+  }
+
+  // values at the edge Gauss points (the traces, if the cell is not limited)
+  auto traces = [&]() {
+    Fx f[NB];
+    const int E = fx_block<NB>(x, f);
+#pragma unroll
+    for (int p = 0; p < NE; ++p) {
+      const double sg = gauss_s(NQ, p % NQ);
+      s_u[p][lc].c[c] = fx_out(fx_point<NB>(f, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)), E);
+    }
+  };
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    traces();
+    if (pass == 1 || !__any_sync(FULL, todo)) break;
+    // the limiter's points: the edge Gauss points and two extra points
+    double ext[2];
+    if (ph.decomp) {
+      // classical decomposition: P1 repeats edge point 0 (its edge weights sum to one), P2 takes
+      // the weighted internal state of Sec. 4.1: u_* - ubar = -1/6 sum w_nu dev
+      double acc = 0.0;
+#pragma unroll
+      for (int p = 0; p < NE; ++p) acc = fma(gauss_w(NQ, p % NQ), s_u[p][lc].c[c] - x[0], acc);
+      ext[0] = ext[1] = K == 1 ? s_u[0][lc].c[c] : fma(-1.0 / 6.0, acc, x[0]);
+    } else {
+      // P1: the vertices v1, v2; P2: the internal nodes, whose basis values the mesh holds
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        double s = 0.0;
+        if (K == 1) {
+          const int vp = m.limv[p * nt + Kc];
+#pragma unroll
+          for (int l = 1; l < NB; ++l) s = fma(psi(l, vert_xi(vp), vert_eta(vp)), x[l], s);
+        } else {
+#pragma unroll
+          for (int l = 1; l < NB; ++l) s = fma(m.psi_node[(5 * p + l - 1) * nt + Kc], x[l], s);
+        }
+        ext[p] = x[0] + s;
+      }
+    }
+    s_u[NE][lc].c[c] = ext[0];
+    s_u[NE + 1][lc].c[c] = ext[1];
+    __syncwarp();
+    const Vec4d av = s_a[lc];
+    const double Ebar = int_energy(av.c);
+    const bool adm = av.c[0] > 0.0 && Ebar > 0.0;
+    // Step 1: density.  Minimum on the integer units through order-preserving keys
+    long long kmin = ord_key(INFINITY);
+#pragma unroll
+    for (int p = c; p < NE + 2; p += 4) kmin = min(kmin, ord_key(s_u[p][lc].c[0]));
+    kmin = min(kmin, __shfl_xor_sync(FULL, kmin, 1));
+    kmin = min(kmin, __shfl_xor_sync(FULL, kmin, 2));
+    const double rmin = ord_val(kmin);
+    const double eps1 = fmin(av.c[0], 1e-13);
+    const double th1 = rmin < eps1 ? (av.c[0] - eps1) / (av.c[0] - rmin) : 1.0;
+    // Step 2: internal energy of the density-limited polynomial
+    // E - |m|^2 / (2 rho) < eps2 is tested as rho E - |m|^2 / 2 < eps2 rho (rho > 0):
+    // the division is only needed at points that violate the bound
+    const double eps2 = fmin(Ebar, 1e-13);
+    long long kem = ord_key(INFINITY);
+#pragma unroll 1
+    for (int p = c; p < NE + 2; p += 4) {
+      const Vec4d u = s_u[p][lc];
+      const double w0 = th1 < 1.0 ? fma(th1, u.c[0] - av.c[0], av.c[0]) : u.c[0];
+      const double q = 0.5 * fdot2(u.c[1], u.c[1], u.c[2], u.c[2]);
+      if (!(w0 > 0.0) || fma(u.c[3], w0, -q) < eps2 * w0) kem = min(kem, ord_key(u.c[3] - q / w0));
+    }
+    kem = min(kem, __shfl_xor_sync(FULL, kem, 1));
+    kem = min(kem, __shfl_xor_sync(FULL, kem, 2));
+    const double emin = ord_val(kem);
+    const double th2 = emin < eps2 ? (Ebar - eps2) / (Ebar - emin) : 1.0;
+    const bool lim = todo && adm && (th1 < 1.0 || th2 < 1.0);
+    if (todo && live && c == 0) {
+      if (!adm) cnt[1] = 1;
+      if (lim) cnt[0] = 1;
+    }
+    if (!__any_sync(FULL, lim)) break;
+    // scale the modes; the traces are taken again from the scaled (stored)
+    // modes, so that a run resumed from the stored state sees the same traces
+    // bit for bit
+    const double th = c == 0 ? th1 * th2 : th2;
+#pragma unroll
+    for (int l = 1; l < NB; ++l) x[l] = lim && th < 1.0 ? th * x[l] : x[l];
+    __syncwarp();   // every lane has read the points
+  }
+  if (live) {
+    out.avg[c * nt + Kc] = x[0];
+#pragma unroll
+    for (int l = 1; l < NB; ++l) out.hi[(c * (NB - 1) + (l - 1)) * nt + Kc] = x[l];
+  }
+  __syncthreads();
+
+  // ---------------------------- output ----------------------------------------
+  // traces, F.n and wave speed of the limited state, one (cell, edge point) per lane
+  double amax = 0.0;
+  if (K0 + lane < nt) {
+    const int64_t Kl = K0 + lane;
+    const double gamma = phys_gamma<double>(ph), gm1 = phys_gm1<double>(ph);
+#pragma unroll 1
+    for (int p = warp0; p < NE; p += 4) {
+      const int i = p / NQ;
+      const int32_t cn = m.conn[i * nt + Kl];
+      const double nx = m.nrm[(2 * i) * nt + Kl], ny = m.nrm[(2 * i + 1) * nt + Kl];
+      const Vec4d u = s_u[p][lane];
+      double o8[8];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) o8[q] = u.c[q];
+      amax = max_nn(amax, flux_speed(u.c, nx, ny, gm1, gamma, o8 + 4));
+      vstore<8>(tr + (Kl * NE + p) * 8, o8);
+      if (cn <= -2) {   // constant exterior states (walls mirror the trace: same speed)
+        // exterior states for the next stage's alpha at the time of the stage
+        // result: t + c_out dt, and after the last stage of a step clamped to
+        // the end time, the end time itself (the next step starts there)
+        const double t_out = end_of_step && sc->pad ? sc->t_end : fma(c_out, sc->dt, sc->t);
+        double px = 0.0, py = 0.0;
+        if (cn == -7) {
+          const int ia = i == 2 ? 0 : i + 1, ib = i == 0 ? 2 : i - 1, nu = p - i * NQ;
+          const double s = nu == 0 ? gauss_s(NQ, 0) : nu == 1 ? gauss_s(NQ, 1) : gauss_s(NQ, NQ - 1);
+          const double xa = m.vxy[(2 * ia) * nt + Kl], ya = m.vxy[(2 * ia + 1) * nt + Kl];
+          const double xb = m.vxy[(2 * ib) * nt + Kl], yb = m.vxy[(2 * ib + 1) * nt + Kl];
+          px = fma(xb - xa, s, xa);
+          py = fma(yb - ya, s, ya);
+        }
+        double up[4];
+        ghost_state(-cn, u.c, s_a[lane].c, nx, ny, px, py, t_out, ph, up);
+        amax = max_nn(amax, wave_speed(up, nx, ny, gamma));
+      }
+    }
+  }
+  double am[1] = {amax};
+  block_reduce<1>(am, part_alpha + tile, OpMaxNN());
+  block_reduce<2>(cnt, part_cnt + 2 * tile, OpSum());
+}
+
+}  // namespace dg

@@ -149,7 +149,7 @@ __device__ __forceinline__ void hessian_p2(const float hi[4][6], float jx, float
 template <int K>
 __device__ __forceinline__ void load_mixed(const StateDev<float> &s, int64_t nt, int64_t K_, double a[4],
                                            float af[4], float hi[4][Deg<K>::NB]) {
-  load_state<float, Deg<K>::NB>(s, nt, K_, a, hi);
+  load_state<Deg<K>::NB>(s, nt, K_, a, hi);
 #pragma unroll
   for (int c = 0; c < 4; ++c) af[c] = float(a[c]);
 }
@@ -289,7 +289,7 @@ __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, 
     const bool first = a == 0.0 && b == 1.0;
     double un0[4] = {0.0, 0.0, 0.0, 0.0};
     float cu[4][NB];
-    if (!first) load_state<float, NB>(un, nt, Kc, un0, cu);
+    if (!first) load_state<NB>(un, nt, Kc, un0, cu);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const double acc0 = double(s_hi[c]) + double(s_lo[c]);
@@ -305,6 +305,40 @@ __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, 
     store_modes_mixed<NB>(uh, Kc, cv);
   }
   block_reduce<4>(mass, part_sum + 4 * tile, OpSum());
+}
+
+// ==========================================================================
+// K2 (mixed): sup deviations from the domain mean at the volume points
+// ==========================================================================
+template <int K>
+__device__ __forceinline__ void stats_tile_mixed(const MeshDev &m, StateDev<float> uh, double *part_dev,
+                                                 const Scalars *sc, int64_t tile) {
+  constexpr int NB = Deg<K>::NB, NV = Deg<K>::NV;
+  const int64_t nt = m.nt;
+  const int64_t Kc = tile * TPB + threadIdx.x;
+  // deviations in the working precision, reduced in it; one conversion per block
+  float dr[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  if (Kc < nt) {
+    double a0[4];
+    float hi[4][NB];
+    load_state<NB>(uh, nt, Kc, a0, hi);
+    double off[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) off[c] = a0[c] - sc->mean[c];   // deviation of the cell mean
+#pragma unroll
+    for (int mu = 0; mu < NV; ++mu) {
+      float u[4];
+      eval_fixed<float, NB>(off, hi, vol_xi(NV, mu), vol_eta(NV, mu), u);
+      dr[0] = max_nn(dr[0], fabs(u[0]));
+      dr[1] = max_nn(dr[1], fdot2(u[1], u[1], u[2], u[2]));   // squared: one square root per cell below
+      dr[2] = max_nn(dr[2], fabs(u[3]));
+      dr[3] = max_nn(dr[3], fabs(u[1]));
+      dr[4] = max_nn(dr[4], fabs(u[2]));
+    }
+    // sqrt is monotonic and correctly rounded: sqrt(max) = max(sqrt), bit for bit
+    dr[1] = sqrt(dr[1]);
+  }
+  block_reduce<5>(dr, part_dev + 5 * tile, OpMaxNN());
 }
 
 // ==========================================================================
@@ -434,7 +468,7 @@ __device__ __forceinline__ void edge_jumps_mixed(int I, const MeshDev &m, const 
 // The limiter point set of a P_K cell: the 3 (K + 1) edge Gauss points, then
 // two extra points (the internal nodes of the optimal decomposition for P2,
 // the vertices v1, v2 for P1; with the classical decomposition both extra
-// rows are the weighted edge combination of zxs_extra_points).  LimTab holds,
+// rows are the weighted edge combination u_* of Sec. 4.1).  LimTab holds,
 // per point, psi_1 .. psi_{NB-1} there; the node rows come from the mesh.
 template <int K>
 struct LimTab {
@@ -717,7 +751,7 @@ __device__ __forceinline__ bool limit_screen_mixed(const MeshDev &m, const Phys 
           float d[4];
 #pragma unroll
           for (int c = 0; c < 4; ++c) d[c] = K == 1 ? 0.0f : float(-1.0 / 6.0) * zs[c];
-          if (K == 1) edge_dev<K, 0>(0, hi, d);   // P1: the edge weights sum to one (see zxs_extra_points)
+          if (K == 1) edge_dev<K, 0>(0, hi, d);   // P1: the edge weights sum to one
           ok = passes(d) && ok;
         } else {
 #pragma unroll
@@ -846,7 +880,7 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
           s_vtx[VTX_REC * v + 13][threadIdx.x] = cs;
         });
       }
-      // sigma_q^j = sum_i (beta_i / h_i) A^{k,j} h_i^j sqrt(J) / D_q (see oe_bp_tile)
+      // sigma_q^j = sum_i (beta_i / h_i) A^{k,j} h_i^j sqrt(J) / D_q (see dg_stage_fp64.cuh)
       float sig[4][K + 1];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
