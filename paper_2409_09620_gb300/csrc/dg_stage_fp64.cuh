@@ -22,7 +22,9 @@
 // Measured against one thread per cell with every sum on the FP64 pipe: double
 // Mach reflection, 1,036,800 P2 cells, ms per launch: k_rk 2.37 -> 1.50,
 // k_stats 0.96 -> 1.05, k_oe_bp 1.39 -> 0.90, step 14.16 -> 10.38; isentropic
-// vortex, 2,048 P1 cells, step 250 -> 135 us.
+// vortex, 2,048 P1 cells, step 250 -> 135 us.  Sums, products, reciprocals and
+// square roots as register-only DFMAs (dg_common.cuh): k_rk 1.50 -> 1.41,
+// k_stats 1.05 -> 0.91, k_oe_bp 0.90 -> 0.81, step 10.38 -> 9.42.
 #pragma once
 
 namespace dg {
@@ -106,8 +108,8 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   {
     const int64_t Kl = K0 + lane < nt ? K0 + lane : nt - 1;
     const double ar = m.area[Kl];
-    const double jx = ar * m.jinv[Kl], jy = ar * m.jinv[nt + Kl], ex = ar * m.jinv[2 * nt + Kl],
-                 ey = ar * m.jinv[3 * nt + Kl];
+    const double jx = mul(ar, m.jinv[Kl]), jy = mul(ar, m.jinv[nt + Kl]), ex = mul(ar, m.jinv[2 * nt + Kl]),
+                 ey = mul(ar, m.jinv[3 * nt + Kl]);
 #pragma unroll 1
     for (int p = warp0; p < NV; p += 4) {
       Vec4d u = s_u[p][lane], g1, g2;
@@ -155,7 +157,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       // l_i w_nu / 2: the 1/2 of the LF flux rides on the weight (a power of
       // two).  The two cells of an edge form exactly opposite products.
       const double lw = li * (0.5 * gauss_w(NQ, nu));
-      tv[i * NQ + nu] = lw * fma(-alpha, up - um, fm + fp);
+      tv[i * NQ + nu] = mul(lw, fma(-alpha, sub(up, um), add(fm, fp)));
     }
   }
   __syncthreads();
@@ -205,7 +207,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 #pragma unroll
       for (int l = 0; l < NB; ++l) fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg))), f);
     }
-    const double dta = dt * m.iarea[Kc];
+    const double dta = mul(dt, m.iarea[Kc]);
     const bool first = a == 0.0 && b == 1.0;   // the first stage skips the zero term and the load of u_n
     const bool bad = max(Ev, Ee) >= FX_ENAN;
     double x[NB], xn[NB];
@@ -226,7 +228,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 #pragma unroll
     for (int l = 1; l < NB; ++l) uh.hi[(c * (NB - 1) + (l - 1)) * nt + Kc] = h[l];
   }
-  double mass = live ? m.area[Kc] * h[0] : 0.0;
+  double mass = live ? mul(m.area[Kc], h[0]) : 0.0;
 
   // ---- vertex derivatives of u_h for the OE jumps ------------------------------
   {
@@ -259,7 +261,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       // physical second derivatives (xx, xy, yy) from the reference ones:
       // lane r forms the factors of row r of J^-T H J^-1, shared by the components
       const double p0 = c == 2 ? jy : jx, p1 = c == 2 ? ey : ex, q0 = c == 0 ? jx : jy, q1 = c == 0 ? ex : ey;
-      const double wa = p0 * q0, wb = fdot2(p0, q1, q0, p1), wc = p1 * q1;
+      const double wa = mul(p0, q0), wb = fdot2(p0, q1, q0, p1), wc = mul(p1, q1);
       FxAcc s0{0, 0}, s1{0, 0}, s2{0, 0};
 #pragma unroll
       for (int l = 3; l < NB; ++l) {
@@ -284,17 +286,17 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     const Vec4d u = s_u[warp0][lane];
     double ri = 0.0, cs = INFINITY;
     if (gt0(u.c[0])) {
-      ri = 1.0 / u.c[0];
-      double p = gm1 * fma(-0.5 * fdot2(u.c[1], u.c[1], u.c[2], u.c[2]), ri, u.c[3]);
+      ri = recip(u.c[0]);
+      double p = mul(gm1, fma(half_neg(fdot2(u.c[1], u.c[1], u.c[2], u.c[2])), ri, u.c[3]));
       p = gt0(p) ? p : 0.0;
-      cs = sqrt(gamma * p * ri);
+      cs = root(mul(mul(gamma, p), ri));
     }
     *reinterpret_cast<double2 *>(vdo + (K0 + lane) * VD_CELL + warp0 * VD_STRIDE + 12) = make_double2(ri, cs);
   }
   // block sums of |K| u^(0): the cells of a warp, then the warps in order
   __shared__ double s_m[TPB / 32][4];
 #pragma unroll
-  for (int o = 4; o < 32; o <<= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
+  for (int o = 4; o < 32; o <<= 1) mass = add(mass, __shfl_xor_sync(0xffffffffu, mass, o));
   if (lane < 4) s_m[threadIdx.x >> 5][lane] = mass;
   __syncthreads();
   if (threadIdx.x < 4)
@@ -315,7 +317,7 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
   const int64_t Kc = K0 + lc < nt ? K0 + lc : nt - 1;   // a repeated cell changes no maximum
   double x[NB];
   load_comp<NB>(uh, nt, Kc, c, x);
-  x[0] -= sc->mean[c];
+  x[0] = sub(x[0], sc->mean[c]);
   int mx = 0;
 #pragma unroll
   for (int l = 0; l < NB; ++l) mx = max(mx, fx_abs_hi(x[l]));
@@ -343,7 +345,7 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
   const double d = fx_out((int64_t)top, E);
   const double m1 = fx_out(b1, E), m2 = fx_out(b2, E);
   // rho, |m|, E, |m1|, |m2|; the lanes of the other components hold 0
-  double dr[5] = {c == 0 ? d : 0.0, c == 1 ? sqrt(fdot2(m1, m1, m2, m2)) : 0.0, c == 3 ? d : 0.0, c == 1 ? d : 0.0,
+  double dr[5] = {c == 0 ? d : 0.0, c == 1 ? root(fdot2(m1, m1, m2, m2)) : 0.0, c == 3 ? d : 0.0, c == 1 ? d : 0.0,
                   c == 2 ? d : 0.0};
   block_reduce<5>(dr, part_dev + 5 * tile, OpMaxNN());
 }
@@ -394,13 +396,13 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
         const double *ro = vme + ov * VD_STRIDE, *rx = vnb + xv * VD_STRIDE;
         const double2 go = *reinterpret_cast<const double2 *>(ro + 4 + 2 * c),
                       gx = *reinterpret_cast<const double2 *>(rx + 4 + 2 * c);
-        jv[ev] = ro[c] - rx[c];
-        jg[ev][0] = go.x - gx.x;
-        jg[ev][1] = go.y - gx.y;
+        jv[ev] = sub(ro[c], rx[c]);
+        jg[ev][0] = sub(go.x, gx.x);
+        jg[ev][1] = sub(go.y, gx.y);
       }
       if (K == 2) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) jh[q] = hsi[Kc * 12 + 3 * c + q] - hsi[nb * 12 + 3 * c + q];
+        for (int q = 0; q < 3; ++q) jh[q] = sub(hsi[Kc * 12 + 3 * c + q], hsi[nb * 12 + 3 * c + q]);
       }
       int vv = c & 1 ? (c & 2 ? jn + 1 : i + 2) : (c & 2 ? jn + 2 : i + 1);
       vv = vv >= 3 ? vv - 3 : vv;
@@ -466,13 +468,13 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     for (int ev = 0; ev < 2; ++ev) {
       const double q = rot(jv[ev]), g0 = rot(jg[ev][0]), g1 = rot(jg[ev][1]);
       // 2 J: the 1/2 of the trapezoidal rule moves into A (sqrt(1/2))
-      J[0] = ev == 0 ? q * q : fma(q, q, J[0]);
+      J[0] = ev == 0 ? mul(q, q) : fma(q, q, J[0]);
       J[1] = ev == 0 ? fdot2(g0, g0, g1, g1) : fma(g0, g0, fma(g1, g1, J[1]));
     }
     if (K == 2) {   // the Hessian jump counts at both endpoints
       const double h0 = rot(jh[0]), h1 = rot(jh[1]), h2 = rot(jh[2]);
-      const double f = fma(h0, h0, fma(h1 + h1, h1, h2 * h2));
-      J[K] = f + f;
+      const double f = fma(h0, h0, fma(add(h1, h1), h1, mul(h2, h2)));
+      J[K] = add(f, f);
     }
     const bool finite = is_finite_bits(beta);
     double er[4] = {0.0, 0.0, 0.0, 0.0};
@@ -480,12 +482,12 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     for (int j = 0; j <= K; ++j) {
       const double Jp = __shfl_xor_sync(0xffffffffu, J[j], 3);
       if (mom) J[j] = max_nn(J[j], Jp);   // delta_m = max(delta_mn, delta_mt)
-      const double s = sqrt(J[j]);
+      const double s = root(J[j]);
       // A^{k,j} = (2j + 1) / ((2k - 1) j!); a zero jump adds nothing, also where beta is
       // +inf (a vertex with rho <= 0) and 0 * inf would be NaN
       constexpr double r2 = 0.70710678118654752440;
       const double A = (2.0 * j + 1.0) / ((2.0 * K - 1.0) * (j == 2 ? 2.0 : 1.0)) * r2;
-      er[j] = finite || nonzero_bits(s) ? (A * beta) * s : 0.0;
+      er[j] = finite || nonzero_bits(s) ? mul(A * beta, s) : 0.0;
     }
     if (live) vstore<4>(ej + e * EJ_STRIDE + 4 * c, er);
   }
@@ -535,20 +537,20 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
       const double *er = ej + (int64_t)m.cedge[i * nt + Kc] * EJ_STRIDE + 4 * c;
       const double2 e01 = *reinterpret_cast<const double2 *>(er);
       sig[0] = fma(m.hgeo[(3 + i) * nt + Kc], e01.x, sig[0]);
-      sig[1] += e01.y;
+      sig[1] = add(sig[1], e01.y);
       if (K == 2) sig[K] = fma(m.hgeo[i * nt + Kc], er[2], sig[K]);
     }
     const double iD = sc->invD[c];
     // exact solution of the damping ODE: mode of degree d times exp(-dt sum_{j<=d} sigma^j)
-    const double s = nonzero_bits(iD) ? iD * dt : 0.0;
+    const double s = nonzero_bits(iD) ? mul(iD, dt) : 0.0;
     double sacc = sig[0];
 #pragma unroll
     for (int d = 1; d <= K; ++d) {
-      sacc += sig[d];
-      const double fac = exp_neg(nonzero_bits(iD) ? s * sacc : 0.0);
+      sacc = add(sacc, sig[d]);
+      const double fac = exp_neg(nonzero_bits(iD) ? mul(s, sacc) : 0.0);
 #pragma unroll
       for (int l = 1; l < NB; ++l)
-        if (degree_of(l) == d) x[l] *= fac;
+        if (degree_of(l) == d) x[l] = mul(x[l], fac);
     }
   }
 
