@@ -222,6 +222,14 @@ __device__ __forceinline__ T cfma(double c, T x, T acc) {
   return fma(static_cast<T>(c), x, acc);
 }
 
+// x != 0 on the integer units (true for NaN, false for +0 and -0, as the
+// comparison); on the two words, for a 64-bit test of the bits is compiled to
+// an FP64 comparison
+__device__ __forceinline__ bool nonzero_bits(double x) {
+  return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) != 0u;
+}
+__device__ __forceinline__ bool nonzero_bits(float x) { return (__float_as_int(x) << 1) != 0; }
+
 // ------------------------------------------------------------------------
 // FP64 operations at the cost of a register-only DFMA
 // ------------------------------------------------------------------------
@@ -267,7 +275,7 @@ __device__ __forceinline__ float half_neg(float x) { return -0.5f * x; }
 // 572.  Zero stays zero; outside [2^-895, 2^897) it takes sqrt.
 __device__ __forceinline__ double root(double x) {
   const unsigned ex = (unsigned)__double2hiint(x) >> 20;
-  const bool zero = (__double_as_longlong(x) << 1) == 0;
+  const bool zero = !nonzero_bits(x);
   if (ex - 128u >= 1792u && !zero) return sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -325,12 +333,12 @@ __device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }
 // damping away from discontinuities, take a 7-FMA Taylor polynomial
 // (dg_math.h); the rest the library exp; FP32 the fast intrinsic, whose
 // error (a few ulp) is far below the mixed form's FP32 arithmetic error
-__device__ __forceinline__ double exp_neg(double x) { return x <= EXP_NEG_SMALL_MAX ? exp_neg_small(x) : exp(-x); }
+__device__ __forceinline__ double exp_neg(double x) {
+  static_assert(EXP_NEG_SMALL_MAX == 0.00390625, "the high word below");
+  // x < 2^-8 on the integer units (x >= 0, or NaN, whose high word is above)
+  return (unsigned)__double2hiint(x) < 0x3f700000u ? exp_neg_small(x) : exp(-x);
+}
 __device__ __forceinline__ float exp_neg(float x) { return __expf(-x); }
-
-// x != 0 on the integer units (true for NaN, false for +0 and -0, as the comparison)
-__device__ __forceinline__ bool nonzero_bits(double x) { return (__double_as_longlong(x) << 1) != 0; }
-__device__ __forceinline__ bool nonzero_bits(float x) { return (__float_as_int(x) << 1) != 0; }
 
 // F(u) . n and the spectral radius |v.n| + c (+inf for rho <= 0) with one reciprocal
 template <typename T>

@@ -70,14 +70,17 @@ FX_HD double fx_make(int hi, unsigned lo) {
   return x;
 #endif
 }
-// 127 + floor(log2 |r|), 0 for r = 0: the exponent field of r rounded toward
-// zero to FP32 (the conversion runs beside the integer pipe)
-FX_HD int fx_log2_127(int64_t r) {
+// 127 + floor(log2 a), 0 for a = 0, from the exponent field of the leading 32
+// bits rounded toward zero to FP32 (a 64-bit conversion would run on the FP64
+// pipe, 64 cycles)
+FX_HD int fx_log2_127(uint64_t a) {
+  const unsigned hi = (unsigned)(a >> 32), t = hi ? hi : (unsigned)a;
 #ifdef __CUDA_ARCH__
-  return (__float_as_int(__ll2float_rz(r)) >> 23) & 0xff;
+  const int e = __float_as_int(__uint2float_rz(t)) >> 23;
 #else
-  return r == 0 ? 0 : 190 - __builtin_clzll((uint64_t)(r < 0 ? -r : r));
+  const int e = t == 0 ? 0 : 158 - __builtin_clz(t);
 #endif
+  return hi ? e + 32 : e;
 }
 
 // constant: c = (h 2^29 + l) 2^-56, |l| <= 2^28
@@ -114,25 +117,52 @@ FX_HD Fx fx_from(double x, int E) {
   return Fx{(int)(v >> FX_LIMB) * g, ((int)v & ((1 << FX_LIMB) - 1)) * g};
 }
 
+// s + a b as one 32 x 32 + 64 bit multiply-add (left to itself the compiler
+// multiplies sign-extended 64-bit values, several instructions each)
+FX_HD void fx_mad(int64_t &s, int a, int b) {
+#ifdef __CUDA_ARCH__
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+#else
+  s += (int64_t)a * b;
+#endif
+}
 // sum of products, exact but for the dropped l l
 struct FxAcc {
   int64_t a, b;
 };
 FX_HD void fx_mac(FxAcc &s, FxC c, Fx x) {
   if (c.h != 0) {
-    s.a += (int64_t)c.h * x.h;
-    s.b += (int64_t)c.h * x.l;
+    fx_mad(s.a, c.h, x.h);
+    fx_mad(s.b, c.h, x.l);
   }
-  if (c.l != 0) s.b += (int64_t)c.l * x.h;
+  if (c.l != 0) fx_mad(s.b, c.l, x.h);
+}
+// run-time coefficient c = x 2^k (|c| < 4) in the format of a constant, as fx_mac takes it
+FX_HD Fx fx_coef(double x, int k) {
+  return (fx_hiword(x) & 0x7ff00000) == 0 ? Fx{0, 0} : fx_from(x, 1024 - k);
+}
+FX_HD void fx_mac(FxAcc &s, Fx c, Fx x) {
+  fx_mad(s.a, c.h, x.h);
+  fx_mad(s.b, c.h, x.l);
+  fx_mad(s.b, c.l, x.h);
+}
+// differences and sums of two values of a block, one bit longer than a value
+FX_HD Fx operator-(Fx p, Fx q) { return Fx{p.h - q.h, p.l - q.l}; }
+FX_HD Fx operator+(Fx p, Fx q) { return Fx{p.h + q.h, p.l + q.l}; }
+// a sum back as a value, shifted right by s (its block's exponent grows by s); |r| < 2^(58 + s)
+FX_HD Fx fx_value(int64_t r, int s) {
+  const int64_t v = r >> s;
+  return Fx{(int)(v >> FX_LIMB), (int)v & ((1 << FX_LIMB) - 1)};
 }
 FX_HD int64_t fx_sum(const FxAcc &s) {
   return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + (s.b >> (FX_ONE - FX_LIMB));
 }
 // r 2^(E - 1080) rounded to nearest; |r| < 2^63
 FX_HD double fx_to(int64_t r, int E) {
-  const int e8 = fx_log2_127(r);
   const int64_t g = r >> 63;
-  const uint64_t m = (uint64_t)(r ^ g) << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62 (|r| - 1 for r < 0)
+  const uint64_t a = (uint64_t)(r ^ g);   // |r| (|r| - 1 for r < 0)
+  const int e8 = fx_log2_127(a);
+  const uint64_t m = a << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62
   const uint64_t q = (m + 512u) >> 10;
   int f = E + e8 - 185;                // exponent field, less the one that q carries
   f = f < 0 ? 0 : (f > 2046 ? 2046 : f);

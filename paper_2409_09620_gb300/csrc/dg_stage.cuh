@@ -22,8 +22,8 @@ namespace dg {
 // Resident blocks per SM requested from the register allocator (FP32 / FP64
 // instantiations).  Higher occupancy hides the latency of the neighbour
 // gathers and of the FP64 pipe better than the few spilled registers cost.
-// FP64, 1,036,800 P2 cells, ms per launch of k_rk / k_stats / k_oe_bp: 4, 4, 4
-// blocks 1.60 / 1.13 / 0.90, 6, 6, 7 blocks 1.50 / 1.05 / 0.90, 8 each the same.
+// FP64, 1,036,800 P2 cells, ms per launch: k_rk 1.13 with 5 blocks, 1.12 with 6,
+// 1.09 with 7 and 8; k_stats and k_oe_bp, bound by the FP64 pipe, the same from 5 on.
 #ifndef RK_MINB_F
 #define RK_MINB_F 4
 #endif
@@ -34,7 +34,7 @@ namespace dg {
 #define OEBP_MINB_F 4
 #endif
 #ifndef RK_MINB_D
-#define RK_MINB_D 6
+#define RK_MINB_D 7
 #endif
 #ifndef STATS_MINB_D
 #define STATS_MINB_D 6

@@ -24,7 +24,10 @@
 // k_stats 0.96 -> 1.05, k_oe_bp 1.39 -> 0.90, step 14.16 -> 10.38; isentropic
 // vortex, 2,048 P1 cells, step 250 -> 135 us.  Sums, products, reciprocals and
 // square roots as register-only DFMAs (dg_common.cuh): k_rk 1.50 -> 1.41,
-// k_stats 1.05 -> 0.91, k_oe_bp 0.90 -> 0.81, step 10.38 -> 9.42.
+// k_stats 1.05 -> 0.91, k_oe_bp 0.90 -> 0.81, step 10.38 -> 9.42.  LF terms and
+// vertex derivatives of k_rk in fixed point, no 64-bit conversion or comparison
+// left on the FP64 pipe: k_rk 1.41 -> 1.09, k_stats 0.91 -> 0.82, k_oe_bp
+// 0.81 -> 0.69, step 9.42 -> 7.81.
 #pragma once
 
 namespace dg {
@@ -119,20 +122,30 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     }
   }
   // ---- edge fluxes of this component -------------------------------------------
-  double tv[3 * NQ];
+  // y = l_i ((F(u-) + F(u+)) . n - alpha (u+ - u-)) in fixed point: the traces of
+  // an edge share one block, its fluxes another, and l_i and alpha l_i scaled to
+  // the larger of the two products are run-time coefficients.  Beside a
+  // conversion per trace value this takes 6 integer multiply-adds per point
+  // where the FP64 pipe took 4 operations (64 cycles each).  The two cells of
+  // an edge form opposite values to 2^-58 of the larger product.
+  int64_t ry[3 * NQ];
+  int ei[3];
+  bool bad = false;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const int32_t cn = m.conn[i * nt + Kc];
     const double li = m.len[i * nt + Kc];
+    double um[NQ], fm[NQ], up[NQ], fp[NQ];
+    int mu = 0, mf = 0;
 #pragma unroll
     for (int nu = 0; nu < NQ; ++nu) {
       const double *po = tr + ((Kc * 3 + i) * NQ + nu) * 8;
-      const double um = po[c], fm = po[4 + c];
-      double up, fp;
+      um[nu] = po[c];
+      fm[nu] = po[4 + c];
       if (cn >= 0) {
         const double *pn = tr + (((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)) * 8;
-        up = pn[c];
-        fp = -pn[4 + c];   // F(u+).n of this cell's normal
+        up[nu] = pn[c];
+        fp[nu] = -pn[4 + c];   // F(u+).n of this cell's normal
       } else {
         const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
         double px = 0.0, py = 0.0, ow[4], av[4], gh[4], gf[4];
@@ -151,18 +164,30 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         }
         ghost_state(-cn, ow, av, nx, ny, px, py, t_in, ph, gh);
         flux_dir(gh, nx, ny, gm1, gf);
-        up = pick4(gh, c);
-        fp = pick4(gf, c);
+        up[nu] = pick4(gh, c);
+        fp[nu] = pick4(gf, c);
       }
-      // l_i w_nu / 2: the 1/2 of the LF flux rides on the weight (a power of
-      // two).  The two cells of an edge form exactly opposite products.
-      const double lw = li * (0.5 * gauss_w(NQ, nu));
-      tv[i * NQ + nu] = mul(lw, fma(-alpha, sub(up, um), add(fm, fp)));
+      mu = max(mu, max(fx_abs_hi(um[nu]), fx_abs_hi(up[nu])));
+      mf = max(mf, max(fx_abs_hi(fm[nu]), fx_abs_hi(fp[nu])));
+    }
+    const double al = mul(alpha, li);
+    const int Eu = fx_exp(mu), Ef = fx_exp(mf);
+    // both coefficients are below 1: x < 2^(exponent field - 1022)
+    ei[i] = max(Ef + (fx_abs_hi(li) >> 20), Eu + (fx_abs_hi(al) >> 20)) - 1022;
+    const Fx cf = fx_coef(li, Ef - ei[i]), cu = fx_coef(-al, Eu - ei[i]);
+    bad = bad || max(Eu, Ef) >= FX_ENAN || (fx_abs_hi(al) >> 20) >= FX_ENAN;
+#pragma unroll
+    for (int nu = 0; nu < NQ; ++nu) {
+      FxAcc y{0, 0};
+      fx_mac(y, cf, fx_from(fm[nu], Ef) + fx_from(fp[nu], Ef));
+      fx_mac(y, cu, fx_from(up[nu], Eu) - fx_from(um[nu], Eu));
+      ry[i * NQ + nu] = fx_sum(y);   // below 2^60
     }
   }
   __syncthreads();
   // ---- quadrature sums, mass inverse, SSP-RK combination ---------------------------
-  // volume |K| sum_mu w_mu F . grad Psi_l, edges - sum_i l_i sum_nu w_nu Fhat Psi_l
+  // volume |K| sum_mu w_mu F . grad Psi_l, edges - sum_i l_i sum_nu w_nu Fhat Psi_l, both with
+  // the mass inverse (and the 1/2 of the LF flux) on their coefficients
   double h[NB];
   {
     int64_t rv[NB];
@@ -186,30 +211,28 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         const Fx f1 = fx_from(g1[mu], Ev), f2 = fx_from(g2[mu], Ev);
 #pragma unroll
         for (int l = 1; l < NB; ++l) {
-          fx_mac(s[l], fxc(w * psi_x(l, xi, eta)), f1);
-          fx_mac(s[l], fxc(w * psi_y(l, xi, eta)), f2);
+          fx_mac(s[l], fxc(w * psi_x(l, xi, eta) * inv_mass_c(l)), f1);
+          fx_mac(s[l], fxc(w * psi_y(l, xi, eta) * inv_mass_c(l)), f2);
         }
       }
 #pragma unroll
       for (int l = 1; l < NB; ++l) rv[l] = fx_sum(s[l]);
     }
-    int mx = 0;
-#pragma unroll
-    for (int p = 0; p < 3 * NQ; ++p) mx = max(mx, fx_abs_hi(tv[p]));
-    const int Ee = fx_exp(mx);
+    const int Ee = max(max(ei[0], ei[1]), ei[2]) + 2;
     FxAcc s[NB];
 #pragma unroll
     for (int l = 0; l < NB; ++l) s[l] = FxAcc{0, 0};
 #pragma unroll
     for (int p = 0; p < 3 * NQ; ++p) {
-      const double sg = gauss_s(NQ, p % NQ);
-      const Fx f = fx_from(tv[p], Ee);
+      const double sg = gauss_s(NQ, p % NQ), w = 0.5 * gauss_w(NQ, p % NQ);
+      const Fx f = fx_value(ry[p], min(Ee - ei[p / NQ], 63));
 #pragma unroll
-      for (int l = 0; l < NB; ++l) fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg))), f);
+      for (int l = 0; l < NB; ++l)
+        fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w * inv_mass_c(l)), f);
     }
     const double dta = mul(dt, m.iarea[Kc]);
     const bool first = a == 0.0 && b == 1.0;   // the first stage skips the zero term and the load of u_n
-    const bool bad = max(Ev, Ee) >= FX_ENAN;
+    bad = bad || Ev >= FX_ENAN;
     double x[NB], xn[NB];
     load_comp<NB>(v, nt, Kc, c, x);
     if (!first) load_comp<NB>(un, nt, Kc, c, xn);
@@ -219,7 +242,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       int64_t r = fx_sum(s[l]);
       if (l > 0) r = fx_add(rv[l], Ev, r, Ee, E);
       const double d = bad ? NAN : fx_to(r, E);
-      const double L = fma(dta * inv_mass_c(l), d, x[l]);
+      const double L = fma(dta, d, x[l]);
       h[l] = first ? L : fdot2(a, xn[l], b, L);
     }
   }
@@ -231,37 +254,53 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   double mass = live ? mul(m.area[Kc], h[0]) : 0.0;
 
   // ---- vertex derivatives of u_h for the OE jumps ------------------------------
+  // values, then the reference derivatives turned by J^-1, all in fixed point
+  // (coefficients of derivatives reach 48: as c / 64; the entries of J^-1 share a block)
   {
-    const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
-    Fx f[NB];
+    Fx f[NB], J[2][2];   // J[d][0] = dxi/dx_d, J[d][1] = deta/dx_d
     const int E = fx_block<NB>(h, f);
+    bad = bad || E >= FX_ENAN;
+    int EJ;
+    {
+      const double j0 = m.jinv[Kc], j1 = m.jinv[nt + Kc], j2 = m.jinv[2 * nt + Kc], j3 = m.jinv[3 * nt + Kc];
+      EJ = fx_exp(max(max(fx_abs_hi(j0), fx_abs_hi(j1)), max(fx_abs_hi(j2), fx_abs_hi(j3)))) - 1022;   // |j| < 2^EJ
+      J[0][0] = fx_coef(j0, -EJ);
+      J[1][0] = fx_coef(j1, -EJ);
+      J[0][1] = fx_coef(j2, -EJ);
+      J[1][1] = fx_coef(j3, -EJ);
+    }
+    // p dxi/dx_d + q deta/dx_d as a sum
+    auto turn = [&](int d, Fx p, Fx q) {
+      FxAcc t{0, 0};
+      fx_mac(t, J[d][0], p);
+      fx_mac(t, J[d][1], q);
+      return fx_sum(t);
+    };
     double *vo = vdo + Kc * VD_CELL;
-    double gx = 0.0, ge = 0.0;
+    double gx = 0.0, gy = 0.0;
 #pragma unroll
     for (int vv = 0; vv < 3; ++vv) {
       const double val = fx_out(fx_point<NB>(f, vert_xi(vv), vert_eta(vv)), E);
       if (K == 2 || vv == 0) {   // P1 has one gradient
-        FxAcc sx{0, 0}, se{0, 0};   // derivative coefficients reach 48: as c / 64
+        FxAcc sx{0, 0}, se{0, 0};
 #pragma unroll
         for (int l = 1; l < NB; ++l) {
           fx_mac(sx, fxc(psi_x(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
           fx_mac(se, fxc(psi_y(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
         }
-        gx = fx_out(fx_sum(sx), E + 6);
-        ge = fx_out(fx_sum(se), E + 6);
+        // the coefficients of a sum add up to at most 37 / 64: the sums are values as they are
+        const Fx px = fx_value(fx_sum(sx), 0), pe = fx_value(fx_sum(se), 0);
+        gx = bad ? NAN : fx_to(turn(0, px, pe), E + 6 + EJ);
+        gy = bad ? NAN : fx_to(turn(1, px, pe), E + 6 + EJ);
       }
-      s_u[vv][lc].c[c] = val;   // this warp's slots; read after the barrier below
+      s_u[vv][lc].c[c] = val;   // this thread's slot; read after the barrier below
       if (live) {
         double *rec = vo + vv * VD_STRIDE;
         rec[c] = val;
-        *reinterpret_cast<double2 *>(rec + 4 + 2 * c) = make_double2(fdot2(gx, jx, ge, ex), fdot2(gx, jy, ge, ey));
+        *reinterpret_cast<double2 *>(rec + 4 + 2 * c) = make_double2(gx, gy);
       }
     }
     if (K == 2) {
-      // physical second derivatives (xx, xy, yy) from the reference ones:
-      // lane r forms the factors of row r of J^-T H J^-1, shared by the components
-      const double p0 = c == 2 ? jy : jx, p1 = c == 2 ? ey : ex, q0 = c == 0 ? jx : jy, q1 = c == 0 ? ex : ey;
-      const double wa = mul(p0, q0), wb = fdot2(p0, q1, q0, p1), wc = mul(p1, q1);
       FxAcc s0{0, 0}, s1{0, 0}, s2{0, 0};
 #pragma unroll
       for (int l = 3; l < NB; ++l) {
@@ -269,14 +308,14 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         fx_mac(s1, fxc(psi_2(l, 1) / 64.0), f[l]);
         fx_mac(s2, fxc(psi_2(l, 2) / 64.0), f[l]);
       }
-      const double hxx = fx_out(fx_sum(s0), E + 6), hxe = fx_out(fx_sum(s1), E + 6), hee = fx_out(fx_sum(s2), E + 6);
+      // (xx, xy, yy) = J^-T H J^-1 row by row; a turn at most doubles a value
+      const Fx hxx = fx_value(fx_sum(s0), 0), hxe = fx_value(fx_sum(s1), 0), hee = fx_value(fx_sum(s2), 0);
+      const Fx ax = fx_value(turn(0, hxx, hxe), 1), bx = fx_value(turn(0, hxe, hee), 1);
+      const Fx ay = fx_value(turn(1, hxx, hxe), 1), by = fx_value(turn(1, hxe, hee), 1);
+      const int64_t d2[3] = {turn(0, ax, bx), turn(1, ax, bx), turn(1, ay, by)};
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const double ga = __shfl_sync(0xffffffffu, wa, (lane & ~3) + r), gb = __shfl_sync(0xffffffffu, wb, (lane & ~3) + r),
-                     gc = __shfl_sync(0xffffffffu, wc, (lane & ~3) + r);
-        const double d2 = fma(hxx, ga, fdot2(hxe, gb, hee, gc));
-        if (live) hso[Kc * 12 + 3 * c + r] = d2;
-      }
+      for (int r = 0; r < 3; ++r)
+        if (live) hso[Kc * 12 + 3 * c + r] = bad ? NAN : fx_to(d2[r], E + 7 + 2 * EJ);
     }
   }
   __syncthreads();
@@ -570,7 +609,7 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
     for (int l = 1; l < NB; ++l) S += abs_f32_down(x[l]);
     const float D = fmaf(4.00002f, S, 1e-37f), A = abs_f32_down(x[0]);
     const float B = fmaf(1.000002f, A, D);              // upper bound of |component|
-    const float lo = x[0] > 0.0 ? A - D : -1.0f;        // lower bound of rho, E
+    const float lo = gt0(x[0]) ? A - D : -1.0f;         // lower bound of rho, E
     const float r_lo = __shfl_sync(FULL, lo, q0), r_hi = __shfl_sync(FULL, B, q0);
     const float M_hi = __shfl_sync(FULL, B, q0 + 1) + __shfl_sync(FULL, B, q0 + 2);
     const float E_lo = __shfl_sync(FULL, lo, q0 + 3), E_hi = __shfl_sync(FULL, B, q0 + 3);

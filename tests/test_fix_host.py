@@ -38,7 +38,11 @@ int main() {
     for (int i = n - 1; i >= 0; --i) fx_mac(s1, fxc(c[i]), fx_from(x[i], E));
     int E2;
     const int64_t r2 = fx_add(fx_sum(s), E, fx_sum(s), E - 40, E2);
-    std::printf("%d %a %d %a\n", E, fx_to(fx_sum(s), E), (int)(fx_sum(s) == fx_sum(s1)), fx_to(r2, E2));
+    FxAcc s3{0, 0};   // the halved constants as run-time coefficients
+    for (int i = 0; i < n; ++i) fx_mac(s3, fx_coef(c[i], -1), fx_from(x[i], E));
+    const Fx w = fx_value(fx_sum(s3), 6);
+    std::printf("%d %a %d %a %a %d\n", E, fx_to(fx_sum(s), E), (int)(fx_sum(s) == fx_sum(s1)), fx_to(r2, E2),
+                fx_to(fx_sum(s3), E + 1), (int)((((int64_t)w.h << FX_LIMB) + w.l) == fx_sum(s3) >> 6 && w.l >= 0));
   }
   return 0;
 }
@@ -61,7 +65,8 @@ def driver(tmp_path_factory):
 def _run(exe, sums):
     text = "\n".join(" ".join([str(len(s))] + [f"{float(c).hex()} {float(x).hex()}" for c, x in s]) for s in sums)
     out = subprocess.run([str(exe)], input=text + "\n", capture_output=True, text=True, check=True).stdout.split("\n")
-    return [(int(a), float.fromhex(b), int(o), float.fromhex(d)) for a, b, o, d in (line.split() for line in out if line)]
+    return [(int(a), float.fromhex(b), int(o), float.fromhex(d), float.fromhex(e), int(v))
+            for a, b, o, d, e, v in (line.split() for line in out if line)]
 
 
 def _sums(kind, rng, count=300):
@@ -87,7 +92,7 @@ def _sums(kind, rng, count=300):
 @pytest.mark.parametrize("kind", ["plain", "spread", "cancel", "whole", "scale", "edge"])
 def test_sum_within_the_format_bound(driver, kind):
     sums = _sums(kind, np.random.default_rng([3, len(kind)]))
-    for s, (E, r, same, r2) in zip(sums, _run(driver, sums)):
+    for s, (E, r, same, r2, r3, split) in zip(sums, _run(driver, sums)):
         exact = sum((Fraction(c) * Fraction(x) for c, x in s), Fraction(0))
         B = Fraction(2) ** (E - 1022)
         tol = B * Fraction(8 * len(s) + 2, 2 ** 58) + abs(exact) / 2 ** 53
@@ -97,6 +102,10 @@ def test_sum_within_the_format_bound(driver, kind):
             assert Fraction(r) == exact
         # the sum of two blocks 40 exponents apart: one more unit each, of the larger block's
         assert abs(Fraction(r2) - exact * (1 + Fraction(1, 2 ** 40))) <= 2 * tol + B / 2 ** 56
+        # run-time coefficients c / 2 are truncated at 2^-56, their low limbs reach 2^29, and the
+        # sum is doubled: the terms of the bound above are 4, 2 * 4 and 2 * 4 units
+        assert abs(Fraction(r3) - exact) <= B * Fraction(20 * len(s) + 4, 2 ** 58) + abs(exact) / 2 ** 53
+        assert split == 1
 
 
 def test_zeros_and_subnormals(driver):
@@ -107,7 +116,7 @@ def test_zeros_and_subnormals(driver):
 
 def test_tiny_block_keeps_its_absolute_bound(driver):
     # the block exponent stops at 64: one unit is 2^-1016
-    (E, r, _, _), = _run(driver, [[(2.0, 1e-300), (1.0, 0.0)]])
+    (E, r, *_), = _run(driver, [[(2.0, 1e-300), (1.0, 0.0)]])
     assert E == 64 and abs(Fraction(r) - 2 * Fraction(1e-300)) <= Fraction(18, 2 ** 1016)
 
 
