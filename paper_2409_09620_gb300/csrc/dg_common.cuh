@@ -11,9 +11,10 @@
 //   neighbours' modal states instead, see dg_stage_mixed.cuh):
 //             tr[nt][3][Q][8]  traces of the stage input at edge Gauss points:
 //                              u (4) and F(u).n_i (4), written by the cell that owns them
-//             vd[nt][3][16]    value (4), physical gradient (8), 1/rho and sound speed
-//                              of u_h at each vertex (2 padding values)
-//             hs[nt][12]       physical Hessian (xx, xy, yy) of u_h per component (P2)
+//             vd[nt][52]       u_h at the three vertices, [3][16]: value (4) and physical
+//                              gradient (8) in fixed point, 1/rho, sound speed and momentum
+//                              in FP64; then the blocks' exponents per component (4)
+//             hs[nt][12]       physical Hessian (xx, xy, yy) of u_h per component (P2), fixed point
 //             ej[ne][16]       per edge: the OE jump terms of each component
 // The mixed form's kernels are one thread per cell, the FP64 form's four lanes
 // per cell; reductions are per-block partials reduced in a fixed order, so
@@ -68,9 +69,13 @@ constexpr int TR_STRIDE = 8;
 // per-edge OE record ej[ne][4][4]: A^{k,j} beta sqrt(J) of the trapezoidal jump
 // sums J, per component and derivative order j = 0..k (one padding value)
 constexpr int EJ_STRIDE = 16;
-// per-cell vertex record vd[nt][3][VD_STRIDE]: value (4), gradient (8), 1/rho, sound speed
+// per-cell vertex record vd[nt][VD_CELL]: per vertex VD_STRIDE values (value and
+// gradient of component c at c and 4 + 2 c as limb pairs of dg_fix.cuh; 1/rho,
+// sound speed, m1, m2), then per component the exponents of its values, and of
+// its gradients and Hessian, as two and one 16-bit numbers
 constexpr int VD_STRIDE = 16;
-constexpr int VD_CELL = 3 * VD_STRIDE;
+constexpr int VD_EXP = 3 * VD_STRIDE;
+constexpr int VD_CELL = VD_EXP + 4;
 
 // 16-byte vector loads and stores of N consecutive values (N a multiple of 16/sizeof(T))
 template <typename T> struct Vec16;

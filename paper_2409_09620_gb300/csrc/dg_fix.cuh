@@ -146,14 +146,15 @@ FX_HD void fx_mac(FxAcc &s, Fx c, Fx x) {
   fx_mad(s.b, c.h, x.l);
   fx_mad(s.b, c.l, x.h);
 }
-// differences and sums of two values of a block, one bit longer than a value
+// difference of two values of a block, one bit longer than a value
 FX_HD Fx operator-(Fx p, Fx q) { return Fx{p.h - q.h, p.l - q.l}; }
-FX_HD Fx operator+(Fx p, Fx q) { return Fx{p.h + q.h, p.l + q.l}; }
 // a sum back as a value, shifted right by s (its block's exponent grows by s); |r| < 2^(58 + s)
 FX_HD Fx fx_value(int64_t r, int s) {
   const int64_t v = r >> s;
   return Fx{(int)(v >> FX_LIMB), (int)v & ((1 << FX_LIMB) - 1)};
 }
+// a value as one integer
+FX_HD int64_t fx_join(Fx x) { return (int64_t)x.h * (1LL << FX_LIMB) + x.l; }
 FX_HD int64_t fx_sum(const FxAcc &s) {
   return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + (s.b >> (FX_ONE - FX_LIMB));
 }

@@ -23,7 +23,8 @@ namespace dg {
 // instantiations).  Higher occupancy hides the latency of the neighbour
 // gathers and of the FP64 pipe better than the few spilled registers cost.
 // FP64, 1,036,800 P2 cells, ms per launch: k_rk 1.13 with 5 blocks, 1.12 with 6,
-// 1.09 with 7 and 8; k_stats and k_oe_bp, bound by the FP64 pipe, the same from 5 on.
+// 1.09 with 7 and 8; k_stats 0.66 with 6, 0.61 with 7, 0.58 with 8; k_oe_bp the
+// same from 5 on (P1 1 % faster with 8).
 #ifndef RK_MINB_F
 #define RK_MINB_F 4
 #endif
@@ -37,10 +38,10 @@ namespace dg {
 #define RK_MINB_D 7
 #endif
 #ifndef STATS_MINB_D
-#define STATS_MINB_D 6
+#define STATS_MINB_D 8
 #endif
 #ifndef OEBP_MINB_D
-#define OEBP_MINB_D 7
+#define OEBP_MINB_D 8
 #endif
 
 // A cell's state.  The FP64 form keeps the modes component- and mode-major
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D
 // OE statistics of the tile's cells and the jump data of the edges it owns
 template <int K, typename Real>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_MINB_D)
-    k_stats(MeshDev m, Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
+    k_stats(const __grid_constant__ MeshDev m, const __grid_constant__ Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
             const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out) {
   if (!sc->active) return;
   stats_tile<K, Real>(m, uh, part_dev, sc, blockIdx.x);

@@ -27,7 +27,9 @@
 // k_stats 1.05 -> 0.91, k_oe_bp 0.90 -> 0.81, step 10.38 -> 9.42.  LF terms and
 // vertex derivatives of k_rk in fixed point, no 64-bit conversion or comparison
 // left on the FP64 pipe: k_rk 1.41 -> 1.09, k_stats 0.91 -> 0.82, k_oe_bp
-// 0.81 -> 0.69, step 9.42 -> 7.81.
+// 0.81 -> 0.69, step 9.42 -> 7.81.  OE jumps in fixed point from limb records, no
+// negated doubles (each an FP64 operation): k_rk 1.09 -> 0.97, k_stats
+// 0.82 -> 0.58, step 7.81 -> 6.71.
 #pragma once
 
 namespace dg {
@@ -135,7 +137,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   for (int i = 0; i < 3; ++i) {
     const int32_t cn = m.conn[i * nt + Kc];
     const double li = m.len[i * nt + Kc];
-    double um[NQ], fm[NQ], up[NQ], fp[NQ];
+    double um[NQ], fm[NQ], up[NQ], fn[NQ];   // fn = - F(u+).n (a negated double would be an FP64 operation)
     int mu = 0, mf = 0;
 #pragma unroll
     for (int nu = 0; nu < NQ; ++nu) {
@@ -145,7 +147,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       if (cn >= 0) {
         const double *pn = tr + (((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)) * 8;
         up[nu] = pn[c];
-        fp[nu] = -pn[4 + c];   // F(u+).n of this cell's normal
+        fn[nu] = pn[4 + c];   // the neighbour's normal is the negative
       } else {
         const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
         double px = 0.0, py = 0.0, ow[4], av[4], gh[4], gf[4];
@@ -165,22 +167,22 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         ghost_state(-cn, ow, av, nx, ny, px, py, t_in, ph, gh);
         flux_dir(gh, nx, ny, gm1, gf);
         up[nu] = pick4(gh, c);
-        fp[nu] = pick4(gf, c);
+        fn[nu] = -pick4(gf, c);
       }
       mu = max(mu, max(fx_abs_hi(um[nu]), fx_abs_hi(up[nu])));
-      mf = max(mf, max(fx_abs_hi(fm[nu]), fx_abs_hi(fp[nu])));
+      mf = max(mf, max(fx_abs_hi(fm[nu]), fx_abs_hi(fn[nu])));
     }
     const double al = mul(alpha, li);
     const int Eu = fx_exp(mu), Ef = fx_exp(mf);
     // both coefficients are below 1: x < 2^(exponent field - 1022)
     ei[i] = max(Ef + (fx_abs_hi(li) >> 20), Eu + (fx_abs_hi(al) >> 20)) - 1022;
-    const Fx cf = fx_coef(li, Ef - ei[i]), cu = fx_coef(-al, Eu - ei[i]);
+    const Fx cf = fx_coef(li, Ef - ei[i]), cu = fx_coef(al, Eu - ei[i]);
     bad = bad || max(Eu, Ef) >= FX_ENAN || (fx_abs_hi(al) >> 20) >= FX_ENAN;
 #pragma unroll
     for (int nu = 0; nu < NQ; ++nu) {
       FxAcc y{0, 0};
-      fx_mac(y, cf, fx_from(fm[nu], Ef) + fx_from(fp[nu], Ef));
-      fx_mac(y, cu, fx_from(up[nu], Eu) - fx_from(um[nu], Eu));
+      fx_mac(y, cf, fx_from(fm[nu], Ef) - fx_from(fn[nu], Ef));
+      fx_mac(y, cu, fx_from(um[nu], Eu) - fx_from(up[nu], Eu));
       ry[i * NQ + nu] = fx_sum(y);   // below 2^60
     }
   }
@@ -276,11 +278,12 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       fx_mac(t, J[d][1], q);
       return fx_sum(t);
     };
+    // stored as limb pairs (FP64 would be rounded here and taken apart again in K2)
     double *vo = vdo + Kc * VD_CELL;
-    double gx = 0.0, gy = 0.0;
+    Fx gx{0, 0}, gy{0, 0};
 #pragma unroll
     for (int vv = 0; vv < 3; ++vv) {
-      const double val = fx_out(fx_point<NB>(f, vert_xi(vv), vert_eta(vv)), E);
+      const int64_t val = fx_point<NB>(f, vert_xi(vv), vert_eta(vv));   // below 11 * 2^58
       if (K == 2 || vv == 0) {   // P1 has one gradient
         FxAcc sx{0, 0}, se{0, 0};
 #pragma unroll
@@ -288,18 +291,25 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
           fx_mac(sx, fxc(psi_x(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
           fx_mac(se, fxc(psi_y(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
         }
-        // the coefficients of a sum add up to at most 37 / 64: the sums are values as they are
+        // the coefficients of a sum add up to at most 37 / 64 and a turn at most doubles
+        // it: below 2^59, limbs with a bit to spare
         const Fx px = fx_value(fx_sum(sx), 0), pe = fx_value(fx_sum(se), 0);
-        gx = bad ? NAN : fx_to(turn(0, px, pe), E + 6 + EJ);
-        gy = bad ? NAN : fx_to(turn(1, px, pe), E + 6 + EJ);
+        gx = fx_value(turn(0, px, pe), 0);
+        gy = fx_value(turn(1, px, pe), 0);
       }
-      s_u[vv][lc].c[c] = val;   // this thread's slot; read after the barrier below
+      s_u[vv][lc].c[c] = fx_out(val, E);   // this thread's slot; read after the barrier below
       if (live) {
         double *rec = vo + vv * VD_STRIDE;
-        rec[c] = val;
-        *reinterpret_cast<double2 *>(rec + 4 + 2 * c) = make_double2(gx, gy);
+        const Fx v2 = fx_value(val, 2);   // below 2^59.5
+        *reinterpret_cast<int2 *>(rec + c) = make_int2(v2.h, v2.l);
+        *reinterpret_cast<int4 *>(rec + 4 + 2 * c) = make_int4(gx.h, gx.l, gy.h, gy.l);
       }
     }
+    // exponents of the values, gradients (c / 64, J^-1) and Hessians (one shift more)
+    if (live)
+      *reinterpret_cast<short4 *>(vo + VD_EXP + c) =
+          bad ? make_short4(FX_ENAN, FX_ENAN, FX_ENAN, 0)
+              : make_short4((short)(E + 2), (short)(E + 6 + EJ), (short)(E + 7 + 2 * EJ), 0);
     if (K == 2) {
       FxAcc s0{0, 0}, s1{0, 0}, s2{0, 0};
 #pragma unroll
@@ -308,14 +318,16 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         fx_mac(s1, fxc(psi_2(l, 1) / 64.0), f[l]);
         fx_mac(s2, fxc(psi_2(l, 2) / 64.0), f[l]);
       }
-      // (xx, xy, yy) = J^-T H J^-1 row by row; a turn at most doubles a value
+      // (xx, xy, yy) = J^-T H J^-1 row by row
       const Fx hxx = fx_value(fx_sum(s0), 0), hxe = fx_value(fx_sum(s1), 0), hee = fx_value(fx_sum(s2), 0);
       const Fx ax = fx_value(turn(0, hxx, hxe), 1), bx = fx_value(turn(0, hxe, hee), 1);
       const Fx ay = fx_value(turn(1, hxx, hxe), 1), by = fx_value(turn(1, hxe, hee), 1);
       const int64_t d2[3] = {turn(0, ax, bx), turn(1, ax, bx), turn(1, ay, by)};
 #pragma unroll
-      for (int r = 0; r < 3; ++r)
-        if (live) hso[Kc * 12 + 3 * c + r] = bad ? NAN : fx_to(d2[r], E + 7 + 2 * EJ);
+      for (int r = 0; r < 3; ++r) {
+        const Fx d = fx_value(d2[r], 0);   // below 2^59
+        if (live) *reinterpret_cast<int2 *>(hso + Kc * 12 + 3 * c + r) = make_int2(d.h, d.l);
+      }
     }
   }
   __syncthreads();
@@ -330,7 +342,9 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       p = gt0(p) ? p : 0.0;
       cs = root(mul(mul(gamma, p), ri));
     }
-    *reinterpret_cast<double2 *>(vdo + (K0 + lane) * VD_CELL + warp0 * VD_STRIDE + 12) = make_double2(ri, cs);
+    double *rec = vdo + (K0 + lane) * VD_CELL + warp0 * VD_STRIDE;
+    *reinterpret_cast<double2 *>(rec + 12) = make_double2(ri, cs);
+    *reinterpret_cast<double2 *>(rec + 14) = make_double2(u.c[1], u.c[2]);
   }
   // block sums of |K| u^(0): the cells of a warp, then the warps in order
   __shared__ double s_m[TPB / 32][4];
@@ -399,8 +413,85 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
 // and of the normal, so both cells share them.  With RIOE both momentum rows
 // hold the larger of the normal and tangential sums.
 // Edges [etile[tile], etile[tile + 1]), four lanes per edge, one per component;
-// for beta the lanes take the four (endpoint, side) pairs.
+// for beta the lanes take the four (endpoint, side) pairs.  The jumps and their
+// rotation are taken in fixed point from K1's records (27 FP64 operations per
+// lane otherwise), the squares and square roots in FP64.
 // --------------------------------------------------------------------------
+__device__ __forceinline__ Fx ld_fx(const double *p) {
+  const int2 v = *reinterpret_cast<const int2 *>(p);
+  return Fx{v.x, v.y};
+}
+// a - b of blocks with exponents Ea, Eb as limbs of exponent E + S, E >= Ea, Eb;
+// |a - b| < 2^(60 + S), for the high limb has 32 bits
+template <int S>
+__device__ __forceinline__ Fx fx_jump(Fx a, int Ea, Fx b, int Eb, int E) {
+  return fx_value((fx_join(a) >> min(E - Ea, 63)) - (fx_join(b) >> min(E - Eb, 63)), S);
+}
+
+// beta and 2 J of component c at a boundary edge, from the exterior polynomial
+// of all components of this side
+template <int K>
+__device__ __noinline__ void boundary_jumps(const MeshDev &m, const Phys &ph, const double *__restrict__ avg,
+                                            const double *__restrict__ vme, const double *__restrict__ hsi,
+                                            int64_t Kc, int i, int32_t cn, double nx, double ny, double t_out,
+                                            int c, int cw, double gamma, double &beta, double *J) {
+  const int64_t nt = m.nt;
+  double ab[4], hme[12];
+  short4 xo[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    ab[q] = avg[q * nt + Kc];   // the exterior state of a transmissive edge
+    xo[q] = *reinterpret_cast<const short4 *>(vme + VD_EXP + q);
+  }
+  auto get = [&](const double *p, int E) { return E >= FX_ENAN ? NAN : fx_to(fx_join(ld_fx(p)), E); };
+#pragma unroll
+  for (int q = 0; q < 12; ++q) hme[q] = K == 2 ? get(hsi + Kc * 12 + q, xo[q / 3].z) : 0.0;
+  beta = 0.0;
+  // row c of a jump per component, the momentum in (m_n, m_t) for RIOE
+  auto row = [&](const double d[4]) {
+    const double n = fdot2(d[1], nx, d[2], ny), t = fdot2(d[2], nx, -d[1], ny);
+    const double e[4] = {d[0], cw ? d[1] : n, cw ? d[2] : t, d[3]};
+    return pick4(e, c);
+  };
+#pragma unroll 1
+  for (int ev = 0; ev < 2; ++ev) {
+    int ov = i + 1 + ev;
+    ov = ov >= 3 ? ov - 3 : ov;
+    const double *ro = vme + ov * VD_STRIDE;
+    double val[4], grd[8], xv[4], xg[8], xh[12];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) val[q] = get(ro + q, xo[q].x);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) grd[q] = get(ro + 4 + q, xo[q / 2].y);
+    double px = 0.0, py = 0.0;
+    if (cn == -7) { px = m.vxy[(2 * ov) * nt + Kc]; py = m.vxy[(2 * ov + 1) * nt + Kc]; }
+    ghost_vertex(-cn, val, grd, hme, ab, nx, ny, px, py, t_out, ph, xv, xg, xh);
+    const double r_own = fma(fabs(fdot2(ro[14], nx, ro[15], ny)), ro[12], ro[13]);
+    // a mirror state has the same spectral radius
+    beta = max_nn(beta, max_nn(r_own, cn == -1 ? r_own : wave_speed(xv, nx, ny, gamma)));
+    double dv[4], d0[4], d1[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      dv[q] = val[q] - xv[q];
+      d0[q] = grd[2 * q] - xg[2 * q];
+      d1[q] = grd[2 * q + 1] - xg[2 * q + 1];
+    }
+    const double q = row(dv), g0 = row(d0), g1 = row(d1);
+    J[0] = ev == 0 ? q * q : fma(q, q, J[0]);
+    J[1] = ev == 0 ? fdot2(g0, g0, g1, g1) : fma(g0, g0, fma(g1, g1, J[1]));
+    if (K == 2 && ev == 0) {   // the exterior Hessian is constant: taken at v_c, for both endpoints
+      double h[3];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const double dh[4] = {hme[r] - xh[r], hme[3 + r] - xh[3 + r], hme[6 + r] - xh[6 + r], hme[9 + r] - xh[9 + r]};
+        h[r] = row(dh);
+      }
+      const double f = fma(h[0], h[0], fma(h[1] + h[1], h[1], h[2] * h[2]));
+      J[K] = f + f;
+    }
+  }
+}
+
 template <int K>
 __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph, const double *__restrict__ avg,
                                                const double *__restrict__ vdi, const double *__restrict__ hsi,
@@ -422,99 +513,74 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     const int32_t cn = m.conn[i * nt + Kc];
     const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
     const double *vme = vdi + Kc * VD_CELL;
-    double jv[2], jg[2][2], jh[3] = {0.0, 0.0, 0.0}, r;
-    if (cn >= 0) {
-      const int64_t nb = cn >> 2;
-      const int jn = cn & 3;
-      const double *vnb = vdi + nb * VD_CELL;
+    const short4 xo = *reinterpret_cast<const short4 *>(vme + VD_EXP + c);
+    // jumps of this component: values and gradients at v_c then v_d, the Hessian once; with
+    // the exponent of each kind (the momentum components share it, for their rotation)
+    Fx jv[2], jg[2][2], jh[3];
+    int E0, E1, E2 = 0;
+    auto shared_exp = [&](int E) {
+      const int p = __shfl_xor_sync(0xffffffffu, E, 3);
+      return mom ? max(E, p) : E;
+    };
+    double r;
+    bool bad = xo.x >= FX_ENAN;
+    const int64_t nb = cn >= 0 ? cn >> 2 : Kc;
+    const int jn = cn >= 0 ? cn & 3 : i;
+    const double *vnb = vdi + nb * VD_CELL;
+    const short4 xx = *reinterpret_cast<const short4 *>(vnb + VD_EXP + c);
+    bad = bad || xx.x >= FX_ENAN;
+    E0 = shared_exp(max(xo.x, xx.x));
+    E1 = shared_exp(max(xo.y, xx.y));
+    if (K == 2) E2 = shared_exp(max(xo.z, xx.z));
 #pragma unroll
-      for (int ev = 0; ev < 2; ++ev) {   // v_c then v_d, and the neighbour's copy of it
-        int ov = i + 1 + ev, xv = jn + 2 - ev;
-        ov = ov >= 3 ? ov - 3 : ov;
-        xv = xv >= 3 ? xv - 3 : xv;
-        const double *ro = vme + ov * VD_STRIDE, *rx = vnb + xv * VD_STRIDE;
-        const double2 go = *reinterpret_cast<const double2 *>(ro + 4 + 2 * c),
-                      gx = *reinterpret_cast<const double2 *>(rx + 4 + 2 * c);
-        jv[ev] = sub(ro[c], rx[c]);
-        jg[ev][0] = sub(go.x, gx.x);
-        jg[ev][1] = sub(go.y, gx.y);
-      }
-      if (K == 2) {
+    for (int ev = 0; ev < 2; ++ev) {   // v_c then v_d, and the neighbour's copy of it
+      int ov = i + 1 + ev, xv = jn + 2 - ev;
+      ov = ov >= 3 ? ov - 3 : ov;
+      xv = xv >= 3 ? xv - 3 : xv;
+      const double *ro = vme + ov * VD_STRIDE, *rx = vnb + xv * VD_STRIDE;
+      const int4 go = *reinterpret_cast<const int4 *>(ro + 4 + 2 * c),
+                 gx = *reinterpret_cast<const int4 *>(rx + 4 + 2 * c);
+      jv[ev] = fx_jump<1>(ld_fx(ro + c), xo.x, ld_fx(rx + c), xx.x, E0);
+      jg[ev][0] = fx_jump<0>(Fx{go.x, go.y}, xo.y, Fx{gx.x, gx.y}, xx.y, E1);
+      jg[ev][1] = fx_jump<0>(Fx{go.z, go.w}, xo.y, Fx{gx.z, gx.w}, xx.y, E1);
+    }
+    if (K == 2) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) jh[q] = sub(hsi[Kc * 12 + 3 * c + q], hsi[nb * 12 + 3 * c + q]);
-      }
+      for (int q = 0; q < 3; ++q)
+        jh[q] = fx_jump<0>(ld_fx(hsi + Kc * 12 + 3 * c + q), xo.z, ld_fx(hsi + nb * 12 + 3 * c + q), xx.z, E2);
+    }
+    {
       int vv = c & 1 ? (c & 2 ? jn + 1 : i + 2) : (c & 2 ? jn + 2 : i + 1);
       vv = vv >= 3 ? vv - 3 : vv;
       const double *rr = (c & 2 ? vnb : vme) + vv * VD_STRIDE;
-      r = fma(fabs(fdot2(rr[1], nx, rr[2], ny)), rr[12], rr[13]);
-    } else {
-      // boundary edge: the exterior polynomial from all components of this side
-      const double t_out = fma(c_out, sc->dt, sc->t);
-      double ab[4], hme[12];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) ab[q] = avg[q * nt + Kc];   // the exterior state of a transmissive edge
-#pragma unroll
-      for (int q = 0; q < 12; ++q) hme[q] = K == 2 ? hsi[Kc * 12 + q] : 0.0;
-      r = 0.0;
-#pragma unroll 1
-      for (int ev = 0; ev < 2; ++ev) {
-        int ov = i + 1 + ev;
-        ov = ov >= 3 ? ov - 3 : ov;
-        const double *ro = vme + ov * VD_STRIDE;
-        double val[4], grd[8], xv[4], xg[8], xh[12];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) val[q] = ro[q];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) grd[q] = ro[4 + q];
-        double px = 0.0, py = 0.0;
-        if (cn == -7) { px = m.vxy[(2 * ov) * nt + Kc]; py = m.vxy[(2 * ov + 1) * nt + Kc]; }
-        ghost_vertex(-cn, val, grd, hme, ab, nx, ny, px, py, t_out, ph, xv, xg, xh);
-        const double r_own = fma(fabs(fdot2(val[1], nx, val[2], ny)), ro[12], ro[13]);
-        // a mirror state has the same spectral radius
-        r = max_nn(r, max_nn(r_own, cn == -1 ? r_own : wave_speed(xv, nx, ny, gamma)));
-        double gv[4], gw[4], dv[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          dv[q] = val[q] - xv[q];
-          gv[q] = grd[2 * q] - xg[2 * q];
-          gw[q] = grd[2 * q + 1] - xg[2 * q + 1];
-        }
-        const double d0 = pick4(dv, c), d1 = pick4(gv, c), d2 = pick4(gw, c);
-        if (ev == 0) {
-          jv[0] = d0; jg[0][0] = d1; jg[0][1] = d2;
-          // the Hessian of the exterior state is constant: taken at v_c only
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const double dh[4] = {hme[q] - xh[q], hme[3 + q] - xh[3 + q], hme[6 + q] - xh[6 + q], hme[9 + q] - xh[9 + q]};
-            jh[q] = K == 2 ? pick4(dh, c) : 0.0;
-          }
-        } else {
-          jv[1] = d0; jg[1][0] = d1; jg[1][1] = d2;
-        }
-      }
+      r = fma(fabs(fdot2(rr[14], nx, rr[15], ny)), rr[12], rr[13]);
     }
     r = max_nn(r, __shfl_xor_sync(0xffffffffu, r, 1));
-    const double beta = max_nn(r, __shfl_xor_sync(0xffffffffu, r, 2));
+    double beta = max_nn(r, __shfl_xor_sync(0xffffffffu, r, 2));
     // RIOE: rotate the momentum jumps to (m_n, m_t) with the owner's normal
-    const double sy = c == 2 ? -ny : ny;
-    auto rot = [&](double q) {
-      const double p = __shfl_xor_sync(0xffffffffu, q, 3);
-      const double t = fdot2(q, nx, p, sy);
-      return mom ? t : q;
+    const Fx rs = fx_coef(mom ? nx : 1.0, 0), ry = fx_coef(mom ? ny : 0.0, 0);
+    const Fx rp = c == 2 ? Fx{-ry.h, -ry.l} : ry;
+    auto rot = [&](Fx q, int E) {
+      const Fx p{__shfl_xor_sync(0xffffffffu, q.h, 3), __shfl_xor_sync(0xffffffffu, q.l, 3)};
+      FxAcc t{0, 0};
+      fx_mac(t, rs, q);
+      fx_mac(t, rp, p);
+      return bad ? NAN : fx_to(fx_sum(t), E);
     };
     double J[K + 1];
 #pragma unroll
     for (int ev = 0; ev < 2; ++ev) {
-      const double q = rot(jv[ev]), g0 = rot(jg[ev][0]), g1 = rot(jg[ev][1]);
+      const double q = rot(jv[ev], E0 + 1), g0 = rot(jg[ev][0], E1), g1 = rot(jg[ev][1], E1);
       // 2 J: the 1/2 of the trapezoidal rule moves into A (sqrt(1/2))
       J[0] = ev == 0 ? mul(q, q) : fma(q, q, J[0]);
       J[1] = ev == 0 ? fdot2(g0, g0, g1, g1) : fma(g0, g0, fma(g1, g1, J[1]));
     }
     if (K == 2) {   // the Hessian jump counts at both endpoints
-      const double h0 = rot(jh[0]), h1 = rot(jh[1]), h2 = rot(jh[2]);
+      const double h0 = rot(jh[0], E2), h1 = rot(jh[1], E2), h2 = rot(jh[2], E2);
       const double f = fma(h0, h0, fma(add(h1, h1), h1, mul(h2, h2)));
       J[K] = add(f, f);
     }
+    if (cn < 0) boundary_jumps<K>(m, ph, avg, vme, hsi, Kc, i, cn, nx, ny, fma(c_out, sc->dt, sc->t), c, cw, gamma, beta, J);
     const bool finite = is_finite_bits(beta);
     double er[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
