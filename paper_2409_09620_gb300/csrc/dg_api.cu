@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -90,6 +91,7 @@ struct dg_solver {
   Scalars *sc = nullptr;
   cudaGraphExec_t step_exec = nullptr;
   StageCtx ctx{};
+  mutable std::mutex scratch_mutex;   // the transfers' use of the free state buffer
   ~dg_solver() {
     if (step_exec) cudaGraphExecDestroy(step_exec);
     StateBuf *bufs[3] = {&un, &uh, &us};
@@ -303,48 +305,49 @@ cudaError_t alloc_state(dg_solver *s, StateBuf *b) {
   return cudaMalloc(&b->hi, std::max<size_t>(1, real_size(s) * 4 * (s->nb - 1) * nt));
 }
 
-// host modal state [4][nb][nt] (double) -> device buffer
+// A state buffer other than b, free to hold two components' modes in FP64 (the
+// size of the mixed form's mode records): the stage buffers u_h and u_s carry
+// nothing between calls, and no caller fills both before it uses one.
+double *mode_scratch(const dg_solver *s, const StateBuf &b) {
+  return (double *)(b.hi == s->uh.hi ? s->us.hi : s->uh.hi);
+}
+
+// host modal state [4][nb][nt] (double) -> device buffer.  Mixed form: the modes
+// cross in FP64 two components at a time and are rounded to the per-cell
+// records on the device.
 int32_t upload_state(dg_solver *s, const double *coeffs, const StateBuf &b) {
   const int64_t nt = s->mesh->nt;
   const int nb = s->nb;
-  for (int c = 0; c < 4; ++c)
+  const bool mixed = s->cfg.precision == DG_PREC_MIXED;
+  const size_t bytes = sizeof(double) * (nb - 1) * nt;   // modes of one component
+  std::lock_guard<std::mutex> lock(s->scratch_mutex);
+  for (int c = 0; c < 4; ++c) {
     CUDA_TRY(cudaMemcpyAsync(b.avg + c * nt, coeffs + (int64_t)c * nb * nt, sizeof(double) * nt,
                              cudaMemcpyHostToDevice, s->stream));
-  if (s->cfg.precision == DG_PREC_MIXED) {
-    std::vector<float> tmp((size_t)(4 * (nb - 1) * nt));
-    for (int c = 0; c < 4; ++c)
-      for (int l = 1; l < nb; ++l)
-        for (int64_t K = 0; K < nt; ++K)
-          tmp[(size_t)K * 4 * (nb - 1) + c * (nb - 1) + (l - 1)] = (float)coeffs[((int64_t)c * nb + l) * nt + K];
-    CUDA_TRY(cudaMemcpyAsync(b.hi, tmp.data(), sizeof(float) * tmp.size(), cudaMemcpyHostToDevice, s->stream));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-  } else {
-    for (int c = 0; c < 4; ++c)
-      CUDA_TRY(cudaMemcpyAsync((double *)b.hi + (int64_t)c * (nb - 1) * nt, coeffs + ((int64_t)c * nb + 1) * nt,
-                               sizeof(double) * (nb - 1) * nt, cudaMemcpyHostToDevice, s->stream));
+    double *dst = mixed ? mode_scratch(s, b) + (int64_t)(c & 1) * (nb - 1) * nt
+                        : (double *)b.hi + (int64_t)c * (nb - 1) * nt;
+    CUDA_TRY(cudaMemcpyAsync(dst, coeffs + ((int64_t)c * nb + 1) * nt, bytes, cudaMemcpyHostToDevice, s->stream));
+    if (mixed && (c & 1)) launch_convert_modes(s->ctx, b.hi, mode_scratch(s, b), c - 1, true);
   }
+  CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
 
 int32_t download_state(const dg_solver *s, const StateBuf &b, double *coeffs) {
   const int64_t nt = s->mesh->nt;
   const int nb = s->nb;
-  for (int c = 0; c < 4; ++c)
+  const bool mixed = s->cfg.precision == DG_PREC_MIXED;
+  const size_t bytes = sizeof(double) * (nb - 1) * nt;
+  std::lock_guard<std::mutex> lock(s->scratch_mutex);   // two readers of one solver share the scratch
+  for (int c = 0; c < 4; ++c) {
     CUDA_TRY(cudaMemcpyAsync(coeffs + (int64_t)c * nb * nt, b.avg + c * nt, sizeof(double) * nt,
                              cudaMemcpyDeviceToHost, s->stream));
-  if (s->cfg.precision == DG_PREC_MIXED) {
-    std::vector<float> tmp((size_t)(4 * (nb - 1) * nt));
-    CUDA_TRY(cudaMemcpyAsync(tmp.data(), b.hi, sizeof(float) * tmp.size(), cudaMemcpyDeviceToHost, s->stream));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    for (int c = 0; c < 4; ++c)
-      for (int l = 1; l < nb; ++l)
-        for (int64_t K = 0; K < nt; ++K)
-          coeffs[((int64_t)c * nb + l) * nt + K] = tmp[(size_t)K * 4 * (nb - 1) + c * (nb - 1) + (l - 1)];
-  } else {
-    for (int c = 0; c < 4; ++c)
-      CUDA_TRY(cudaMemcpyAsync(coeffs + ((int64_t)c * nb + 1) * nt, (double *)b.hi + (int64_t)c * (nb - 1) * nt,
-                               sizeof(double) * (nb - 1) * nt, cudaMemcpyDeviceToHost, s->stream));
+    if (mixed && !(c & 1)) launch_convert_modes(s->ctx, b.hi, mode_scratch(s, b), c, false);
+    const double *src = mixed ? mode_scratch(s, b) + (int64_t)(c & 1) * (nb - 1) * nt
+                              : (const double *)b.hi + (int64_t)c * (nb - 1) * nt;
+    CUDA_TRY(cudaMemcpyAsync(coeffs + ((int64_t)c * nb + 1) * nt, src, bytes, cudaMemcpyDeviceToHost, s->stream));
   }
+  CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   return DG_OK;
 }

@@ -53,6 +53,9 @@ void launch_oe_bp_only(const StageCtx &c, const StateBuf &uh, const StateBuf &ou
                        double c_out, int end_of_step);
 void launch_fin_alpha(const StageCtx &c, int stage);
 void launch_step_begin(const StageCtx &c);
+// modes of components c0, c0 + 1 between the mixed form's records and the ABI's
+// layout [2][nb - 1][nt] on the device (half the size of the records in FP64)
+void launch_convert_modes(const StageCtx &c, void *rec, double *modes, int c0, bool to_record);
 void launch_set_active(const StageCtx &c, int active);
 void launch_set_inv_normalisers(const StageCtx &c);
 // tiles of a mesh: the blocks of a stage kernel in the given precision, one reduction partial each
