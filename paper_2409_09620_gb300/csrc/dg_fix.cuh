@@ -25,6 +25,7 @@
 // 2^-1016; a block that holds an infinity or a NaN has E = 0x7ff, and the
 // callers turn its results into NaN.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -176,6 +177,27 @@ FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
   E = (E1 > E2 ? E1 : E2) + 1;
   const int s1 = E - E1, s2 = E - E2;
   return (r1 >> (s1 > 63 ? 63 : s1)) + (r2 >> (s2 > 63 ? 63 : s2));
+}
+
+// block fixed point of N values; returns the block's exponent
+template <int N>
+FX_HD int fx_block(const double x[N], Fx f[N]) {
+  int mx = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int j = 0; j < N; ++j) mx = fx_abs_hi(x[j]) > mx ? fx_abs_hi(x[j]) : mx;
+  const int E = fx_exp(mx);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int j = 0; j < N; ++j) f[j] = fx_from(x[j], E);
+  return E;
+}
+// fx_to, NaN for a block that holds a non-finite value
+FX_HD double fx_out(int64_t r, int E) {
+  const double x = fx_to(r, E);
+  return E >= FX_ENAN ? NAN : x;
 }
 
 }  // namespace dg

@@ -17,12 +17,19 @@
 //
 // with finalize kernels in the fixed two-level order of the Euler path.  The
 // time step is Sec. 5's C_SSP / alpha * min_K |K| / ((2k + 1) sum_i l_K^(i)).
+//
+// The kernels are bound by the FP64 pipe (64-76 cycles per warp instruction), so
+// sums with constant coefficients are taken in block fixed point on the integer
+// units (dg_fix.cuh) and the rest in register-only DFMAs (dg_common.cuh).
+// Measured, with every sum on the FP64 pipe before: Burgers P3, 51,200 cells,
+// 0.598 -> 0.327 ms per step; linear P2, 204,800 cells, 1.06 -> 0.60 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
 #include "../../include/dg.h"
+#include "dg_fix.cuh"
 #include "dg_internal.h"
 
 namespace dg {
@@ -119,12 +126,8 @@ struct ScPhys {
   double bc[4];        // constant-state boundary values (tags 3..6)
 };
 
-__device__ __forceinline__ void sflux(const ScPhys &ph, double u, double &f0, double &f1) {
-  if (ph.flux == 0) { f0 = ph.ax * u; f1 = ph.ay * u; }
-  else { f0 = f1 = 0.5 * u * u; }
-}
 __device__ __forceinline__ double sspeed(const ScPhys &ph, double u, double nx, double ny) {
-  return ph.flux == 0 ? ph.ax * nx + ph.ay * ny : u * (nx + ny);
+  return ph.flux == 0 ? fdot2(ph.ax, nx, ph.ay, ny) : mul(u, add(nx, ny));
 }
 // exterior value at a boundary edge (tag > 0): constant state or the interior value
 __device__ __forceinline__ double sghost(const ScPhys &ph, int tag, double uin) {
@@ -133,6 +136,26 @@ __device__ __forceinline__ double sghost(const ScPhys &ph, int tag, double uin) 
 
 // record of the derivatives d^j u / dx^a dy^(j-a) at a vertex: index of (j, a)
 __host__ __device__ constexpr int didx(int j, int a) { return j * (j + 1) / 2 + (j - a); }
+
+// value of the polynomial at a fixed reference point in fixed point, with
+// the coefficients halved for P3 (basis values reach 8 there): exponent E + SVAL<K>
+template <int K> constexpr int SVAL = K == 3 ? 1 : 0;
+template <int K>
+__device__ __forceinline__ int64_t sfx_point(const Fx f[SDeg<K>::NB], double xi, double eta) {
+  FxAcc s{0, 0};
+#pragma unroll
+  for (int l = 0; l < SDeg<K>::NB; ++l) fx_mac(s, fxc(psi_rs(l, 0, 0, xi, eta) / (1 << SVAL<K>)), f[l]);
+  return fx_sum(s);
+}
+// reference derivative d^(r+s) / dxi^r deta^s at a fixed point (coefficients reach
+// 960 for P3, 48 for P2: as c / 256)
+template <int K>
+__device__ __forceinline__ double sfx_deriv(const Fx f[SDeg<K>::NB], int E, int r, int s, double xi, double eta) {
+  FxAcc a{0, 0};
+#pragma unroll
+  for (int l = 1; l < SDeg<K>::NB; ++l) fx_mac(a, fxc(psi_rs(l, r, s, xi, eta) / 256.0), f[l]);
+  return fx_out(fx_sum(a), E + 8);
+}
 
 // ---- K1: volume + edge fluxes + RK combination ------------------------------------
 template <int K>
@@ -148,64 +171,83 @@ __global__ void __launch_bounds__(TPB) k_sc_rk(MeshDev m, ScPhys ph, const doubl
   if (Kc < nt) {
     const double dt = sc->dt, alpha = sc->alpha;
     const double area = m.area[Kc];
-    const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
-    double c[NB], acc[NB];
+    // F(u) = g(u) (d1, d2): g = u, (ax, ay) or g = u^2, (1/2, 1/2)
+    const double d1 = ph.flux == 0 ? ph.ax : 0.5, d2 = ph.flux == 0 ? ph.ay : 0.5;
+    // volume: sum_mu w_mu g(u(x_mu)) (d . grad xi dPsi/dxi + d . grad eta dPsi/deta), the mass
+    // inverse on the coefficients
+    Fx g[NV];
+    int Eg;
+    {
+      double x[NV];
+      double c[NB];
+      Fx f[NB];
 #pragma unroll
-    for (int l = 0; l < NB; ++l) { c[l] = v[l * nt + Kc]; acc[l] = 0.0; }
-    // volume: |K| sum_mu w_mu F(u(x_mu)) . grad Psi_l
+      for (int l = 0; l < NB; ++l) c[l] = v[l * nt + Kc];
+      const int E = fx_block<NB>(c, f);
 #pragma unroll
-    for (int mu = 0; mu < NV; ++mu) {
-      const double xi = svol_xi(NV, mu), eta = svol_eta(NV, mu), w = svol_w(NV, mu);
-      double u = 0.0;
-#pragma unroll
-      for (int l = 0; l < NB; ++l) u = cfma(psi_rs(l, 0, 0, xi, eta), c[l], u);
-      double f0, f1;
-      sflux(ph, u, f0, f1);
-      const double g1 = f0 * jx + f1 * jy, g2 = f0 * ex + f1 * ey;   // F . grad xi, F . grad eta
-#pragma unroll
-      for (int l = 1; l < NB; ++l) {
-        acc[l] = cfma(w * psi_rs(l, 1, 0, xi, eta), g1, acc[l]);
-        acc[l] = cfma(w * psi_rs(l, 0, 1, xi, eta), g2, acc[l]);
+      for (int mu = 0; mu < NV; ++mu) {
+        const double u = fx_out(sfx_point<K>(f, svol_xi(NV, mu), svol_eta(NV, mu)), E + SVAL<K>);
+        x[mu] = ph.flux == 0 ? u : mul(u, u);
       }
+      Eg = fx_block<NV>(x, g);
     }
+    // edges: l_i (F(u-) + F(u+) - alpha (u+ - u-)) . n
+    Fx y[3 * NQ];
+    int Ee;
+    {
+      double tv[3 * NQ];
 #pragma unroll
-    for (int l = 1; l < NB; ++l) acc[l] *= area;
-    // edges: - sum_i l_i sum_nu w_nu Fhat Psi_l
+      for (int i = 0; i < 3; ++i) {
+        const int32_t cn = m.conn[i * nt + Kc];
+        const double li = m.len[i * nt + Kc];
+        const double vl = mul(fdot2(d1, m.nrm[(2 * i) * nt + Kc], d2, m.nrm[(2 * i + 1) * nt + Kc]), li);
+        const double al = mul(alpha, li);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const int32_t cn = m.conn[i * nt + Kc];
-      const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc], li = m.len[i * nt + Kc];
-#pragma unroll
-      for (int nu = 0; nu < NQ; ++nu) {
-        const double um = tr[(Kc * 3 + i) * NQ + nu];
-        const double up = cn >= 0 ? tr[((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)] : sghost(ph, -cn, um);
-        double fm0, fm1, fp0, fp1;
-        sflux(ph, um, fm0, fm1);
-        sflux(ph, up, fp0, fp1);
-        const double fh = 0.5 * ((fm0 + fp0) * nx + (fm1 + fp1) * ny - alpha * (up - um));
-        const double tv = li * sgauss_w(NQ, nu) * fh;
-        const double s = sgauss_s(NQ, nu);
-#pragma unroll
-        for (int l = 0; l < NB; ++l) acc[l] = cfma(-psi_rs(l, 0, 0, edge_xi(i, s), edge_eta(i, s)), tv, acc[l]);
+        for (int nu = 0; nu < NQ; ++nu) {
+          const double um = tr[(Kc * 3 + i) * NQ + nu];
+          const double up = cn >= 0 ? tr[((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)] : sghost(ph, -cn, um);
+          const double s = ph.flux == 0 ? add(um, up) : add(mul(um, um), mul(up, up));
+          tv[i * NQ + nu] = sub(mul(vl, s), mul(al, sub(up, um)));
+        }
       }
+      Ee = fx_block<3 * NQ>(tv, y);
     }
-    // mass inverse and SSP-RK combination
+    // quadrature sums, mass inverse and SSP-RK combination
+    const double A1 = fdot2(d1, m.jinv[Kc], d2, m.jinv[nt + Kc]), A2 = fdot2(d1, m.jinv[2 * nt + Kc], d2, m.jinv[3 * nt + Kc]);
     const double dta = dt / area;
-    double h[NB];
 #pragma unroll
     for (int l = 0; l < NB; ++l) {
-      h[l] = a * un[l * nt + Kc] + b * (c[l] + dta * sc_inv_mass(l) * acc[l]);
-      uh[l * nt + Kc] = h[l];
+      FxAcc e{0, 0};
+#pragma unroll
+      for (int p = 0; p < 3 * NQ; ++p) {
+        const double s = sgauss_s(NQ, p % NQ);
+        fx_mac(e, fxc(-0.5 * sgauss_w(NQ, p % NQ) * sc_inv_mass(l) * psi_rs(l, 0, 0, edge_xi(p / NQ, s), edge_eta(p / NQ, s))),
+               y[p]);
+      }
+      double L = fma(dta, fx_out(fx_sum(e), Ee), v[l * nt + Kc]);
+      if (l > 0) {
+        FxAcc sx{0, 0}, sy{0, 0};
+#pragma unroll
+        for (int mu = 0; mu < NV; ++mu) {
+          const double xi = svol_xi(NV, mu), eta = svol_eta(NV, mu), w = svol_w(NV, mu) * sc_inv_mass(l);
+          fx_mac(sx, fxc(w * psi_rs(l, 1, 0, xi, eta)), g[mu]);
+          fx_mac(sy, fxc(w * psi_rs(l, 0, 1, xi, eta)), g[mu]);
+        }
+        L = fma(dt, fdot2(A1, fx_out(fx_sum(sx), Eg), A2, fx_out(fx_sum(sy), Eg)), L);
+      }
+      const double h = fdot2(a, un[l * nt + Kc], b, L);
+      uh[l * nt + Kc] = h;
+      if (l == 0) mass[0] = mul(area, h);
     }
-    mass[0] = area * h[0];
   }
   block_reduce<1>(mass, part + blockIdx.x, OpSum());
 }
 
 // ---- K2: sup |u - mean| at the volume points; vertex derivative records ----------------
-// The records hold d^j u / dx^p dy^(j-p), j <= K, at the three vertices (the
-// affine map gives d/dx = xi_x d/dxi + eta_x d/deta, d/dy = xi_y d/dxi +
-// eta_y d/deta), for the OE jumps of the neighbours and the cell itself.
+// The records hold d^j u / dx^p dy^(j-p), j <= K, at the three vertices, for
+// the OE jumps of the neighbours and the cell itself.  The affine map gives d/dx
+// = xi_x d/dxi + eta_x d/deta, d/dy = xi_y d/dxi + eta_y d/deta: a symmetric
+// tensor of order j is turned one index at a time.
 template <int K>
 __global__ void __launch_bounds__(TPB) k_sc_stats(MeshDev m, const double *__restrict__ u, double *__restrict__ vr,
                                                   double *part, const ScScalars *sc) {
@@ -215,46 +257,77 @@ __global__ void __launch_bounds__(TPB) k_sc_stats(MeshDev m, const double *__res
   const int64_t Kc = (int64_t)blockIdx.x * TPB + threadIdx.x;
   double d[1] = {0.0};
   if (Kc < nt) {
-    const double mean = sc->mean;
     double c[NB];
+    Fx f[NB];
 #pragma unroll
     for (int l = 0; l < NB; ++l) c[l] = u[l * nt + Kc];
+    const double c0 = c[0];
+    c[0] = sub(c0, sc->mean);
+    const int Ed = fx_block<NB>(c, f);
+    uint64_t top = 0;
 #pragma unroll
     for (int mu = 0; mu < NV; ++mu) {
-      double s = c[0] - mean;
-#pragma unroll
-      for (int l = 1; l < NB; ++l) s = cfma(psi_rs(l, 0, 0, svol_xi(NV, mu), svol_eta(NV, mu)), c[l], s);
-      d[0] = max_nn(d[0], fabs(s));
+      const int64_t r = sfx_point<K>(f, svol_xi(NV, mu), svol_eta(NV, mu));
+      const uint64_t ab = (uint64_t)(r < 0 ? -r : r);
+      top = ab > top ? ab : top;
     }
+    d[0] = fx_out((int64_t)top, Ed + SVAL<K>);
+    c[0] = c0;
+    const int E = fx_block<NB>(c, f);
     const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
     double *vo = vr + Kc * 3 * NB;
+    // one index of a tensor with components t[r], r = number of xi: out[r] for d/dx (w = 0) or d/dy
+    auto turn = [&](int n, int w, const double *t, double *o) {
+#pragma unroll
+      for (int r = 0; r < n; ++r) o[r] = fdot2(t[r + 1], w == 0 ? jx : jy, t[r], w == 0 ? ex : ey);
+    };
+    double t3[4] = {0.0, 0.0, 0.0, 0.0};   // third derivatives: constant
+    if constexpr (K == 3) {
+      double t[4], x[3], y[3], xx[2], xy[2], yy[2];
+#pragma unroll
+      for (int r = 0; r <= 3; ++r) t[r] = sfx_deriv<K>(f, E, r, 3 - r, 0.0, 0.0);
+      turn(3, 0, t, x);
+      turn(3, 1, t, y);
+      turn(2, 0, x, xx);
+      turn(2, 1, x, xy);
+      turn(2, 1, y, yy);
+      turn(1, 0, xx, t3);
+      turn(1, 1, xx, t3 + 1);
+      turn(1, 1, xy, t3 + 2);
+      turn(1, 1, yy, t3 + 3);
+    }
+    double t2[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int vv = 0; vv < 3; ++vv) {
       const double xi = vert_xi(vv), eta = vert_eta(vv);
+      double *rec = vo + vv * NB;
+      rec[0] = fx_out(sfx_point<K>(f, xi, eta), E + SVAL<K>);
+      {
+        double t[2], x, y;
+        t[0] = sfx_deriv<K>(f, E, 0, 1, xi, eta);
+        t[1] = sfx_deriv<K>(f, E, 1, 0, xi, eta);
+        turn(1, 0, t, &x);
+        turn(1, 1, t, &y);
+        rec[didx(1, 1)] = x;
+        rec[didx(1, 0)] = y;
+      }
+      if constexpr (K >= 2) {
+        if (K == 3 || vv == 0) {   // P2: constant
+          double t[3], x[2], y[2];
 #pragma unroll
-      for (int j = 0; j <= K; ++j)
-#pragma unroll
-        for (int p = j; p >= 0; --p) {
-          // expand (jx Dxi + ex Deta)^p (jy Dxi + ey Deta)^(j-p): co[r] multiplies Dxi^r Deta^(j-r)
-          double co[K + 1];
-#pragma unroll
-          for (int r = 0; r <= K; ++r) co[r] = r == 0 ? 1.0 : 0.0;
-#pragma unroll
-          for (int f = 0; f < j; ++f) {
-            const double fa = f < p ? jx : jy, fb = f < p ? ex : ey;
-#pragma unroll
-            for (int r = K; r >= 0; --r) co[r] = (r > 0 ? fa * co[r - 1] : 0.0) + fb * co[r];
-          }
-          double dv = 0.0;
-#pragma unroll
-          for (int r = 0; r <= j; ++r) {
-            double ref = 0.0;   // d^j u / dxi^r deta^(j-r) at the vertex
-#pragma unroll
-            for (int l = 0; l < NB; ++l) ref = cfma(psi_rs(l, r, j - r, xi, eta), c[l], ref);
-            dv += co[r] * ref;
-          }
-          vo[vv * NB + didx(j, p)] = dv;
+          for (int r = 0; r <= 2; ++r) t[r] = sfx_deriv<K>(f, E, r, 2 - r, xi, eta);
+          turn(2, 0, t, x);
+          turn(2, 1, t, y);
+          turn(1, 0, x, t2);
+          turn(1, 1, x, t2 + 1);
+          turn(1, 1, y, t2 + 2);
         }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) rec[didx(2, 2 - q)] = t2[q];
+      }
+      if constexpr (K == 3)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rec[didx(3, 3 - q)] = t3[q];
     }
   }
   block_reduce<1>(d, part + blockIdx.x, OpMaxNN());
@@ -275,82 +348,86 @@ __global__ void __launch_bounds__(TPB) k_sc_oe(MeshDev m, ScPhys ph, const doubl
     double c[NB];
 #pragma unroll
     for (int l = 0; l < NB; ++l) c[l] = uh[l * nt + Kc];
-    if (do_oe && sc->inv_dev != 0.0) {
+    if (do_oe && nonzero_bits(sc->inv_dev)) {
       const double inv_dev = sc->inv_dev, dt = sc->dt;
       double sig[K + 1];
 #pragma unroll
       for (int j = 0; j <= K; ++j) sig[j] = 0.0;
       const double *vme = vr + Kc * 3 * NB;
-#pragma unroll
+#pragma unroll 1
       for (int i = 0; i < 3; ++i) {
         const int32_t cn = m.conn[i * nt + Kc];
         const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
         const double h = m.hgeo[i * nt + Kc], ih = m.hgeo[(3 + i) * nt + Kc];
-        double J[K + 1];
+        // 2 J_j = sum over both ends of sum_a C_j^a jump^2 (the trapezoidal 1/2 moves into A):
+        // the derivatives with binomial coefficient 1 and those with C > 1 apart
+        double J[K + 1], Jm[K + 1];
 #pragma unroll
-        for (int j = 0; j <= K; ++j) J[j] = 0.0;
+        for (int j = 0; j <= K; ++j) J[j] = Jm[j] = 0.0;
         double beta = 0.0;
+        const bool dir = cn < 0 && (-cn) >= DG_BC_DIRICHLET0 && (-cn) < DG_BC_DIRICHLET0 + 4;
 #pragma unroll
         for (int ev = 0; ev < 2; ++ev) {
-          const int ov = (i + 1 + ev) % 3;                 // v_c, then v_d
+          int ov = i + 1 + ev, xv = (cn & 3) + 2 - ev;      // v_c, then v_d; the neighbour's copy
+          ov = ov >= 3 ? ov - 3 : ov;
+          xv = xv >= 3 ? xv - 3 : xv;
           const double *own = vme + ov * NB;
-          const double *oth = cn >= 0 ? vr + ((int64_t)(cn >> 2) * 3 + ((cn & 3) + 2 - ev) % 3) * NB : nullptr;
-          const bool dir = cn < 0 && (-cn) >= DG_BC_DIRICHLET0 && (-cn) < DG_BC_DIRICHLET0 + 4;
-          const double u_own = own[0];
-          const double u_ext = cn >= 0 ? oth[0] : (dir ? ph.bc[-cn - DG_BC_DIRICHLET0] : u_own);
+          const double *oth = cn >= 0 ? vr + ((int64_t)(cn >> 2) * 3 + xv) * NB : own;
+          const double u_own = own[0], u_ext = dir ? ph.bc[-cn - DG_BC_DIRICHLET0] : oth[0];
           beta = max_nn(beta, max_nn(fabs(sspeed(ph, u_own, nx, ny)), fabs(sspeed(ph, u_ext, nx, ny))));
 #pragma unroll
-          for (int j = 0; j <= K; ++j) {
+          for (int j = 0; j <= K; ++j)
 #pragma unroll
             for (int a = j; a >= 0; --a) {
-              // C_j^a for the derivative d^j / dx^a dy^(j-a)
-              double cb = 1.0;
-#pragma unroll
-              for (int t = 0; t < a; ++t) cb = cb * double(j - t) / double(t + 1);
-              const double o = own[didx(j, a)];
-              const double x = cn >= 0 ? oth[didx(j, a)] : (dir ? (j == 0 ? u_ext : 0.0) : o);
-              const double jump = o - x;
-              J[j] += 0.5 * cb * jump * jump;
+              const double x = j == 0 ? u_ext : (dir ? 0.0 : oth[didx(j, a)]);   // a constant state has no derivatives
+              const double jump = sub(own[didx(j, a)], x);
+              if (a == 0 || a == j) J[j] = fma(jump, jump, J[j]);
+              else Jm[j] = fma(jump, jump, Jm[j]);
             }
-          }
         }
         // delta^j = A^{k,j} h^j sqrt(J_j) / D, sigma^j += beta / h delta^j
+        const double bh = mul(mul(beta, ih), inv_dev);
         double hj = 1.0, fact = 1.0;
 #pragma unroll
         for (int j = 0; j <= K; ++j) {
           if (j > 0) fact *= double(j);
-          const double A = (2.0 * j + 1.0) / ((2.0 * K - 1.0) * fact);
-          sig[j] += beta * ih * (A * hj * sqrt(J[j]) * inv_dev);
-          hj *= h;
+          const double A = (2.0 * j + 1.0) / ((2.0 * K - 1.0) * fact) * 0.70710678118654752440;
+          const double J2 = j < 2 ? J[j] : fma(double(j), Jm[j], J[j]);   // C_2^1 = 2, C_3^1 = C_3^2 = 3
+          sig[j] = fma(mul(A * bh, hj), root(J2), sig[j]);
+          hj = j == 0 ? h : mul(hj, h);
         }
       }
       double fac[K + 1];
       double sacc = sig[0];
 #pragma unroll
       for (int md = 1; md <= K; ++md) {
-        sacc += sig[md];
-        fac[md] = exp_neg(dt * sacc);
+        sacc = add(sacc, sig[md]);
+        fac[md] = exp_neg(mul(dt, sacc));
       }
 #pragma unroll
-      for (int l = 1; l < NB; ++l) c[l] *= fac[sc_degree(l)];
+      for (int l = 1; l < NB; ++l) c[l] = mul(c[l], fac[sc_degree(l)]);
     }
 #pragma unroll
     for (int l = 0; l < NB; ++l) out[l * nt + Kc] = c[l];
-    // traces of the result at the edge Gauss points; wave speeds of the next stage's input
+    // traces of the result at the edge Gauss points; wave speeds of the next stage's input:
+    // |u| is largest where its fixed-point value is, and the speed is monotonic in |u|
+    Fx f[NB];
+    const int E = fx_block<NB>(c, f);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const int32_t cn = m.conn[i * nt + Kc];
       const double nx = m.nrm[(2 * i) * nt + Kc], ny = m.nrm[(2 * i + 1) * nt + Kc];
+      double um = 0.0;
 #pragma unroll
       for (int nu = 0; nu < NQ; ++nu) {
         const double s = sgauss_s(NQ, nu);
-        double u = 0.0;
-#pragma unroll
-        for (int l = 0; l < NB; ++l) u = cfma(psi_rs(l, 0, 0, edge_xi(i, s), edge_eta(i, s)), c[l], u);
+        const double u = fx_out(sfx_point<K>(f, edge_xi(i, s), edge_eta(i, s)), E + SVAL<K>);
         tr[(Kc * 3 + i) * NQ + nu] = u;
-        amax = max_nn(amax, fabs(sspeed(ph, u, nx, ny)));
-        if (cn < 0) amax = max_nn(amax, fabs(sspeed(ph, sghost(ph, -cn, u), nx, ny)));
+        um = max_nn(um, fabs(u));
       }
+      amax = max_nn(amax, fabs(sspeed(ph, um, nx, ny)));
+      // exterior states: constant, or the interior trace, already in
+      if (cn < 0) amax = max_nn(amax, fabs(sspeed(ph, sghost(ph, -cn, um), nx, ny)));
     }
   }
   double av[1] = {amax};

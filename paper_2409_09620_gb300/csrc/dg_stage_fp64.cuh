@@ -49,17 +49,6 @@ __device__ __forceinline__ void load_comp(const StateDev<double> &s, int64_t nt,
 #pragma unroll
   for (int l = 1; l < NB; ++l) x[l] = s.hi[(c * (NB - 1) + (l - 1)) * nt + K];
 }
-// block fixed point of a component's coefficients; returns the block's exponent
-template <int NB>
-__device__ __forceinline__ int fx_block(const double x[NB], Fx f[NB]) {
-  int mx = 0;
-#pragma unroll
-  for (int l = 0; l < NB; ++l) mx = max(mx, fx_abs_hi(x[l]));
-  const int E = fx_exp(mx);
-#pragma unroll
-  for (int l = 0; l < NB; ++l) f[l] = fx_from(x[l], E);
-  return E;
-}
 // value of the component's polynomial at a fixed reference point: sum_l psi_l(x) f_l
 template <int NB>
 __device__ __forceinline__ int64_t fx_point(const Fx f[NB], double xi, double eta) {
@@ -67,11 +56,6 @@ __device__ __forceinline__ int64_t fx_point(const Fx f[NB], double xi, double et
 #pragma unroll
   for (int l = 0; l < NB; ++l) fx_mac(s, fxc(psi(l, xi, eta)), f[l]);
   return fx_sum(s);
-}
-// fx_to, NaN for a block that holds a non-finite value
-__device__ __forceinline__ double fx_out(int64_t r, int E) {
-  const double x = fx_to(r, E);
-  return E >= FX_ENAN ? NAN : x;
 }
 // component c of four values held by every lane
 __device__ __forceinline__ double pick4(const double v[4], int c) {
