@@ -371,6 +371,22 @@ const double C_IN[3] = {0.0, 1.0, 0.5}, C_OUT[3] = {1.0, 0.5, 1.0};
 void enqueue_step(dg_solver *s) {
   const StageCtx &c = s->ctx;
   const int oe = s->cfg.oe != DG_OE_OFF, bp = s->cfg.bp != DG_BP_OFF;
+  const int64_t ntiles = num_tiles(s->mesh->nt, c.prec);
+  if (num_groups(ntiles) <= FUSE_GROUPS) {
+    // few tiles: each kernel finishes the reduction of the one before it; the
+    // last stage's alpha, counters and time are finished for the host
+    const int n = (int)ntiles;
+    for (int st = 0; st < 3; ++st) {
+      launch_rk_only(c, st == 0 ? s->un : s->us, s->un, s->uh, RK_A[st], RK_B[st], C_IN[st],
+                     Fuse{1, n, st == 0 ? nullptr : c.part_alpha, c.part_cnt, c.sc});
+      if (oe) launch_stats_only(c, s->uh, C_OUT[st], Fuse{1, n, c.part_sum, nullptr, c.sc});
+      else launch_fin_mean(c);
+      launch_oe_bp_only(c, s->uh, st == 2 ? s->un : s->us, oe, bp, C_OUT[st], st == 2,
+                        oe ? Fuse{1, n, c.part_dev, nullptr, c.sc} : Fuse{});
+    }
+    launch_fin_alpha(c, 2);
+    return;
+  }
   launch_step_begin(c);
   for (int st = 0; st < 3; ++st) {
     const StateBuf &v = st == 0 ? s->un : s->us;

@@ -743,4 +743,100 @@ __device__ __forceinline__ void step_begin_thread(Scalars *sc) {
   }
 }
 
+// ------------------------------------------------------------------------
+// Finalisation inside the consuming kernel (few tiles)
+// ------------------------------------------------------------------------
+// A finalize kernel of a small mesh is one block and almost all latency
+// (launch, partials from L2, a serial chain of FP64 operations, the ticket): about
+// 5 us, nine times per step.  With at most FUSE_GROUPS groups of tiles every
+// block of the consuming kernel takes the reduction itself, in the order of the
+// finalize kernels, into a copy of the scalars in its shared memory, and block
+// 0 writes them back.  No field that a block of the same launch reads from
+// memory for its result is written in that launch.  Isentropic vortex, 2,048 P1
+// cells: @FUSE@
+constexpr int FUSE_GROUPS = 2;
+struct Fuse {
+  int on, ntiles;
+  const double *part;       // partials of the kernel before (nullptr: none, the step start)
+  const long long *cnt;     // counters beside the wave speeds
+  Scalars *sc;
+};
+
+// all partials -> out[] in every thread, the arithmetic of reduce_group and reduce_top
+template <int N, typename T, typename Op>
+__device__ __forceinline__ void fused_reduce(const T *part, int ntiles, Op op, T out[N]) {
+  __shared__ T grp[FUSE_GROUPS * N];
+  const int ng = (ntiles + TILE_GROUP - 1) / TILE_GROUP;
+  for (int g = 0; g < ng; ++g) reduce_group<N>(part, g, ntiles, grp, op);
+  if (ng > 1) {
+    T v[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = threadIdx.x < ng ? grp[threadIdx.x * N + q] : Op::template ident<T>();
+    block_reduce<N>(v, grp, op);
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q) out[q] = op(Op::template ident<T>(), grp[q]);
+}
+__device__ __forceinline__ void copy_scalars(const Scalars *sc, Scalars *s) {
+  static_assert(sizeof(Scalars) % 8 == 0 && sizeof(Scalars) / 8 <= TPB, "one word per thread");
+  if (threadIdx.x < sizeof(Scalars) / 8)
+    reinterpret_cast<double *>(s)[threadIdx.x] = reinterpret_cast<const double *>(sc)[threadIdx.x];
+  __syncthreads();
+}
+
+// domain means (before K2), normalisers (before K3), alpha of the stage input or
+// the step start (before K1): the scalars to use, in s
+__device__ __forceinline__ void fuse_means(const Fuse &f, Scalars *s) {
+  copy_scalars(f.sc, s);
+  double r[4];
+  fused_reduce<4>(f.part, f.ntiles, OpSum(), r);
+  if (threadIdx.x < 4) {
+    const double mean = (threadIdx.x == 0 ? r[0] : threadIdx.x == 1 ? r[1] : threadIdx.x == 2 ? r[2] : r[3]) / s->area_total;
+    s->mean[threadIdx.x] = mean;
+    if (blockIdx.x == 0) f.sc->mean[threadIdx.x] = mean;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void fuse_deviations(const Fuse &f, Scalars *s, int cw) {
+  copy_scalars(f.sc, s);
+  double r[5];
+  fused_reduce<5>(f.part, f.ntiles, OpMaxNN(), r);
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 5; ++q) s->dev[q] = r[q];
+    write_inv_normalisers(s, cw);
+    if (blockIdx.x == 0) {
+      for (int q = 0; q < 5; ++q) f.sc->dev[q] = s->dev[q];
+      for (int q = 0; q < 4; ++q) { f.sc->invD[q] = s->invD[q]; f.sc->invDf[q] = s->invDf[q]; }
+    }
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void fuse_alpha(const Fuse &f, Scalars *s) {
+  copy_scalars(f.sc, s);
+  if (f.part) {
+    if (!s->active) return;   // an idle step leaves the counters alone
+    double a[1];
+    fused_reduce<1>(f.part, f.ntiles, OpMaxNN(), a);
+    long long n[2] = {0, 0};
+    if (blockIdx.x == 0) fused_reduce<2>(f.cnt, f.ntiles, OpSum(), n);
+    if (threadIdx.x == 0) {
+      s->alpha = a[0];
+      if (blockIdx.x == 0) {   // as finish_alpha_top after stage 0 or 1
+        f.sc->alpha = a[0];
+        f.sc->limited += n[0];
+        f.sc->nonphys += n[1];
+        if (a[0] * s->dt > s->min_ca * (1.0 + 1e-12)) f.sc->breaches += 1;
+      }
+    }
+  } else if (threadIdx.x == 0) {
+    step_begin_thread(s);
+    if (blockIdx.x == 0) {
+      f.sc->dt = s->dt;
+      f.sc->pad = s->pad;
+      f.sc->active = s->active;
+    }
+  }
+  __syncthreads();
+}
+
 }  // namespace dg

@@ -188,22 +188,22 @@ void launch_geometry(cudaStream_t s, int64_t nt, const double *vxy, const GeomPt
 template <int K, typename Real>
 static void rk_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> v, StateDev<Real> un,
                     StateDev<Real> uh, const void *tr, void *vd, void *hs, double *part_sum, const Scalars *sc,
-                    double a, double b, double c_in) {
+                    double a, double b, double c_in, const Fuse &f) {
   k_rk<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
-                                              sc, a, b, c_in);
+                                              sc, a, b, c_in, f);
 }
 template <int K, typename Real>
 static void stats_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, double *part_dev,
-                       const void *vd, const void *hs, void *ej, const Scalars *sc, double c_out) {
+                       const void *vd, const void *hs, void *ej, const Scalars *sc, double c_out, const Fuse &f) {
   k_stats<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
-                                                 sc, c_out);
+                                                 sc, c_out, f);
 }
 template <int K, typename Real>
 static void oebp_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, StateDev<Real> out,
                       const void *ej, void *tr, double *pa, long long *pc, const Scalars *sc, int do_oe,
-                      int do_bp, double c_out, int end_of_step) {
+                      int do_bp, double c_out, int end_of_step, const Fuse &f) {
   k_oe_bp<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe,
-                                                 do_bp, c_out, end_of_step);
+                                                 do_bp, c_out, end_of_step, f);
 }
 
 #define DG_DISPATCH(K_, PREC_, CALL)                        \
@@ -221,10 +221,10 @@ static void oebp_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev
 
 // k_rk: volume + edge fluxes + RK combination, block sums of |K| u_h^(0)
 void launch_rk_only(const StageCtx &c, const StateBuf &v, const StateBuf &un, const StateBuf &uh, double a,
-                    double b, double c_in) {
+                    double b, double c_in, const Fuse &f) {
   DG_DISPATCH(c.k, c.prec,
               (rk_impl<KK, Real>(c.stream, c.mesh, c.phys, {v.avg, (Real *)v.hi}, {un.avg, (Real *)un.hi},
-                                 {uh.avg, (Real *)uh.hi}, c.tr, c.vd, c.hs, c.part_sum, c.sc, a, b, c_in)));
+                                 {uh.avg, (Real *)uh.hi}, c.tr, c.vd, c.hs, c.part_sum, c.sc, a, b, c_in, f)));
 }
 
 void launch_fin_mean(const StageCtx &c) {
@@ -239,10 +239,10 @@ void launch_rk(const StageCtx &c, const StateBuf &v, const StateBuf &un, const S
 }
 
 // k_stats: deviation maxima at the volume points and the edge OE records
-void launch_stats_only(const StageCtx &c, const StateBuf &uh, double c_out) {
+void launch_stats_only(const StageCtx &c, const StateBuf &uh, double c_out, const Fuse &f) {
   DG_DISPATCH(c.k, c.prec,
               (stats_impl<KK, Real>(c.stream, c.mesh, c.phys, {uh.avg, (Real *)uh.hi}, c.part_dev, c.vd, c.hs, c.ej,
-                                    c.sc, c_out)));
+                                    c.sc, c_out, f)));
 }
 
 void launch_fin_dev(const StageCtx &c) {
@@ -257,10 +257,10 @@ void launch_stats(const StageCtx &c, const StateBuf &uh, double c_out) {
 
 // k_oe_bp: RIOE + limiter + traces, block maxima of the wave speed and counters
 void launch_oe_bp_only(const StageCtx &c, const StateBuf &uh, const StateBuf &out, int do_oe, int do_bp,
-                       double c_out, int end_of_step) {
+                       double c_out, int end_of_step, const Fuse &f) {
   DG_DISPATCH(c.k, c.prec,
               (oebp_impl<KK, Real>(c.stream, c.mesh, c.phys, {uh.avg, (Real *)uh.hi}, {out.avg, (Real *)out.hi}, c.ej,
-                                   c.tr, c.part_alpha, c.part_cnt, c.sc, do_oe, do_bp, c_out, end_of_step)));
+                                   c.tr, c.part_alpha, c.part_cnt, c.sc, do_oe, do_bp, c_out, end_of_step, f)));
 }
 
 // alpha and counters; after stage 2 also t += dt (stage < 0: outside a step)

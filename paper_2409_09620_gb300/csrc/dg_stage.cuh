@@ -196,7 +196,12 @@ template <int K, typename Real>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D)
     k_rk(MeshDev m, Phys ph, StateDev<Real> v, StateDev<Real> un, StateDev<Real> uh, const Real *__restrict__ tr,
          Real *__restrict__ vdo, Real *__restrict__ hso, double *part_sum, const Scalars *sc, double a, double b,
-         double c_in) {
+         double c_in, Fuse f) {
+  __shared__ Scalars s_sc;
+  if (f.on) {
+    fuse_alpha(f, &s_sc);
+    sc = &s_sc;
+  }
   if (!sc->active) return;
   rk_tile<K, Real>(m, ph, v, un, uh, tr, vdo, hso, part_sum, sc, a, b, c_in, blockIdx.x);
 }
@@ -205,8 +210,13 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D
 template <int K, typename Real>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_MINB_D)
     k_stats(const __grid_constant__ MeshDev m, const __grid_constant__ Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
-            const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out) {
+            const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out, Fuse f) {
   if (!sc->active) return;
+  __shared__ Scalars s_sc;
+  if (f.on) {
+    fuse_means(f, &s_sc);
+    sc = &s_sc;
+  }
   stats_tile<K, Real>(m, uh, part_dev, sc, blockIdx.x);
   edge_tile<K, Real>(m, ph, uh.avg, vdi, hsi, ej, sc, c_out, blockIdx.x);
 }
@@ -216,8 +226,13 @@ template <int K, typename Real>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? OEBP_MINB_F : OEBP_MINB_D)
     k_oe_bp(MeshDev m, Phys ph, StateDev<Real> uh, StateDev<Real> out, const Real *__restrict__ ej,
             Real *__restrict__ tr, double *part_alpha, long long *part_cnt, const Scalars *sc, int do_oe,
-            int do_bp, double c_out, int end_of_step) {
+            int do_bp, double c_out, int end_of_step, Fuse f) {
   if (!sc->active) return;
+  __shared__ Scalars s_sc;
+  if (f.on) {
+    fuse_deviations(f, &s_sc, ph.oe == 2);
+    sc = &s_sc;
+  }
   oe_bp_tile<K, Real>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, sc, do_oe, do_bp, c_out, end_of_step, blockIdx.x);
 }
 
