@@ -755,10 +755,13 @@ __device__ __forceinline__ void step_begin_thread(Scalars *sc) {
 // memory for its result is written in that launch.  Per step: vortex, 2,048 P1
 // cells FP64, 127 -> 104 us; Riemann problem, 1,058 P2 cells mixed, 118 -> 90 us.
 // The limit: P2 FP64, 2 groups (7,688 cells) 178 -> 166 us, 4 groups 229 -> 243 us;
-// mixed, 2 groups (31,250 cells) 125 -> 116 us, 4 groups 144 -> 161 us.
+// mixed, 2 groups (31,250 cells) 125 -> 116 us, 4 groups 144 -> 161 us.  The
+// kernels have a variant for it: chosen at run time it cost the mixed form's
+// large meshes 1.5 %.
 constexpr int FUSE_GROUPS = 2;
 struct Fuse {
-  int on, ntiles;
+  int on;                   // which kernel to launch: the one that finishes the reduction itself
+  int ntiles;
   const double *part;       // partials of the kernel before (nullptr: none, the step start)
   const long long *cnt;     // counters beside the wave speeds
   Scalars *sc;

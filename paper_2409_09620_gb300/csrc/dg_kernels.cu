@@ -189,21 +189,33 @@ template <int K, typename Real>
 static void rk_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> v, StateDev<Real> un,
                     StateDev<Real> uh, const void *tr, void *vd, void *hs, double *part_sum, const Scalars *sc,
                     double a, double b, double c_in, const Fuse &f) {
-  k_rk<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
+  auto launch = [&](auto kernel) {
+    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
                                               sc, a, b, c_in, f);
+  };
+  if (f.on) launch(k_rk<K, Real, true>);
+  else launch(k_rk<K, Real, false>);
 }
 template <int K, typename Real>
 static void stats_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, double *part_dev,
                        const void *vd, const void *hs, void *ej, const Scalars *sc, double c_out, const Fuse &f) {
-  k_stats<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
-                                                 sc, c_out, f);
+  auto launch = [&](auto kernel) {
+    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
+                                              sc, c_out, f);
+  };
+  if (f.on) launch(k_stats<K, Real, true>);
+  else launch(k_stats<K, Real, false>);
 }
 template <int K, typename Real>
 static void oebp_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, StateDev<Real> out,
                       const void *ej, void *tr, double *pa, long long *pc, const Scalars *sc, int do_oe,
                       int do_bp, double c_out, int end_of_step, const Fuse &f) {
-  k_oe_bp<K, Real><<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe,
-                                                 do_bp, c_out, end_of_step, f);
+  auto launch = [&](auto kernel) {
+    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe, do_bp,
+                                              c_out, end_of_step, f);
+  };
+  if (f.on) launch(k_oe_bp<K, Real, true>);
+  else launch(k_oe_bp<K, Real, false>);
 }
 
 #define DG_DISPATCH(K_, PREC_, CALL)                        \
@@ -297,8 +309,10 @@ int64_t num_tiles(int64_t nt, int prec) { return (nt + tile_cells(prec) - 1) / t
 
 size_t stage_kernels_local_bytes(int k, int prec) {
   size_t n = 0;
-  DG_DISPATCH(k, prec, (n = std::max({kernel_local_bytes(k_rk<KK, Real>), kernel_local_bytes(k_stats<KK, Real>),
-                                      kernel_local_bytes(k_oe_bp<KK, Real>)})));
+  DG_DISPATCH(k, prec, (n = std::max({kernel_local_bytes(k_rk<KK, Real, true>), kernel_local_bytes(k_stats<KK, Real, true>),
+                                      kernel_local_bytes(k_oe_bp<KK, Real, true>), kernel_local_bytes(k_rk<KK, Real, false>),
+                                      kernel_local_bytes(k_stats<KK, Real, false>),
+                                      kernel_local_bytes(k_oe_bp<KK, Real, false>)})));
   return n;
 }
 

@@ -192,13 +192,13 @@ __device__ __forceinline__ void oe_bp_tile(const MeshDev &m, const Phys &ph, Sta
     oe_bp_tile_fp64<K>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, sc, do_oe, do_bp, c_out, end_of_step, tile);
 }
 
-template <int K, typename Real>
+template <int K, typename Real, bool FUSED>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D)
     k_rk(MeshDev m, Phys ph, StateDev<Real> v, StateDev<Real> un, StateDev<Real> uh, const Real *__restrict__ tr,
          Real *__restrict__ vdo, Real *__restrict__ hso, double *part_sum, const Scalars *sc, double a, double b,
          double c_in, Fuse f) {
-  __shared__ Scalars s_sc;
-  if (f.on) {
+  if constexpr (FUSED) {
+    __shared__ Scalars s_sc;
     fuse_alpha(f, &s_sc);
     sc = &s_sc;
   }
@@ -207,13 +207,13 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D
 }
 
 // OE statistics of the tile's cells and the jump data of the edges it owns
-template <int K, typename Real>
+template <int K, typename Real, bool FUSED>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_MINB_D)
     k_stats(const __grid_constant__ MeshDev m, const __grid_constant__ Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
             const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out, Fuse f) {
   if (!sc->active) return;
-  __shared__ Scalars s_sc;
-  if (f.on) {
+  if constexpr (FUSED) {
+    __shared__ Scalars s_sc;
     fuse_means(f, &s_sc);
     sc = &s_sc;
   }
@@ -222,14 +222,14 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_
 }
 
 // RIOE damping, BP limiter, traces and wave speeds of the stage result
-template <int K, typename Real>
+template <int K, typename Real, bool FUSED>
 __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? OEBP_MINB_F : OEBP_MINB_D)
     k_oe_bp(MeshDev m, Phys ph, StateDev<Real> uh, StateDev<Real> out, const Real *__restrict__ ej,
             Real *__restrict__ tr, double *part_alpha, long long *part_cnt, const Scalars *sc, int do_oe,
             int do_bp, double c_out, int end_of_step, Fuse f) {
   if (!sc->active) return;
-  __shared__ Scalars s_sc;
-  if (f.on) {
+  if constexpr (FUSED) {
+    __shared__ Scalars s_sc;
     fuse_deviations(f, &s_sc, ph.oe == 2);
     sc = &s_sc;
   }
