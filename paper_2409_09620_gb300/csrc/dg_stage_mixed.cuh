@@ -374,7 +374,7 @@ constexpr int VTX_REC = 14;
 // and gradients at both endpoints, the (constant) Hessian jump once
 template <int K>
 __device__ __forceinline__ void edge_jumps_mixed(int I, const MeshDev &m, const Phys &ph, const StateDev<float> &uh,
-                                                 int64_t Kc, const float a0f[4], const float (*sv)[TPB],
+                                                 int64_t Kc, const float a0f[4], const float (*sv)[32],
                                                  const float hme[12], int32_t cn, float nx, float ny, double t_out,
                                                  int cw, float &beta, float Jq[4][K + 1]) {
   constexpr int NB = Deg<K>::NB;
@@ -438,10 +438,10 @@ __device__ __forceinline__ void edge_jumps_mixed(int I, const MeshDev &m, const 
     // this cell's value, physical gradient, 1/rho and sound speed at the vertex
     float val[4], grd[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) val[q] = sv[VTX_REC * ov + q][threadIdx.x];
+    for (int q = 0; q < 4; ++q) val[q] = sv[VTX_REC * ov + q][threadIdx.x & 31];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) grd[q] = sv[VTX_REC * ov + 4 + q][threadIdx.x];
-    const float ri = sv[VTX_REC * ov + 12][threadIdx.x], cs = sv[VTX_REC * ov + 13][threadIdx.x];
+    for (int q = 0; q < 8; ++q) grd[q] = sv[VTX_REC * ov + 4 + q][threadIdx.x & 31];
+    const float ri = sv[VTX_REC * ov + 12][threadIdx.x & 31], cs = sv[VTX_REC * ov + 13][threadIdx.x & 31];
     const float r_own = fma(fabsf(fdot2(val[1], nx, val[2], ny)), ri, cs);
     float xv[4], xg[8], r_oth;
     if (cn >= 0) {
@@ -483,197 +483,191 @@ __device__ __forceinline__ void edge_jumps_mixed(int I, const MeshDev &m, const 
 }
 
 // ---------------------------------------------------------------------------
-// FP64 theta of the mixed form (Sec. 4.4 Steps 1-2), one warp per cell
+// FP64 theta of the mixed form (Sec. 4.4 Steps 1-2), eight cells of a warp at a time
 // ---------------------------------------------------------------------------
+// shared scratch of a warp: the vertex records of its 32 cells during the OE
+// ([3 VTX_REC][32] floats), then the limiter's.  One array for both degrees,
+// for the batch kernels hold both.
+constexpr int OE_WARP_SCRATCH = 3 * VTX_REC * 32 * 4;
+__device__ __forceinline__ unsigned char *oe_warp_scratch() {
+  __shared__ __align__(16) unsigned char buf[TPB / 32][OE_WARP_SCRATCH];
+  return buf[threadIdx.x >> 5];
+}
 // The limiter point set of a P_K cell: the 3 (K + 1) edge Gauss points, then
 // two extra points (the internal nodes of the optimal decomposition for P2,
-// the vertices v1, v2 for P1; with the classical decomposition both extra
-// rows are the weighted edge combination u_* of Sec. 4.1).  LimTab holds,
-// per point, psi_1 .. psi_{NB-1} there; the node rows come from the mesh.
-template <int K>
-struct LimTab {
-  static constexpr int NQ = K + 1, NE = 3 * NQ, NP = NE + 2, NB = Deg<K>::NB;
-  double v[NP][NB];
-};
-template <int K>
-constexpr LimTab<K> make_lim_tab() {
-  LimTab<K> t{};
-  constexpr int NQ = LimTab<K>::NQ, NE = LimTab<K>::NE, NB = LimTab<K>::NB;
-  for (int p = 0; p < NE; ++p) {
-    const double sg = gauss_s(NQ, p % NQ);
-    for (int l = 0; l < NB; ++l) t.v[p][l] = psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg));
-  }
-  for (int l = 0; l < NB; ++l) {
-    double acc = 0.0;   // classical extra row: P1 the first edge point, P2 -1/6 sum_p w_p psi(x_p)
-    for (int p = 0; p < NE; ++p) acc += gauss_w(NQ, p % NQ) * t.v[p][l];
-    const double v = K == 1 ? t.v[0][l] : (-1.0 / 6.0) * acc;
-    t.v[NE][l] = v;
-    t.v[NE + 1][l] = v;
-  }
-  return t;
-}
-static __device__ const LimTab<1> g_lim_tab1 = make_lim_tab<1>();
-static __device__ const LimTab<2> g_lim_tab2 = make_lim_tab<2>();
-
-// per-warp scratch of the cooperative limiter: the cell's averages, modes in
-// FP64, the scaled modes (FP32 and back in FP64) and the scalars of its theta
+// the vertices v1, v2 for P1; with the classical decomposition both are the
+// weighted edge combination u_* of Sec. 4.1).
 template <int K>
 struct LimScratch {
-  static constexpr int NM = 4 * (Deg<K>::NB - 1);
-  double a0[4], hd[NM], hsd[NM], sa[4];
-  float hs[NM];
+  static constexpr int NE = 3 * (K + 1), NP = NE + 2;
+  double dev[NP][8][4];             // deviations at the points, per cell and component
+  double a0[8][4];
+  int64_t cell[8];
+  float hs[8][4][Deg<K>::NB - 1];   // modes
+  int res[8];                       // 1: limited, 2: fell back to its average
 };
+static_assert(sizeof(LimScratch<2>) <= OE_WARP_SCRATCH, "scratch of a warp");
 
-// Warp reductions over the limiter points (lanes beyond the set hold the
-// identity): minimum on the integer units through order-preserving keys,
-// maximum of non-negative values on their bit patterns.
-__device__ __forceinline__ double warp_min_ord(double x) {
-  long long k = ord_key(x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) k = min(k, __shfl_xor_sync(0xffffffffu, k, o));
-  return ord_val(k);
-}
-__device__ __forceinline__ double warp_max_nn(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = max_nn(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
-
-// FP64 theta for the cells of this warp that failed the FP32 screen (flag).
-// The warp takes them one at a time; lane p evaluates limiter point p and
-// lane j scales mode j, so the serial FP64 work of a cell (well over a
-// thousand FP64 instructions, which GB300's narrow FP64 pipe runs at about
-// one warp instruction per 64 cycles per scheduler) shrinks to about a
-// hundred and fifty warp instructions.  The targets cover the rounding of
-// the FP32 store (2^-22 per unit of sum |mode|, |Psi| <= 4 on K); the stored
-// FP32 modes are then verified in FP64 at every point of the set, and a cell
-// that still fails keeps its average only.  On return a flagged lane's hi
-// holds the stored modes; limited is set when theta < 1 or the cell fell back
-// to its average.  Every lane of the warp calls this (the shuffles and
-// warp barriers take all 32).
+// FP64 theta for the cells of this warp that failed the FP32 screen (flag): four
+// lanes per cell, one per component, as in the FP64 form; point values in block
+// fixed point, what needs all components dealt out over the points.  About 120 FP64
+// instructions (64 cycles each) for up to eight cells, where one warp per
+// cell took about 150 for each: Sedov blast, 18,432 P2 cells, 100 steps, 467 -> 187 us
+// per step.  The targets cover the rounding of the FP32 store (2^-22 per unit of
+// sum |mode|, |Psi| <= 4 on K); the stored FP32 modes are then verified in FP64 at
+// every point of the set, and a cell that still fails keeps its average only.
+// On return a flagged lane's hi holds the stored modes; limited is set when theta <
+// 1 or the cell fell back to its average.  Every lane of the warp calls this (the
+// shuffles and warp barriers take all 32).
 template <int K>
 __device__ __forceinline__ void limit_fp64_warp(const MeshDev &m, const Phys &ph, bool flag, int64_t Kc,
                                                 const double a0[4], float hi[4][Deg<K>::NB], StateDev<float> out,
-                                                long long &limited) {
-  constexpr int NB = Deg<K>::NB, NQ = K + 1, NE = 3 * NQ, NP = NE + 2, NM = 4 * (NB - 1);
-  static_assert(NP <= 32 && NM <= 32, "one lane per point and per mode");
+                                                unsigned char *scratch, long long &limited) {
+  constexpr int NB = Deg<K>::NB, NQ = K + 1, NE = LimScratch<K>::NE, NP = LimScratch<K>::NP, NL = (NP + 3) / 4;
   const unsigned FULL = 0xffffffffu;
-  unsigned todo = __ballot_sync(FULL, flag);
+  const unsigned todo = __ballot_sync(FULL, flag);
   if (todo == 0u) return;
-  __shared__ LimScratch<K> scr_all[TPB / 32];
-  LimScratch<K> &S = scr_all[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
+  LimScratch<K> &S = *reinterpret_cast<LimScratch<K> *>(scratch);
+  const int lane = threadIdx.x & 31, quad = lane >> 2, c = lane & 3, q0 = lane & ~3;
   const int64_t nt = m.nt;
   const double r22 = 2.384185791015625e-07;   // 2^-22
-  // this lane's basis values at its point (edge rows; extra rows per cell below)
-  double psv[NB];
-  const bool on_pt = lane < NP;
-  const int prow = on_pt ? lane : 0;
-#pragma unroll
-  for (int l = 1; l < NB; ++l) psv[l] = K == 1 ? g_lim_tab1.v[prow][l] : g_lim_tab2.v[prow][l];
-  const bool node_row = on_pt && lane >= NE && !ph.decomp;
-  while (todo) {
-    const int src = __ffs(todo) - 1;
-    todo &= todo - 1u;
-    const int64_t Ks = __shfl_sync(FULL, Kc, src);
-    if (lane == src) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) S.a0[c] = a0[c];
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int l = 1; l < NB; ++l) S.hs[c * (NB - 1) + l - 1] = hi[c][l];
-    }
+  const int rank = __popc(todo & ((1u << lane) - 1u)), n = __popc(todo);
+#pragma unroll 1
+  for (int base = 0; base < n; base += 8) {
+    const int slot = rank - base;
+    const bool mine = flag && slot >= 0 && slot < 8;
     __syncwarp();
-    if (lane < NM) S.hd[lane] = double(S.hs[lane]);
-    if (node_row) {   // the extra point of this cell: P2 internal node, P1 vertex
-      const int e = lane - NE;
-      if (K == 1) {
-        const int vp = m.limv[e * nt + Ks];
+    if (mine) {
+      S.cell[slot] = Kc;
 #pragma unroll
-        for (int l = 1; l < NB; ++l) psv[l] = psi(l, vert_xi(vp), vert_eta(vp));
-      } else {
+      for (int q = 0; q < 4; ++q) {
+        S.a0[slot][q] = a0[q];
 #pragma unroll
-        for (int l = 1; l < NB; ++l) psv[l] = m.psi_node[(5 * e + l - 1) * nt + Ks];
+        for (int l = 1; l < NB; ++l) S.hs[slot][q][l - 1] = hi[q][l];
       }
     }
     __syncwarp();
-    if (lane < 4) {
-      double sa = 0.0;
+    const bool on = base + quad < n;
+    const int qs = on ? quad : 0;      // a quad without a cell repeats the first and stores nothing
+    const int64_t Ks = S.cell[qs];
+    double A[4], hd[NB];
 #pragma unroll
-      for (int l = 1; l < NB; ++l) sa += fabs(S.hd[lane * (NB - 1) + l - 1]);
-      S.sa[lane] = sa;
-    }
-    double A[4];
+    for (int q = 0; q < 4; ++q) A[q] = S.a0[qs][q];
+    hd[0] = 0.0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) A[c] = S.a0[c];
-    // deviations of the unlimited polynomial at this lane's point
-    double d[4] = {0.0, 0.0, 0.0, 0.0};
-    if (on_pt) {
+    for (int l = 1; l < NB; ++l) hd[l] = double(S.hs[qs][c][l - 1]);
+    double sa = 0.0;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        double acc = 0.0;
+    for (int l = 1; l < NB; ++l) sa = add(sa, fabs(hd[l]));
+    const double S0 = __shfl_sync(FULL, sa, q0), S1 = __shfl_sync(FULL, sa, q0 + 1), S2 = __shfl_sync(FULL, sa, q0 + 2),
+                 S3 = __shfl_sync(FULL, sa, q0 + 3);
+    // this component's deviations at every point, from the modes x
+    auto deviations = [&](const double x[NB]) {
+      Fx f[NB];
+      const int E = fx_block<NB>(x, f);
+      double ws = 0.0;   // classical: sum of w dev
 #pragma unroll
-        for (int l = 1; l < NB; ++l) acc = fma(psv[l], S.hd[c * (NB - 1) + l - 1], acc);
-        d[c] = acc;
+      for (int p = 0; p < NE; ++p) {
+        const double sg = gauss_s(NQ, p % NQ);
+        FxAcc s{0, 0};
+#pragma unroll
+        for (int l = 1; l < NB; ++l) fx_mac(s, fxc(psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg))), f[l]);
+        const double d = fx_out(fx_sum(s), E);
+        S.dev[p][quad][c] = d;
+        if (ph.decomp) ws = K == 1 ? (p == 0 ? d : ws) : fma(gauss_w(NQ, p % NQ), d, ws);
       }
-    }
-    __syncwarp();
-    double Sa[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) Sa[c] = S.sa[c];
-    // Step 1: density
-    const double rmin = warp_min_ord(on_pt ? A[0] + d[0] : INFINITY);
+      for (int p = 0; p < 2; ++p) {
+        double d;
+        if (ph.decomp) {
+          d = K == 1 ? ws : (-1.0 / 6.0) * ws;
+        } else {
+          d = 0.0;
+          const int vp = K == 1 ? m.limv[p * nt + Ks] : 0;
+#pragma unroll
+          for (int l = 1; l < NB; ++l)
+            d = fma(K == 1 ? psi(l, vert_xi(vp), vert_eta(vp)) : m.psi_node[(5 * p + l - 1) * nt + Ks], x[l], d);
+        }
+        S.dev[NE + p][quad][c] = d;
+      }
+      __syncwarp();
+    };
+    deviations(hd);
+    // Step 1: density.  This lane's points are c, c + 4, c + 8
+    long long kmin = ord_key(INFINITY);
+#pragma unroll
+    for (int p = c; p < NP; p += 4) kmin = min(kmin, ord_key(add(A[0], S.dev[p][quad][0])));
+    kmin = min(kmin, __shfl_xor_sync(FULL, kmin, 1));
+    kmin = min(kmin, __shfl_xor_sync(FULL, kmin, 2));
+    const double rmin = ord_val(kmin);
     const double eps1 = fmin(A[0], 1e-13);
-    const double tgt1 = fmin(A[0], fma(2.0 * r22, Sa[0], eps1));
+    const double tgt1 = fmin(A[0], fma(2.0 * r22, S0, eps1));
     const double th1 = rmin < tgt1 ? (A[0] - tgt1) / (A[0] - rmin) : 1.0;
     // Step 2: internal energy of the density-limited polynomial; the target
     // covers the FP32 store through the largest squared speed on the set
-    const double w0 = fma(th1, d[0], A[0]), w1 = A[1] + d[1], w2 = A[2] + d[2], w3 = A[3] + d[3];
-    const double q = fdot2(w1, w1, w2, w2);
-    const double v2 = q / (w0 * w0);
-    const double vmax2 = warp_max_nn(on_pt && v2 == v2 ? v2 : 0.0);   // a NaN is ignored, as by fmax
+    double w0[NL], w3[NL], q[NL], vmax2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      const int p = c + 4 * i;
+      if (p >= NP) continue;
+      const double *d = S.dev[p][quad];
+      const double w1 = add(A[1], d[1]), w2 = add(A[2], d[2]);
+      w0[i] = fma(th1, d[0], A[0]);
+      w3[i] = add(A[3], d[3]);
+      q[i] = fdot2(w1, w1, w2, w2);
+      const double v2 = mul(q[i], recip(mul(w0[i], w0[i])));
+      if (v2 == v2) vmax2 = max_nn(vmax2, v2);   // a NaN is ignored, as by fmax
+    }
+    vmax2 = max_nn(vmax2, __shfl_xor_sync(FULL, vmax2, 1));
+    vmax2 = max_nn(vmax2, __shfl_xor_sync(FULL, vmax2, 2));
     const double Ebar = int_energy(A);
-    const double RE = r22 * fma(sqrt(vmax2), Sa[1] + Sa[2], fma(vmax2 * th1, Sa[0], Sa[3]));
+    const double RE = r22 * fma(root(vmax2), S1 + S2, fma(vmax2 * th1, S0, S3));
     const double eps2 = fmin(Ebar, 1e-13);
     const double tgt2 = fmin(Ebar, fma(2.0, RE, eps2));
     // E - |m|^2 / (2 rho) < tgt2 tested as rho E - |m|^2 / 2 < tgt2 rho (rho > 0):
     // the division only at points that violate the target
-    double e_pt = INFINITY;
-    if (on_pt && (!(w0 > 0.0) || fma(w3, w0, -0.5 * q) < tgt2 * w0)) e_pt = w3 - 0.5 * q / w0;
-    const double emin = warp_min_ord(e_pt);
+    long long kem = ord_key(INFINITY);
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      if (c + 4 * i >= NP) continue;
+      const double hq = half_neg(q[i]);
+      if (!(w0[i] > 0.0) || fma(w3[i], w0[i], hq) < mul(tgt2, w0[i])) kem = min(kem, ord_key(w3[i] + hq / w0[i]));
+    }
+    kem = min(kem, __shfl_xor_sync(FULL, kem, 1));
+    kem = min(kem, __shfl_xor_sync(FULL, kem, 2));
+    const double emin = ord_val(kem);
     const double th2 = emin < tgt2 ? (Ebar - tgt2) / (Ebar - emin) : 1.0;
-    // the scaled modes, one per lane, stored in FP32 and read back in FP64
-    if (lane < NM) {
-      const double th = lane < NB - 1 ? th1 * th2 : th2;
-      const float h = float(th * S.hd[lane]);
-      S.hs[lane] = h;
-      S.hsd[lane] = double(h);
+    // the scaled modes, stored in FP32 and verified in FP64 at every point of the set
+    const double th = c == 0 ? th1 * th2 : th2;
+#pragma unroll
+    for (int l = 1; l < NB; ++l) {
+      const float h = float(mul(th, hd[l]));
+      hd[l] = double(h);
+      if (on) S.hs[quad][c][l - 1] = h;
     }
-    __syncwarp();
-    // verify the stored modes at every point of the set
+    __syncwarp();   // every lane has read the deviations
+    deviations(hd);
     bool bad_pt = false;
-    if (on_pt) {
-      double v[4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        double acc = 0.0;
-#pragma unroll
-        for (int l = 1; l < NB; ++l) acc = fma(psv[l], S.hsd[c * (NB - 1) + l - 1], acc);
-        v[c] = A[c] + acc;
-      }
-      bad_pt = !(v[0] > 0.0) || !(fma(v[3], v[0], -0.5 * fdot2(v[1], v[1], v[2], v[2])) > 0.0);
+    for (int i = 0; i < NL; ++i) {
+      const int p = c + 4 * i;
+      if (p >= NP) continue;
+      const double *d = S.dev[p][quad];
+      const double v0 = add(A[0], d[0]), v1 = add(A[1], d[1]), v2 = add(A[2], d[2]), v3 = add(A[3], d[3]);
+      bad_pt = bad_pt || !(v0 > 0.0) || !(fma(v3, v0, half_neg(fdot2(v1, v1, v2, v2))) > 0.0);
     }
-    const bool bad = __any_sync(FULL, bad_pt);
-    if (lane == src) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int l = 1; l < NB; ++l) hi[c][l] = bad ? 0.0f : S.hs[c * (NB - 1) + l - 1];
-      store_modes_mixed<NB>(out, Kc, hi);
-      if (th1 < 1.0 || th2 < 1.0 || bad) limited = 1;
-    }
+    const unsigned bad = (__ballot_sync(FULL, bad_pt) >> q0) & 0xfu;
+    if (on && c == 0) S.res[quad] = (th1 < 1.0 || th2 < 1.0 || bad ? 1 : 0) | (bad ? 2 : 0);
     __syncwarp();
+    if (mine) {
+      const int r = S.res[slot];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int l = 1; l < NB; ++l) hi[k][l] = r & 2 ? 0.0f : S.hs[slot][k][l - 1];
+      store_modes_mixed<NB>(out, Kc, hi);
+      if (r) limited = 1;
+    }
   }
 }
 
@@ -857,6 +851,7 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
   // alpha there too, or at the end time after the last stage of a clamped step
   const double dt = sc->dt, t_out = fma(c_out, sc->dt, sc->t);
   const double t_alpha = end_of_step && sc->pad ? sc->t_end : t_out;
+  unsigned char *scratch = oe_warp_scratch();
   double a0[4] = {0.0, 0.0, 0.0, 0.0};
   float a0f[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hi[4][NB];
   float nxs[3], nys[3];
@@ -882,9 +877,10 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
       for (int q = 0; q < 12; ++q) hme[q] = 0.0f;
       if constexpr (K == 2) hessian_p2(hi, jx, jy, ex, ey, hme);
       // the cell's own vertex data, formed once (each vertex serves two
-      // edges) at compile-time vertex indices, in this thread's column of a
-      // block-shared array (no exchange between threads, so no barrier)
-      __shared__ float s_vtx[3 * VTX_REC][TPB];
+      // edges) at compile-time vertex indices, in this thread's column of the
+      // warp's scratch (no exchange between threads, so no barrier)
+      float (*s_vtx)[32] = reinterpret_cast<float (*)[32]>(scratch);
+      const int lane = threadIdx.x & 31;
       {
         const float gamma = ph.gamma_f, gm1 = ph.gm1_f;
         static_for<3>([&](auto vc) {
@@ -893,11 +889,11 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
           vertex_eval<K>(v, a0f, hi, val, gx, ge);
           vertex_phys<K>(val, gx, ge, jx, jy, ex, ey, gamma, gm1, grd, ri, cs);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) s_vtx[VTX_REC * v + q][threadIdx.x] = val[q];
+          for (int q = 0; q < 4; ++q) s_vtx[VTX_REC * v + q][lane] = val[q];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) s_vtx[VTX_REC * v + 4 + q][threadIdx.x] = grd[q];
-          s_vtx[VTX_REC * v + 12][threadIdx.x] = ri;
-          s_vtx[VTX_REC * v + 13][threadIdx.x] = cs;
+          for (int q = 0; q < 8; ++q) s_vtx[VTX_REC * v + 4 + q][lane] = grd[q];
+          s_vtx[VTX_REC * v + 12][lane] = ri;
+          s_vtx[VTX_REC * v + 13][lane] = cs;
         });
       }
       // sigma_q^j = sum_i (beta_i / h_i) A^{k,j} h_i^j sqrt(J) / D_q (see dg_stage_fp64.cuh)
@@ -971,7 +967,7 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
     lim64 = limit_screen_mixed<K>(m, ph, a0, a0f, hi, out, Kc, do_bp, cnt);
   }
   // the FP64 theta of the cells that failed the screen, by the whole warp
-  limit_fp64_warp<K>(m, ph, lim64, Kc, a0, hi, out, cnt[0]);
+  limit_fp64_warp<K>(m, ph, lim64, Kc, a0, hi, out, scratch, cnt[0]);
   if (live) alpha_mixed<K>(m, ph, a0f, hi, nxs, nys, cns, Kc, t_alpha, amax);
   double av[1] = {amax};
   block_reduce<1>(av, part_alpha + tile, OpMaxNN());
