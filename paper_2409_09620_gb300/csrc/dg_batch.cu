@@ -209,19 +209,19 @@ __global__ void __launch_bounds__(TPB) k_batch_begin(const SolveDev *__restrict_
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<2, Real>::rk)
     k_batch_rk(const SolveDev *__restrict__ sv, const WorkItem *__restrict__ work, int nwork, int stage) {
   phase_rk<Real>(sv, work, nwork, stage);
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<2, Real>::stats)
     k_batch_stats(const SolveDev *__restrict__ sv, const WorkItem *__restrict__ work, int nwork, int stage) {
   phase_stats<Real>(sv, work, nwork, stage);
 }
 
 template <typename Real>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? OEBP_MINB_F : OEBP_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<2, Real>::oe_bp)
     k_batch_oe_bp(const SolveDev *__restrict__ sv, const WorkItem *__restrict__ work, int nwork, int stage) {
   phase_oe_bp<Real>(sv, work, nwork, stage);
 }

@@ -19,30 +19,32 @@
 
 namespace dg {
 
-// Resident blocks per SM requested from the register allocator (FP32 / FP64
-// instantiations).  Higher occupancy hides the latency of the neighbour
-// gathers and of the FP64 pipe better than the few spilled registers cost.
-// FP64, 1,036,800 P2 cells, ms per launch: k_rk 1.13 with 5 blocks, 1.12 with 6,
-// 1.09 with 7 and 8; k_stats 0.66 with 6, 0.61 with 7, 0.58 with 8; k_oe_bp the
-// same from 5 on (P1 1 % faster with 8).
-#ifndef RK_MINB_F
-#define RK_MINB_F 4
-#endif
-#ifndef STATS_MINB_F
-#define STATS_MINB_F 6
-#endif
-#ifndef OEBP_MINB_F
-#define OEBP_MINB_F 4
-#endif
-#ifndef RK_MINB_D
-#define RK_MINB_D 7
-#endif
-#ifndef STATS_MINB_D
-#define STATS_MINB_D 8
-#endif
-#ifndef OEBP_MINB_D
-#define OEBP_MINB_D 8
-#endif
+// Resident blocks per SM requested from the register allocator.  Higher
+// occupancy hides the latency of the neighbour gathers and of the FP64 pipe
+// until the spills cost more, which for the fewer modes of P1 happens later.
+// 1,036,800 cells, ms per launch:
+//   FP64  k_rk     P2 1.13 with 5 blocks, 1.12 with 6, 1.09 with 7 and 8;
+//                  P1 0.484 with 6, 0.472 with 7 and 8, 0.458 with 10, 0.476 with 12
+//         k_stats  P2 0.575 with 8, 0.548 with 10, 0.561 with 12, 0.72 with 14;
+//                  P1 0.417 with 8, 0.384 with 10, 0.373 with 12, 0.392 with 14
+//         k_oe_bp  the same from 5 to 10
+//   mixed k_rk     P2 0.181 with 3 blocks, 0.157 with 4, 0.166 with 5;
+//                  P1 0.136 with 4, 0.112 with 6, 0.103 with 8, 0.106 with 9
+//         k_oe_bp  P2 0.229 with 3 and 4 blocks, 0.265 with 5;
+//                  P1 0.149 with 4, 0.136 with 5, 0.135 with 6, 0.141 with 7
+//         k_stats  the same from 5 to 8 (bound by memory)
+// A small mesh (FUSED) has at most FUSE_GROUPS * TILE_GROUP blocks, not two per SM: its
+// kernels get all the registers they want.  us per step with 2 / 4 / 6 blocks: 1,058 P2
+// cells, mixed, 85 / 90 / 100; 20,000 P2 cells, mixed, 104 / 108 / 130; 2,048 P1 cells, FP64,
+// 100 / 100 / 102.
+// The batch kernels hold both degrees and take the values of P2.
+template <int K, typename Real, bool FUSED = false>
+struct MinBlocks {
+  static constexpr bool F = sizeof(Real) == 4;
+  static constexpr int rk = FUSED ? 2 : F ? (K == 1 ? 8 : 4) : (K == 1 ? 10 : 7);
+  static constexpr int stats = FUSED ? 2 : F ? 6 : (K == 1 ? 12 : 10);
+  static constexpr int oe_bp = FUSED ? 2 : F ? (K == 1 ? 6 : 4) : 8;
+};
 
 // A cell's state.  The FP64 form keeps the modes component- and mode-major
 // ([4][NB-1][nt]); the mixed form keeps each cell's 4 (NB - 1) FP32 modes
@@ -193,7 +195,7 @@ __device__ __forceinline__ void oe_bp_tile(const MeshDev &m, const Phys &ph, Sta
 }
 
 template <int K, typename Real, bool FUSED>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::rk)
     k_rk(MeshDev m, Phys ph, StateDev<Real> v, StateDev<Real> un, StateDev<Real> uh, const Real *__restrict__ tr,
          Real *__restrict__ vdo, Real *__restrict__ hso, double *part_sum, const Scalars *sc, double a, double b,
          double c_in, Fuse f) {
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? RK_MINB_F : RK_MINB_D
 
 // OE statistics of the tile's cells and the jump data of the edges it owns
 template <int K, typename Real, bool FUSED>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::stats)
     k_stats(const __grid_constant__ MeshDev m, const __grid_constant__ Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
             const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out, Fuse f) {
   if (!sc->active) return;
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? STATS_MINB_F : STATS_
 
 // RIOE damping, BP limiter, traces and wave speeds of the stage result
 template <int K, typename Real, bool FUSED>
-__global__ void __launch_bounds__(TPB, sizeof(Real) == 4 ? OEBP_MINB_F : OEBP_MINB_D)
+__global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::oe_bp)
     k_oe_bp(MeshDev m, Phys ph, StateDev<Real> uh, StateDev<Real> out, const Real *__restrict__ ej,
             Real *__restrict__ tr, double *part_alpha, long long *part_cnt, const Scalars *sc, int do_oe,
             int do_bp, double c_out, int end_of_step, Fuse f) {
