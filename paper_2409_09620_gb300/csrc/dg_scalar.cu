@@ -207,14 +207,14 @@ __global__ void __launch_bounds__(TPB) k_sc_rk(MeshDev m, ScPhys ph, const doubl
           const double um = tr[(Kc * 3 + i) * NQ + nu];
           const double up = cn >= 0 ? tr[((int64_t)(cn >> 2) * 3 + (cn & 3)) * NQ + (NQ - 1 - nu)] : sghost(ph, -cn, um);
           const double s = ph.flux == 0 ? add(um, up) : add(mul(um, um), mul(up, up));
-          tv[i * NQ + nu] = sub(mul(vl, s), mul(al, sub(up, um)));
+          tv[i * NQ + nu] = fma(al, sub(um, up), mul(vl, s));
         }
       }
       Ee = fx_block<3 * NQ>(tv, y);
     }
     // quadrature sums, mass inverse and SSP-RK combination
     const double A1 = fdot2(d1, m.jinv[Kc], d2, m.jinv[nt + Kc]), A2 = fdot2(d1, m.jinv[2 * nt + Kc], d2, m.jinv[3 * nt + Kc]);
-    const double dta = dt / area;
+    const double dta = mul(dt, m.iarea[Kc]);
 #pragma unroll
     for (int l = 0; l < NB; ++l) {
       FxAcc e{0, 0};
@@ -247,10 +247,14 @@ __global__ void __launch_bounds__(TPB) k_sc_rk(MeshDev m, ScPhys ph, const doubl
 // The records hold d^j u / dx^p dy^(j-p), j <= K, at the three vertices, for
 // the OE jumps of the neighbours and the cell itself.  The affine map gives d/dx
 // = xi_x d/dxi + eta_x d/deta, d/dy = xi_y d/dxi + eta_y d/deta: a symmetric
-// tensor of order j is turned one index at a time.
+// tensor of order j is turned one index at a time.  P3 takes 190 registers if
+// let, two blocks per SM and a second, nearly empty wave on 400 blocks: with
+// three, Burgers on 51,200 cells takes 293 instead of 315 us per step, 204,800 cells of
+// P3 convection 931 instead of 946; four and more spill (299, 306 us).
 template <int K>
-__global__ void __launch_bounds__(TPB) k_sc_stats(MeshDev m, const double *__restrict__ u, double *__restrict__ vr,
-                                                  double *part, const ScScalars *sc) {
+__global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, const double *__restrict__ u,
+                                                                  double *__restrict__ vr, double *part,
+                                                                  const ScScalars *sc) {
   constexpr int NB = SDeg<K>::NB, NV = SDeg<K>::NV;
   if (!sc->active) return;
   const int64_t nt = m.nt;
