@@ -123,11 +123,11 @@ __device__ __forceinline__ void phase_rk(const SolveDev *__restrict__ sv, const 
     const StateDev<Real> v{S.avg[vi], (Real *)S.hi[vi]}, un{S.avg[0], (Real *)S.hi[0]}, uh{S.avg[1], (Real *)S.hi[1]};
     for (int64_t t = it.first_tile; t < it.first_tile + it.ntiles; ++t) {
       if (S.k == 1)
-        rk_tile<1, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum, S.sc,
-                         a, b, c_in, t);
+        rk_tile<1, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
+                         PlainScalars{S.sc}, a, b, c_in, t);
       else
-        rk_tile<2, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum, S.sc,
-                         a, b, c_in, t);
+        rk_tile<2, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
+                         PlainScalars{S.sc}, a, b, c_in, t);
       finish_means(S.part_sum, S.fin, t, S.ntiles, S.sc);
     }
   }
@@ -145,11 +145,11 @@ __device__ __forceinline__ void phase_stats(const SolveDev *__restrict__ sv, con
     const StateDev<Real> uh{S.avg[1], (Real *)S.hi[1]};
     for (int64_t t = it.first_tile; t < it.first_tile + it.ntiles; ++t) {
       if (S.k == 1) {
-        stats_tile<1, Real>(S.mesh, uh, S.part_dev, S.sc, t);
+        stats_tile<1, Real>(S.mesh, uh, S.part_dev, PlainScalars{S.sc}, t);
         edge_tile<1, Real>(S.mesh, S.ph, uh.avg, (const Real *)S.vd, (const Real *)S.hs, (Real *)S.ej, S.sc, c_out,
                            t);
       } else {
-        stats_tile<2, Real>(S.mesh, uh, S.part_dev, S.sc, t);
+        stats_tile<2, Real>(S.mesh, uh, S.part_dev, PlainScalars{S.sc}, t);
         edge_tile<2, Real>(S.mesh, S.ph, uh.avg, (const Real *)S.vd, (const Real *)S.hs, (Real *)S.ej, S.sc, c_out,
                            t);
       }
@@ -172,10 +172,10 @@ __device__ __forceinline__ void phase_oe_bp(const SolveDev *__restrict__ sv, con
     for (int64_t t = it.first_tile; t < it.first_tile + it.ntiles; ++t) {
       if (S.k == 1)
         oe_bp_tile<1, Real>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
-                            S.sc, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
+                            PlainScalars{S.sc}, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
       else
         oe_bp_tile<2, Real>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
-                            S.sc, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
+                            PlainScalars{S.sc}, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
       finish_alpha(S.part_alpha, S.part_cnt, S.fin, t, S.ntiles, S.sc, stage);
     }
   }

@@ -190,7 +190,7 @@ static void rk_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<R
                     StateDev<Real> uh, const void *tr, void *vd, void *hs, double *part_sum, const Scalars *sc,
                     double a, double b, double c_in, const Fuse &f) {
   auto launch = [&](auto kernel) {
-    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
+    kernel<<<ntiles<Real>(m.nt) + (f.on ? 1 : 0), TPB, 0, s>>>(m, ph, v, un, uh, (const Real *)tr, (Real *)vd, (Real *)hs, part_sum,
                                               sc, a, b, c_in, f);
   };
   if (f.on) launch(k_rk<K, Real, true>);
@@ -200,7 +200,7 @@ template <int K, typename Real>
 static void stats_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev<Real> uh, double *part_dev,
                        const void *vd, const void *hs, void *ej, const Scalars *sc, double c_out, const Fuse &f) {
   auto launch = [&](auto kernel) {
-    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
+    kernel<<<ntiles<Real>(m.nt) + (f.on ? 1 : 0), TPB, 0, s>>>(m, ph, uh, part_dev, (const Real *)vd, (const Real *)hs, (Real *)ej,
                                               sc, c_out, f);
   };
   if (f.on) launch(k_stats<K, Real, true>);
@@ -211,7 +211,7 @@ static void oebp_impl(cudaStream_t s, const MeshDev &m, const Phys &ph, StateDev
                       const void *ej, void *tr, double *pa, long long *pc, const Scalars *sc, int do_oe,
                       int do_bp, double c_out, int end_of_step, const Fuse &f) {
   auto launch = [&](auto kernel) {
-    kernel<<<ntiles<Real>(m.nt), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe, do_bp,
+    kernel<<<ntiles<Real>(m.nt) + (f.on ? 1 : 0), TPB, 0, s>>>(m, ph, uh, out, (const Real *)ej, (Real *)tr, pa, pc, sc, do_oe, do_bp,
                                               c_out, end_of_step, f);
   };
   if (f.on) launch(k_oe_bp<K, Real, true>);

@@ -162,19 +162,19 @@ namespace dg {
 // ==========================================================================
 // The tile functions of both precisions, and the kernels of one solve
 // ==========================================================================
-template <int K, typename Real>
+template <int K, typename Real, typename Sc>
 __device__ __forceinline__ void rk_tile(const MeshDev &m, const Phys &ph, StateDev<Real> v, StateDev<Real> un,
                                         StateDev<Real> uh, const Real *__restrict__ tr, Real *__restrict__ vdo,
-                                        Real *__restrict__ hso, double *part_sum, const Scalars *sc, double a,
+                                        Real *__restrict__ hso, double *part_sum, Sc get, double a,
                                         double b, double c_in, int64_t tile) {
-  if constexpr (sizeof(Real) == sizeof(float)) rk_tile_mixed<K>(m, ph, v, un, uh, part_sum, sc, a, b, c_in, tile);
-  else rk_tile_fp64<K>(m, ph, v, un, uh, tr, vdo, hso, part_sum, sc, a, b, c_in, tile);
+  if constexpr (sizeof(Real) == sizeof(float)) rk_tile_mixed<K>(m, ph, v, un, uh, part_sum, get, a, b, c_in, tile);
+  else rk_tile_fp64<K>(m, ph, v, un, uh, tr, vdo, hso, part_sum, get, a, b, c_in, tile);
 }
-template <int K, typename Real>
-__device__ __forceinline__ void stats_tile(const MeshDev &m, StateDev<Real> uh, double *part_dev, const Scalars *sc,
+template <int K, typename Real, typename Sc>
+__device__ __forceinline__ void stats_tile(const MeshDev &m, StateDev<Real> uh, double *part_dev, Sc get,
                                            int64_t tile) {
-  if constexpr (sizeof(Real) == sizeof(float)) stats_tile_mixed<K>(m, uh, part_dev, sc, tile);
-  else stats_tile_fp64<K>(m, uh, part_dev, sc, tile);
+  if constexpr (sizeof(Real) == sizeof(float)) stats_tile_mixed<K>(m, uh, part_dev, get, tile);
+  else stats_tile_fp64<K>(m, uh, part_dev, get, tile);
 }
 // the mixed form takes its jumps in K3
 template <int K, typename Real>
@@ -183,15 +183,15 @@ __device__ __forceinline__ void edge_tile(const MeshDev &m, const Phys &ph, cons
                                           Real *__restrict__ ej, const Scalars *sc, double c_out, int64_t tile) {
   if constexpr (sizeof(Real) == sizeof(double)) edge_tile_fp64<K>(m, ph, avg, vdi, hsi, ej, sc, c_out, tile);
 }
-template <int K, typename Real>
+template <int K, typename Real, typename Sc>
 __device__ __forceinline__ void oe_bp_tile(const MeshDev &m, const Phys &ph, StateDev<Real> uh, StateDev<Real> out,
                                            const Real *__restrict__ ej, Real *__restrict__ tr, double *part_alpha,
-                                           long long *part_cnt, const Scalars *sc, int do_oe, int do_bp,
+                                           long long *part_cnt, Sc get, int do_oe, int do_bp,
                                            double c_out, int end_of_step, int64_t tile) {
   if constexpr (sizeof(Real) == sizeof(float))
-    oe_bp_tile_mixed<K>(m, ph, uh, out, part_alpha, part_cnt, sc, do_oe, do_bp, c_out, end_of_step, tile);
+    oe_bp_tile_mixed<K>(m, ph, uh, out, part_alpha, part_cnt, get, do_oe, do_bp, c_out, end_of_step, tile);
   else
-    oe_bp_tile_fp64<K>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, sc, do_oe, do_bp, c_out, end_of_step, tile);
+    oe_bp_tile_fp64<K>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, get, do_oe, do_bp, c_out, end_of_step, tile);
 }
 
 template <int K, typename Real, bool FUSED>
@@ -201,11 +201,17 @@ __global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::rk)
          double c_in, Fuse f) {
   if constexpr (FUSED) {
     __shared__ Scalars s_sc;
-    fuse_alpha(f, &s_sc);
-    sc = &s_sc;
+    FuseAlpha g(f, &s_sc);
+    if (g.writer()) {
+      g.begin();
+      g.end();
+      return;
+    }
+    rk_tile<K, Real>(m, ph, v, un, uh, tr, vdo, hso, part_sum, g, a, b, c_in, blockIdx.x);
+  } else {
+    if (!sc->active) return;
+    rk_tile<K, Real>(m, ph, v, un, uh, tr, vdo, hso, part_sum, PlainScalars{sc}, a, b, c_in, blockIdx.x);
   }
-  if (!sc->active) return;
-  rk_tile<K, Real>(m, ph, v, un, uh, tr, vdo, hso, part_sum, sc, a, b, c_in, blockIdx.x);
 }
 
 // OE statistics of the tile's cells and the jump data of the edges it owns
@@ -213,13 +219,21 @@ template <int K, typename Real, bool FUSED>
 __global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::stats)
     k_stats(const __grid_constant__ MeshDev m, const __grid_constant__ Phys ph, StateDev<Real> uh, double *part_dev, const Real *__restrict__ vdi,
             const Real *__restrict__ hsi, Real *__restrict__ ej, const Scalars *sc, double c_out, Fuse f) {
-  if (!sc->active) return;
   if constexpr (FUSED) {
     __shared__ Scalars s_sc;
-    fuse_means(f, &s_sc);
+    FuseMeans g(f, &s_sc);
+    if (g.writer()) {
+      g.begin();
+      g.end();
+      return;
+    }
+    stats_tile<K, Real>(m, uh, part_dev, g, blockIdx.x);
     sc = &s_sc;
+    if (!sc->active) return;
+  } else {
+    if (!sc->active) return;
+    stats_tile<K, Real>(m, uh, part_dev, PlainScalars{sc}, blockIdx.x);
   }
-  stats_tile<K, Real>(m, uh, part_dev, sc, blockIdx.x);
   edge_tile<K, Real>(m, ph, uh.avg, vdi, hsi, ej, sc, c_out, blockIdx.x);
 }
 
@@ -229,13 +243,20 @@ __global__ void __launch_bounds__(TPB, MinBlocks<K, Real, FUSED>::oe_bp)
     k_oe_bp(MeshDev m, Phys ph, StateDev<Real> uh, StateDev<Real> out, const Real *__restrict__ ej,
             Real *__restrict__ tr, double *part_alpha, long long *part_cnt, const Scalars *sc, int do_oe,
             int do_bp, double c_out, int end_of_step, Fuse f) {
-  if (!sc->active) return;
   if constexpr (FUSED) {
     __shared__ Scalars s_sc;
-    fuse_deviations(f, &s_sc, ph.oe == 2);
-    sc = &s_sc;
+    FuseDeviations g(f, &s_sc, ph.oe == 2);
+    if (g.writer()) {
+      g.begin();
+      g.end();
+      return;
+    }
+    oe_bp_tile<K, Real>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, g, do_oe, do_bp, c_out, end_of_step, blockIdx.x);
+  } else {
+    if (!sc->active) return;
+    oe_bp_tile<K, Real>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, PlainScalars{sc}, do_oe, do_bp, c_out,
+                        end_of_step, blockIdx.x);
   }
-  oe_bp_tile<K, Real>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, sc, do_oe, do_bp, c_out, end_of_step, blockIdx.x);
 }
 
 }  // namespace dg

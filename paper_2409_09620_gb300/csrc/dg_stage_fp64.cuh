@@ -70,11 +70,11 @@ __device__ __forceinline__ double pick4(const double v[4], int c) {
 // K1: u_h = a u_n + b (v + dt L(v))
 // ==========================================================================
 // one tile; block partial -> part_sum[4 * tile]
-template <int K>
+template <int K, typename Sc>
 __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> v, StateDev<double> un,
                                              StateDev<double> uh, const double *__restrict__ tr,
                                              double *__restrict__ vdo, double *__restrict__ hso, double *part_sum,
-                                             const Scalars *sc, double a, double b, double c_in, int64_t tile) {
+                                             Sc get, double a, double b, double c_in, int64_t tile) {
   constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ, NV = Deg<K>::NV;
   __shared__ Vec4d s_u[NV][FT], s_g[NV][FT];
   __shared__ double s_cell[4][FT];   // dt / |K|, then alpha l_i
@@ -84,7 +84,8 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   const int64_t nt = m.nt, K0 = tile * FT;
   const bool live = K0 + lc < nt;
   const int64_t Kc = live ? K0 + lc : nt - 1;
-  const double gm1 = phys_gm1<double>(ph), dt = sc->dt, alpha = sc->alpha;
+  const double gm1 = phys_gm1<double>(ph);
+  get.begin();
 
   // ---- values at the volume points -----------------------------------------
   {
@@ -96,6 +97,9 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     for (int mu = 0; mu < NV; ++mu)
       s_u[mu][lc].c[c] = fx_out(fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu)), E);
   }
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
+  const double dt = sc->dt, alpha = sc->alpha;
   // products that belong to a cell or an edge, once per cell instead of in every lane
   {
     const int64_t Kl = K0 + lane < nt ? K0 + lane : nt - 1;
@@ -352,15 +356,18 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 // ==========================================================================
 // K2: sup deviations from the domain mean at the volume points
 // ==========================================================================
-template <int K>
-__device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<double> uh, double *part_dev,
-                                                const Scalars *sc, int64_t tile) {
+template <int K, typename Sc>
+__device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<double> uh, double *part_dev, Sc get,
+                                                int64_t tile) {
   constexpr int NB = Deg<K>::NB, NV = Deg<K>::NV;
   const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
   const int64_t nt = m.nt, K0 = tile * FT;
   const int64_t Kc = K0 + lc < nt ? K0 + lc : nt - 1;   // a repeated cell changes no maximum
   double x[NB];
+  get.begin();
   load_comp<NB>(uh, nt, Kc, c, x);
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
   x[0] = sub(x[0], sc->mean[c]);
   int mx = 0;
 #pragma unroll
@@ -599,12 +606,12 @@ __device__ __forceinline__ float abs_f32_down(double x) {
   return __int_as_float(min(max(t, 0), 0x0ff00000) << 3);
 }
 
-template <int K>
+template <int K, typename Sc>
 __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> uh,
                                                 StateDev<double> out, const double *__restrict__ ej,
                                                 double *__restrict__ tr, double *part_alpha, long long *part_cnt,
-                                                const Scalars *sc, int do_oe, int do_bp, double c_out,
-                                                int end_of_step, int64_t tile) {
+                                                Sc get, int do_oe, int do_bp, double c_out, int end_of_step,
+                                                int64_t tile) {
   constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ;
   constexpr int NE = 3 * NQ;          // edge Gauss points
   __shared__ Vec4d s_u[NE + 2][FT], s_a[FT];
@@ -614,18 +621,18 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
   const int64_t nt = m.nt, K0 = tile * FT;
   const bool live = K0 + lc < nt;
   const int64_t Kc = live ? K0 + lc : nt - 1;
-  const double dt = sc->dt;
   long long cnt[2] = {0, 0};
   double x[NB];
+  get.begin();
   load_comp<NB>(uh, nt, Kc, c, x);
   s_a[lc].c[c] = x[0];
 
   // ---------------------------- RIOE ---------------------------------------
+  double sig[K + 1];
   if (do_oe) {
     // sigma^j = sum_i (beta_i / h_i) delta_i^j with delta = A^{k,j} h^j sqrt(J) / D: the
     // edge records hold A beta sqrt(J), the edge sum is scaled by 1 / D once (a constant
     // component, 1 / D = 0, gets sigma = 0)
-    double sig[K + 1];
 #pragma unroll
     for (int j = 0; j <= K; ++j) sig[j] = 0.0;
 #pragma unroll
@@ -636,6 +643,11 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
       sig[1] = add(sig[1], e01.y);
       if (K == 2) sig[K] = fma(m.hgeo[i * nt + Kc], er[2], sig[K]);
     }
+  }
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
+  const double dt = sc->dt;
+  if (do_oe) {
     const double iD = sc->invD[c];
     // exact solution of the damping ODE: mode of degree d times exp(-dt sum_{j<=d} sigma^j)
     const double s = nonzero_bits(iD) ? mul(iD, dt) : 0.0;

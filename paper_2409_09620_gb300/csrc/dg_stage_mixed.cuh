@@ -174,6 +174,24 @@ __device__ __forceinline__ void load_mixed(const StateDev<float> &s, int64_t nt,
   for (int c = 0; c < 4; ++c) af[c] = INT ? f32_of(a[c]) : float(a[c]);
 }
 
+// A cell's state ahead of its use: on a small mesh, whose kernels reduce the
+// partials of the one before first, the loads go beside that.  (A thread beyond
+// the last cell takes the last one and does nothing with it.)
+template <int K>
+struct EarlyState {
+  double a[4];
+  float af[4], hi[4][Deg<K>::NB];
+  __device__ __forceinline__ void take(double a_[4], float af_[4], float hi_[4][Deg<K>::NB]) const {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      a_[c] = a[c];
+      af_[c] = af[c];
+#pragma unroll
+      for (int l = 0; l < Deg<K>::NB; ++l) hi_[c][l] = hi[c][l];
+    }
+  }
+};
+
 // F(u) . d with every product and sum rounded on its own (no contraction;
 // the reciprocal is the same instruction sequence wherever it is used)
 __device__ __forceinline__ void flux_dir_nc(const float u[4], float dx, float dy, float gm1, float f[4]) {
@@ -191,14 +209,19 @@ __device__ __forceinline__ void flux_dir_nc(const float u[4], float dx, float dy
 // ==========================================================================
 // K1 (mixed): u_h = a u_n + b (v + dt L(v))
 // ==========================================================================
-template <int K>
+template <int K, typename Sc>
 __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, StateDev<float> v, StateDev<float> un,
-                                              StateDev<float> uh, double *part_sum, const Scalars *sc, double a,
-                                              double b, double c_in, int64_t tile) {
+                                              StateDev<float> uh, double *part_sum, Sc get, double a, double b,
+                                              double c_in, int64_t tile) {
   constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ, NV = Deg<K>::NV;
   const int64_t nt = m.nt;
   const int64_t Kc = tile * TPB + threadIdx.x;
   double mass[4] = {0.0, 0.0, 0.0, 0.0};
+  get.begin();
+  EarlyState<K> early;
+  if constexpr (Sc::FUSED) load_mixed<K, true>(v, nt, Kc < nt ? Kc : nt - 1, early.a, early.af, early.hi);
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
   if (Kc < nt) {
     const double dt = sc->dt;
     const float alpha = float(sc->alpha), gm1 = ph.gm1_f;
@@ -206,7 +229,8 @@ __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, 
     const float jx = m.jinv_f[Kc], jy = m.jinv_f[nt + Kc], ex = m.jinv_f[2 * nt + Kc], ey = m.jinv_f[3 * nt + Kc];
     double v0[4];
     float v0r[4], cv[4][NB];
-    load_mixed<K, true>(v, nt, Kc, v0, v0r, cv);
+    if constexpr (Sc::FUSED) early.take(v0, v0r, cv);
+    else load_mixed<K, true>(v, nt, Kc, v0, v0r, cv);
     int32_t cns[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) cns[i] = m.conn[i * nt + Kc];
@@ -330,18 +354,21 @@ __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, 
 // ==========================================================================
 // K2 (mixed): sup deviations from the domain mean at the volume points
 // ==========================================================================
-template <int K>
-__device__ __forceinline__ void stats_tile_mixed(const MeshDev &m, StateDev<float> uh, double *part_dev,
-                                                 const Scalars *sc, int64_t tile) {
+template <int K, typename Sc>
+__device__ __forceinline__ void stats_tile_mixed(const MeshDev &m, StateDev<float> uh, double *part_dev, Sc get,
+                                                 int64_t tile) {
   constexpr int NB = Deg<K>::NB, NV = Deg<K>::NV;
   const int64_t nt = m.nt;
   const int64_t Kc = tile * TPB + threadIdx.x;
   // deviations in the working precision, reduced in it; one conversion per block
   float dr[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  get.begin();
+  double a0[4];
+  float hi[4][NB];
+  load_state<NB>(uh, nt, Kc < nt ? Kc : nt - 1, a0, hi);
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
   if (Kc < nt) {
-    double a0[4];
-    float hi[4][NB];
-    load_state<NB>(uh, nt, Kc, a0, hi);
     double off[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) off[c] = a0[c] - sc->mean[c];   // deviation of the cell mean
@@ -836,10 +863,10 @@ __device__ __forceinline__ void alpha_mixed(const MeshDev &m, const Phys &ph, co
   amax = max_nn(amax, double(amax32));
 }
 
-template <int K>
+template <int K, typename Sc>
 __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &ph, StateDev<float> uh,
                                                  StateDev<float> out, double *part_alpha, long long *part_cnt,
-                                                 const Scalars *sc, int do_oe, int do_bp, double c_out, int end_of_step,
+                                                 Sc get, int do_oe, int do_bp, double c_out, int end_of_step,
                                                  int64_t tile) {
   constexpr int NB = Deg<K>::NB;
   const int64_t nt = m.nt;
@@ -847,6 +874,11 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
   const bool live = Kc < nt;
   double amax = 0.0;
   long long cnt[2] = {0, 0};
+  get.begin();
+  EarlyState<K> early;
+  if constexpr (Sc::FUSED) load_mixed<K>(uh, nt, live ? Kc : nt - 1, early.a, early.af, early.hi);
+  const Scalars *sc = get.end();
+  if (Sc::FUSED && !sc->active) return;
   // OE exterior states at the time of the stage result; the next stage's
   // alpha there too, or at the end time after the last stage of a clamped step
   const double dt = sc->dt, t_out = fma(c_out, sc->dt, sc->t);
@@ -858,7 +890,8 @@ __device__ __forceinline__ void oe_bp_tile_mixed(const MeshDev &m, const Phys &p
   int32_t cns[3];
   bool lim64 = false;
   if (live) {
-    load_mixed<K>(uh, nt, Kc, a0, a0f, hi);
+    if constexpr (Sc::FUSED) early.take(a0, a0f, hi);
+    else load_mixed<K>(uh, nt, Kc, a0, a0f, hi);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       nxs[i] = m.nrm_f[(2 * i) * nt + Kc];
