@@ -29,9 +29,11 @@ namespace dg {
 //                  P1 0.417 with 8, 0.384 with 10, 0.373 with 12, 0.392 with 14
 //         k_oe_bp  the same from 5 to 10
 //   mixed k_rk     P2 0.181 with 3 blocks, 0.157 with 4, 0.166 with 5;
-//                  P1 0.136 with 4, 0.112 with 6, 0.103 with 8, 0.106 with 9
+//                  P1 0.136 with 4, 0.112 with 6, 0.105 with 7, 0.103 with 8, 0.106 with 9;
+//                  259,200 cells 0.0380 with 4, 0.0330 with 6, 0.0337 with 7, 0.0347 with 8
 //         k_oe_bp  P2 0.229 with 3 and 4 blocks, 0.265 with 5;
-//                  P1 0.149 with 4, 0.136 with 5, 0.135 with 6, 0.141 with 7
+//                  P1 0.149 with 4, 0.136 with 5, 0.135 with 6, 0.141 with 7;
+//                  259,200 cells 0.0468 with 4, 0.0453 with 5, 0.0496 with 6
 //         k_stats  the same from 5 to 8 (bound by memory)
 // A small mesh (FUSED) has at most FUSE_GROUPS * TILE_GROUP blocks, not two per SM: its
 // kernels get all the registers they want.  us per step with 2 / 4 / 6 blocks: 1,058 P2
@@ -41,9 +43,9 @@ namespace dg {
 template <int K, typename Real, bool FUSED = false>
 struct MinBlocks {
   static constexpr bool F = sizeof(Real) == 4;
-  static constexpr int rk = FUSED ? 2 : F ? (K == 1 ? 8 : 4) : (K == 1 ? 10 : 7);
+  static constexpr int rk = FUSED ? 2 : F ? (K == 1 ? 7 : 4) : (K == 1 ? 10 : 7);
   static constexpr int stats = FUSED ? 2 : F ? 6 : (K == 1 ? 12 : 10);
-  static constexpr int oe_bp = FUSED ? 2 : F ? (K == 1 ? 6 : 4) : 8;
+  static constexpr int oe_bp = FUSED ? 2 : F ? (K == 1 ? 5 : 4) : 8;
 };
 
 // A cell's state.  The FP64 form keeps the modes component- and mode-major
