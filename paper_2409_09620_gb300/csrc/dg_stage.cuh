@@ -23,8 +23,8 @@ namespace dg {
 // occupancy hides the latency of the neighbour gathers and of the FP64 pipe
 // until the spills cost more, which for the fewer modes of P1 happens later.
 // 1,036,800 cells, ms per launch:
-//   FP64  k_rk     P2 1.13 with 5 blocks, 1.12 with 6, 1.09 with 7 and 8;
-//                  P1 0.484 with 6, 0.472 with 7 and 8, 0.458 with 10, 0.476 with 12
+//   FP64  k_rk     P2 0.900 with 7 blocks, 0.903 with 8, 0.956 with 9, 1.05 with 10;
+//                  P1 0.407 with 9, 0.406 with 10, 0.421 with 12
 //         k_stats  P2 0.575 with 8, 0.548 with 10, 0.561 with 12, 0.72 with 14;
 //                  P1 0.417 with 8, 0.384 with 10, 0.373 with 12, 0.392 with 14
 //         k_oe_bp  the same from 5 to 10

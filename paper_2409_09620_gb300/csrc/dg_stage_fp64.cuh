@@ -32,7 +32,8 @@
 // 0.82 -> 0.58, step 7.81 -> 6.71.  Products of a cell or an edge (dt / |K|,
 // alpha l_i, |K| J^-1) and the block sums of k_rk dealt out one per lane: 33 of
 // its 306 FP64 operations per tile less, k_rk 0.97 -> 0.94 (P1 0.51 -> 0.47), step
-// 6.71 -> 6.61 (P1 4.08 -> 3.98).
+// 6.71 -> 6.61 (P1 4.08 -> 3.98).  Blocks per SM by degree (dg_stage.cuh): step 6.53
+// (P1 3.81); the edges of k_rk in a loop: 6.43 (P1 3.66).
 #pragma once
 
 namespace dg {
@@ -126,10 +127,14 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   // conversion per trace value this takes 6 integer multiply-adds per point
   // where the FP64 pipe took 4 operations (64 cycles each).  The two cells of
   // an edge form opposite values to 2^-58 of the larger product.
-  int64_t ry[3 * NQ];
-  int ei[3];
+  // One edge after another in a loop, its values in shared memory: unrolled, the
+  // kernel was 67 KB of straight-line code that waited for instructions more than
+  // for anything else (28 % of the stalls, P2), and held 9 sums in registers.
+  // 1,036,800 cells: P2 0.94 -> 0.90 ms, P1 0.457 -> 0.406 ms.
+  __shared__ int64_t s_y[3 * NQ][TPB];   // this thread's, in its own column
+  int ei[3] = {0, 0, 0};
   bool bad = false;
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < 3; ++i) {
     const int32_t cn = m.conn[i * nt + Kc];
     const double li = m.len[i * nt + Kc];
@@ -150,8 +155,9 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         const double t_in = fma(c_in, sc->dt, sc->t);
         if (cn == -7) {
           const double s = gauss_s(NQ, nu);
-          const double xa = m.vxy[(2 * ((i + 1) % 3)) * nt + Kc], ya = m.vxy[(2 * ((i + 1) % 3) + 1) * nt + Kc];
-          const double xb = m.vxy[(2 * ((i + 2) % 3)) * nt + Kc], yb = m.vxy[(2 * ((i + 2) % 3) + 1) * nt + Kc];
+          const int ia = i == 2 ? 0 : i + 1, ib = i == 0 ? 2 : i - 1;
+          const double xa = m.vxy[(2 * ia) * nt + Kc], ya = m.vxy[(2 * ia + 1) * nt + Kc];
+          const double xb = m.vxy[(2 * ib) * nt + Kc], yb = m.vxy[(2 * ib + 1) * nt + Kc];
           px = fma(xb - xa, s, xa);
           py = fma(yb - ya, s, ya);
         }
@@ -171,15 +177,17 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     const double al = s_cell[1 + i][lc];
     const int Eu = fx_exp(mu), Ef = fx_exp(mf);
     // both coefficients are below 1: x < 2^(exponent field - 1022)
-    ei[i] = max(Ef + (fx_abs_hi(li) >> 20), Eu + (fx_abs_hi(al) >> 20)) - 1022;
-    const Fx cf = fx_coef(li, Ef - ei[i]), cu = fx_coef(al, Eu - ei[i]);
+    const int e = max(Ef + (fx_abs_hi(li) >> 20), Eu + (fx_abs_hi(al) >> 20)) - 1022;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ei[j] = j == i ? e : ei[j];
+    const Fx cf = fx_coef(li, Ef - e), cu = fx_coef(al, Eu - e);
     bad = bad || max(Eu, Ef) >= FX_ENAN || (fx_abs_hi(al) >> 20) >= FX_ENAN;
 #pragma unroll
     for (int nu = 0; nu < NQ; ++nu) {
       FxAcc y{0, 0};
       fx_mac(y, cf, fx_from(fm[nu], Ef) - fx_from(fn[nu], Ef));
       fx_mac(y, cu, fx_from(um[nu], Eu) - fx_from(up[nu], Eu));
-      ry[i * NQ + nu] = fx_sum(y);   // below 2^60
+      s_y[i * NQ + nu][threadIdx.x] = fx_sum(y);   // below 2^60
     }
   }
   __syncthreads();
@@ -223,7 +231,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 #pragma unroll
     for (int p = 0; p < 3 * NQ; ++p) {
       const double sg = gauss_s(NQ, p % NQ), w = 0.5 * gauss_w(NQ, p % NQ);
-      const Fx f = fx_value(ry[p], min(Ee - ei[p / NQ], 63));
+      const Fx f = fx_value(s_y[p][threadIdx.x], min(Ee - ei[p / NQ], 63));
 #pragma unroll
       for (int l = 0; l < NB; ++l)
         fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w * inv_mass_c(l)), f);
