@@ -237,7 +237,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
         fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w * inv_mass_c(l)), f);
     }
     const double dta = s_cell[0][lc];
-    const bool first = a == 0.0 && b == 1.0;   // the first stage skips the zero term and the load of u_n
+    const bool first = first_stage(a, b);   // the first stage skips the zero term and the load of u_n
     bad = bad || Ev >= FX_ENAN;
     double x[NB], xn[NB];
     load_comp<NB>(v, nt, Kc, c, x);

@@ -330,7 +330,7 @@ __device__ __forceinline__ void rk_tile_mixed(const MeshDev &m, const Phys &ph, 
     // ---- mass inverse and SSP-RK combination -----------------------------------
     const double dta = dt * m.iarea[Kc];
     const float ar = float(a), br = float(b), dtar = float(dta);
-    const bool first = a == 0.0 && b == 1.0;
+    const bool first = first_stage(a, b);
     double un0[4] = {0.0, 0.0, 0.0, 0.0};
     float cu[4][NB];
     if (!first) load_state<NB>(un, nt, Kc, un0, cu);
