@@ -167,7 +167,9 @@ int32_t dg_set_state(dg_solver *solver, const double *coeffs, double t);
  * count of kernel kind q: 0 step_begin (dt), 1 rk (volume + edge flux + RK
  * combine), 2 fin_mean (domain means), 3 stats (deviation maxima and edge OE
  * records), 4 fin_dev (normalisers), 5 oe_bp (RIOE + limiter + traces), 6
- * fin_alpha (alpha, counters, time).  A step is 19 launches (13 with OE off). */
+ * fin_alpha (alpha, counters, time).  A step is 19 launches (13 with OE off);
+ * the captured step of a small mesh, whose kernels finish each other's
+ * reductions, is 10 with the same results bit for bit. */
 #define DG_NUM_KERNEL_KINDS 7
 int32_t dg_profile_steps(dg_solver *solver, int64_t n, double *ms, int64_t *launches);
 /* Measured FMA throughput of the current device: a kernel of independent
@@ -266,7 +268,7 @@ int32_t dg_batch_shape(const dg_batch *batch, int32_t *cells_per_block, int32_t 
 /* Time `steps` steps for form 0 and, for forms 3 and 1, every
  * cells-per-chunk in {128, 256, 512, 1024} and every blocks-per-SM up to the
  * occupancy limit; keep the fastest and restore every solve's state, time and
- * counters.  The shape changes no result (partials are per 128 cells of each
+ * counters.  The shape changes no result (partials are per tile of each
  * solve). */
 int32_t dg_batch_autotune(dg_batch *batch, int32_t steps, int32_t *best_cells_per_block,
                           int32_t *best_blocks_per_sm, int32_t *best_launches_per_stage,
