@@ -37,28 +37,32 @@ if ROOT not in sys.path:
 METRIC = "P2 Euler DG cell-stage updates/s (FP64 vs FP32), HBM GB/s; p50/p99 solve latency"
 UNIT = "cell-stage updates/s"
 
-# Algorithmic FP64 work per cell-stage of each kernel kind (P2 interior cell,
-# RIOE, limiter on, cell not limited), counted from the kernel source: add /
-# sub / mul / division / square root / exponential = 1 flop, fma = 2; a
-# compile-time coefficient of 0 costs nothing and one of +-1 a single add; the
-# first term into a zero accumulator is one multiply.  k_rk: volume evaluation
-# 208, volume fluxes 186, volume accumulation 368, edge terms 529, mass
-# inverse and RK combination 106 (mean of the three stages; the first has no
-# u_n term), vertex records 269, Hessians 73, block sums 6.  k_stats:
-# deviations at the volume points 231, edge OE records 187 per edge x 1.5.
-# k_oe_bp: sigma 87, damping 38, limiter at the 11 points 497, traces and
-# wave speeds 313 (the nine reciprocal densities from one division and 24
-# multiplies); a cell that the bound over the whole cell settles skips the
-# 11 points (about 30 flops instead of 497).
-ALGO_FLOPS_P2 = {"rk": 1745.0, "stats": 512.0, "oe_bp": 935.0}
-# FP64 flops per cell-stage the hardware executed for the same kernels
-# (2 DFMA + DMUL + DADD from ncu captures / cells; k_rk: mean of its three
-# stages 1896 / 1968 / 1968); division, square root and exp expand into
-# DFMA sequences.  None = not re-measured since the kernel last changed.
-EXECUTED_FLOPS_P2 = {"rk": 1944.0, "stats": 744.0, "oe_bp": 967.0}
-# DRAM bytes (read + write) per launch from the same captures (k_rk: mean of
-# its stages 1.599 / 1.808 / 1.808 GB).
-TRAFFIC_PER_LAUNCH = {"rk": 1.738e9, "stats": 0.948e9, "oe_bp": 1.301e9}
+# The method's FP64 work per cell-stage of each kernel kind (P2 interior cell,
+# RIOE, limiter on, cell not limited): add / sub / mul / division / square
+# root / exponential = 1 flop, fma = 2; a compile-time coefficient of 0 costs
+# nothing and one of +-1 a single add; the first term into a zero accumulator
+# is one multiply.  k_rk: volume evaluation 208, volume fluxes 186, volume
+# accumulation 368, edge terms 529, mass inverse and RK combination 106 (mean of
+# the three stages; the first has no u_n term), vertex records 269, Hessians
+# 73, block sums 6.  k_stats: deviations at the volume points 231, edge OE
+# records 187 per edge x 1.5.  k_oe_bp: sigma 87, damping 38, limiter at the 11
+# points 497, traces and wave speeds 313; a cell that the bound over the whole
+# cell settles skips the 11 points (about 30 flops instead of 497).
+METHOD_FLOPS_P2 = {"rk": 1745.0, "stats": 512.0, "oe_bp": 935.0}
+# The part of it that has run-time operands and stays on the FP64 pipe; sums with
+# constant coefficients run in fixed point on the integer units.  k_rk: volume
+# fluxes 186, RK combination 96, vertex speeds 33, products of a cell or an
+# edge 8, block sums 8.  k_stats: norm and mean 8, jumps, wave speeds and square
+# roots 124 per edge x 1.5.  k_oe_bp: sigma and damping 108, fluxes and wave
+# speeds of the nine traces 216.
+ALGO_FLOPS_P2 = {"rk": 331.0, "stats": 194.0, "oe_bp": 324.0}
+# FP64 flops per cell-stage the hardware executed for the same kernels (2 DFMA +
+# DMUL + DADD from ncu captures / cells, first stage of a step); sums and products are DFMAs
+# too, division, square root and exp expand into DFMA sequences.
+EXECUTED_FLOPS_P2 = {"rk": 586.3, "stats": 502.7, "oe_bp": 732.5}
+# DRAM bytes (read + write) per launch, from ncu captures per cell (k_rk: mean of
+# its three stages)
+TRAFFIC_PER_LAUNCH = {"rk": 1.649e9, "stats": 1.047e9, "oe_bp": 1.190e9}
 # Mixed form (P2, FP32 modes 1-5 and FP64 averages: S = 4 x 8 + 4 x 5 x 4 =
 # 112 B of state per cell).  Algorithmic HBM bytes per cell-stage of the
 # method's three passes, each array element moved once and neighbour data
@@ -74,8 +78,8 @@ S_MIXED_P2 = 112.0
 ALGO_BYTES_MIXED_P2 = {"rk": (8.0 / 3.0) * S_MIXED_P2 + 80.0, "stats": S_MIXED_P2,
                        "oe_bp": 2.0 * S_MIXED_P2 + 92.0}
 # DRAM bytes per launch of the mixed-form kernels from one ncu capture (k_rk:
-# mean of its stages 272 / 394 / 394 B per cell)
-TRAFFIC_MIXED_PER_LAUNCH = {"rk": 0.366e9, "stats": 0.120e9, "oe_bp": 0.304e9}
+# mean of its stages 232 / 359 / 359 B per cell)
+TRAFFIC_MIXED_PER_LAUNCH = {"rk": 0.328e9, "stats": 0.116e9, "oe_bp": 0.262e9}
 
 
 def load_peaks():
@@ -368,6 +372,8 @@ def main():
                 "peak_measured": fp64_meas, "peak_derived": FP64_PEAK_TFLOPS,
                 "frac_of_derived": achieved / FP64_PEAK_TFLOPS if achieved else None,
                 "algorithmic_flops_per_cell": ALGO_FLOPS_P2.get(dom),
+                "method_flops_per_cell": METHOD_FLOPS_P2.get(dom),
+                "method_tflops": METHOD_FLOPS_P2.get(dom, 0.0) * nt / (avg_ms / 1e3) / 1e12,
                 "executed_flops_per_cell": ex,
                 "executed_tflops": ex * nt / (avg_ms / 1e3) / 1e12 if ex else None,
                 "avg_launch_ms": avg_ms,
