@@ -367,12 +367,13 @@ int32_t write_scalars(dg_solver *s, const Scalars *h) {
 const double RK_A[3] = {0.0, 0.75, 1.0 / 3.0}, RK_B[3] = {1.0, 0.25, 2.0 / 3.0};
 const double C_IN[3] = {0.0, 1.0, 0.5}, C_OUT[3] = {1.0, 0.5, 1.0};
 
-// one SSP-RK3 step of the BP RI-OEDG scheme (Sec. 4.5) on the solver's stream
-void enqueue_step(dg_solver *s) {
+// one SSP-RK3 step of the BP RI-OEDG scheme (Sec. 4.5) on the solver's stream;
+// fuse: a small mesh's kernels may finish each other's reductions
+void enqueue_step(dg_solver *s, bool fuse) {
   const StageCtx &c = s->ctx;
   const int oe = s->cfg.oe != DG_OE_OFF, bp = s->cfg.bp != DG_BP_OFF;
   const int64_t ntiles = num_tiles(s->mesh->nt, c.prec);
-  if (num_groups(ntiles) <= FUSE_GROUPS) {
+  if (fuse && num_groups(ntiles) <= FUSE_GROUPS) {
     // few tiles: each kernel finishes the reduction of the one before it; the
     // last stage's alpha, counters and time are finished for the host
     const int n = (int)ntiles;
@@ -517,7 +518,7 @@ extern "C" int32_t dg_init(const dg_mesh *mesh, const dg_config *cfg, const doub
   }
   cudaGraph_t graph = nullptr;
   STRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-  enqueue_step(s);
+  enqueue_step(s, true);
   e = cudaStreamEndCapture(s->stream, &graph);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&s->step_exec, graph, 0);
   if (graph) cudaGraphDestroy(graph);
@@ -789,11 +790,11 @@ void solver_states(const dg_solver *s, StateBuf *un, StateBuf *uh, StateBuf *us)
 int solver_nb(const dg_solver *s) { return s->nb; }
 int32_t solver_read_scalars(const dg_solver *s, Scalars *h) { return read_scalars(s, h); }
 int32_t solver_write_scalars(dg_solver *s, const Scalars *h) { return write_scalars(s, h); }
-int32_t solver_capture_step(dg_solver *s, cudaGraph_t *graph) {
+int32_t solver_capture_step(dg_solver *s, bool fuse, cudaGraph_t *graph) {
   *graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return set_error(DG_ECUDA, cudaGetErrorString(e));
-  enqueue_step(s);
+  enqueue_step(s, fuse);
   e = cudaStreamEndCapture(s->stream, graph);
   if (e != cudaSuccess || !*graph) {
     cudaGetLastError();

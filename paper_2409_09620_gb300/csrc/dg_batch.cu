@@ -450,9 +450,17 @@ struct BatchCore {
     cudaGraph_t g = nullptr;
     if (cudaGraphCreate(&g, 0) != cudaSuccess) return set_error(DG_ECUDA, "graph create");
     int32_t rc = DG_OK;
+    int64_t tiles = 0;
+    for (dg_solver *sv_ : solves) tiles += num_tiles(solver_ctx(sv_).mesh.nt, prec);
+    // Small meshes finish their reductions inside their kernels only while the batch is about
+    // one wave of blocks: then launches count.  Beyond, other solves cover them, and the fused
+    // kernels' registers and repeated reductions cost throughput.  us per step, separate /
+    // fused: mixed, 318 tiles 153 / 120, 767 tiles 207 / 212, 1,197 tiles 300 / 326; 64 solves,
+    // 3.0M cells, 3,365 / 3,752; FP64, 877 tiles 393 / 360, 2,506 tiles 710 / 877.
+    const bool fuse = tiles <= (int64_t)num_sms * (prec == DG_PREC_MIXED ? 4 : 8);
     for (dg_solver *sv_ : solves) {
       cudaGraph_t child = nullptr;
-      if ((rc = solver_capture_step(sv_, &child)) != DG_OK) break;
+      if ((rc = solver_capture_step(sv_, fuse, &child)) != DG_OK) break;
       cudaGraphNode_t node;
       const cudaError_t e = cudaGraphAddChildGraphNode(&node, g, nullptr, 0, child);
       cudaGraphDestroy(child);
