@@ -156,7 +156,10 @@ int32_t dg_advance(dg_solver *solver, double t_end, int64_t max_steps, dg_stats 
 int32_t dg_advance_async(dg_solver *solver, int64_t n);
 int32_t dg_sync(dg_solver *solver, dg_stats *stats);
 /* host copy of the current state (len = number of doubles available in
- * coeffs, at least 4 * nb * nt) and time (t may be NULL) */
+ * coeffs, at least 4 * nb * nt) and time (t may be NULL).  Other threads may
+ * read a solver while one thread advances it (dg_advance, dg_advance_async,
+ * the calls of its batch) or replaces its state: a copy is the state of one
+ * step boundary, whole, and harms nothing; t is read after the state. */
 int32_t dg_get_state(const dg_solver *solver, double *coeffs, size_t len, double *t);
 /* replace the state (host coefficients, used as given, not limited) and time */
 int32_t dg_set_state(dg_solver *solver, const double *coeffs, double t);

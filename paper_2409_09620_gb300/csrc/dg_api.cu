@@ -91,12 +91,20 @@ struct dg_solver {
   Scalars *sc = nullptr;
   cudaGraphExec_t step_exec = nullptr;
   StageCtx ctx{};
-  mutable std::mutex scratch_mutex;   // the transfers' use of the free state buffer
+  // A reader (dg_get_state on any thread) may run beside a writer: the mixed form's modes are
+  // converted through a buffer that no step and no upload touches (nullptr: only the caller
+  // that advances the solver reads it, and u_h serves), and `order` is held while the work of
+  // one transfer or one step is enqueued, so that a copy of the state is of one step boundary.
+  // The solves of a batch, whose steps are enqueued together, share the batch's.
+  double *modes = nullptr;
+  int mode_rows = 0;   // modes it holds at a time
+  std::mutex own_order;
+  std::mutex *order = &own_order;
   ~dg_solver() {
     if (step_exec) cudaGraphExecDestroy(step_exec);
     StateBuf *bufs[3] = {&un, &uh, &us};
     for (auto *b : bufs) { cudaFree(b->avg); cudaFree(b->hi); }
-    cudaFree(tr); cudaFree(vd); cudaFree(hs); cudaFree(ej);
+    cudaFree(tr); cudaFree(vd); cudaFree(hs); cudaFree(ej); cudaFree(modes);
     cudaFree(part_sum); cudaFree(part_dev); cudaFree(part_alpha); cudaFree(part_cnt); cudaFree(sc);
     cudaFree(fin.grp_sum); cudaFree(fin.grp_dev); cudaFree(fin.grp_alpha); cudaFree(fin.grp_cnt); cudaFree(fin.tick);
     if (own_stream && stream) cudaStreamDestroy(stream);
@@ -305,49 +313,63 @@ cudaError_t alloc_state(dg_solver *s, StateBuf *b) {
   return cudaMalloc(&b->hi, std::max<size_t>(1, real_size(s) * 4 * (s->nb - 1) * nt));
 }
 
-// A state buffer other than b, free to hold two components' modes in FP64 (the
-// size of the mixed form's mode records): the stage buffers u_h and u_s carry
-// nothing between calls, and no caller fills both before it uses one.
-double *mode_scratch(const dg_solver *s, const StateBuf &b) {
-  return (double *)(b.hi == s->uh.hi ? s->us.hi : s->uh.hi);
-}
-
-// host modal state [4][nb][nt] (double) -> device buffer.  Mixed form: the modes
-// cross in FP64 two components at a time and are rounded to the per-cell
-// records on the device.
+// host modal state [4][nb][nt] (double) -> device buffer b, one of the solver's stage
+// buffers.  Mixed form: the modes cross in FP64 two components at a time, into a stage
+// buffer other than b (a state's records are the size of two components' modes in FP64;
+// the stage buffers carry nothing between calls, and no caller fills both before it uses
+// one), and are rounded to the per-cell records on the device.
 int32_t upload_state(dg_solver *s, const double *coeffs, const StateBuf &b) {
   const int64_t nt = s->mesh->nt;
   const int nb = s->nb;
   const bool mixed = s->cfg.precision == DG_PREC_MIXED;
   const size_t bytes = sizeof(double) * (nb - 1) * nt;   // modes of one component
-  std::lock_guard<std::mutex> lock(s->scratch_mutex);
+  double *const scratch = (double *)(b.hi == s->uh.hi ? s->us.hi : s->uh.hi);
+  std::lock_guard<std::mutex> lock(*s->order);
   for (int c = 0; c < 4; ++c) {
     CUDA_TRY(cudaMemcpyAsync(b.avg + c * nt, coeffs + (int64_t)c * nb * nt, sizeof(double) * nt,
                              cudaMemcpyHostToDevice, s->stream));
-    double *dst = mixed ? mode_scratch(s, b) + (int64_t)(c & 1) * (nb - 1) * nt
-                        : (double *)b.hi + (int64_t)c * (nb - 1) * nt;
+    double *dst = mixed ? scratch + (int64_t)(c & 1) * (nb - 1) * nt : (double *)b.hi + (int64_t)c * (nb - 1) * nt;
     CUDA_TRY(cudaMemcpyAsync(dst, coeffs + ((int64_t)c * nb + 1) * nt, bytes, cudaMemcpyHostToDevice, s->stream));
-    if (mixed && (c & 1)) launch_convert_modes(s->ctx, b.hi, mode_scratch(s, b), c - 1, true);
+    if (mixed && (c & 1)) launch_convert_modes(s->ctx, b.hi, scratch, (c - 1) * (nb - 1), 2 * (nb - 1), true);
   }
   CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
 
+// Modes that a reader converts at a time, as many as fit in 10.5 MB: those of two components
+// (up to 131,072 P2 cells), of one, or one mode (8 bytes per cell, 1 % of a large solver; 1.4
+// instead of 1.1 ms for 1,036,800 cells).  The modes of a component are contiguous in the
+// host's array, so every copy is one piece.
+int reader_rows(int64_t nt, int nm) {
+  const int64_t fit = 10 * 131072 / nt;
+  return fit >= 2 * nm ? 2 * nm : fit >= nm ? nm : 1;
+}
+
+// device buffer -> host modal state; waits for the copies
 int32_t download_state(const dg_solver *s, const StateBuf &b, double *coeffs) {
   const int64_t nt = s->mesh->nt;
-  const int nb = s->nb;
-  const bool mixed = s->cfg.precision == DG_PREC_MIXED;
-  const size_t bytes = sizeof(double) * (nb - 1) * nt;
-  std::lock_guard<std::mutex> lock(s->scratch_mutex);   // two readers of one solver share the scratch
-  for (int c = 0; c < 4; ++c) {
-    CUDA_TRY(cudaMemcpyAsync(coeffs + (int64_t)c * nb * nt, b.avg + c * nt, sizeof(double) * nt,
-                             cudaMemcpyDeviceToHost, s->stream));
-    if (mixed && !(c & 1)) launch_convert_modes(s->ctx, b.hi, mode_scratch(s, b), c, false);
-    const double *src = mixed ? mode_scratch(s, b) + (int64_t)(c & 1) * (nb - 1) * nt
-                              : (const double *)b.hi + (int64_t)c * (nb - 1) * nt;
-    CUDA_TRY(cudaMemcpyAsync(coeffs + ((int64_t)c * nb + 1) * nt, src, bytes, cudaMemcpyDeviceToHost, s->stream));
+  const int nb = s->nb, nm = nb - 1;
+  {
+    std::lock_guard<std::mutex> lock(*s->order);
+    for (int c = 0; c < 4; ++c) {
+      CUDA_TRY(cudaMemcpyAsync(coeffs + (int64_t)c * nb * nt, b.avg + c * nt, sizeof(double) * nt,
+                               cudaMemcpyDeviceToHost, s->stream));
+      if (s->cfg.precision != DG_PREC_MIXED)
+        CUDA_TRY(cudaMemcpyAsync(coeffs + ((int64_t)c * nb + 1) * nt, (const double *)b.hi + (int64_t)c * nm * nt,
+                                 sizeof(double) * nm * nt, cudaMemcpyDeviceToHost, s->stream));
+    }
+    if (s->cfg.precision == DG_PREC_MIXED) {
+      double *const scratch = s->modes ? s->modes : (double *)(b.hi == s->uh.hi ? s->us.hi : s->uh.hi);
+      const int rows = s->modes ? s->mode_rows : 2 * nm;
+      for (int r0 = 0; r0 < 4 * nm; r0 += rows) {
+        launch_convert_modes(s->ctx, b.hi, scratch, r0, rows, false);
+        for (int r = 0; r < rows; r += std::min(rows, nm))
+          CUDA_TRY(cudaMemcpyAsync(coeffs + ((int64_t)(r0 + r) / nm * nb + 1 + (r0 + r) % nm) * nt, scratch + r * nt,
+                                   sizeof(double) * std::min(rows, nm) * nt, cudaMemcpyDeviceToHost, s->stream));
+      }
+    }
+    CUDA_TRY(cudaGetLastError());
   }
-  CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   return DG_OK;
 }
@@ -397,10 +419,24 @@ void enqueue_step(dg_solver *s, bool fuse) {
   }
 }
 
+// n graph launches, each whole before or after a reader's copy
+int32_t launch_steps(dg_solver *s, int64_t n) {
+  for (int64_t i = 0; i < n; ++i) {
+    std::lock_guard<std::mutex> lock(*s->order);
+    CUDA_TRY(cudaGraphLaunch(s->step_exec, s->stream));
+  }
+  return DG_OK;
+}
+
 }  // namespace
 
 extern "C" int32_t dg_init(const dg_mesh *mesh, const dg_config *cfg, const double *coeffs, void *cuda_stream,
                            dg_solver **out) {
+  return solver_init(mesh, cfg, coeffs, cuda_stream, true, out);
+}
+
+int32_t dg::solver_init(const dg_mesh *mesh, const dg_config *cfg, const double *coeffs, void *cuda_stream,
+                        bool readers, dg_solver **out) {
   if (!out) return fail(DG_EINVAL, "out is NULL");
   *out = nullptr;
   if (!mesh || !cfg || !coeffs) return fail(DG_EINVAL, "NULL argument");
@@ -437,6 +473,10 @@ extern "C" int32_t dg_init(const dg_mesh *mesh, const dg_config *cfg, const doub
   STRY(alloc_state(s, &s->un));
   STRY(alloc_state(s, &s->uh));
   STRY(alloc_state(s, &s->us));
+  if (readers && cfg->precision == DG_PREC_MIXED) {
+    s->mode_rows = reader_rows(nt, s->nb - 1);
+    STRY(dalloc(&s->modes, s->mode_rows * nt));
+  }
   const int64_t xc = uses_exchange(cfg->precision) ? nt : 1;   // exchange buffers: FP64 form only
   STRY(cudaMalloc(&s->tr, rs * xc * 3 * nq * TR_STRIDE));
   STRY(cudaMalloc(&s->vd, rs * xc * VD_CELL));
@@ -559,7 +599,7 @@ extern "C" int32_t dg_advance(dg_solver *s, double t_end, int64_t max_steps, dg_
   // launch in chunks; steps past t_end are no-ops on the device
   while (done < max_steps && h.t < t_end) {
     const int64_t chunk = std::min<int64_t>(max_steps - done, 32);
-    for (int64_t i = 0; i < chunk; ++i) CUDA_TRY(cudaGraphLaunch(s->step_exec, s->stream));
+    if ((rc = launch_steps(s, chunk)) != DG_OK) return rc;
     done += chunk;
     if ((rc = read_scalars(s, &h)) != DG_OK) return rc;
     if (!std::isfinite(h.alpha) || h.alpha <= 0.0) break;
@@ -573,8 +613,7 @@ extern "C" int32_t dg_advance(dg_solver *s, double t_end, int64_t max_steps, dg_
 
 extern "C" int32_t dg_advance_async(dg_solver *s, int64_t n) {
   if (!s || n < 0) return fail(DG_EINVAL, "bad argument");
-  for (int64_t i = 0; i < n; ++i) CUDA_TRY(cudaGraphLaunch(s->step_exec, s->stream));
-  return DG_OK;
+  return launch_steps(s, n);
 }
 
 extern "C" int32_t dg_sync(dg_solver *s, dg_stats *stats) {
@@ -613,7 +652,10 @@ extern "C" int32_t dg_set_state(dg_solver *s, const double *coeffs, double t) {
   h.active = 1;
   if ((rc = write_scalars(s, &h)) != DG_OK) return rc;
   if ((rc = upload_state(s, coeffs, s->uh)) != DG_OK) return rc;
-  launch_oe_bp(s->ctx, s->uh, s->un, 0, 0, 0.0, -1);   // traces and alpha only
+  {
+    std::lock_guard<std::mutex> lock(*s->order);
+    launch_oe_bp(s->ctx, s->uh, s->un, 0, 0, 0.0, -1);   // traces and alpha only
+  }
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   return DG_OK;
@@ -632,6 +674,7 @@ extern "C" int32_t dg_profile_steps(dg_solver *s, int64_t n, double *ms, int64_t
   int32_t rc = DG_OK;
   for (int64_t step = 0; step < n && rc == DG_OK; ++step) {
     int kind[MAXL], nl = 0;
+    std::unique_lock<std::mutex> lock(*s->order);
     auto rec = [&](int kd, auto &&fn) {
       cudaEventRecord(ev[2 * nl], s->stream);
       fn();
@@ -650,6 +693,7 @@ extern "C" int32_t dg_profile_steps(dg_solver *s, int64_t n, double *ms, int64_t
       rec(5, [&] { launch_oe_bp_only(c, s->uh, st == 2 ? s->un : s->us, oe, bp, C_OUT[st], st == 2); });
       rec(6, [&] { launch_fin_alpha(c, st); });
     }
+    lock.unlock();
     cudaError_t e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) { rc = fail(DG_ECUDA, "profiled step: %s", cudaGetErrorString(e)); break; }
     for (int i = 0; i < nl; ++i) {
@@ -788,6 +832,7 @@ void solver_states(const dg_solver *s, StateBuf *un, StateBuf *uh, StateBuf *us)
   *us = s->us;
 }
 int solver_nb(const dg_solver *s) { return s->nb; }
+void solver_share_order(dg_solver *s, std::mutex *order) { s->order = order; }
 int32_t solver_read_scalars(const dg_solver *s, Scalars *h) { return read_scalars(s, h); }
 int32_t solver_write_scalars(dg_solver *s, const Scalars *h) { return write_scalars(s, h); }
 int32_t solver_capture_step(dg_solver *s, bool fuse, cudaGraph_t *graph) {

@@ -240,6 +240,7 @@ namespace dg {
 struct BatchCore {
   int prec = 0;
   cudaStream_t stream = nullptr;
+  std::mutex order;   // held while a step is enqueued; the owned solves' readers hold it too
   std::vector<dg_solver *> solves;
   std::vector<SolveDev> host_sv;
   SolveDev *d_sv = nullptr;
@@ -480,6 +481,7 @@ struct BatchCore {
     if (host_sv.empty()) return DG_OK;
     if (form == 0 && !graph_ok) return set_error(DG_ECUDA, "the per-solve batch graph is missing");
     for (int64_t s = 0; s < n; ++s) {
+      std::lock_guard<std::mutex> lock(order);
       if (graph_ok) {
         if (cudaGraphLaunch(exec, stream) != cudaSuccess) return set_error(DG_ECUDA, "batch graph launch");
       } else {
@@ -546,7 +548,9 @@ extern "C" int32_t dg_batch_create(int32_t n, const dg_mesh *const *meshes, cons
   for (int i = 0; i < n && rc == DG_OK; ++i) {
     dg_solver *s = nullptr;
     rc = dg_init(meshes[i], &cfgs[i], coeffs[i], b->stream, &s);
-    if (rc == DG_OK) b->owned.push_back(s);
+    if (rc != DG_OK) break;
+    solver_share_order(s, &b->core.order);
+    b->owned.push_back(s);
   }
   if (rc == DG_OK) rc = b->core.set_solves(b->owned);
   if (rc != DG_OK) { delete b; return rc; }

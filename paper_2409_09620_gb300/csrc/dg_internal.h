@@ -2,6 +2,7 @@
 // kernel launch wrappers (dg_kernels.cu).
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <cuda_runtime.h>
 
 #include "../../include/dg.h"
@@ -53,18 +54,25 @@ void launch_oe_bp_only(const StageCtx &c, const StateBuf &uh, const StateBuf &ou
                        double c_out, int end_of_step, const Fuse &f = Fuse{});
 void launch_fin_alpha(const StageCtx &c, int stage);
 void launch_step_begin(const StageCtx &c);
-// modes of components c0, c0 + 1 between the mixed form's records and the ABI's
-// layout [2][nb - 1][nt] on the device (half the size of the records in FP64)
-void launch_convert_modes(const StageCtx &c, void *rec, double *modes, int c0, bool to_record);
+// modes [row0, row0 + rows) of the 4 (nb - 1) of every cell, rows one mode, those of one
+// component or of two, between the mixed form's records and FP64 modes [rows][nt] on the
+// device (the ABI's layout)
+void launch_convert_modes(const StageCtx &c, void *rec, double *modes, int row0, int rows, bool to_record);
 void launch_set_active(const StageCtx &c, int active);
 void launch_set_inv_normalisers(const StageCtx &c);
 // tiles of a mesh: the blocks of a stage kernel in the given precision, one reduction partial each
 int64_t num_tiles(int64_t nt, int prec);
 
+// dg_init; readers = false for a solver that only the caller that advances it reads: it
+// keeps no buffer for a reader beside a step (dg_api.cu)
+int32_t solver_init(const dg_mesh *mesh, const dg_config *cfg, const double *coeffs, void *cuda_stream, bool readers,
+                    dg_solver **out);
 // access to a solver's launch context and buffers (dg_api.cu)
 const StageCtx &solver_ctx(const dg_solver *s);
 void solver_states(const dg_solver *s, StateBuf *un, StateBuf *uh, StateBuf *us);
 int solver_nb(const dg_solver *s);
+// the mutex that whoever enqueues the solver's steps holds meanwhile (it outlives the solver's use)
+void solver_share_order(dg_solver *s, std::mutex *order);
 int32_t solver_read_scalars(const dg_solver *s, Scalars *h);
 int32_t solver_write_scalars(dg_solver *s, const Scalars *h);
 // one SSP-RK3 step of the solver (the kernels of its own step graph) captured

@@ -152,19 +152,19 @@ __global__ void k_set_active(Scalars *sc, int active) {
   if (threadIdx.x == 0) sc->active = active;
 }
 
-// Two components' modes between the mixed form's per-cell FP32 records and the
-// component- and mode-major FP64 layout of the C ABI, one thread per cell.
-// Bound by memory (24 bytes per mode both ways: 0.05 ms for 1,036,800 P2 cells
-// and two components); the host loop it replaces took 45 ms per state.
-template <int NB, bool TO_RECORD>
+// R modes of every cell between the mixed form's per-cell FP32 records (NR modes) and the
+// component- and mode-major FP64 layout of the C ABI, one thread per cell.  Bound by memory
+// (two components' modes: 24 bytes per mode both ways, 0.05 ms for 1,036,800 P2 cells; one
+// mode: a 32-byte sector of the record and 8 bytes); the host loop it replaces took 45 ms
+// per state.
+template <int R, bool TO_RECORD>
 __global__ void __launch_bounds__(TPB) k_convert_modes(int64_t nt, float *__restrict__ rec, double *__restrict__ modes,
-                                                       int c0) {
-  constexpr int NM = NB - 1;
+                                                       int NR) {
   const int64_t K = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (K >= nt) return;
-  float *r = rec + K * 4 * NM + c0 * NM;
+  float *r = rec + K * NR;
 #pragma unroll
-  for (int q = 0; q < 2 * NM; ++q) {
+  for (int q = 0; q < R; ++q) {
     if constexpr (TO_RECORD) r[q] = float(modes[q * nt + K]);
     else modes[q * nt + K] = double(r[q]);
   }
@@ -287,15 +287,22 @@ void launch_oe_bp(const StageCtx &c, const StateBuf &uh, const StateBuf &out, in
   launch_fin_alpha(c, stage);
 }
 
-void launch_convert_modes(const StageCtx &c, void *rec, double *modes, int c0, bool to_record) {
-  const unsigned nb = nblocks(c.mesh.nt);
-  float *r = (float *)rec;
-  if (c.k == 1) {
-    if (to_record) k_convert_modes<3, true><<<nb, TPB, 0, c.stream>>>(c.mesh.nt, r, modes, c0);
-    else k_convert_modes<3, false><<<nb, TPB, 0, c.stream>>>(c.mesh.nt, r, modes, c0);
+void launch_convert_modes(const StageCtx &c, void *rec, double *modes, int row0, int rows, bool to_record) {
+  const int64_t nt = c.mesh.nt;
+  const int NR = c.k == 1 ? 8 : 20;
+  float *r = (float *)rec + row0;
+  auto launch = [&](auto kernel) { kernel<<<nblocks(nt), TPB, 0, c.stream>>>(nt, r, modes, NR); };
+  if (to_record) {   // two components at a time
+    if (c.k == 1) launch(k_convert_modes<4, true>);
+    else launch(k_convert_modes<10, true>);
+  } else if (rows == 1) {
+    launch(k_convert_modes<1, false>);
+  } else if (c.k == 1) {
+    if (rows == 2) launch(k_convert_modes<2, false>);
+    else launch(k_convert_modes<4, false>);
   } else {
-    if (to_record) k_convert_modes<6, true><<<nb, TPB, 0, c.stream>>>(c.mesh.nt, r, modes, c0);
-    else k_convert_modes<6, false><<<nb, TPB, 0, c.stream>>>(c.mesh.nt, r, modes, c0);
+    if (rows == 5) launch(k_convert_modes<5, false>);
+    else launch(k_convert_modes<10, false>);
   }
 }
 

@@ -81,7 +81,7 @@ struct DeviceEngine final : ServeEngine {
     Payload &p = pay[id];
     int32_t rc = dg_mesh_create(p.nv, p.xy.data(), p.nt, p.tri.data(), p.canon.empty() ? nullptr : p.canon.data(),
                                 p.bc.empty() ? nullptr : p.bc.data(), &p.mesh);
-    if (rc == DG_OK) rc = dg_init(p.mesh, &p.cfg, p.coeffs.data(), stream, &p.solver);
+    if (rc == DG_OK) rc = solver_init(p.mesh, &p.cfg, p.coeffs.data(), stream, false, &p.solver);
     Scalars h{};
     if (rc == DG_OK) rc = solver_read_scalars(p.solver, &h);
     if (rc == DG_OK) {
