@@ -690,9 +690,11 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
     const float r_lo = __shfl_sync(FULL, lo, q0), r_hi = __shfl_sync(FULL, B, q0);
     const float M_hi = __shfl_sync(FULL, B, q0 + 1) + __shfl_sync(FULL, B, q0 + 2);
     const float E_lo = __shfl_sync(FULL, lo, q0 + 3), E_hi = __shfl_sync(FULL, B, q0 + 3);
-    const float M2 = M_hi * M_hi;
-    const bool settled = r_lo >= fmaf(1e-5f, r_hi, 2e-13f) &&
-                         r_lo * E_lo - 0.5f * M2 >= fmaf(1e-5f, fmaf(E_hi, r_lo, M2), 2e-13f * r_lo);
+    const float M2 = M_hi * M_hi, S2 = fmaf(E_hi, r_lo, M2);
+    // a NaN or an infinity (also above the FP32 range) leaves S2 infinite or NaN: such a cell
+    // is looked at point by point, and its average counted if it is not in G
+    const bool settled = r_lo >= fmaf(1e-5f, r_hi, 2e-13f) && S2 < INFINITY &&
+                         r_lo * E_lo - 0.5f * M2 >= fmaf(1e-5f, S2, 2e-13f * r_lo);
     todo = !settled;
   }
 
