@@ -380,29 +380,29 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
   int mx = 0;
 #pragma unroll
   for (int l = 0; l < NB; ++l) mx = max(mx, fx_abs_hi(x[l]));
-  // the two momentum components share a block, so that their squares compare
+  const int E = fx_exp(mx);
+  // the squares of the two momentum components compare in the larger of their blocks
   const bool mom = c == 1 || c == 2;
-  const int mp = __shfl_xor_sync(0xffffffffu, mx, 3);
-  const int E = fx_exp(mom ? max(mx, mp) : mx);
+  const int Ep = __shfl_xor_sync(0xffffffffu, E, 3);
+  const int down = mom && Ep > E ? min(Ep - E, 63) : 0;
   Fx f[NB];
 #pragma unroll
   for (int l = 0; l < NB; ++l) f[l] = fx_from(x[l], E);
   // maxima in fixed point; the point of the largest |m|^2 is found from the
   // top 64 bits of the squares (2^-62 of the largest), its norm taken in FP64
   uint64_t top = 0, best = 0;
-  int64_t b1 = 0, b2 = 0;
+  int64_t b1 = 0;
 #pragma unroll
   for (int mu = 0; mu < NV; ++mu) {
     const int64_t r = fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu));
     const uint64_t ab = (uint64_t)(r < 0 ? -r : r);
     top = ab > top ? ab : top;
-    const uint64_t sq = __umul64hi(ab, ab);
+    const uint64_t sq = __umul64hi(ab >> down, ab >> down);
     const uint64_t s = sq + (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)sq, 3);
-    const int64_t q = __shfl_xor_sync(0xffffffffu, (long long)r, 3);
-    if (mu == 0 || s > best) { best = s; b1 = r; b2 = q; }
+    if (mu == 0 || s > best) { best = s; b1 = r; }
   }
   const double d = fx_out((int64_t)top, E);
-  const double m1 = fx_out(b1, E), m2 = fx_out(b2, E);
+  const double m1 = fx_out(b1, E), m2 = __shfl_xor_sync(0xffffffffu, m1, 3);
   // rho, |m|, E, |m1|, |m2|; the lanes of the other components hold 0
   double dr[5] = {c == 0 ? d : 0.0, c == 1 ? root(fdot2(m1, m1, m2, m2)) : 0.0, c == 3 ? d : 0.0, c == 1 ? d : 0.0,
                   c == 2 ? d : 0.0};
