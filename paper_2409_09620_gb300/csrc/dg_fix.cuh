@@ -179,6 +179,25 @@ FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
   return (r1 >> (s1 > 63 ? 63 : s1)) + (r2 >> (s2 > 63 ? 63 : s2));
 }
 
+// |r| as an integer; the top 62 bits of values whose largest is top (left shift, if negative right)
+FX_HD uint64_t fx_mag(int64_t r) { return (uint64_t)(r < 0 ? -r : r); }
+FX_HD int fx_norm_shift(uint64_t top) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)top) - 2;
+#else
+  return top == 0 ? 62 : __builtin_clzll(top) - 2;
+#endif
+}
+// the top 64 bits of (a 2^s)^2, a 2^s < 2^62: squares compare to 2^-58 of the largest
+FX_HD uint64_t fx_square(uint64_t a, int s) {
+  a = s >= 0 ? a << s : a >> (s < -63 ? 63 : -s);
+#ifdef __CUDA_ARCH__
+  return __umul64hi(a, a);
+#else
+  return (uint64_t)(((unsigned __int128)a * a) >> 64);
+#endif
+}
+
 // block fixed point of N values; returns the block's exponent
 template <int N>
 FX_HD int fx_block(const double x[N], Fx f[N]) {

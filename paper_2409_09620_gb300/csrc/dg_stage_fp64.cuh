@@ -388,18 +388,25 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
   Fx f[NB];
 #pragma unroll
   for (int l = 0; l < NB; ++l) f[l] = fx_from(x[l], E);
-  // maxima in fixed point; the point of the largest |m|^2 is found from the
-  // top 64 bits of the squares (2^-62 of the largest), its norm taken in FP64
-  uint64_t top = 0, best = 0;
+  // maxima in fixed point; the point of the largest |m|^2 is found from the top 64 bits
+  // of the squares (of the values scaled to 62 bits: to 2^-58 of the largest), its norm
+  // taken in FP64
+  int64_t r[NV];
+  uint64_t top = 0;
+#pragma unroll
+  for (int mu = 0; mu < NV; ++mu) {
+    r[mu] = fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu));
+    top = max(top, fx_mag(r[mu]));
+  }
+  const uint64_t ta = top >> down, tb = __shfl_xor_sync(0xffffffffu, (unsigned long long)ta, 3);
+  const int sh = fx_norm_shift(max(ta, tb)) - down;
+  uint64_t best = 0;
   int64_t b1 = 0;
 #pragma unroll
   for (int mu = 0; mu < NV; ++mu) {
-    const int64_t r = fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu));
-    const uint64_t ab = (uint64_t)(r < 0 ? -r : r);
-    top = ab > top ? ab : top;
-    const uint64_t sq = __umul64hi(ab >> down, ab >> down);
+    const uint64_t sq = fx_square(fx_mag(r[mu]), sh);
     const uint64_t s = sq + (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)sq, 3);
-    if (mu == 0 || s > best) { best = s; b1 = r; }
+    if (mu == 0 || s > best) { best = s; b1 = r[mu]; }
   }
   const double d = fx_out((int64_t)top, E);
   const double m1 = fx_out(b1, E), m2 = __shfl_xor_sync(0xffffffffu, m1, 3);
