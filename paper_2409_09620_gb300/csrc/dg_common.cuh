@@ -23,6 +23,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "dg_basis.h"
 #include "dg_math.h"
 
 namespace dg {
@@ -71,8 +72,9 @@ constexpr int TR_STRIDE = 8;
 constexpr int EJ_STRIDE = 16;
 // per-cell vertex record vd[nt][VD_CELL]: per vertex VD_STRIDE values (value and
 // gradient of component c at c and 4 + 2 c as limb pairs of dg_fix.cuh; 1/rho,
-// sound speed, m1, m2), then per component the exponents of its values, and of
-// its gradients and Hessian, as two and one 16-bit numbers
+// sound speed, m1, m2), then per component four 16-bit exponents: of its values, the x
+// and the y entries of its gradients, and the xx entry of its Hessian (xy and yy: one and
+// two steps from x to y further)
 constexpr int VD_STRIDE = 16;
 constexpr int VD_EXP = 3 * VD_STRIDE;
 constexpr int VD_CELL = VD_EXP + 4;
@@ -140,28 +142,7 @@ struct Scalars {
   int active, pad;
 };
 
-// ------------------------------------------------------------------------
-// Basis of eq. (basisfunc), modes 0..5, on the reference triangle
-// (v1 -> (0,0), v2 -> (1,0), v3 -> (0,1)).  Written as constexpr functions so
-// that evaluations at the fixed quadrature points fold to constants.
-// ------------------------------------------------------------------------
-__host__ __device__ constexpr double psi(int l, double x, double y) {
-  return l == 0 ? 1.0
-       : l == 1 ? 4.0 * x + 2.0 * y - 2.0
-       : l == 2 ? 3.0 * y - 1.0
-       : l == 3 ? 24.0 * x * x + 24.0 * x * y + 4.0 * y * y - 24.0 * x - 8.0 * y + 4.0
-       : l == 4 ? 20.0 * x * y + 10.0 * y * y - 4.0 * x - 12.0 * y + 2.0
-                : 10.0 * y * y - 8.0 * y + 1.0;
-}
-__host__ __device__ constexpr double psi_x(int l, double x, double y) {   // d/dxi
-  return l == 0 ? 0.0 : l == 1 ? 4.0 : l == 2 ? 0.0 : l == 3 ? 48.0 * x + 24.0 * y - 24.0
-       : l == 4 ? 20.0 * y - 4.0 : 0.0;
-}
-__host__ __device__ constexpr double psi_y(int l, double x, double y) {   // d/deta
-  return l == 0 ? 0.0 : l == 1 ? 2.0 : l == 2 ? 3.0 : l == 3 ? 24.0 * x + 8.0 * y - 8.0
-       : l == 4 ? 20.0 * x + 20.0 * y - 12.0 : 20.0 * y - 8.0;
-}
-// the same basis evaluated in the arithmetic of T at run-time points
+// the basis of dg_basis.h evaluated in the arithmetic of T at run-time points
 template <typename T>
 __device__ __forceinline__ T psi_t(int l, T x, T y) {
   // nested forms with explicit fmas (see fdot2)
@@ -172,51 +153,6 @@ __device__ __forceinline__ T psi_t(int l, T x, T y) {
        : l == 4 ? fma(x, fma(T(20), y, T(-4)), fma(y, fma(T(10), y, T(-12)), T(2)))
                 : fma(y, fma(T(10), y, T(-8)), T(1));
 }
-// second reference derivatives: r = 0 (xi xi), 1 (xi eta), 2 (eta eta)
-__host__ __device__ constexpr double psi_2(int l, int r) {
-  return l == 3 ? (r == 0 ? 48.0 : r == 1 ? 24.0 : 8.0)
-       : l == 4 ? (r == 0 ? 0.0 : 20.0)
-       : l == 5 ? (r == 2 ? 20.0 : 0.0) : 0.0;
-}
-// mass a_K^(l) = c_l |K| of the orthogonal basis
-__host__ __device__ constexpr double mass_c(int l) {
-  return l == 0 ? 1.0 : l == 1 ? 2.0 / 3.0 : l == 2 ? 0.5 : l == 3 ? 16.0 / 15.0 : l == 4 ? 4.0 / 9.0 : 1.0 / 3.0;
-}
-// 1 / c_l (exact in binary)
-__host__ __device__ constexpr double inv_mass_c(int l) {
-  return l == 0 ? 1.0 : l == 1 ? 1.5 : l == 2 ? 2.0 : l == 3 ? 0.9375 : l == 4 ? 2.25 : 3.0;
-}
-__host__ __device__ constexpr int degree_of(int l) { return l == 0 ? 0 : (l <= 2 ? 1 : 2); }
-
-// Gauss-Legendre nodes of Appendix B mapped to s in (0, 1), weights summing to 1.
-__host__ __device__ constexpr double gauss_s(int Q, int nu) {
-  return Q == 2 ? (nu == 0 ? 0.21132486540518713 : 0.78867513459481287)
-                : (nu == 0 ? 0.11270166537925831 : nu == 1 ? 0.5 : 0.88729833462074169);
-}
-__host__ __device__ constexpr double gauss_w(int Q, int nu) {
-  return Q == 2 ? 0.5 : (nu == 1 ? 8.0 / 18.0 : 5.0 / 18.0);
-}
-// edge i is opposite vertex i, run from vertex i+1 to vertex i+2 (counter-clockwise)
-__host__ __device__ constexpr double edge_xi(int i, double s) { return i == 0 ? 1.0 - s : i == 1 ? 0.0 : s; }
-__host__ __device__ constexpr double edge_eta(int i, double s) { return i == 0 ? s : i == 1 ? 1.0 - s : 0.0; }
-__host__ __device__ constexpr double vert_xi(int v) { return v == 1 ? 1.0 : 0.0; }
-__host__ __device__ constexpr double vert_eta(int v) { return v == 2 ? 1.0 : 0.0; }
-
-// Volume rules of Appendix A (tab:2th for N = 3, tab:4th for N = 6); (xi, eta) = (b2, b3).
-__host__ __device__ constexpr double vol_xi(int N, int mu) {
-  return N == 3 ? (mu == 0 ? 1.0 / 6.0 : mu == 1 ? 2.0 / 3.0 : 1.0 / 6.0)
-       : (mu == 0 ? 0.445948490915965 : mu == 1 ? 0.108103018168070 : mu == 2 ? 0.445948490915965
-          : mu == 3 ? 0.091576213509771 : mu == 4 ? 0.816847572980458 : 0.091576213509771);
-}
-__host__ __device__ constexpr double vol_eta(int N, int mu) {
-  return N == 3 ? (mu == 0 ? 2.0 / 3.0 : mu == 1 ? 1.0 / 6.0 : 1.0 / 6.0)
-       : (mu == 0 ? 0.108103018168070 : mu == 1 ? 0.445948490915965 : mu == 2 ? 0.445948490915965
-          : mu == 3 ? 0.816847572980458 : mu == 4 ? 0.091576213509771 : 0.091576213509771);
-}
-__host__ __device__ constexpr double vol_w(int N, int mu) {
-  return N == 3 ? 1.0 / 3.0 : (mu < 3 ? 0.223381589678010 : 0.109951743655322);
-}
-
 // acc + c * x with a coefficient c known at compile time after unrolling:
 // zero terms vanish and unit coefficients become additions.
 template <typename T>

@@ -19,11 +19,15 @@
 //     the terms does not matter;
 //   * the result converts to FP64 with one rounding.
 //
-// The error of a sum is a few 2^-57 of the block's largest magnitude, below
-// that of the FMA chain it replaces (tests/test_fix_host.py).  Zeros stay
-// zero, subnormals count as zero and blocks below 2^-959 keep an absolute
-// 2^-1016; a block that holds an infinity or a NaN has E = 0x7ff, and the
-// callers turn its results into NaN.
+// The error of a sum is a few 2^-57 of the block's largest magnitude
+// (tests/test_fix_host.py).  Where that value is a term of the sum (point values,
+// quadrature sums), an FMA chain rounds at 2^-53 of it.  Where it would not be,
+// the terms have a block of their own: derivatives, which do not contain the
+// cell average (dg_fix_vertex.cuh; tests/test_fix_vertex_host.py compares them with
+// the chain).  Zeros stay zero,
+// subnormals count as zero and blocks below 2^-959 keep an absolute 2^-1016; a
+// block that holds an infinity or a NaN has E = 0x7ff, and the callers turn its
+// results into NaN.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -156,13 +160,38 @@ FX_HD Fx fx_value(int64_t r, int s) {
 }
 // a value as one integer
 FX_HD int64_t fx_join(Fx x) { return (int64_t)x.h * (1LL << FX_LIMB) + x.l; }
+// a - b of blocks with exponents Ea, Eb, in that of E >= Ea, Eb; below 2^61
+FX_HD int64_t fx_diff(Fx a, int Ea, Fx b, int Eb, int E) {
+  return (fx_join(a) >> (E - Ea < 63 ? E - Ea : 63)) - (fx_join(b) >> (E - Eb < 63 ? E - Eb : 63));
+}
+// the same as limbs of exponent E + S; |a - b| < 2^(60 + S), for the high limb has 32 bits
+template <int S>
+FX_HD Fx fx_jump(Fx a, int Ea, Fx b, int Eb, int E) {
+  return fx_value(fx_diff(a, Ea, b, Eb, E), S);
+}
 FX_HD int64_t fx_sum(const FxAcc &s) {
   return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + (s.b >> (FX_ONE - FX_LIMB));
 }
+// the same with the sum's last unit rounded to nearest instead of down
+FX_HD int64_t fx_round(const FxAcc &s) {
+  return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + ((s.b + (1LL << (FX_ONE - FX_LIMB - 1))) >> (FX_ONE - FX_LIMB));
+}
+// sum of products with run-time coefficients, l l included (their low limbs reach
+// 2^29, so that dropping it costs up to 4 units of the result per term), and rounded
+struct FxAccL {
+  int64_t a, b, l;
+};
+FX_HD void fx_mac(FxAccL &s, Fx c, Fx x) {
+  fx_mad(s.a, c.h, x.h);
+  fx_mad(s.b, c.h, x.l);
+  fx_mad(s.b, c.l, x.h);
+  fx_mad(s.l, c.l, x.l);
+}
+FX_HD int64_t fx_round(const FxAccL &s) { return fx_round(FxAcc{s.a, s.b + (s.l >> FX_LIMB)}); }
 // r 2^(E - 1080) rounded to nearest; |r| < 2^63
 FX_HD double fx_to(int64_t r, int E) {
   const int64_t g = r >> 63;
-  const uint64_t a = (uint64_t)(r ^ g);   // |r| (|r| - 1 for r < 0)
+  const uint64_t a = (uint64_t)(r ^ g) - (uint64_t)g;   // |r|
   const int e8 = fx_log2_127(a);
   const uint64_t m = a << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62
   const uint64_t q = (m + 512u) >> 10;
@@ -188,6 +217,13 @@ FX_HD int fx_norm_shift(uint64_t top) {
   return top == 0 ? 62 : __builtin_clzll(top) - 2;
 #endif
 }
+// bits by which |r| < 2^61 may grow as a value of limbs (-1: it has to shrink by one), at most 40
+FX_HD int fx_room(int64_t r) {
+  const int z = fx_norm_shift(fx_mag(r)) - 2;
+  return z < 40 ? z : 40;
+}
+// r 2^z as a value; its block's exponent falls by z >= -1
+FX_HD Fx fx_value_up(int64_t r, int z) { return fx_value(z >= 0 ? r * (1LL << z) : r, z >= 0 ? 0 : 1); }
 // the top 64 bits of (a 2^s)^2, a 2^s < 2^62: squares compare to 2^-58 of the largest
 FX_HD uint64_t fx_square(uint64_t a, int s) {
   a = s >= 0 ? a << s : a >> (s < -63 ? 63 : -s);

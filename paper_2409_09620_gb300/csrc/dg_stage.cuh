@@ -16,6 +16,7 @@
 
 #include "dg_common.cuh"
 #include "dg_fix.cuh"
+#include "dg_fix_vertex.cuh"
 
 namespace dg {
 

@@ -260,80 +260,40 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   __shared__ double s_m[TPB];
   s_m[threadIdx.x] = live ? mul(m.area[Kc], h[0]) : 0.0;   // summed after the barrier below
 
-  // ---- vertex derivatives of u_h for the OE jumps ------------------------------
-  // values, then the reference derivatives turned by J^-1, all in fixed point
-  // (coefficients of derivatives reach 48: as c / 64; the entries of J^-1 share a block)
+  // ---- vertex values and derivatives of u_h for the OE jumps --------------------
+  // stored as limb pairs (FP64 would be rounded here and taken apart again in K2)
   {
-    Fx f[NB], J[2][2];   // J[d][0] = dxi/dx_d, J[d][1] = deta/dx_d
-    const int E = fx_block<NB>(h, f);
-    bad = bad || E >= FX_ENAN;
-    int EJ;
-    {
-      const double j0 = m.jinv[Kc], j1 = m.jinv[nt + Kc], j2 = m.jinv[2 * nt + Kc], j3 = m.jinv[3 * nt + Kc];
-      EJ = fx_exp(max(max(fx_abs_hi(j0), fx_abs_hi(j1)), max(fx_abs_hi(j2), fx_abs_hi(j3)))) - 1022;   // |j| < 2^EJ
-      J[0][0] = fx_coef(j0, -EJ);
-      J[1][0] = fx_coef(j1, -EJ);
-      J[0][1] = fx_coef(j2, -EJ);
-      J[1][1] = fx_coef(j3, -EJ);
-    }
-    // p dxi/dx_d + q deta/dx_d as a sum
-    auto turn = [&](int d, Fx p, Fx q) {
-      FxAcc t{0, 0};
-      fx_mac(t, J[d][0], p);
-      fx_mac(t, J[d][1], q);
-      return fx_sum(t);
-    };
-    // stored as limb pairs (FP64 would be rounded here and taken apart again in K2)
     double *vo = vdo + Kc * VD_CELL;
-    Fx gx{0, 0}, gy{0, 0};
+    short4 ex = make_short4(0, 0, 0, 0);
+    {
+      Fx f[NB];
+      const int E = fx_block<NB>(h, f);
+      bad = bad || E >= FX_ENAN;
+      ex.x = (short)(E + 2);
 #pragma unroll
-    for (int vv = 0; vv < 3; ++vv) {
-      const int64_t val = fx_point<NB>(f, vert_xi(vv), vert_eta(vv));   // below 11 * 2^58
-      if (K == 2 || vv == 0) {   // P1 has one gradient
-        FxAcc sx{0, 0}, se{0, 0};
-#pragma unroll
-        for (int l = 1; l < NB; ++l) {
-          fx_mac(sx, fxc(psi_x(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
-          fx_mac(se, fxc(psi_y(l, vert_xi(vv), vert_eta(vv)) / 64.0), f[l]);
-        }
-        // the coefficients of a sum add up to at most 37 / 64 and a turn at most doubles
-        // it: below 2^59, limbs with a bit to spare
-        const Fx px = fx_value(fx_sum(sx), 0), pe = fx_value(fx_sum(se), 0);
-        gx = fx_value(turn(0, px, pe), 0);
-        gy = fx_value(turn(1, px, pe), 0);
-      }
-      s_u[vv][lc].c[c] = fx_out(val, E);   // this thread's slot; read after the barrier below
-      if (live) {
-        double *rec = vo + vv * VD_STRIDE;
-        const Fx v2 = fx_value(val, 2);   // below 2^59.5
-        *reinterpret_cast<int2 *>(rec + c) = make_int2(v2.h, v2.l);
-        *reinterpret_cast<int4 *>(rec + 4 + 2 * c) = make_int4(gx.h, gx.l, gy.h, gy.l);
+      for (int vv = 0; vv < 3; ++vv) {
+        const int64_t val = fx_point<NB>(f, vert_xi(vv), vert_eta(vv));   // below 11 * 2^58
+        s_u[vv][lc].c[c] = fx_out(val, E);   // this thread's slot; read after the barrier below
+        const Fx v2 = fx_value(val, 2);      // below 2^59.5
+        if (live) *reinterpret_cast<int2 *>(vo + vv * VD_STRIDE + c) = make_int2(v2.h, v2.l);
       }
     }
-    // exponents of the values, gradients (c / 64, J^-1) and Hessians (one shift more)
-    if (live)
-      *reinterpret_cast<short4 *>(vo + VD_EXP + c) =
-          bad ? make_short4(FX_ENAN, FX_ENAN, FX_ENAN, 0)
-              : make_short4((short)(E + 2), (short)(E + 6 + EJ), (short)(E + 7 + 2 * EJ), 0);
-    if (K == 2) {
-      FxAcc s0{0, 0}, s1{0, 0}, s2{0, 0};
+    const double jxi[2] = {m.jinv[Kc], m.jinv[nt + Kc]}, jeta[2] = {m.jinv[2 * nt + Kc], m.jinv[3 * nt + Kc]};
+    const FxRows J = fx_rows(jxi, jeta);
+    auto gradient = [&](int vv, Fx gx, Fx gy) {
+      if (live) *reinterpret_cast<int4 *>(vo + vv * VD_STRIDE + 4 + 2 * c) = make_int4(gx.h, gx.l, gy.h, gy.l);
+    };
+    FxDerivs<NB> d(h, J, gradient);
+    ex.y = (short)d.EG[0];
+    ex.z = (short)d.EG[1];
+    if constexpr (K == 2) {
+      ex.w = (short)d.EH;
 #pragma unroll
-      for (int l = 3; l < NB; ++l) {
-        fx_mac(s0, fxc(psi_2(l, 0) / 64.0), f[l]);
-        fx_mac(s1, fxc(psi_2(l, 1) / 64.0), f[l]);
-        fx_mac(s2, fxc(psi_2(l, 2) / 64.0), f[l]);
-      }
-      // (xx, xy, yy) = J^-T H J^-1 row by row
-      const Fx hxx = fx_value(fx_sum(s0), 0), hxe = fx_value(fx_sum(s1), 0), hee = fx_value(fx_sum(s2), 0);
-      const Fx ax = fx_value(turn(0, hxx, hxe), 1), bx = fx_value(turn(0, hxe, hee), 1);
-      const Fx ay = fx_value(turn(1, hxx, hxe), 1), by = fx_value(turn(1, hxe, hee), 1);
-      const int64_t d2[3] = {turn(0, ax, bx), turn(1, ax, bx), turn(1, ay, by)};
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const Fx d = fx_value(d2[r], 0);   // below 2^59
-        if (live) *reinterpret_cast<int2 *>(hso + Kc * 12 + 3 * c + r) = make_int2(d.h, d.l);
-      }
+      for (int r = 0; r < 3; ++r)
+        if (live) *reinterpret_cast<int2 *>(hso + Kc * 12 + 3 * c + r) = make_int2(d.hess[r].h, d.hess[r].l);
     }
+    if (bad) ex = make_short4(FX_ENAN, FX_ENAN, FX_ENAN, FX_ENAN);
+    if (live) *reinterpret_cast<short4 *>(vo + VD_EXP + c) = ex;
   }
   __syncthreads();
   // 1/rho and sound speed at the vertices, for the wave speeds beta of the OE (+inf for rho <= 0)
@@ -434,13 +394,6 @@ __device__ __forceinline__ Fx ld_fx(const double *p) {
   const int2 v = *reinterpret_cast<const int2 *>(p);
   return Fx{v.x, v.y};
 }
-// a - b of blocks with exponents Ea, Eb as limbs of exponent E + S, E >= Ea, Eb;
-// |a - b| < 2^(60 + S), for the high limb has 32 bits
-template <int S>
-__device__ __forceinline__ Fx fx_jump(Fx a, int Ea, Fx b, int Eb, int E) {
-  return fx_value((fx_join(a) >> min(E - Ea, 63)) - (fx_join(b) >> min(E - Eb, 63)), S);
-}
-
 // beta and 2 J of component c at a boundary edge, from the exterior polynomial
 // of all components of this side
 template <int K>
@@ -456,9 +409,10 @@ __device__ __noinline__ void boundary_jumps(const MeshDev &m, const Phys &ph, co
     ab[q] = avg[q * nt + Kc];   // the exterior state of a transmissive edge
     xo[q] = *reinterpret_cast<const short4 *>(vme + VD_EXP + q);
   }
-  auto get = [&](const double *p, int E) { return E >= FX_ENAN ? NAN : fx_to(fx_join(ld_fx(p)), E); };
+  auto get = [&](const double *p, int q, int E) { return xo[q].x >= FX_ENAN ? NAN : fx_to(fx_join(ld_fx(p)), E); };
 #pragma unroll
-  for (int q = 0; q < 12; ++q) hme[q] = K == 2 ? get(hsi + Kc * 12 + q, xo[q / 3].z) : 0.0;
+  for (int q = 0; q < 12; ++q)   // xx, xy, yy: the exponents step as those of the gradient's x and y
+    hme[q] = K == 2 ? get(hsi + Kc * 12 + q, q / 3, xo[q / 3].w + q % 3 * (xo[q / 3].z - xo[q / 3].y)) : 0.0;
   beta = 0.0;
   // row c of a jump per component, the momentum in (m_n, m_t) for RIOE
   auto row = [&](const double d[4]) {
@@ -473,9 +427,9 @@ __device__ __noinline__ void boundary_jumps(const MeshDev &m, const Phys &ph, co
     const double *ro = vme + ov * VD_STRIDE;
     double val[4], grd[8], xv[4], xg[8], xh[12];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) val[q] = get(ro + q, xo[q].x);
+    for (int q = 0; q < 4; ++q) val[q] = get(ro + q, q, xo[q].x);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) grd[q] = get(ro + 4 + q, xo[q / 2].y);
+    for (int q = 0; q < 8; ++q) grd[q] = get(ro + 4 + q, q / 2, q & 1 ? xo[q / 2].z : xo[q / 2].y);
     double px = 0.0, py = 0.0;
     if (cn == -7) { px = m.vxy[(2 * ov) * nt + Kc]; py = m.vxy[(2 * ov + 1) * nt + Kc]; }
     ghost_vertex(-cn, val, grd, hme, ab, nx, ny, px, py, t_out, ph, xv, xg, xh);
@@ -530,10 +484,12 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     // jumps of this component: values and gradients at v_c then v_d, the Hessian once; with
     // the exponent of each kind (the momentum components share it, for their rotation)
     Fx jv[2], jg[2][2], jh[3];
-    int E0, E1, E2 = 0;
-    auto shared_exp = [&](int E) {
-      const int p = __shfl_xor_sync(0xffffffffu, E, 3);
-      return mom ? max(E, p) : E;
+    int E0, Ev[2], E1[2], E2[3] = {0, 0, 0};
+    // the larger exponents of two components, two kinds at a time
+    auto shared_exp = [&](int Ea, int Eb, int &a, int &b) {
+      const int p = __shfl_xor_sync(0xffffffffu, (Ea << 16) | (Eb & 0xffff), 3);
+      a = mom ? max(Ea, p >> 16) : Ea;
+      b = mom ? max(Eb, (int)(short)p) : Eb;
     };
     double r;
     bool bad = xo.x >= FX_ENAN;
@@ -542,9 +498,11 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     const double *vnb = vdi + nb * VD_CELL;
     const short4 xx = *reinterpret_cast<const short4 *>(vnb + VD_EXP + c);
     bad = bad || xx.x >= FX_ENAN;
-    E0 = shared_exp(max(xo.x, xx.x));
-    E1 = shared_exp(max(xo.y, xx.y));
-    if (K == 2) E2 = shared_exp(max(xo.z, xx.z));
+    int ho[3] = {xo.w, xo.w + xo.z - xo.y, xo.w + 2 * (xo.z - xo.y)};   // Hessian: xx, xy, yy
+    int hx[3] = {xx.w, xx.w + xx.z - xx.y, xx.w + 2 * (xx.z - xx.y)};
+    shared_exp(max(xo.x, xx.x), max(xo.y, xx.y), E0, E1[0]);
+    shared_exp(max(xo.z, xx.z), max(ho[0], hx[0]), E1[1], E2[0]);
+    if (K == 2) shared_exp(max(ho[1], hx[1]), max(ho[2], hx[2]), E2[1], E2[2]);
 #pragma unroll
     for (int ev = 0; ev < 2; ++ev) {   // v_c then v_d, and the neighbour's copy of it
       int ov = i + 1 + ev, xv = jn + 2 - ev;
@@ -553,14 +511,21 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
       const double *ro = vme + ov * VD_STRIDE, *rx = vnb + xv * VD_STRIDE;
       const int4 go = *reinterpret_cast<const int4 *>(ro + 4 + 2 * c),
                  gx = *reinterpret_cast<const int4 *>(rx + 4 + 2 * c);
-      jv[ev] = fx_jump<1>(ld_fx(ro + c), xo.x, ld_fx(rx + c), xx.x, E0);
-      jg[ev][0] = fx_jump<0>(Fx{go.x, go.y}, xo.y, Fx{gx.x, gx.y}, xx.y, E1);
-      jg[ev][1] = fx_jump<0>(Fx{go.z, go.w}, xo.y, Fx{gx.z, gx.w}, xx.y, E1);
+      // the values' difference is far below their block: scaled up, so that it keeps its
+      // bits in the rotation (gradients and Hessians contain no average)
+      const int64_t d = fx_diff(ld_fx(ro + c), xo.x, ld_fx(rx + c), xx.x, E0);
+      int z = fx_room(d);
+      const int zp = __shfl_xor_sync(0xffffffffu, z, 3);
+      z = mom ? min(z, zp) : z;
+      jv[ev] = fx_value_up(d, z);
+      Ev[ev] = E0 - z;
+      jg[ev][0] = fx_jump<0>(Fx{go.x, go.y}, xo.y, Fx{gx.x, gx.y}, xx.y, E1[0]);
+      jg[ev][1] = fx_jump<0>(Fx{go.z, go.w}, xo.z, Fx{gx.z, gx.w}, xx.z, E1[1]);
     }
     if (K == 2) {
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        jh[q] = fx_jump<0>(ld_fx(hsi + Kc * 12 + 3 * c + q), xo.z, ld_fx(hsi + nb * 12 + 3 * c + q), xx.z, E2);
+        jh[q] = fx_jump<1>(ld_fx(hsi + Kc * 12 + 3 * c + q), ho[q], ld_fx(hsi + nb * 12 + 3 * c + q), hx[q], E2[q]);
     }
     {
       int vv = c & 1 ? (c & 2 ? jn + 1 : i + 2) : (c & 2 ? jn + 2 : i + 1);
@@ -583,13 +548,13 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
     double J[K + 1];
 #pragma unroll
     for (int ev = 0; ev < 2; ++ev) {
-      const double q = rot(jv[ev], E0 + 1), g0 = rot(jg[ev][0], E1), g1 = rot(jg[ev][1], E1);
+      const double q = rot(jv[ev], Ev[ev]), g0 = rot(jg[ev][0], E1[0]), g1 = rot(jg[ev][1], E1[1]);
       // 2 J: the 1/2 of the trapezoidal rule moves into A (sqrt(1/2))
       J[0] = ev == 0 ? mul(q, q) : fma(q, q, J[0]);
       J[1] = ev == 0 ? fdot2(g0, g0, g1, g1) : fma(g0, g0, fma(g1, g1, J[1]));
     }
     if (K == 2) {   // the Hessian jump counts at both endpoints
-      const double h0 = rot(jh[0], E2), h1 = rot(jh[1], E2), h2 = rot(jh[2], E2);
+      const double h0 = rot(jh[0], E2[0] + 1), h1 = rot(jh[1], E2[1] + 1), h2 = rot(jh[2], E2[2] + 1);
       const double f = fma(h0, h0, fma(add(h1, h1), h1, mul(h2, h2)));
       J[K] = add(f, f);
     }
