@@ -23,8 +23,8 @@
 // (tests/test_fix_host.py).  Where that value is a term of the sum (point values,
 // quadrature sums), an FMA chain rounds at 2^-53 of it.  Where it would not be,
 // the terms have a block of their own: derivatives, which do not contain the
-// cell average (dg_fix_vertex.cuh; tests/test_fix_vertex_host.py compares them with
-// the chain).  Zeros stay zero,
+// cell average (dg_fix_vertex.cuh, dg_fix_scalar.cuh; tests/test_fix_vertex_host.py and
+// tests/test_fix_scalar_host.py compare them with the chain).  Zeros stay zero,
 // subnormals count as zero and blocks below 2^-959 keep an absolute 2^-1016; a
 // block that holds an infinity or a NaN has E = 0x7ff, and the callers turn its
 // results into NaN.

@@ -30,49 +30,11 @@
 
 #include "../../include/dg.h"
 #include "dg_fix.cuh"
+#include "dg_fix_scalar.cuh"
 #include "dg_internal.h"
 
 namespace dg {
 namespace sc {
-
-// --------------------------------------------------------------------------
-// Basis of eq. (basisfunc), modes 0..9, and its reference derivatives.  Each
-// mode is a sum of terms c xi^p eta^q; d^(r+s)/dxi^r deta^s is taken term by
-// term.  constexpr, so evaluations at fixed points fold to constants.
-// --------------------------------------------------------------------------
-// flat (non-recursive) helpers for exponents and orders up to 3, so that the
-// optimiser folds every evaluation at the fixed points into a constant
-__host__ __device__ constexpr double ipow(double x, int n) {
-  return n <= 0 ? 1.0 : n == 1 ? x : n == 2 ? x * x : x * x * x;
-}
-__host__ __device__ constexpr double fall(int n, int r) {   // n (n-1) ... (n-r+1)
-  return r <= 0 ? 1.0 : r == 1 ? double(n) : r == 2 ? double(n * (n - 1)) : double(n * (n - 1) * (n - 2));
-}
-__host__ __device__ constexpr double term(double c, int p, int q, int r, int s, double x, double y) {
-  return (r > p || s > q) ? 0.0 : c * fall(p, r) * fall(q, s) * ipow(x, p - r) * ipow(y, q - s);
-}
-__host__ __device__ constexpr double psi_rs(int l, int r, int s, double x, double y) {
-#define T(c, p, q) term(c, p, q, r, s, x, y)
-  return l == 0 ? T(1, 0, 0)
-       : l == 1 ? T(4, 1, 0) + T(2, 0, 1) + T(-2, 0, 0)
-       : l == 2 ? T(3, 0, 1) + T(-1, 0, 0)
-       : l == 3 ? T(24, 2, 0) + T(24, 1, 1) + T(4, 0, 2) + T(-24, 1, 0) + T(-8, 0, 1) + T(4, 0, 0)
-       : l == 4 ? T(20, 1, 1) + T(10, 0, 2) + T(-4, 1, 0) + T(-12, 0, 1) + T(2, 0, 0)
-       : l == 5 ? T(10, 0, 2) + T(-8, 0, 1) + T(1, 0, 0)
-       : l == 6 ? T(160, 3, 0) + T(240, 2, 1) + T(96, 1, 2) + T(8, 0, 3) + T(-240, 2, 0) + T(-192, 1, 1) +
-                      T(-24, 0, 2) + T(96, 1, 0) + T(24, 0, 1) + T(-8, 0, 0)
-       : l == 7 ? T(168, 2, 1) + T(168, 1, 2) + T(28, 0, 3) + T(-24, 2, 0) + T(-192, 1, 1) + T(-60, 0, 2) +
-                      T(24, 1, 0) + T(36, 0, 1) + T(-4, 0, 0)
-       : l == 8 ? T(84, 1, 2) + T(42, 0, 3) + T(-48, 1, 1) + T(-66, 0, 2) + T(4, 1, 0) + T(26, 0, 1) + T(-2, 0, 0)
-                : T(35, 0, 3) + T(-45, 0, 2) + T(15, 0, 1) + T(-1, 0, 0);
-#undef T
-}
-// a_K^(l) / |K| (exact rationals: 1, 2/3, 1/2, 16/15, 4/9, 1/3, 16/7, 4/5, 1/3, 1/4)
-__host__ __device__ constexpr double sc_inv_mass(int l) {
-  return l == 0 ? 1.0 : l == 1 ? 1.5 : l == 2 ? 2.0 : l == 3 ? 0.9375 : l == 4 ? 2.25 : l == 5 ? 3.0
-       : l == 6 ? 7.0 / 16.0 : l == 7 ? 1.25 : l == 8 ? 3.0 : 4.0;
-}
-__host__ __device__ constexpr int sc_degree(int l) { return l == 0 ? 0 : l <= 2 ? 1 : l <= 5 ? 2 : 3; }
 
 template <int K> struct SDeg {
   static constexpr int NB = (K + 1) * (K + 2) / 2;     // modes; also derivatives up to order K per vertex
@@ -147,16 +109,6 @@ __device__ __forceinline__ int64_t sfx_point(const Fx f[SDeg<K>::NB], double xi,
   for (int l = 0; l < SDeg<K>::NB; ++l) fx_mac(s, fxc(psi_rs(l, 0, 0, xi, eta) / (1 << SVAL<K>)), f[l]);
   return fx_sum(s);
 }
-// reference derivative d^(r+s) / dxi^r deta^s at a fixed point (coefficients reach
-// 960 for P3, 48 for P2: as c / 256)
-template <int K>
-__device__ __forceinline__ double sfx_deriv(const Fx f[SDeg<K>::NB], int E, int r, int s, double xi, double eta) {
-  FxAcc a{0, 0};
-#pragma unroll
-  for (int l = 1; l < SDeg<K>::NB; ++l) fx_mac(a, fxc(psi_rs(l, r, s, xi, eta) / 256.0), f[l]);
-  return fx_out(fx_sum(a), E + 8);
-}
-
 // ---- K1: volume + edge fluxes + RK combination ------------------------------------
 template <int K>
 __global__ void __launch_bounds__(TPB) k_sc_rk(MeshDev m, ScPhys ph, const double *__restrict__ v,
@@ -277,19 +229,65 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
     }
     d[0] = fx_out((int64_t)top, Ed + SVAL<K>);
     c[0] = c0;
-    const int E = fx_block<NB>(c, f);
-    const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
     double *vo = vr + Kc * 3 * NB;
+    {
+      const int E = fx_block<NB>(c, f);
+#pragma unroll
+      for (int vv = 0; vv < 3; ++vv) vo[vv * NB] = fx_out(sfx_point<K>(f, vert_xi(vv), vert_eta(vv)), E + SVAL<K>);
+    }
+    const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
     // one index of a tensor with components t[r], r = number of xi: out[r] for d/dx (w = 0) or d/dy
     auto turn = [&](int n, int w, const double *t, double *o) {
 #pragma unroll
       for (int r = 0; r < n; ++r) o[r] = fdot2(t[r + 1], w == 0 ? jx : jy, t[r], w == 0 ? ex : ey);
     };
-    double t3[4] = {0.0, 0.0, 0.0, 0.0};   // third derivatives: constant
-    if constexpr (K == 3) {
-      double t[4], x[3], y[3], xx[2], xy[2], yy[2];
+    if constexpr (K == 1) {   // constant: three operations
+      const double t[2] = {fma(2.0, c[1], mul(3.0, c[2])), mul(4.0, c[1])};
+      double x, y;
+      turn(1, 0, t, &x);
+      turn(1, 1, t, &y);
 #pragma unroll
-      for (int r = 0; r <= 3; ++r) t[r] = sfx_deriv<K>(f, E, r, 3 - r, 0.0, 0.0);
+      for (int vv = 0; vv < 3; ++vv) {
+        vo[vv * NB + didx(1, 1)] = x;
+        vo[vv * NB + didx(1, 0)] = y;
+      }
+    } else {
+      const int E = sfx_deriv_block<K, 1>(c, f);
+#pragma unroll
+      for (int vv = 0; vv < 3; ++vv) {
+        double t[2], x, y;
+#pragma unroll
+        for (int r = 0; r <= 1; ++r) t[r] = sfx_deriv<K, 1>(f, E, r, vv);
+        turn(1, 0, t, &x);
+        turn(1, 1, t, &y);
+        vo[vv * NB + didx(1, 1)] = x;
+        vo[vv * NB + didx(1, 0)] = y;
+      }
+    }
+    if constexpr (K >= 2) {
+      const int E = sfx_deriv_block<K, 2>(c, f);
+      double t2[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int vv = 0; vv < 3; ++vv) {
+        if (K == 3 || vv == 0) {   // P2: constant
+          double t[3], x[2], y[2];
+#pragma unroll
+          for (int r = 0; r <= 2; ++r) t[r] = sfx_deriv<K, 2>(f, E, r, vv);
+          turn(2, 0, t, x);
+          turn(2, 1, t, y);
+          turn(1, 0, x, t2);
+          turn(1, 1, x, t2 + 1);
+          turn(1, 1, y, t2 + 2);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) vo[vv * NB + didx(2, 2 - q)] = t2[q];
+      }
+    }
+    if constexpr (K == 3) {   // third derivatives: constant
+      const int E = sfx_deriv_block<K, 3>(c, f);
+      double t[4], x[3], y[3], xx[2], xy[2], yy[2], t3[4];
+#pragma unroll
+      for (int r = 0; r <= 3; ++r) t[r] = sfx_deriv<K, 3>(f, E, r, 0);
       turn(3, 0, t, x);
       turn(3, 1, t, y);
       turn(2, 0, x, xx);
@@ -299,39 +297,10 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
       turn(1, 1, xx, t3 + 1);
       turn(1, 1, xy, t3 + 2);
       turn(1, 1, yy, t3 + 3);
-    }
-    double t2[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-    for (int vv = 0; vv < 3; ++vv) {
-      const double xi = vert_xi(vv), eta = vert_eta(vv);
-      double *rec = vo + vv * NB;
-      rec[0] = fx_out(sfx_point<K>(f, xi, eta), E + SVAL<K>);
-      {
-        double t[2], x, y;
-        t[0] = sfx_deriv<K>(f, E, 0, 1, xi, eta);
-        t[1] = sfx_deriv<K>(f, E, 1, 0, xi, eta);
-        turn(1, 0, t, &x);
-        turn(1, 1, t, &y);
-        rec[didx(1, 1)] = x;
-        rec[didx(1, 0)] = y;
-      }
-      if constexpr (K >= 2) {
-        if (K == 3 || vv == 0) {   // P2: constant
-          double t[3], x[2], y[2];
+      for (int vv = 0; vv < 3; ++vv)
 #pragma unroll
-          for (int r = 0; r <= 2; ++r) t[r] = sfx_deriv<K>(f, E, r, 2 - r, xi, eta);
-          turn(2, 0, t, x);
-          turn(2, 1, t, y);
-          turn(1, 0, x, t2);
-          turn(1, 1, x, t2 + 1);
-          turn(1, 1, y, t2 + 2);
-        }
-#pragma unroll
-        for (int q = 0; q < 3; ++q) rec[didx(2, 2 - q)] = t2[q];
-      }
-      if constexpr (K == 3)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) rec[didx(3, 3 - q)] = t3[q];
+        for (int q = 0; q < 4; ++q) vo[vv * NB + didx(3, 3 - q)] = t3[q];
     }
   }
   block_reduce<1>(d, part + blockIdx.x, OpMaxNN());
