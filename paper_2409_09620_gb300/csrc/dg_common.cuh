@@ -198,9 +198,10 @@ __device__ __forceinline__ double mul(double a, double b) { return fma(a, b, fp_
 __device__ __forceinline__ float add(float a, float b) { return a + b; }
 __device__ __forceinline__ float mul(float a, float b) { return a * b; }
 
-// 1 / x: the hardware's reciprocal approximation y (relative error e below
-// 2^-20) and one cubic step y (1 + e + e^2); the remainder e^3 is below 2^-60,
-// so the result is within 0.51 ulp.  3 DFMA (192 cycles) in place of 344.
+// 1 / x: the hardware's reciprocal approximation y (relative error e below 2^-20) and one
+// step of the fourth-order iteration y (1 + e + e^2 + e^3) (Traub 1964, the reciprocal's
+// hyperpower series).  The remainder e^4 is below 2^-80 and e is exact to 2^-73, so the
+// result is within 0.50001 ulp (tests/test_gpu_math.py).  4 DFMA (256 cycles) in place of 344.
 // Outside the normal range (with two binary orders to spare) it divides.
 __device__ __forceinline__ double recip(double x) {
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
@@ -208,26 +209,29 @@ __device__ __forceinline__ double recip(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, fp_const<0>());
-  return fma(y, fma(e, e, e), y);
+  return fma(y, fma(fma(e, e, e), e, e), y);
 }
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 // -x / 2
 __device__ __forceinline__ double half_neg(double x) { return fma(-x, fp_const<2>(), fp_const<1>()); }
 __device__ __forceinline__ float half_neg(float x) { return -0.5f * x; }
-// sqrt(x), x >= 0 (or NaN): from the hardware's approximation y of 1 / sqrt(x)
-// (relative error below 2^-20), g = x y and two Newton steps g + (x - g^2) y / 2,
-// whose remainders are below 2^-41 and 2^-61; the residual x - g^2 is exact in
-// the fma, so the result is within 0.51 ulp.  5 DFMA (320 cycles) in place of
-// 572.  Zero stays zero; outside [2^-895, 2^897) it takes sqrt.
+// sqrt(x), x >= 0 (or NaN): from the hardware's approximation y of 1 / sqrt(x) (relative error
+// d below 2^-20) Goldschmidt's coupled iteration (1964): g -> sqrt(x) and h -> 1 / (2 sqrt(x))
+// with r = 1/2 - g h, both then within 1.5 d^2 < 2^-39, and a last Newton step g + (x - g^2) h,
+// whose residual is exact in the fma and whose remainder is below 2^-77: within 0.50001 ulp
+// (tests/test_gpu_math.py).  6 DFMA (384 cycles) in place of 572.  Zero stays zero; outside
+// [2^-895, 2^897) it takes sqrt.
 __device__ __forceinline__ double root(double x) {
   const unsigned ex = (unsigned)__double2hiint(x) >> 20;
   const bool zero = !nonzero_bits(x);
   if (ex - 128u >= 1792u && !zero) return sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double h = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));   // y / 2
+  double h = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));   // y / 2
   double g = mul(x, y);
-  g = fma(fma(-g, g, x), h, g);
+  const double r = fma(-g, h, fp_const<2>());
+  g = fma(g, r, g);
+  h = fma(h, r, h);
   g = fma(fma(-g, g, x), h, g);
   return zero ? x : g;
 }

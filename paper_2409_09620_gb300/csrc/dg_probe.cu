@@ -1,7 +1,8 @@
 // dg_probe.cu -- FMA throughput of this GPU in FP64 and FP32, measured with
 // CUDA events.  The FP64 stage kernels are bound by the FP64 pipe (GB300 runs
 // DFMA at a small fraction of its FP32 rate), so the roofline of the solver's
-// FP64 path is this measured rate, not a memory bandwidth.
+// FP64 path is this measured rate, not a memory bandwidth.  Also the kernels' own
+// arithmetic functions on arrays, for tests against exact results.
 #include <cuda_runtime.h>
 
 #include "../../include/dg.h"
@@ -32,9 +33,41 @@ __global__ void __launch_bounds__(PROBE_THREADS) k_probe_fma(int64_t iters, T m,
   if (s == T(-12345.678)) g_probe_sink = double(s);
 }
 
+template <typename F>
+__global__ void __launch_bounds__(PROBE_THREADS) k_probe_math(int64_t n, double *x, F f) {
+  const int64_t i = (int64_t)blockIdx.x * PROBE_THREADS + threadIdx.x;
+  if (i < n) x[i] = f(x[i]);
+}
+struct ProbeRecip {
+  __device__ double operator()(double x) const { return recip(x); }
+};
+struct ProbeRoot {
+  __device__ double operator()(double x) const { return root(x); }
+};
+
 }  // namespace dg
 
 using namespace dg;
+
+extern "C" int32_t dg_probe_math(int32_t kind, int64_t n, const double *x, double *y, void *cuda_stream) {
+  if (!x || !y || n <= 0 || n > (int64_t(1) << 30) || kind < 0 || kind > DG_MATH_ROOT)
+    return set_error(DG_EINVAL, "bad argument");
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  double *d = nullptr;
+  cudaError_t e = cudaMalloc(&d, sizeof(double) * n);
+  if (e != cudaSuccess) return set_error(DG_ENOMEM, cudaGetErrorString(e));
+  e = cudaMemcpyAsync(d, x, sizeof(double) * n, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) {
+    const unsigned grid = (unsigned)((n + PROBE_THREADS - 1) / PROBE_THREADS);
+    if (kind == DG_MATH_RECIP) k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeRecip{});
+    else k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeRoot{});
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(y, d, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFree(d);
+  return e == cudaSuccess ? DG_OK : set_error(DG_ECUDA, cudaGetErrorString(e));
+}
 
 extern "C" int32_t dg_probe_fma_peak(int32_t precision, double *tflops, double *ms, void *cuda_stream) {
   if (!tflops || (precision != DG_PREC_FP64 && precision != DG_PREC_MIXED))

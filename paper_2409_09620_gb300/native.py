@@ -84,6 +84,7 @@ SIGNATURES = {
     "dg_op_alpha": (i32, [P, P, dbl, C.POINTER(dbl)]),
     "dg_profile_steps": (i32, [P, i64, P, P]),
     "dg_probe_fma_peak": (i32, [i32, C.POINTER(dbl), C.POINTER(dbl), P]),
+    "dg_probe_math": (i32, [i32, i64, P, P, P]),
     "dg_stats_noalloc": (i32, [P, i32, P, P, P]),
     "dg_batch_create": (i32, [i32, P, P, P, P, C.POINTER(P)]),
     "dg_batch_destroy": (None, [P]),
@@ -156,6 +157,17 @@ def probe_fma_peak(precision=PREC_FP64, stream=None):
     tf, ms = dbl(), dbl()
     _check(lib().dg_probe_fma_peak(precision, C.byref(tf), C.byref(ms), None if stream is None else P(stream)))
     return tf.value, ms.value
+
+
+MATH_RECIP, MATH_ROOT = 0, 1
+
+
+def probe_math(kind, x):
+    """The kernels' own arithmetic functions on an array (for tests)."""
+    x = np.ascontiguousarray(x, np.float64)
+    y = np.empty_like(x)
+    _check(lib().dg_probe_math(kind, x.size, _p(x), _p(y), None))
+    return y
 
 
 def config_for(workload, **kw):
