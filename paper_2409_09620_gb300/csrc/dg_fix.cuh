@@ -25,9 +25,9 @@
 // the terms have a block of their own: derivatives, which do not contain the
 // cell average (dg_fix_vertex.cuh, dg_fix_scalar.cuh; tests/test_fix_vertex_host.py and
 // tests/test_fix_scalar_host.py compare them with the chain).  Zeros stay zero,
-// subnormals count as zero and blocks below 2^-959 keep an absolute 2^-1016; a
-// block that holds an infinity or a NaN has E = 0x7ff, and the callers turn its
-// results into NaN.
+// subnormals count as zero and blocks below 2^-959 keep an absolute 2^-1016;
+// a result beyond FP64's range is infinite; a block that holds an infinity or a
+// NaN has E = 0x7ff, and the callers turn its results into NaN.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -188,18 +188,29 @@ FX_HD void fx_mac(FxAccL &s, Fx c, Fx x) {
   fx_mad(s.l, c.l, x.l);
 }
 FX_HD int64_t fx_round(const FxAccL &s) { return fx_round(FxAcc{s.a, s.b + (s.l >> FX_LIMB)}); }
-// r 2^(E - 1080) rounded to nearest; |r| < 2^63
-FX_HD double fx_to(int64_t r, int E) {
+// r 2^(E - 1080) rounded to nearest, |r| < 2^63.  fx_near where neither end of FP64's range
+// is near (every block but those of extreme values); fx_to for any E: it scales the
+// integer's own FP64 value by two powers of two, which is exact but for the overflow or
+// underflow
+constexpr int FX_NEAR_MIN = 58, FX_NEAR_MAX = 2040;
+FX_HD double fx_near(int64_t r, int E) {
   const int64_t g = r >> 63;
   const uint64_t a = (uint64_t)(r ^ g) - (uint64_t)g;   // |r|
   const int e8 = fx_log2_127(a);
   const uint64_t m = a << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62
   const uint64_t q = (m + 512u) >> 10;
-  int f = E + e8 - 185;                // exponent field, less the one that q carries
-  f = f < 0 ? 0 : (f > 2046 ? 2046 : f);
-  f = e8 == 0 ? 0 : f;
-  const int hi = ((int)(q >> 32) + (f << 20)) | ((int)(g >> 32) & (int)0x80000000);
-  return fx_make(hi, (unsigned)q);
+  const int f = e8 == 0 ? 0 : E + e8 - 185;   // exponent field, less the one that q carries
+  return fx_make(((int)(q >> 32) + (f << 20)) | ((int)(g >> 32) & (int)0x80000000), (unsigned)q);
+}
+FX_HD double fx_pow2(int e) { return fx_make((e + 1023) << 20, 0u); }
+FX_HD double fx_to(int64_t r, int E) {
+  const bool far = (unsigned)(E - FX_NEAR_MIN) > (unsigned)(FX_NEAR_MAX - FX_NEAR_MIN);
+  double x = fx_near(r, far ? 1080 : E);
+  if (far) {
+    const int e = E < -960 ? -2040 : E > 3120 ? 2040 : E - 1080;
+    x = x * fx_pow2(e / 2) * fx_pow2(e - e / 2);
+  }
+  return x;
 }
 // r1 2^(E1 - 1080) + r2 2^(E2 - 1080) as r 2^(E - 1080)
 FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
@@ -249,10 +260,14 @@ FX_HD int fx_block(const double x[N], Fx f[N]) {
   for (int j = 0; j < N; ++j) f[j] = fx_from(x[j], E);
   return E;
 }
-// fx_to, NaN for a block that holds a non-finite value
+// The same for many results of one block: fx_near(r, fx_safe(E)), and then, only if
+// E > FX_NEAR_MAX, fx_far of each: what the scaling is short of, NaN for a block that
+// holds a non-finite value
+FX_HD int fx_safe(int E) { return E > FX_NEAR_MAX ? 1080 : E; }
+FX_HD double fx_far(double x, int E) { return E >= FX_ENAN ? NAN : x * fx_pow2(480) * fx_pow2(E - 1560); }
 FX_HD double fx_out(int64_t r, int E) {
-  const double x = fx_to(r, E);
-  return E >= FX_ENAN ? NAN : x;
+  const double x = fx_near(r, fx_safe(E));
+  return E > FX_NEAR_MAX ? fx_far(x, E) : x;
 }
 
 }  // namespace dg
