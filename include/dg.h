@@ -188,10 +188,13 @@ int32_t dg_profile_steps(dg_solver *solver, int64_t n, double *ms, int64_t *laun
  * DG_ECUDA. */
 int32_t dg_probe_fma_peak(int32_t precision, double *tflops, double *ms, void *cuda_stream);
 /* y[i] = f(x[i]) on the current device with the kernels' own arithmetic (host arrays
- * of n doubles, n <= 2^30), for tests: 1 / x, or sqrt(x) for x >= 0 or NaN.
+ * of n doubles, n <= 2^30), for tests: 1 / x; sqrt(x) for x >= 0 or NaN; x rounded
+ * to FP32 on the integer units; x, cast to FP32, taken back to FP64 on them.
  * Errors: DG_EINVAL, DG_ENOMEM, DG_ECUDA. */
 #define DG_MATH_RECIP 0
 #define DG_MATH_ROOT 1
+#define DG_MATH_F32 2
+#define DG_MATH_F64 3
 int32_t dg_probe_math(int32_t kind, int64_t n, const double *x, double *y, void *cuda_stream);
 /* the solver's CUDA stream (cudaStream_t) */
 void *dg_stream(const dg_solver *solver);

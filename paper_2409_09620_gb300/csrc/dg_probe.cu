@@ -44,13 +44,19 @@ struct ProbeRecip {
 struct ProbeRoot {
   __device__ double operator()(double x) const { return root(x); }
 };
+struct ProbeF32 {
+  __device__ double operator()(double x) const { return f32_of(x); }
+};
+struct ProbeF64 {
+  __device__ double operator()(double x) const { return f64_of(float(x)); }
+};
 
 }  // namespace dg
 
 using namespace dg;
 
 extern "C" int32_t dg_probe_math(int32_t kind, int64_t n, const double *x, double *y, void *cuda_stream) {
-  if (!x || !y || n <= 0 || n > (int64_t(1) << 30) || kind < 0 || kind > DG_MATH_ROOT)
+  if (!x || !y || n <= 0 || n > (int64_t(1) << 30) || kind < 0 || kind > DG_MATH_F64)
     return set_error(DG_EINVAL, "bad argument");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   double *d = nullptr;
@@ -60,7 +66,9 @@ extern "C" int32_t dg_probe_math(int32_t kind, int64_t n, const double *x, doubl
   if (e == cudaSuccess) {
     const unsigned grid = (unsigned)((n + PROBE_THREADS - 1) / PROBE_THREADS);
     if (kind == DG_MATH_RECIP) k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeRecip{});
-    else k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeRoot{});
+    else if (kind == DG_MATH_ROOT) k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeRoot{});
+    else if (kind == DG_MATH_F32) k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeF32{});
+    else k_probe_math<<<grid, PROBE_THREADS, 0, s>>>(n, d, ProbeF64{});
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(y, d, sizeof(double) * n, cudaMemcpyDeviceToHost, s);

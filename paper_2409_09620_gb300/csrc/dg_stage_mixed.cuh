@@ -145,26 +145,6 @@ __device__ __forceinline__ void hessian_p2(const float hi[4][6], float jx, float
   }
 }
 
-// FP64 to FP32 and back on the integer units (a conversion instruction takes 64
-// cycles of the FP64 pipe, which the flux pass keeps half busy).  f32_of rounds to
-// nearest, ties away from zero; magnitudes below 2^-126 become 0, those above
-// the FP32 range and NaN infinity.  In the flux pass, 24 conversions per cell,
-// 1,036,800 cells: 0.173 -> 0.157 ms (P2), 0.146 -> 0.135 ms (P1); in the OE pass,
-// bound by latency and registers, slower (0.237 -> 0.254 ms), so it converts as is.
-__device__ __forceinline__ float f32_of(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned long long r = (((unsigned long long)(hi & 0x7fffffffu) << 32) | lo) + 0x10000000ull - 0x3800000000000000ull;
-  const int t = min(max((int)(r >> 32), 0), 0x0ff00000);
-  const unsigned b = __funnelshift_l((unsigned)r, (unsigned)t, 3);
-  return __uint_as_float((t == 0x0ff00000 ? 0x7f800000u : (t == 0 ? 0u : b)) | (hi & 0x80000000u));
-}
-// a finite FP32 value, exact (subnormals as if normal: below 2^-125)
-__device__ __forceinline__ double f64_of(float x) {
-  const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
-  const unsigned e = a >= 0x7f800000u ? 0x7ff00000u : (a == 0u ? 0u : (a >> 3) + 0x38000000u);
-  return __hiloint2double((int)(e | (b & 0x80000000u)), (int)(b << 29));
-}
-
 // a cell's modal state: FP64 averages (and their FP32 roundings) and FP32 modes
 template <int K, bool INT = false>
 __device__ __forceinline__ void load_mixed(const StateDev<float> &s, int64_t nt, int64_t K_, double a[4],

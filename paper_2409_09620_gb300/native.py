@@ -159,7 +159,7 @@ def probe_fma_peak(precision=PREC_FP64, stream=None):
     return tf.value, ms.value
 
 
-MATH_RECIP, MATH_ROOT = 0, 1
+MATH_RECIP, MATH_ROOT, MATH_F32, MATH_F64 = 0, 1, 2, 3
 
 
 def probe_math(kind, x):
