@@ -49,18 +49,10 @@ struct Payload {
   dg_solver *solver = nullptr;
 };
 
-// device bytes of one solve: mesh geometry and connectivity + solver buffers
-size_t solve_bytes(int64_t nt, int k, int prec) {
-  const size_t rs = prec == DG_PREC_MIXED ? 4 : 8;
-  const size_t nb = k == 1 ? 3 : 6, nq = k == 1 ? 2 : 3;
-  const size_t mesh = 45 * 8 + 23 * 4 + 2 + 12 + 4 * 3 + 4 * 2;   // geometry (FP64 + FP32 copies), connectivity, edges
-  const size_t state = 3 * (4 * 8 + rs * 4 * (nb - 1));
-  // traces, vertex records, Hessians, ~1.5 edge records counted as 2 (FP64 form only; the
-  // difference covers the exponents of the vertex records and that form's partials per 32 cells)
-  const size_t exch = uses_exchange(prec) ? rs * (3 * nq * TR_STRIDE + 48 + 12 + 2 * 16) : 0;
-  const size_t part = 10 * 8 + 16;   // per 128-cell block, rounded up per cell below
-  return (size_t)nt * (mesh + state + exch) + ((size_t)nt / 128 + 1) * part + 4096;
-}
+static_assert(SOLVE_TRACE == TR_STRIDE && SOLVE_VERTEX == VD_CELL && SOLVE_EDGE == EJ_STRIDE &&
+                  SOLVE_TILE_FP64 == tile_cells(DG_PREC_FP64) && SOLVE_TILE_MIXED == tile_cells(DG_PREC_MIXED) &&
+                  SOLVE_GROUP == TILE_GROUP,
+              "the charge of a solve counts the buffers of dg_mesh_create and dg_init");
 
 void free_payload_device(Payload &p) {
   if (p.solver) dg_solver_destroy(p.solver);
@@ -192,7 +184,8 @@ extern "C" int32_t dg_server_submit(dg_server *s, int64_t nv, const double *xy, 
   const int nb = cfg->k == 1 ? 3 : 6;
   p.coeffs.assign(coeffs, coeffs + 4 * nb * nt);
   p.t_end = t_end;
-  *id = s->sched.submit(nt, solve_bytes(nt, cfg->k, s->prec), t_end, s->now());
+  const int64_t tagged = bc ? 3 * nt - std::count(bc, bc + 3 * nt, (int8_t)DG_BC_NONE) : 0;
+  *id = s->sched.submit(nt, solve_bytes(nt, tagged, cfg->k, s->prec), t_end, s->now());
   s->eng.pay.emplace(*id, std::move(p));
   return DG_OK;
 }

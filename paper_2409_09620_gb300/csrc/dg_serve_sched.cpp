@@ -5,6 +5,22 @@
 
 namespace dg {
 
+size_t solve_bytes(int64_t nt, int64_t tagged, int k, int precision) {
+  const bool fp64 = precision == DG_PREC_FP64;
+  const int64_t rs = fp64 ? 8 : 4, nm = k == 1 ? 2 : 5, nq = k + 1;
+  const int64_t ne = (3 * nt + (tagged < nt ? tagged : nt) + 1) / 2;
+  const int64_t tiles = (nt + SOLVE_TILE_FP64 - 1) / SOLVE_TILE_FP64;   // of the mesh's edge ranges
+  // geometry in FP64 (45 values) and FP32 (23), limiter vertices, connectivity, edges of the cells; edges
+  const int64_t mesh = nt * (45 * 8 + 23 * 4 + 2 + 12 + 12) + ne * 5 + (tiles + 1) * 4;
+  const int64_t state = nt * 3 * (4 * 8 + rs * 4 * nm);
+  const int64_t exchange = fp64 ? 8 * (nt * (3 * nq * SOLVE_TRACE + SOLVE_VERTEX + 12) + ne * SOLVE_EDGE) : 0;
+  const int64_t parts = fp64 ? tiles : (nt + SOLVE_TILE_MIXED - 1) / SOLVE_TILE_MIXED;
+  const int64_t groups = (parts + SOLVE_GROUP - 1) / SOLVE_GROUP;
+  // sums (4), deviations (5), wave speed, two counters; a ticket per group of three reductions
+  const int64_t part = (parts + groups) * (10 * 8 + 16) + 3 * (groups + 1) * 4;
+  return (size_t)(mesh + state + exchange + part + 4096);
+}
+
 int64_t ServeScheduler::submit(int64_t cells, size_t bytes, double t_end, double now) {
   SchedRequest r;
   r.id = next_id_++;

@@ -12,6 +12,15 @@
 
 namespace dg {
 
+// Device bytes of one solve, charged against the budget: the buffers of dg_mesh_create and
+// dg_init.  `tagged` is the number of edges with a boundary tag: an edge is counted once,
+// (3 nt + boundary edges) / 2 in all, 1.5 per cell of a large mesh and 2 of a strip one cell
+// wide.  Tags on interior edges are ignored by the mesh, so no more than 2 per cell are
+// charged; the fixed 4 KB cover the few more of a mesh of up to 30 cells.
+constexpr int64_t SOLVE_TRACE = 8, SOLVE_VERTEX = 52, SOLVE_EDGE = 16;   // FP64 values per trace point, cell and edge
+constexpr int64_t SOLVE_TILE_FP64 = 32, SOLVE_TILE_MIXED = 128, SOLVE_GROUP = 128;   // cells per partial; partials per group
+size_t solve_bytes(int64_t nt, int64_t tagged, int k, int precision);
+
 // The device side of the server.  Every call returns DG_OK or an error code.
 struct ServeEngine {
   virtual ~ServeEngine() = default;
