@@ -266,10 +266,11 @@ int32_t dg_batch_sync(dg_batch *batch);
 /* the solver handle of solve i (owned by the batch): dg_get_state /
  * dg_set_state work on it; do not destroy it or advance it on its own */
 int32_t dg_batch_solver(dg_batch *batch, int32_t i, dg_solver **out);
-/* launch shape: cells per work chunk (a positive multiple of 128), resident
- * blocks per SM of each launch's grid (clamped per kernel to its occupancy
- * limit) and the launch form (3, 1 or 0, as for dg_batch_create; the chunk
- * and blocks-per-SM values do not apply to form 0).  DG_EINVAL for another
+/* launch shape: cells per work chunk (a positive multiple of 128; in FP64, four
+ * lanes per cell, a chunk is dealt to four blocks), resident blocks per SM of
+ * each launch's grid (clamped per kernel to its occupancy limit) and the launch
+ * form (3, 1 or 0, as for dg_batch_create; the chunk and blocks-per-SM values
+ * do not apply to form 0).  DG_EINVAL for another
  * form, or form 1 on a device without cooperative launch; DG_ECUDA when form
  * 0's graph cannot be built.  *grid receives the largest grid of the form's
  * launches. */

@@ -108,7 +108,7 @@ __device__ __forceinline__ bool grid_sync(BarrierState *b, unsigned nblocks) {
 }
 
 // The three phases of a stage over the work list, blocks [first, first +
-// stride, ...).  Each tile finalises its reductions through the tickets, so
+// stride, ...).  Each chunk finalises its reductions through the tickets, so
 // the phases need only be ordered, by a grid barrier or a kernel boundary.
 template <typename Real>
 __device__ __forceinline__ void phase_rk(const SolveDev *__restrict__ sv, const WorkItem *__restrict__ work,
@@ -123,13 +123,13 @@ __device__ __forceinline__ void phase_rk(const SolveDev *__restrict__ sv, const 
     const StateDev<Real> v{S.avg[vi], (Real *)S.hi[vi]}, un{S.avg[0], (Real *)S.hi[0]}, uh{S.avg[1], (Real *)S.hi[1]};
     for (int64_t t = it.first_tile; t < it.first_tile + it.ntiles; ++t) {
       if (S.k == 1)
-        rk_tile<1, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
+        rk_tile<1, Real, FP64_TILE_BYTES>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
                          PlainScalars{S.sc}, a, b, c_in, t);
       else
-        rk_tile<2, Real>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
+        rk_tile<2, Real, FP64_TILE_BYTES>(S.mesh, S.ph, v, un, uh, (const Real *)S.tr, (Real *)S.vd, (Real *)S.hs, S.part_sum,
                          PlainScalars{S.sc}, a, b, c_in, t);
-      finish_means(S.part_sum, S.fin, t, S.ntiles, S.sc);
     }
+    finish_means(S.part_sum, S.fin, it.first_tile, it.ntiles, S.ntiles, S.sc);
   }
 }
 
@@ -153,8 +153,8 @@ __device__ __forceinline__ void phase_stats(const SolveDev *__restrict__ sv, con
         edge_tile<2, Real>(S.mesh, S.ph, uh.avg, (const Real *)S.vd, (const Real *)S.hs, (Real *)S.ej, S.sc, c_out,
                            t);
       }
-      finish_deviations(S.part_dev, S.fin, t, S.ntiles, S.sc, S.oe == 2);
     }
+    finish_deviations(S.part_dev, S.fin, it.first_tile, it.ntiles, S.ntiles, S.sc, S.oe == 2);
   }
 }
 
@@ -171,22 +171,24 @@ __device__ __forceinline__ void phase_oe_bp(const SolveDev *__restrict__ sv, con
     const StateDev<Real> uh{S.avg[1], (Real *)S.hi[1]}, out{S.avg[oi], (Real *)S.hi[oi]};
     for (int64_t t = it.first_tile; t < it.first_tile + it.ntiles; ++t) {
       if (S.k == 1)
-        oe_bp_tile<1, Real>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
+        oe_bp_tile<1, Real, FP64_TILE_BYTES>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
                             PlainScalars{S.sc}, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
       else
-        oe_bp_tile<2, Real>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
+        oe_bp_tile<2, Real, FP64_TILE_BYTES>(S.mesh, S.ph, uh, out, (const Real *)S.ej, (Real *)S.tr, S.part_alpha, S.part_cnt,
                             PlainScalars{S.sc}, S.oe != 0, S.bp != 0, c_out, stage == 2, t);
-      finish_alpha(S.part_alpha, S.part_cnt, S.fin, t, S.ntiles, S.sc, stage);
     }
+    finish_alpha(S.part_alpha, S.part_cnt, S.fin, it.first_tile, it.ntiles, S.ntiles, S.sc, stage);
   }
 }
 
 // Fused form: one cooperative launch per stage runs the three phases with
-// grid barriers between them (and the step start before stage 0).
+// grid barriers between them (and the step start before stage 0).  FP64: four
+// blocks per SM; us per step of 16 solves of 2k-200k cells (256 cells per chunk) with 2
+// (all the registers it wants) / 3 / 4 / 5 blocks: 11,030 / 8,940 / 7,910 / 8,290.
 template <typename Real>
-__global__ void __launch_bounds__(TPB) k_batch_stage(const SolveDev *__restrict__ sv, int nsv,
-                                                     const WorkItem *__restrict__ work, int nwork,
-                                                     BarrierState *bar, int stage) {
+__global__ void __launch_bounds__(TPB, sizeof(Real) == 8 ? 4 : 1)
+    k_batch_stage(const SolveDev *__restrict__ sv, int nsv, const WorkItem *__restrict__ work, int nwork,
+                  BarrierState *bar, int stage) {
   const unsigned nb = gridDim.x;
   if (stage == 0) {
     if (threadIdx.x == 0)
@@ -389,14 +391,16 @@ struct BatchCore {
     return rc;
   }
 
-  // work list of chunks of cpb cells (a multiple of TPB), then the step graph
+  // work list of chunks of cpb cells (a multiple of TPB), then the step graph; in the FP64
+  // form, four lanes per cell, a chunk goes to four blocks: a block has as many threads' work
+  // as in the mixed form
   int32_t set_shape(int cells_per_block, int bpsm, int launch_form) {
     if (launch_form != 0 && launch_form != 1 && launch_form != 3)
       return set_error(DG_EINVAL, "launch form must be 0, 1 or 3");
     if (max_blocks_per_sm(launch_form) < 1)
       return set_error(DG_EINVAL, "the device does not support cooperative launches");
     std::vector<WorkItem> work;
-    const int64_t tpw = cells_per_block / tile_cells(prec);
+    const int64_t tpw = cells_per_block / TPB;   // tiles
     for (size_t i = 0; i < host_sv.size(); ++i)
       for (int64_t t = 0; t < host_sv[i].ntiles; t += tpw)
         work.push_back(WorkItem{(int)i, 0, t, std::min<int64_t>(tpw, host_sv[i].ntiles - t)});

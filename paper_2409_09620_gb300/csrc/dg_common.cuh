@@ -537,9 +537,9 @@ __device__ __forceinline__ void write_inv_normalisers(Scalars *sc, int cw) {
 // ------------------------------------------------------------------------
 // Finalisation inside the producing kernel, in a fixed order
 // ------------------------------------------------------------------------
-// The tiles of a reduction (TPB cells each, one partial per tile) form groups
-// of TILE_GROUP consecutive tiles.  After writing its partial, a block takes a
-// ticket for its group; the block that takes the group's last ticket reduces
+// The tiles of a reduction (TileCells cells each, one partial per tile) form groups
+// of TILE_GROUP consecutive tiles.  After writing the partials of its tiles, a block takes
+// their tickets of the group; the block that takes the group's last ticket reduces
 // the group's partials with block_reduce and takes a ticket at the top level;
 // the block that takes the last top-level ticket reduces the group results in
 // chunks of TPB, in order, and writes the scalars.  The arithmetic depends only
@@ -555,18 +555,18 @@ __host__ __device__ __forceinline__ int64_t num_groups(int64_t ntiles) {
 __host__ __device__ __forceinline__ int64_t ticket_slots(int64_t ntiles) { return num_groups(ntiles) + 1; }
 
 // Called by every thread of the block once the block's results are written:
-// true in the block that took the last of `total` tickets of *cnt.
+// takes n tickets of *cnt, true in the block that took the last of `total`.
 // The block's writes are ordered before the ticket by the barrier and one
 // device-scope fence of thread 0 (cumulative over what the barrier ordered);
 // the last block fences again before its threads read the other blocks'
 // results.
-__device__ __forceinline__ bool take_ticket(unsigned *cnt, unsigned total) {
+__device__ __forceinline__ bool take_ticket(unsigned *cnt, unsigned total, unsigned n = 1) {
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned t = atomicAdd(cnt, 1u);
-    const int last = t + 1 == total;
+    const unsigned t = atomicAdd(cnt, n);
+    const int last = t + n == total;
     if (last) {
       atomicExch(cnt, 0u);               // every ticket is taken: reset for the next launch
       __threadfence();
@@ -666,33 +666,42 @@ __device__ __forceinline__ void finish_alpha_top(const FinBufs &f, int64_t ntile
 }
 
 // Group level.  In the per-solve finalize kernels block g reduces group g
-// directly; in the batch kernel the block that finishes a group's last tile
-// does (after a group ticket), so both produce the same group results.
-__device__ __forceinline__ bool group_ticket(const FinBufs &f, int kind, int64_t tile, int64_t ntiles) {
-  const int64_t g = tile / TILE_GROUP;
-  return take_ticket(f.tick + kind * ticket_slots(ntiles) + g,
-                     (unsigned)min((int64_t)TILE_GROUP, ntiles - g * TILE_GROUP));
+// directly; in the batch kernel the block that finishes a group's last tiles
+// does (after the group's tickets), so both produce the same group results.
+// A block takes the tickets of a whole chunk of tiles at once: one fence and three barriers
+// per chunk, not per tile.  fn(g) for every group that the n tiles from `first` complete.
+template <typename F>
+__device__ __forceinline__ void complete_groups(const FinBufs &f, int kind, int64_t first, int64_t n, int64_t ntiles,
+                                                F fn) {
+  for (int64_t g = first / TILE_GROUP; g * TILE_GROUP < first + n; ++g) {
+    const int64_t t0 = g * TILE_GROUP, t1 = min(t0 + TILE_GROUP, ntiles);
+    const int64_t mine = min(t1, first + n) - max(t0, first);
+    if (take_ticket(f.tick + kind * ticket_slots(ntiles) + g, (unsigned)(t1 - t0), (unsigned)mine)) fn(g);
+  }
 }
 
-// in-kernel finalisation after tile `tile` wrote its partials (batch kernel)
-__device__ __forceinline__ void finish_means(const double *part_sum, const FinBufs &f, int64_t tile, int64_t ntiles,
-                                             Scalars *sc) {
-  if (!group_ticket(f, 0, tile, ntiles)) return;
-  reduce_group<4>(part_sum, tile / TILE_GROUP, ntiles, f.grp_sum, OpSum());
-  finish_means_top(f, ntiles, sc);
+// in-kernel finalisation after the n tiles from `first` wrote their partials (batch kernel)
+__device__ __forceinline__ void finish_means(const double *part_sum, const FinBufs &f, int64_t first, int64_t n,
+                                             int64_t ntiles, Scalars *sc) {
+  complete_groups(f, 0, first, n, ntiles, [&](int64_t g) {
+    reduce_group<4>(part_sum, g, ntiles, f.grp_sum, OpSum());
+    finish_means_top(f, ntiles, sc);
+  });
 }
-__device__ __forceinline__ void finish_deviations(const double *part_dev, const FinBufs &f, int64_t tile,
+__device__ __forceinline__ void finish_deviations(const double *part_dev, const FinBufs &f, int64_t first, int64_t n,
                                                   int64_t ntiles, Scalars *sc, int cw) {
-  if (!group_ticket(f, 1, tile, ntiles)) return;
-  reduce_group<5>(part_dev, tile / TILE_GROUP, ntiles, f.grp_dev, OpMaxNN());
-  finish_deviations_top(f, ntiles, sc, cw);
+  complete_groups(f, 1, first, n, ntiles, [&](int64_t g) {
+    reduce_group<5>(part_dev, g, ntiles, f.grp_dev, OpMaxNN());
+    finish_deviations_top(f, ntiles, sc, cw);
+  });
 }
 __device__ __forceinline__ void finish_alpha(const double *part_alpha, const long long *part_cnt, const FinBufs &f,
-                                             int64_t tile, int64_t ntiles, Scalars *sc, int stage) {
-  if (!group_ticket(f, 2, tile, ntiles)) return;
-  reduce_group<1>(part_alpha, tile / TILE_GROUP, ntiles, f.grp_alpha, OpMaxNN());
-  reduce_group<2>(part_cnt, tile / TILE_GROUP, ntiles, f.grp_cnt, OpSum());
-  finish_alpha_top(f, ntiles, sc, stage);
+                                             int64_t first, int64_t n, int64_t ntiles, Scalars *sc, int stage) {
+  complete_groups(f, 2, first, n, ntiles, [&](int64_t g) {
+    reduce_group<1>(part_alpha, g, ntiles, f.grp_alpha, OpMaxNN());
+    reduce_group<2>(part_cnt, g, ntiles, f.grp_cnt, OpSum());
+    finish_alpha_top(f, ntiles, sc, stage);
+  });
 }
 
 // dt of the BP CFL condition (Sec. 5), clamped to t_end; inactive once t >= t_end

@@ -165,13 +165,14 @@ namespace dg {
 // ==========================================================================
 // The tile functions of both precisions, and the kernels of one solve
 // ==========================================================================
-template <int K, typename Real, typename Sc>
+// BYTES: the FP64 form's shared memory (dg_stage_fp64.cuh)
+template <int K, typename Real, int BYTES = sizeof(RkShared<K>), typename Sc>
 __device__ __forceinline__ void rk_tile(const MeshDev &m, const Phys &ph, StateDev<Real> v, StateDev<Real> un,
                                         StateDev<Real> uh, const Real *__restrict__ tr, Real *__restrict__ vdo,
                                         Real *__restrict__ hso, double *part_sum, Sc get, double a,
                                         double b, double c_in, int64_t tile) {
   if constexpr (sizeof(Real) == sizeof(float)) rk_tile_mixed<K>(m, ph, v, un, uh, part_sum, get, a, b, c_in, tile);
-  else rk_tile_fp64<K>(m, ph, v, un, uh, tr, vdo, hso, part_sum, get, a, b, c_in, tile);
+  else rk_tile_fp64<K, BYTES>(m, ph, v, un, uh, tr, vdo, hso, part_sum, get, a, b, c_in, tile);
 }
 template <int K, typename Real, typename Sc>
 __device__ __forceinline__ void stats_tile(const MeshDev &m, StateDev<Real> uh, double *part_dev, Sc get,
@@ -186,7 +187,7 @@ __device__ __forceinline__ void edge_tile(const MeshDev &m, const Phys &ph, cons
                                           Real *__restrict__ ej, const Scalars *sc, double c_out, int64_t tile) {
   if constexpr (sizeof(Real) == sizeof(double)) edge_tile_fp64<K>(m, ph, avg, vdi, hsi, ej, sc, c_out, tile);
 }
-template <int K, typename Real, typename Sc>
+template <int K, typename Real, int BYTES = sizeof(OeShared<K>), typename Sc>
 __device__ __forceinline__ void oe_bp_tile(const MeshDev &m, const Phys &ph, StateDev<Real> uh, StateDev<Real> out,
                                            const Real *__restrict__ ej, Real *__restrict__ tr, double *part_alpha,
                                            long long *part_cnt, Sc get, int do_oe, int do_bp,
@@ -194,7 +195,7 @@ __device__ __forceinline__ void oe_bp_tile(const MeshDev &m, const Phys &ph, Sta
   if constexpr (sizeof(Real) == sizeof(float))
     oe_bp_tile_mixed<K>(m, ph, uh, out, part_alpha, part_cnt, get, do_oe, do_bp, c_out, end_of_step, tile);
   else
-    oe_bp_tile_fp64<K>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, get, do_oe, do_bp, c_out, end_of_step, tile);
+    oe_bp_tile_fp64<K, BYTES>(m, ph, uh, out, ej, tr, part_alpha, part_cnt, get, do_oe, do_bp, c_out, end_of_step, tile);
 }
 
 template <int K, typename Real, bool FUSED>

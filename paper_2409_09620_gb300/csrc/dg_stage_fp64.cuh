@@ -46,6 +46,27 @@ struct __align__(16) Vec4d {
   double c[4];
 };
 
+// Shared memory of the tile functions.  A kernel that holds several of them (both degrees,
+// or both phases, in the batch kernels) gives all the same BYTES and so one buffer, which
+// every function leaves free with a barrier.
+template <int K>
+struct RkShared {
+  Vec4d u[Deg<K>::NV][FT], g[Deg<K>::NV][FT];
+  int64_t y[3 * Deg<K>::NQ][TPB];
+  double cell[4][FT], jac[4][FT], m[TPB];
+};
+template <int K>
+struct OeShared {
+  Vec4d u[3 * Deg<K>::NQ + 2][FT], a[FT];
+};
+constexpr int FP64_TILE_BYTES = sizeof(RkShared<2>);   // the largest of them
+static_assert(sizeof(OeShared<2>) <= FP64_TILE_BYTES && sizeof(RkShared<1>) <= FP64_TILE_BYTES, "one buffer");
+template <int BYTES>
+__device__ __forceinline__ unsigned char *tile_shared() {
+  __shared__ __align__(16) unsigned char buf[BYTES];
+  return buf;
+}
+
 // one component's average and modes
 template <int NB>
 __device__ __forceinline__ void load_comp(const StateDev<double> &s, int64_t nt, int64_t K, int c, double x[NB]) {
@@ -77,15 +98,16 @@ __device__ __forceinline__ double pick4(const double v[4], int c) {
 // K1: u_h = a u_n + b (v + dt L(v))
 // ==========================================================================
 // one tile; block partial -> part_sum[4 * tile]
-template <int K, typename Sc>
+template <int K, int BYTES, typename Sc>
 __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> v, StateDev<double> un,
                                              StateDev<double> uh, const double *__restrict__ tr,
                                              double *__restrict__ vdo, double *__restrict__ hso, double *part_sum,
                                              Sc get, double a, double b, double c_in, int64_t tile) {
   constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ, NV = Deg<K>::NV;
-  __shared__ Vec4d s_u[NV][FT], s_g[NV][FT];
-  __shared__ double s_cell[4][FT];   // dt / |K|, then alpha l_i
-  __shared__ double s_jac[4][FT];    // |K| times the inverse Jacobian
+  RkShared<K> &sh = *reinterpret_cast<RkShared<K> *>(tile_shared<BYTES>());
+  auto &s_u = sh.u, &s_g = sh.g;
+  auto &s_cell = sh.cell;   // dt / |K|, then alpha l_i
+  auto &s_jac = sh.jac;     // |K| times the inverse Jacobian
   const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warp0 = (warp + (int)tile) & 3;
   const int64_t nt = m.nt, K0 = tile * FT;
@@ -138,7 +160,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   // kernel was 67 KB of straight-line code that waited for instructions more than
   // for anything else (28 % of the stalls, P2), and held 9 sums in registers.
   // 1,036,800 cells: P2 0.94 -> 0.90 ms, P1 0.457 -> 0.406 ms.
-  __shared__ int64_t s_y[3 * NQ][TPB];   // this thread's, in its own column
+  auto &s_y = sh.y;   // this thread's, in its own column
   int ei[3] = {0, 0, 0};
   bool bad = false;
 #pragma unroll 1
@@ -267,7 +289,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 #pragma unroll
     for (int l = 1; l < NB; ++l) uh.hi[(c * (NB - 1) + (l - 1)) * nt + Kc] = h[l];
   }
-  __shared__ double s_m[TPB];
+  auto &s_m = sh.m;
   s_m[threadIdx.x] = live ? mul(m.area[Kc], h[0]) : 0.0;   // summed after the barrier below
 
   // ---- vertex values and derivatives of u_h for the OE jumps --------------------
@@ -605,7 +627,7 @@ __device__ __forceinline__ float abs_f32_down(double x) {
   return __int_as_float(min(max(t, 0), 0x0ff00000) << 3);
 }
 
-template <int K, typename Sc>
+template <int K, int BYTES, typename Sc>
 __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph, StateDev<double> uh,
                                                 StateDev<double> out, const double *__restrict__ ej,
                                                 double *__restrict__ tr, double *part_alpha, long long *part_cnt,
@@ -613,7 +635,9 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
                                                 int64_t tile) {
   constexpr int NB = Deg<K>::NB, NQ = Deg<K>::NQ;
   constexpr int NE = 3 * NQ;          // edge Gauss points
-  __shared__ Vec4d s_u[NE + 2][FT], s_a[FT];
+  OeShared<K> &sh = *reinterpret_cast<OeShared<K> *>(tile_shared<BYTES>());
+  auto &s_u = sh.u;
+  auto &s_a = sh.a;
   const unsigned FULL = 0xffffffffu;
   const int c = threadIdx.x & 3, lc = threadIdx.x >> 2;
   const int lane = threadIdx.x & 31, warp0 = ((threadIdx.x >> 5) + (int)tile) & 3, q0 = lane & ~3;
