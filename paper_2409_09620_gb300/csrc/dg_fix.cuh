@@ -188,30 +188,23 @@ FX_HD void fx_mac(FxAccL &s, Fx c, Fx x) {
   fx_mad(s.l, c.l, x.l);
 }
 FX_HD int64_t fx_round(const FxAccL &s) { return fx_round(FxAcc{s.a, s.b + (s.l >> FX_LIMB)}); }
-// r 2^(E - 1080) rounded to nearest, |r| < 2^63.  fx_near where neither end of FP64's range
-// is near (every block but those of extreme values); fx_to for any E: it scales the
-// integer's own FP64 value by two powers of two, which is exact but for the overflow or
-// underflow
+// r 2^(E - 1080) rounded to nearest, |r| < 2^63 and E >= FX_NEAR_MIN, so that it is not below
+// FP64's normal numbers: fx_near for E <= FX_NEAR_MAX, fx_to infinite beyond FP64's range
 constexpr int FX_NEAR_MIN = 58, FX_NEAR_MAX = 2040;
-FX_HD double fx_near(int64_t r, int E) {
+template <bool WIDE>
+FX_HD double fx_convert(int64_t r, int E) {
   const int64_t g = r >> 63;
   const uint64_t a = (uint64_t)(r ^ g) - (uint64_t)g;   // |r|
   const int e8 = fx_log2_127(a);
   const uint64_t m = a << (189 - e8 < 63 ? 189 - e8 : 63);   // leading bit at 62
   const uint64_t q = (m + 512u) >> 10;
   const int f = e8 == 0 ? 0 : E + e8 - 185;   // exponent field, less the one that q carries
-  return fx_make(((int)(q >> 32) + (f << 20)) | ((int)(g >> 32) & (int)0x80000000), (unsigned)q);
+  const bool over = WIDE && f >= 2046;
+  const int hi = over ? 0x7ff00000 : (int)(q >> 32) + (int)((unsigned)f << 20);
+  return fx_make(hi | ((int)(g >> 32) & (int)0x80000000), over ? 0u : (unsigned)q);
 }
-FX_HD double fx_pow2(int e) { return fx_make((e + 1023) << 20, 0u); }
-FX_HD double fx_to(int64_t r, int E) {
-  const bool far = (unsigned)(E - FX_NEAR_MIN) > (unsigned)(FX_NEAR_MAX - FX_NEAR_MIN);
-  double x = fx_near(r, far ? 1080 : E);
-  if (far) {
-    const int e = E < -960 ? -2040 : E > 3120 ? 2040 : E - 1080;
-    x = x * fx_pow2(e / 2) * fx_pow2(e - e / 2);
-  }
-  return x;
-}
+FX_HD double fx_near(int64_t r, int E) { return fx_convert<false>(r, E); }
+FX_HD double fx_to(int64_t r, int E) { return fx_convert<true>(r, E); }
 // r1 2^(E1 - 1080) + r2 2^(E2 - 1080) as r 2^(E - 1080)
 FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
   E = (E1 > E2 ? E1 : E2) + 1;
@@ -260,14 +253,10 @@ FX_HD int fx_block(const double x[N], Fx f[N]) {
   for (int j = 0; j < N; ++j) f[j] = fx_from(x[j], E);
   return E;
 }
-// The same for many results of one block: fx_near(r, fx_safe(E)), and then, only if
-// E > FX_NEAR_MAX, fx_far of each: what the scaling is short of, NaN for a block that
-// holds a non-finite value
-FX_HD int fx_safe(int E) { return E > FX_NEAR_MAX ? 1080 : E; }
-FX_HD double fx_far(double x, int E) { return E >= FX_ENAN ? NAN : x * fx_pow2(480) * fx_pow2(E - 1560); }
-FX_HD double fx_out(int64_t r, int E) {
-  const double x = fx_near(r, fx_safe(E));
-  return E > FX_NEAR_MAX ? fx_far(x, E) : x;
-}
+// x, or NaN (a selection: as the arms of a conditional the compiler would branch around the
+// whole conversion)
+FX_HD double fx_nan_if(bool bad, double x) { return bad ? NAN : x; }
+// fx_to for a block's own exponent, NaN for a block that holds a non-finite value
+FX_HD double fx_out(int64_t r, int E) { return fx_nan_if(E >= FX_ENAN, fx_to(r, E)); }
 
 }  // namespace dg

@@ -108,16 +108,21 @@ FX_HD int sfx_deriv_block(const double c[SC_NB<K>], Fx f[SC_NB<K>]) {
   for (int l = SC_L0<J>; l < SC_NB<K>; ++l) f[l] = fx_from(c[l], E - 3 * (sc_degree(l) - J));
   return bad ? FX_EBAD : E;
 }
-// d^J u / dxi^r deta^(J-r) at vertex v
+// d^J u / dxi^r deta^(J-r) at vertex v, r = 0 ... J
 template <int K, int J>
-FX_HD double sfx_deriv(const Fx f[SC_NB<K>], int E, int r, int v) {
+FX_HD void sfx_derivs(const Fx f[SC_NB<K>], int E, int v, double t[J + 1]) {
   constexpr int S = sc_scale<K, J>();
-  FxAcc a{0, 0};
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
-  for (int l = SC_L0<J>; l < SC_NB<K>; ++l) fx_mac(a, fxc(sc_coef<J>(l, r, v) / double(1 << S)), f[l]);
-  return E >= FX_EBAD ? NAN : fx_to(fx_round(a), E + S);
+  for (int r = 0; r <= J; ++r) {
+    FxAcc a{0, 0};
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int l = SC_L0<J>; l < SC_NB<K>; ++l) fx_mac(a, fxc(sc_coef<J>(l, r, v) / double(1 << S)), f[l]);
+    t[r] = fx_nan_if(E >= FX_EBAD, fx_to(fx_round(a), E + S));
+  }
 }
 
 }  // namespace sc

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(TPB) k_sc_rk(MeshDev m, ScPhys ph, const doubl
       const int E = fx_block<NB>(c, f);
 #pragma unroll
       for (int mu = 0; mu < NV; ++mu) {
-        const double u = fx_out(sfx_point<K>(f, svol_xi(NV, mu), svol_eta(NV, mu)), E + SVAL<K>);
+        const double u = fx_nan_if(E >= FX_ENAN, fx_to(sfx_point<K>(f, svol_xi(NV, mu), svol_eta(NV, mu)), E + SVAL<K>));
         x[mu] = ph.flux == 0 ? u : mul(u, u);
       }
       Eg = fx_block<NV>(x, g);
@@ -227,13 +227,14 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
       const uint64_t ab = (uint64_t)(r < 0 ? -r : r);
       top = ab > top ? ab : top;
     }
-    d[0] = fx_out((int64_t)top, Ed + SVAL<K>);
+    d[0] = fx_nan_if(Ed >= FX_ENAN, fx_to((int64_t)top, Ed + SVAL<K>));
     c[0] = c0;
     double *vo = vr + Kc * 3 * NB;
     {
       const int E = fx_block<NB>(c, f);
 #pragma unroll
-      for (int vv = 0; vv < 3; ++vv) vo[vv * NB] = fx_out(sfx_point<K>(f, vert_xi(vv), vert_eta(vv)), E + SVAL<K>);
+      for (int vv = 0; vv < 3; ++vv)
+        vo[vv * NB] = fx_nan_if(E >= FX_ENAN, fx_to(sfx_point<K>(f, vert_xi(vv), vert_eta(vv)), E + SVAL<K>));
     }
     const double jx = m.jinv[Kc], jy = m.jinv[nt + Kc], ex = m.jinv[2 * nt + Kc], ey = m.jinv[3 * nt + Kc];
     // one index of a tensor with components t[r], r = number of xi: out[r] for d/dx (w = 0) or d/dy
@@ -256,8 +257,7 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
 #pragma unroll
       for (int vv = 0; vv < 3; ++vv) {
         double t[2], x, y;
-#pragma unroll
-        for (int r = 0; r <= 1; ++r) t[r] = sfx_deriv<K, 1>(f, E, r, vv);
+        sfx_derivs<K, 1>(f, E, vv, t);
         turn(1, 0, t, &x);
         turn(1, 1, t, &y);
         vo[vv * NB + didx(1, 1)] = x;
@@ -271,8 +271,7 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
       for (int vv = 0; vv < 3; ++vv) {
         if (K == 3 || vv == 0) {   // P2: constant
           double t[3], x[2], y[2];
-#pragma unroll
-          for (int r = 0; r <= 2; ++r) t[r] = sfx_deriv<K, 2>(f, E, r, vv);
+          sfx_derivs<K, 2>(f, E, vv, t);
           turn(2, 0, t, x);
           turn(2, 1, t, y);
           turn(1, 0, x, t2);
@@ -286,8 +285,7 @@ __global__ void __launch_bounds__(TPB, K == 3 ? 3 : 1) k_sc_stats(MeshDev m, con
     if constexpr (K == 3) {   // third derivatives: constant
       const int E = sfx_deriv_block<K, 3>(c, f);
       double t[4], x[3], y[3], xx[2], xy[2], yy[2], t3[4];
-#pragma unroll
-      for (int r = 0; r <= 3; ++r) t[r] = sfx_deriv<K, 3>(f, E, r, 0);
+      sfx_derivs<K, 3>(f, E, 0, t);
       turn(3, 0, t, x);
       turn(3, 1, t, y);
       turn(2, 0, x, xx);
@@ -394,7 +392,7 @@ __global__ void __launch_bounds__(TPB) k_sc_oe(MeshDev m, ScPhys ph, const doubl
 #pragma unroll
       for (int nu = 0; nu < NQ; ++nu) {
         const double s = sgauss_s(NQ, nu);
-        const double u = fx_out(sfx_point<K>(f, edge_xi(i, s), edge_eta(i, s)), E + SVAL<K>);
+        const double u = fx_nan_if(E >= FX_ENAN, fx_to(sfx_point<K>(f, edge_xi(i, s), edge_eta(i, s)), E + SVAL<K>));
         tr[(Kc * 3 + i) * NQ + nu] = u;
         um = max_nn(um, fabs(u));
       }

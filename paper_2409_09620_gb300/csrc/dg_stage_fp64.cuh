@@ -82,12 +82,6 @@ __device__ __forceinline__ int64_t fx_point(const Fx f[NB], double xi, double et
   for (int l = 0; l < NB; ++l) fx_mac(s, fxc(psi(l, xi, eta)), f[l]);
   return fx_sum(s);
 }
-// component c of cell lc at N points: the rest of the scale of a block of extreme values
-template <int N>
-__device__ __forceinline__ void far_comp(Vec4d (*s)[FT], int lc, int c, int E) {
-#pragma unroll 1
-  for (int p = 0; p < N; ++p) s[p][lc].c[c] = fx_far(s[p][lc].c[c], E);
-}
 // component c of four values held by every lane
 __device__ __forceinline__ double pick4(const double v[4], int c) {
   const double a = c & 1 ? v[1] : v[0], b = c & 1 ? v[3] : v[2];
@@ -124,8 +118,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     const int E = fx_block<NB>(x, f);
 #pragma unroll
     for (int mu = 0; mu < NV; ++mu)
-      s_u[mu][lc].c[c] = fx_near(fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu)), fx_safe(E));
-    if (E > FX_NEAR_MAX) far_comp<NV>(s_u, lc, c, E);
+      s_u[mu][lc].c[c] = fx_out(fx_point<NB>(f, vol_xi(NV, mu), vol_eta(NV, mu)), E);
   }
   const Scalars *sc = get.end();
   if (Sc::FUSED && !sc->active) return;
@@ -265,10 +258,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       for (int l = 0; l < NB; ++l)
         fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w * inv_mass_c(l)), f);
     }
-    double dta = s_cell[0][lc];
-    // extreme fluxes: part of their scale goes to dt / |K|
-    const int far = max(Ee, Ev) < FX_NEAR_MAX ? 0 : max(Ee, Ev) - 1080;
-    if (far != 0) dta *= fx_pow2(far);
+    const double dta = s_cell[0][lc];
     const bool first = first_stage(a, b);   // the first stage skips the zero term and the load of u_n
     bad = bad || Ev >= FX_ENAN;
     double x[NB], xn[NB];
@@ -279,7 +269,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       int E = Ee;
       int64_t r = fx_sum(s[l]);
       if (l > 0) r = fx_add(rv[l], Ev, r, Ee, E);
-      const double d = bad ? NAN : fx_near(r, max(E - far, FX_NEAR_MIN));
+      const double d = fx_nan_if(bad, fx_to(r, E));
       const double L = fma(dta, d, x[l]);
       h[l] = first ? L : fdot2(a, xn[l], b, L);
     }
@@ -305,11 +295,10 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
 #pragma unroll
       for (int vv = 0; vv < 3; ++vv) {
         const int64_t val = fx_point<NB>(f, vert_xi(vv), vert_eta(vv));   // below 11 * 2^58
-        s_u[vv][lc].c[c] = fx_near(val, fx_safe(E));   // this thread's slot; read after the barrier below
+        s_u[vv][lc].c[c] = fx_out(val, E);   // this thread's slot; read after the barrier below
         const Fx v2 = fx_value(val, 2);      // below 2^59.5
         if (live) *reinterpret_cast<int2 *>(vo + vv * VD_STRIDE + c) = make_int2(v2.h, v2.l);
       }
-      if (E > FX_NEAR_MAX) far_comp<3>(s_u, lc, c, E);
     }
     const double jxi[2] = {m.jinv[Kc], m.jinv[nt + Kc]}, jeta[2] = {m.jinv[2 * nt + Kc], m.jinv[3 * nt + Kc]};
     const FxRows J = fx_rows(jxi, jeta);
@@ -401,12 +390,7 @@ __device__ __forceinline__ void stats_tile_fp64(const MeshDev &m, StateDev<doubl
     const uint64_t s = sq + (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)sq, 3);
     if (mu == 0 || s > best) { best = s; b1 = r[mu]; }
   }
-  double d = fx_near((int64_t)top, fx_safe(E)), m1 = fx_near(b1, fx_safe(E));
-  if (E > FX_NEAR_MAX) {
-    d = fx_far(d, E);
-    m1 = fx_far(m1, E);
-  }
-  const double m2 = __shfl_xor_sync(0xffffffffu, m1, 3);
+  const double d = fx_out((int64_t)top, E), m1 = fx_out(b1, E), m2 = __shfl_xor_sync(0xffffffffu, m1, 3);
   // rho, |m|, E, |m1|, |m2|; the lanes of the other components hold 0
   double dr[5] = {c == 0 ? d : 0.0, c == 1 ? root(fdot2(m1, m1, m2, m2)) : 0.0, c == 3 ? d : 0.0, c == 1 ? d : 0.0,
                   c == 2 ? d : 0.0};
@@ -448,7 +432,7 @@ __device__ __noinline__ void boundary_jumps(const MeshDev &m, const Phys &ph, co
   }
   // only squared jumps are taken of these: beyond 2^+-900 infinite or zero either way
   auto get = [&](const double *p, int q, int E) {
-    return xo[q].x >= FX_ENAN ? NAN : fx_near(fx_join(ld_fx(p)), min(max(E, FX_NEAR_MIN), FX_NEAR_MAX));
+    return fx_nan_if(xo[q].x >= FX_ENAN, fx_near(fx_join(ld_fx(p)), min(max(E, FX_NEAR_MIN), FX_NEAR_MAX)));
   };
 #pragma unroll
   for (int q = 0; q < 12; ++q)   // xx, xy, yy: the exponents step as those of the gradient's x and y
@@ -584,7 +568,7 @@ __device__ __forceinline__ void edge_tile_fp64(const MeshDev &m, const Phys &ph,
       fx_mac(t, rs, q);
       fx_mac(t, rp, p);
       // only squared, beyond 2^+-900 to an infinity or zero either way
-      return bad ? NAN : fx_near(fx_sum(t), min(max(E, FX_NEAR_MIN), FX_NEAR_MAX));
+      return fx_nan_if(bad, fx_near(fx_sum(t), min(max(E, FX_NEAR_MIN), FX_NEAR_MAX)));
     };
     double J[K + 1];
 #pragma unroll
@@ -720,9 +704,8 @@ __device__ __forceinline__ void oe_bp_tile_fp64(const MeshDev &m, const Phys &ph
 #pragma unroll
     for (int p = 0; p < NE; ++p) {
       const double sg = gauss_s(NQ, p % NQ);
-      s_u[p][lc].c[c] = fx_near(fx_point<NB>(f, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)), fx_safe(E));
+      s_u[p][lc].c[c] = fx_out(fx_point<NB>(f, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)), E);
     }
-    if (E > FX_NEAR_MAX) far_comp<NE>(s_u, lc, c, E);
   };
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {

@@ -1,7 +1,6 @@
-"""``fx_to`` of ``csrc/dg_fix.cuh`` (plain C++ on the CPU) at the ends of FP64's range: integers of
-any length and sign at exponents from far below the normal numbers to beyond the largest.  The
-result is the nearest number, infinite from 2^1024 - 2^970 up, with the sign; below 2^-1022, where
-it rounds twice, within 2^-1074."""
+"""``fx_to`` of ``csrc/dg_fix.cuh`` (plain C++ on the CPU) up to the end of FP64's range: integers
+of any length and sign at exponents from the smallest that a block's sum has to beyond the
+largest.  The result is the nearest number, infinite from 2^1024 - 2^970 up, with the sign."""
 import math
 import os
 import shutil
@@ -40,9 +39,9 @@ def test_ends_of_the_range(tmp_path):
         bits = int(rng.integers(1, 64))
         r = int(rng.integers(1 << (bits - 1), (1 << bits) - 1, endpoint=True, dtype=np.uint64 if bits > 62 else np.int64))
         top = 2104 - bits   # the exponent at which r reaches 2^1024
-        E = int(rng.choice([top, top - 1, top + 1, top + 500, 58 - bits, 59 - bits, 57 - bits, -400, 64, 1080]))
+        E = int(rng.choice([top, top - 1, top + 1, top + 500, 58, 59, 64, 1080]))
         pairs.append((r if rng.integers(2) else -r, E))
-    pairs += [((1 << 62) + d, E) for d in (-1, 0, 1) for E in (2040, 2041, 2042, -5, -4, -3)] + [(0, -50), (0, 3000)]
+    pairs += [((1 << 62) + d, E) for d in (-1, 0, 1) for E in (2040, 2041, 2042, 58)] + [(0, 58), (0, 3000)]
     out = subprocess.run([str(exe)], input="\n".join(f"{r} {E}" for r, E in pairs) + "\n", capture_output=True,
                          text=True, check=True).stdout.split()
     assert len(out) == len(pairs)
@@ -50,15 +49,11 @@ def test_ends_of_the_range(tmp_path):
     for (r, E), w in zip(pairs, out):
         got, a = float.fromhex(w), abs(r)
         v = F(a) * F(2) ** (E - 1080)
-        if v < F(2) ** -1022:
-            seen.add("small")
-            assert abs(F(abs(got)) - v) <= F(2) ** -1074, (r, E, got)
-            continue
-        elif v >= F(2) ** 1024 - F(2) ** 970:
+        if v >= F(2) ** 1024 - F(2) ** 970:
             want = math.inf
         else:   # halves round up
             ulp = F(math.ulp(float(v))) if float(v) <= v else F(math.ulp(math.nextafter(float(v), 0.0)))
             want = float((v / ulp + F(1, 2)).__floor__() * ulp)
         seen.add("inf" if math.isinf(want) else "normal")
         assert abs(got) == want and (r >= 0 or math.copysign(1.0, got) < 0.0), (r, E, got, want)
-    assert seen == {"small", "inf", "normal"}
+    assert seen == {"inf", "normal"}

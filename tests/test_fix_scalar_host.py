@@ -24,11 +24,14 @@ using namespace dg::sc;
 template <int K, int J> static void order(const double *c) {
   Fx f[SC_NB<K>];
   const int E = sfx_deriv_block<K, J>(c, f);
-  for (int v = 0; v < 3; ++v)
+  for (int v = 0; v < 3; ++v) {
+    double t[J + 1];
+    sfx_derivs<K, J>(f, E, v, t);
     for (int r = 0; r <= J; ++r) {
-      std::printf(" %d %a", E + sc_scale<K, J>(), sfx_deriv<K, J>(f, E, r, v));
+      std::printf(" %d %a", E + sc_scale<K, J>(), t[r]);
       for (int l = 1; l < SC_NB<K>; ++l) std::printf(" %a", psi_rs(l, r, J - r, vert_xi(v), vert_eta(v)));
     }
+  }
 }
 int main() {
   int k;
