@@ -389,10 +389,11 @@ int32_t write_scalars(dg_solver *s, const Scalars *h) {
 const double RK_A[3] = {0.0, 0.75, 1.0 / 3.0}, RK_B[3] = {1.0, 0.25, 2.0 / 3.0};
 const double C_IN[3] = {0.0, 1.0, 0.5}, C_OUT[3] = {1.0, 0.5, 1.0};
 
-// one SSP-RK3 step of the BP RI-OEDG scheme (Sec. 4.5) on the solver's stream;
+// one SSP-RK3 step of the BP RI-OEDG scheme (Sec. 4.5) on a stream;
 // fuse: a small mesh's kernels may finish each other's reductions
-void enqueue_step(dg_solver *s, bool fuse) {
-  const StageCtx &c = s->ctx;
+void enqueue_step(dg_solver *s, bool fuse, cudaStream_t stream) {
+  StageCtx c = s->ctx;
+  c.stream = stream;
   const int oe = s->cfg.oe != DG_OE_OFF, bp = s->cfg.bp != DG_BP_OFF;
   const int64_t ntiles = num_tiles(s->mesh->nt, c.prec);
   if (fuse && num_groups(ntiles) <= FUSE_GROUPS) {
@@ -558,7 +559,7 @@ int32_t dg::solver_init(const dg_mesh *mesh, const dg_config *cfg, const double 
   }
   cudaGraph_t graph = nullptr;
   STRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-  enqueue_step(s, true);
+  enqueue_step(s, true, s->stream);
   e = cudaStreamEndCapture(s->stream, &graph);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&s->step_exec, graph, 0);
   if (graph) cudaGraphDestroy(graph);
@@ -835,12 +836,12 @@ int solver_nb(const dg_solver *s) { return s->nb; }
 void solver_share_order(dg_solver *s, std::mutex *order) { s->order = order; }
 int32_t solver_read_scalars(const dg_solver *s, Scalars *h) { return read_scalars(s, h); }
 int32_t solver_write_scalars(dg_solver *s, const Scalars *h) { return write_scalars(s, h); }
-int32_t solver_capture_step(dg_solver *s, bool fuse, cudaGraph_t *graph) {
+int32_t solver_capture_step(dg_solver *s, bool fuse, cudaStream_t stream, cudaGraph_t *graph) {
   *graph = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return set_error(DG_ECUDA, cudaGetErrorString(e));
-  enqueue_step(s, fuse);
-  e = cudaStreamEndCapture(s->stream, graph);
+  enqueue_step(s, fuse, stream);
+  e = cudaStreamEndCapture(stream, graph);
   if (e != cudaSuccess || !*graph) {
     cudaGetLastError();
     return set_error(DG_ECUDA, "step capture failed");

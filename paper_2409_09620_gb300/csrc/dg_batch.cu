@@ -242,6 +242,7 @@ namespace dg {
 struct BatchCore {
   int prec = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t capture = nullptr;   // step graphs are captured here: a reader may use `stream` meanwhile
   std::mutex order;   // held while a step is enqueued; the owned solves' readers hold it too
   std::vector<dg_solver *> solves;
   std::vector<SolveDev> host_sv;
@@ -264,6 +265,7 @@ struct BatchCore {
   ~BatchCore() {
     if (stream) cudaStreamSynchronize(stream);
     if (exec) cudaGraphExecDestroy(exec);
+    if (capture) cudaStreamDestroy(capture);
     cudaFree(d_sv);
     cudaFree(d_work);
     cudaFree(d_bar);
@@ -272,6 +274,8 @@ struct BatchCore {
   int32_t init(int precision, cudaStream_t s) {
     prec = precision;
     stream = s;
+    if (cudaStreamCreateWithFlags(&capture, cudaStreamNonBlocking) != cudaSuccess)
+      return set_error(DG_ECUDA, "stream creation failed");
     int dev = 0, coop = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -329,16 +333,16 @@ struct BatchCore {
                                          kernel_local_bytes(k_batch_oe_bp<double>)));
   }
 
-  cudaError_t launch_stage(int stage) {
+  cudaError_t launch_stage(int stage, cudaStream_t to) {
     int nsv = (int)host_sv.size(), nw = nwork;
     if (form == 1) {
       void *args[] = {&d_sv, &nsv, &d_work, &nw, &d_bar, &stage};
-      return cudaLaunchCooperativeKernel(fused_kernel(), dim3(grid), dim3(TPB), args, 0, stream);
+      return cudaLaunchCooperativeKernel(fused_kernel(), dim3(grid), dim3(TPB), args, 0, to);
     }
-    if (stage == 0) k_batch_begin<<<(nsv + TPB - 1) / TPB, TPB, 0, stream>>>(d_sv, nsv);
+    if (stage == 0) k_batch_begin<<<(nsv + TPB - 1) / TPB, TPB, 0, to>>>(d_sv, nsv);
     void *args[] = {&d_sv, &d_work, &nw, &stage};
     for (int p = 0; p < 3; ++p) {
-      cudaError_t e = cudaLaunchKernel(phase_kernel(p), dim3(grid_phase[p]), dim3(TPB), args, 0, stream);
+      cudaError_t e = cudaLaunchKernel(phase_kernel(p), dim3(grid_phase[p]), dim3(TPB), args, 0, to);
       if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -435,10 +439,10 @@ struct BatchCore {
     int32_t rc = ensure_stack_limit(stack_bytes());
     if (rc != DG_OK) return rc;
     cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       cudaError_t e = cudaSuccess;
-      for (int st = 0; st < 3 && e == cudaSuccess; ++st) e = launch_stage(st);
-      cudaError_t e2 = cudaStreamEndCapture(stream, &g);
+      for (int st = 0; st < 3 && e == cudaSuccess; ++st) e = launch_stage(st, capture);
+      cudaError_t e2 = cudaStreamEndCapture(capture, &g);
       if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&exec, g, 0) == cudaSuccess)
         graph_ok = true;
       if (g) cudaGraphDestroy(g);
@@ -465,7 +469,7 @@ struct BatchCore {
     const bool fuse = tiles <= (int64_t)num_sms * (prec == DG_PREC_MIXED ? 4 : 8);
     for (dg_solver *sv_ : solves) {
       cudaGraph_t child = nullptr;
-      if ((rc = solver_capture_step(sv_, fuse, &child)) != DG_OK) break;
+      if ((rc = solver_capture_step(sv_, fuse, capture, &child)) != DG_OK) break;
       cudaGraphNode_t node;
       const cudaError_t e = cudaGraphAddChildGraphNode(&node, g, nullptr, 0, child);
       cudaGraphDestroy(child);
@@ -490,7 +494,7 @@ struct BatchCore {
         if (cudaGraphLaunch(exec, stream) != cudaSuccess) return set_error(DG_ECUDA, "batch graph launch");
       } else {
         for (int st = 0; st < 3; ++st) {
-          cudaError_t e = launch_stage(st);
+          cudaError_t e = launch_stage(st, stream);
           if (e != cudaSuccess) return set_error(DG_ECUDA, cudaGetErrorString(e));
         }
       }

@@ -75,9 +75,9 @@ int solver_nb(const dg_solver *s);
 void solver_share_order(dg_solver *s, std::mutex *order);
 int32_t solver_read_scalars(const dg_solver *s, Scalars *h);
 int32_t solver_write_scalars(dg_solver *s, const Scalars *h);
-// one SSP-RK3 step of the solver (the kernels of its own step graph) captured
+// one SSP-RK3 step of the solver (the kernels of its own step graph) captured on `stream`
 // into a new graph, which the caller destroys
-int32_t solver_capture_step(dg_solver *s, bool fuse, cudaGraph_t *graph);
+int32_t solver_capture_step(dg_solver *s, bool fuse, cudaStream_t stream, cudaGraph_t *graph);
 
 // the mesh's device arrays as the kernels see them; boundary tags usable by
 // the scalar solver (dg_api.cu)

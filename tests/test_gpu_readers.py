@@ -103,3 +103,22 @@ def test_readers_beside_a_batch(prec, n, k, form):
         for i in range(2):
             assert np.array_equal(b.solver(i).get_state()[0], steps[-1])
     _beside(b.solver(1), {u.tobytes() for u in steps}, write, 6)
+
+
+@pytest.mark.parametrize("prec", [N.PREC_MIXED, N.PREC_FP64])
+def test_readers_beside_set_shape(prec):
+    """The step graphs are captured while the readers' copies go on."""
+    mesh, cfg, u0 = _setup(prec, 23, 2)
+    b = N.Batch([mesh, mesh], [cfg, cfg], [u0, u0])
+    start = b.solver(1).get_state()[0].tobytes()
+    s = N.Solver(mesh, cfg, u0)
+    s.advance(math.inf, max_steps=3)
+
+    def write():
+        for form in (0, 3, 1):
+            b.set_shape(128, 2, form)
+    _beside(b.solver(1), {start}, write, 30)
+    for form in (0, 3, 1):
+        b.set_shape(128, 2, form)
+        b.advance(max_steps=1)
+    assert np.array_equal(b.solver(1).get_state()[0], s.get_state()[0])
