@@ -729,9 +729,12 @@ extern "C" int32_t dg_batch_autotune(dg_batch *b, int32_t steps, int32_t *best_c
     StateBuf un, uh, us;
     solver_states(s, &un, &uh, &us);
     const Snap &q = snaps[i];
-    cudaMemcpyAsync(un.avg, q.avg, q.navg, cudaMemcpyDeviceToDevice, core.stream);
-    cudaMemcpyAsync(un.hi, q.hi, q.nhi, cudaMemcpyDeviceToDevice, core.stream);
-    if (q.ntr) cudaMemcpyAsync(solver_ctx(s).tr, q.tr, q.ntr, cudaMemcpyDeviceToDevice, core.stream);
+    {
+      std::lock_guard<std::mutex> lock(core.order);   // averages and modes at once, for a reader on another thread
+      cudaMemcpyAsync(un.avg, q.avg, q.navg, cudaMemcpyDeviceToDevice, core.stream);
+      cudaMemcpyAsync(un.hi, q.hi, q.nhi, cudaMemcpyDeviceToDevice, core.stream);
+      if (q.ntr) cudaMemcpyAsync(solver_ctx(s).tr, q.tr, q.ntr, cudaMemcpyDeviceToDevice, core.stream);
+    }
     if (solver_write_scalars(s, &q.sc) != DG_OK) { free_snaps(); return DG_ECUDA; }
   }
   free_snaps();

@@ -122,3 +122,21 @@ def test_readers_beside_set_shape(prec):
         b.set_shape(128, 2, form)
         b.advance(max_steps=1)
     assert np.array_equal(b.solver(1).get_state()[0], s.get_state()[0])
+
+
+@pytest.mark.parametrize("prec", [N.PREC_MIXED, N.PREC_FP64])
+def test_readers_beside_autotune(prec):
+    """The tuning steps (at most 400 states) and the restored start."""
+    mesh, cfg, u0 = _setup(prec, 12, 1)
+    s = N.Solver(mesh, cfg, u0)
+    allowed = {s.get_state()[0].tobytes()}
+    for _ in range(400):
+        s.advance(math.inf, max_steps=1)
+        allowed.add(s.get_state()[0].tobytes())
+    b = N.Batch([mesh, mesh], [cfg, cfg], [u0, u0])
+    start = b.solver(1).get_state()[0].tobytes()
+
+    def write():
+        b.autotune(steps=1)
+        assert b.solver(1).get_state()[0].tobytes() == start
+    _beside(b.solver(1), allowed, write, 3)
