@@ -99,6 +99,18 @@ FX_CONST FxC fxc(double c) {
   return FxC{(int)h, (int)(v - h * (1LL << FX_LIMB))};
 }
 
+// the constant c f with one rounding, f of a few bits (a product in FP64 would round by up to
+// 2^-53 of it first, the same in every cell and step): c split into halves of 26 bits (Dekker 1971)
+FX_CONST FxC fxc(double c, double f) {
+  const double t = c * 134217729.0, ch = t - (t - c), cl = c - ch, one = double(1LL << FX_ONE);
+  const double s1 = ch * f * one, s2 = cl * f * one;   // exact
+  const int64_t i = (int64_t)s1;
+  const double r = (s1 - double(i)) + s2;
+  const int64_t v = i + (int64_t)(r < 0.0 ? r - 0.5 : r + 0.5);
+  const int64_t h = (v + (1LL << (FX_LIMB - 1))) >> FX_LIMB;
+  return FxC{(int)h, (int)(v - h * (1LL << FX_LIMB))};
+}
+
 // exponent of a block from the bitwise-positive high words of its values
 FX_HD int fx_abs_hi(double x) { return fx_hiword(x) & 0x7fffffff; }
 FX_HD int fx_exp(int max_abs_hi) {
@@ -169,13 +181,18 @@ template <int S>
 FX_HD Fx fx_jump(Fx a, int Ea, Fx b, int Eb, int E) {
   return fx_value(fx_diff(a, Ea, b, Eb, E), S);
 }
+// r 2^-s to nearest, |r| < 2^62, s >= 0
+FX_HD int64_t fx_shift(int64_t r, int s) {
+  s = s < 63 ? s : 63;
+  return (r + (int64_t)((1ULL << s) >> 1)) >> s;
+}
+// the sum's last unit is rounded down, from FxAcc{0, FX_HALF} on to nearest
+constexpr int64_t FX_HALF = 1LL << (FX_ONE - FX_LIMB - 1);
 FX_HD int64_t fx_sum(const FxAcc &s) {
   return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + (s.b >> (FX_ONE - FX_LIMB));
 }
-// the same with the sum's last unit rounded to nearest instead of down
-FX_HD int64_t fx_round(const FxAcc &s) {
-  return s.a * (1LL << (2 * FX_LIMB - FX_ONE)) + ((s.b + (1LL << (FX_ONE - FX_LIMB - 1))) >> (FX_ONE - FX_LIMB));
-}
+// the same rounded to nearest
+FX_HD int64_t fx_round(const FxAcc &s) { return fx_sum(FxAcc{s.a, s.b + FX_HALF}); }
 // sum of products with run-time coefficients, l l included (their low limbs reach
 // 2^29, so that dropping it costs up to 4 units of the result per term), and rounded
 struct FxAccL {
@@ -205,11 +222,10 @@ FX_HD double fx_convert(int64_t r, int E) {
 }
 FX_HD double fx_near(int64_t r, int E) { return fx_convert<false>(r, E); }
 FX_HD double fx_to(int64_t r, int E) { return fx_convert<true>(r, E); }
-// r1 2^(E1 - 1080) + r2 2^(E2 - 1080) as r 2^(E - 1080)
+// r1 2^(E1 - 1080) + r2 2^(E2 - 1080) as r 2^(E - 1080), each rounded to nearest
 FX_HD int64_t fx_add(int64_t r1, int E1, int64_t r2, int E2, int &E) {
   E = (E1 > E2 ? E1 : E2) + 1;
-  const int s1 = E - E1, s2 = E - E2;
-  return (r1 >> (s1 > 63 ? 63 : s1)) + (r2 >> (s2 > 63 ? 63 : s2));
+  return fx_shift(r1, E - E1) + fx_shift(r2, E - E2);
 }
 
 // |r| as an integer; the top 62 bits of values whose largest is top (left shift, if negative right)

@@ -206,7 +206,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     bad = bad || max(Eu, Ef) >= FX_ENAN || (fx_abs_hi(al) >> 20) >= FX_ENAN;
 #pragma unroll
     for (int nu = 0; nu < NQ; ++nu) {
-      FxAcc y{0, 0};
+      FxAcc y{0, FX_HALF};
       fx_mac(y, cf, fx_from(fm[nu], Ef) - fx_from(fn[nu], Ef));
       fx_mac(y, cu, fx_from(um[nu], Eu) - fx_from(up[nu], Eu));
       s_y[i * NQ + nu][threadIdx.x] = fx_sum(y);   // below 2^60
@@ -215,7 +215,9 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   __syncthreads();
   // ---- quadrature sums, mass inverse, SSP-RK combination ---------------------------
   // volume |K| sum_mu w_mu F . grad Psi_l, edges - sum_i l_i sum_nu w_nu Fhat Psi_l, both with
-  // the mass inverse (and the 1/2 of the LF flux) on their coefficients
+  // the mass inverse (and the 1/2 of the LF flux) on their coefficients.  Every sum and shift to
+  // nearest: rounded down, each stage had the same bias of about 2^-56 in every cell, and the
+  // error against 64 bits grew (forward facing step, 48 stages: 8.6e-16, now 7.6e-16).
   double h[NB];
   {
     int64_t rv[NB];
@@ -232,15 +234,15 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
       Ev = fx_exp(mx);
       FxAcc s[NB];
 #pragma unroll
-      for (int l = 1; l < NB; ++l) s[l] = FxAcc{0, 0};
+      for (int l = 1; l < NB; ++l) s[l] = FxAcc{0, FX_HALF};
 #pragma unroll
       for (int mu = 0; mu < NV; ++mu) {
         const double xi = vol_xi(NV, mu), eta = vol_eta(NV, mu), w = vol_w(NV, mu);
         const Fx f1 = fx_from(g1[mu], Ev), f2 = fx_from(g2[mu], Ev);
 #pragma unroll
         for (int l = 1; l < NB; ++l) {
-          fx_mac(s[l], fxc(w * psi_x(l, xi, eta) * inv_mass_c(l)), f1);
-          fx_mac(s[l], fxc(w * psi_y(l, xi, eta) * inv_mass_c(l)), f2);
+          fx_mac(s[l], fxc(w * psi_x(l, xi, eta), inv_mass_c(l)), f1);
+          fx_mac(s[l], fxc(w * psi_y(l, xi, eta), inv_mass_c(l)), f2);
         }
       }
 #pragma unroll
@@ -249,14 +251,14 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
     const int Ee = max(max(max(ei[0], ei[1]), ei[2]) + 2, FX_NEAR_MIN);
     FxAcc s[NB];
 #pragma unroll
-    for (int l = 0; l < NB; ++l) s[l] = FxAcc{0, 0};
+    for (int l = 0; l < NB; ++l) s[l] = FxAcc{0, FX_HALF};
 #pragma unroll
     for (int p = 0; p < 3 * NQ; ++p) {
       const double sg = gauss_s(NQ, p % NQ), w = 0.5 * gauss_w(NQ, p % NQ);
-      const Fx f = fx_value(s_y[p][threadIdx.x], min(Ee - ei[p / NQ], 63));
+      const Fx f = fx_value(fx_shift(s_y[p][threadIdx.x], Ee - ei[p / NQ]), 0);
 #pragma unroll
       for (int l = 0; l < NB; ++l)
-        fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w * inv_mass_c(l)), f);
+        fx_mac(s[l], fxc(-psi(l, edge_xi(p / NQ, sg), edge_eta(p / NQ, sg)) * w, inv_mass_c(l)), f);
     }
     const double dta = s_cell[0][lc];
     const bool first = first_stage(a, b);   // the first stage skips the zero term and the load of u_n
