@@ -59,10 +59,10 @@ ALGO_FLOPS_P2 = {"rk": 331.0, "stats": 194.0, "oe_bp": 324.0}
 # FP64 flops per cell-stage the hardware executed for the same kernels (2 DFMA +
 # DMUL + DADD from ncu captures / cells, first stage of a step); sums and products are DFMAs
 # too, division, square root and exp expand into DFMA sequences.
-EXECUTED_FLOPS_P2 = {"rk": 586.3, "stats": 502.7, "oe_bp": 732.5}
+EXECUTED_FLOPS_P2 = {"rk": 604.0, "stats": 471.8, "oe_bp": 762.0}
 # DRAM bytes (read + write) per launch, from ncu captures per cell (k_rk: mean of
 # its three stages)
-TRAFFIC_PER_LAUNCH = {"rk": 1.649e9, "stats": 1.047e9, "oe_bp": 1.190e9}
+TRAFFIC_PER_LAUNCH = {"rk": 1.648e9, "stats": 1.189e9, "oe_bp": 1.194e9}
 # Mixed form (P2, FP32 modes 1-5 and FP64 averages: S = 4 x 8 + 4 x 5 x 4 =
 # 112 B of state per cell).  Algorithmic HBM bytes per cell-stage of the
 # method's three passes, each array element moved once and neighbour data

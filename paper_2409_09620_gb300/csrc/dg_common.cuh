@@ -728,12 +728,12 @@ __device__ __forceinline__ void step_begin_thread(Scalars *sc) {
 // block of the consuming kernel takes the reduction itself, in the order of the
 // finalize kernels, into a copy of the scalars in its shared memory, and one block
 // more, without a tile, writes them back.  No field that a block of the same launch reads from
-// memory for its result is written in that launch.  Per step: vortex, 2,048 P1
-// cells FP64, 127 -> 104 us; Riemann problem, 1,058 P2 cells mixed, 118 -> 90 us.
-// The limit: P2 FP64, 2 groups (7,688 cells) 178 -> 166 us, 4 groups 229 -> 243 us;
-// mixed, 2 groups (31,250 cells) 125 -> 116 us, 4 groups 144 -> 161 us.  The
-// kernels have a variant for it: chosen at run time it cost the mixed form's
-// large meshes 1.5 %.
+// memory for its result is written in that launch.  Vortex, 2,048 P1 cells FP64: 92 us per
+// step; Riemann problem, 1,058 P2 cells mixed: 78 us; with finalize launches 127 and 118.
+// The limit, separate and fused: P2 FP64, 2 groups (7,688 cells) 178 and 166 us, 4 groups
+// 229 and 243 us; mixed, 2 groups (31,250 cells) 125 and 116 us, 4 groups 144 and 161 us.
+// The kernels have a variant for it: chosen at run time it cost the mixed form's large
+// meshes 1.5 %.
 constexpr int FUSE_GROUPS = 2;
 struct Fuse {
   int on;                   // which kernel to launch: the one that finishes the reduction itself
@@ -746,9 +746,7 @@ struct Fuse {
 // Where a tile function gets its scalars: begin() starts the loads, end() returns
 // them (every thread of the block calls both).  In between go the tile's own
 // loads and whatever work needs no scalar, so that the latency of the
-// reduction and that of the state overlap: with one write-back block and the
-// normalisers one per thread, us per step, 2,048 P1 cells FP64 100 -> 94, 1,058 P2
-// cells mixed 85 -> 80, 20,000 P2 cells mixed 104 -> 98.
+// reduction and that of the state overlap (5 to 6 % of a small mesh's step).
 struct PlainScalars {
   static constexpr bool FUSED = false;
   const Scalars *sc;

@@ -22,7 +22,7 @@
 // sums with constant coefficients are taken in block fixed point on the integer
 // units (dg_fix.cuh) and the rest in register-only DFMAs (dg_common.cuh).
 // Measured, with every sum on the FP64 pipe before: Burgers P3, 51,200 cells,
-// 0.598 -> 0.327 ms per step; linear P2, 204,800 cells, 1.06 -> 0.60 ms.
+// 0.598 -> 0.296 ms per step; linear P2, 204,800 cells, 1.06 -> 0.60 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

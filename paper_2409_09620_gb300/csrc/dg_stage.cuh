@@ -24,11 +24,10 @@ namespace dg {
 // occupancy hides the latency of the neighbour gathers and of the FP64 pipe
 // until the spills cost more, which for the fewer modes of P1 happens later.
 // 1,036,800 cells, ms per launch:
-//   FP64  k_rk     P2 0.900 with 7 blocks, 0.903 with 8, 0.956 with 9, 1.05 with 10;
-//                  P1 0.407 with 9, 0.406 with 10, 0.421 with 12
-//         k_stats  P2 0.575 with 8, 0.548 with 10, 0.561 with 12, 0.72 with 14;
-//                  P1 0.417 with 8, 0.384 with 10, 0.373 with 12, 0.392 with 14
-//         k_oe_bp  the same from 5 to 10
+//   FP64  k_rk     P2 0.911 with 7 blocks, 0.916 with 8, 0.955 with 9; P1 the same from 9 to 12
+//         k_stats  P2 0.601 with 8, 0.592 with 10, 0.610 with 12; P1 0.406 with 10, 0.401 with
+//                  12, 0.434 with 14
+//         k_oe_bp  P2 0.711 with 6, 0.714 with 8, 0.720 with 10; P1 0.465, 0.450 and 0.454
 //   mixed k_rk     P2 0.181 with 3 blocks, 0.157 with 4, 0.166 with 5;
 //                  P1 0.136 with 4, 0.112 with 6, 0.105 with 7, 0.103 with 8, 0.106 with 9;
 //                  259,200 cells 0.0380 with 4, 0.0330 with 6, 0.0337 with 7, 0.0347 with 8

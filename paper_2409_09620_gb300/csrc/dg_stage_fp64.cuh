@@ -19,21 +19,10 @@
 //
 // Threads beyond the last cell repeat the last cell and store nothing.
 //
-// Measured against one thread per cell with every sum on the FP64 pipe: double
-// Mach reflection, 1,036,800 P2 cells, ms per launch: k_rk 2.37 -> 1.50,
-// k_stats 0.96 -> 1.05, k_oe_bp 1.39 -> 0.90, step 14.16 -> 10.38; isentropic
-// vortex, 2,048 P1 cells, step 250 -> 135 us.  Sums, products, reciprocals and
-// square roots as register-only DFMAs (dg_common.cuh): k_rk 1.50 -> 1.41,
-// k_stats 1.05 -> 0.91, k_oe_bp 0.90 -> 0.81, step 10.38 -> 9.42.  LF terms and
-// vertex derivatives of k_rk in fixed point, no 64-bit conversion or comparison
-// left on the FP64 pipe: k_rk 1.41 -> 1.09, k_stats 0.91 -> 0.82, k_oe_bp
-// 0.81 -> 0.69, step 9.42 -> 7.81.  OE jumps in fixed point from limb records, no
-// negated doubles (each an FP64 operation): k_rk 1.09 -> 0.97, k_stats
-// 0.82 -> 0.58, step 7.81 -> 6.71.  Products of a cell or an edge (dt / |K|,
-// alpha l_i, |K| J^-1) and the block sums of k_rk dealt out one per lane: 33 of
-// its 306 FP64 operations per tile less, k_rk 0.97 -> 0.94 (P1 0.51 -> 0.47), step
-// 6.71 -> 6.61 (P1 4.08 -> 3.98).  Blocks per SM by degree (dg_stage.cuh): step 6.53
-// (P1 3.81); the edges of k_rk in a loop: 6.43 (P1 3.66).
+// 1,036,800 P2 cells (double Mach reflection), ms per launch, against one thread per cell
+// with every sum on the FP64 pipe: k_rk 2.37 -> 0.91, k_stats 0.96 -> 0.59, k_oe_bp 1.39 ->
+// 0.71, step 14.2 -> 6.67; 460,800 P1 cells: 0.468 -> 0.200, 0.273 -> 0.200,
+// 0.370 -> 0.210.  The errors against 64 bits are those of the FMA chains (vortex 1.54e-15, DMR 3.6e-16, forward facing step 7.6e-16).
 #pragma once
 
 namespace dg {
@@ -152,7 +141,7 @@ __device__ __forceinline__ void rk_tile_fp64(const MeshDev &m, const Phys &ph, S
   // One edge after another in a loop, its values in shared memory: unrolled, the
   // kernel was 67 KB of straight-line code that waited for instructions more than
   // for anything else (28 % of the stalls, P2), and held 9 sums in registers.
-  // 1,036,800 cells: P2 0.94 -> 0.90 ms, P1 0.457 -> 0.406 ms.
+  // A loop gave 4 % of k_rk in P2 and 11 % in P1.
   auto &s_y = sh.y;   // this thread's, in its own column
   int ei[3] = {0, 0, 0};
   bool bad = false;
